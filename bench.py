@@ -134,7 +134,7 @@ def walk_source_hash() -> str:
     import re
 
     h = hashlib.sha256()
-    for f in ("qcs_walk.cu", "qcs_internal.h"):
+    for f in ("qcs_walk.cu", "qcs_engine4.cu", "qcs_device.cuh", "qcs_internal.h"):
         with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_1606_07413_gb300", "csrc", f)) as fh:
             text = fh.read()
         if f == "qcs_internal.h":

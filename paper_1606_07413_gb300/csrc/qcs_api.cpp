@@ -100,8 +100,12 @@ LevelCtx qcs::make_level(const qcs_problem *P, int k, uint32_t version, int dp_b
     lv.C32 = P->dC32;
     lv.Cq = reinterpret_cast<const uint4 *>(P->dCq);
     lv.Cm = reinterpret_cast<const uint4 *>(P->dCm);
+    lv.Csum = P->dCm ? reinterpret_cast<const int16_t *>(P->dCm + (size_t)P->D * P->D / 2) : nullptr;
     lv.U = P->dU;
-    for (int side = 0; side < 2; side++) lv.T1[side] = P->dT1[side];
+    for (int side = 0; side < 2; side++) {
+        lv.T1[side] = P->dT1[side];
+        lv.T4[side] = reinterpret_cast<const uint4 *>(P->dT4[side]);
+    }
     lv.coef = P->dCoef;
     lv.n = P->n;
     lv.k = k;
@@ -148,11 +152,11 @@ void host_adj_stage(int n, uint32_t p, bool adj_of_transpose, std::vector<uint32
 }
 
 std::mutex g_tab_mu;
-std::map<std::pair<int, int>, std::array<uint32_t *, 2>> g_tabs; // (device, n) -> T1v, T1w
+std::map<std::pair<int, int>, std::array<uint32_t *, 4>> g_tabs; // (device, n) -> T1v, T1w, T4v, T4w
 
 } // namespace
 
-int qcs::stage_tables(int n, const uint32_t *t1[2], int64_t *uploaded)
+int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64_t *uploaded)
 {
     int dev = 0;
     CK(cudaGetDevice(&dev));
@@ -165,7 +169,13 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], int64_t *uploaded)
             u0a[i] = (uint32_t)smix_host(kSeedU + (2ull * i + 1) * kGamma) & 0xFFFFu;
             u0b[i] = (uint32_t)smix_host(kSeedU + (2ull * i + 2) * kGamma) & 0xFFFFu;
         }
-        std::array<uint32_t *, 2> tabs{nullptr, nullptr};
+        std::array<uint32_t *, 4> tabs{nullptr, nullptr, nullptr, nullptr};
+        auto upload = [&](uint32_t **d, const std::vector<uint32_t> &h) {
+            cudaError_t e = cudaMalloc(d, sizeof(uint32_t) * h.size());
+            if (e == cudaSuccess) e = cudaMemcpy(*d, h.data(), sizeof(uint32_t) * h.size(), cudaMemcpyHostToDevice);
+            if (uploaded) *uploaded += (int64_t)(sizeof(uint32_t) * h.size());
+            return e;
+        };
         for (int side = 0; side < 2; side++) {
             std::vector<uint32_t> t1((size_t)xi * D);
             for (uint32_t qa = 1; qa <= xi; qa++) {
@@ -173,14 +183,26 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], int64_t *uploaded)
                 host_adj_stage(n, qa, side == 1, ua, ub);
                 for (uint32_t j = 0; j < D; j++) t1[(size_t)(qa - 1) * D + j] = ua[j] | (ub[j] << 16);
             }
-            CK(cudaMalloc(&tabs[side], sizeof(uint32_t) * t1.size()));
-            CK(cudaMemcpy(tabs[side], t1.data(), sizeof(uint32_t) * t1.size(), cudaMemcpyHostToDevice));
-            if (uploaded) *uploaded += (int64_t)(sizeof(uint32_t) * t1.size());
+            CK(upload(&tabs[side], t1));
+            if (n == 4) {
+                // the Pauli of code t << 5 | l is row4(l, t)
+                std::vector<uint32_t> t4v((size_t)D * D);
+                for (uint32_t code = 0; code < D; code++) {
+                    const uint32_t q = row4(code & 31, code >> 5);
+                    for (uint32_t i = 0; i < D; i++) {
+                        const uint32_t j = row4(i >> 3, i & 7);
+                        t4v[(size_t)code * D + i] = q ? t1[(size_t)(q - 1) * D + j] : (u0a[j] | u0b[j] << 16);
+                    }
+                }
+                CK(upload(&tabs[2 + side], t4v));
+            }
         }
         it = g_tabs.emplace(std::make_pair(dev, n), tabs).first;
     }
     t1[0] = it->second[0];
     t1[1] = it->second[1];
+    t4[0] = it->second[2];
+    t4[1] = it->second[3];
     return QCS_OK;
 }
 
@@ -249,31 +271,34 @@ int upload_problem(qcs_problem *P)
                             cq[o + 1] = wb;
                         }
             if (n == 4) {
-                // the tensor-core layout (LevelCtx::Cm): biased bytes, K-blocks of 16 rows
-                cm.assign((size_t)D * 2 * D / 4, 0);
-                // K index k = part * 256 + 8 l + t holds row 32 t + l of the a-part
-                // (part 0) or b-part (part 1): the eight rows one lane of the
-                // walk kernel holds form one K chunk of eight
-                auto entry = [&](int k, int col) -> uint32_t {
-                    const int kk = k & (D - 1), row = (kk % 8) * 32 + kk / 8;
-                    const size_t src = (size_t)row * D + col;
-                    return (uint32_t)(uint8_t)((k < D ? P->C.a[src] : P->C.b[src]) + 128);
-                };
-                for (int col = 0; col < D; col++)
-                    for (int kb = 0; kb < 2 * D / 16; kb++)
-                        for (int q = 0; q < 4; q++) {
-                            const int k0 = 16 * kb + 2 * q;
-                            const uint32_t w = entry(k0, col) | entry(k0 + 1, col) << 8 | entry(k0 + 8, col) << 16 |
-                                               entry(k0 + 9, col) << 24;
-                            const int chunk = (4 * (kb / 4) + q) ^ (4 * (col & 1));
-                            cm[(size_t)col * 128 + (size_t)chunk * 4 + (kb % 4)] = w;
-                        }
+                // the engine's layout (LevelCtx::Cm, Csum): biased bytes by
+                // column, then each column's sum, if the sums suit its f32
+                // accumulation
+                cm.assign((size_t)D * D / 2 + (size_t)D / 2, 0);
+                uint8_t *bytes = reinterpret_cast<uint8_t *>(cm.data());
+                int16_t *sums = reinterpret_cast<int16_t *>(cm.data() + (size_t)D * D / 2);
+                int64_t most = 0;
+                for (int Q = 0; Q < D; Q++) {
+                    int64_t sum = 0, abs_sum = 0;
+                    for (int i = 0; i < D; i++) {
+                        const uint32_t j = row4((uint32_t)i >> 3, (uint32_t)i & 7);
+                        const int64_t a = P->C.a[(size_t)j * D + Q], b = P->C.b[(size_t)j * D + Q];
+                        bytes[(size_t)Q * 2 * D + i] = (uint8_t)(a + 128);
+                        bytes[(size_t)Q * 2 * D + D + i] = (uint8_t)(b + 128);
+                        if (j == 0) continue; // the identity's row is not part of the product
+                        sum += a + b;
+                        abs_sum += std::abs(a) + std::abs(b);
+                    }
+                    sums[Q] = (int16_t)sum;
+                    most = std::max(most, abs_sum);
+                }
+                if (most > kMaxColumnSum) cm.clear();
             }
         }
     }
     CK(cudaGetDevice(&P->device));
     int64_t h2d = 0;
-    if (int rc = stage_tables(n, P->dT1, &h2d)) return rc;
+    if (int rc = stage_tables(n, P->dT1, P->dT4, &h2d)) return rc;
     if (!cq.empty()) {
         CK(cudaMalloc(&P->dCq, sizeof(uint32_t) * cq.size()));
         CK(cudaMemcpy(P->dCq, cq.data(), sizeof(uint32_t) * cq.size(), cudaMemcpyHostToDevice));

@@ -1,0 +1,140 @@
+// qcs_device.cuh -- device functions shared by the kernels of qcs_walk.cu and
+// qcs_engine4.cu: the hash finaliser, the state's decoding, trail starts and
+// references, and the distinguished-point table's insert.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "qcs_internal.h"
+
+namespace qcs {
+namespace {
+
+__device__ __forceinline__ uint64_t smix(uint64_t z)
+{
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
+// smix(base ^ phi) for phi < 2^30, given pre = base ^ (base >> 30): the
+// first xorshift of the finaliser cannot see phi (it shifts by 30), so
+// (base ^ phi) ^ ((base ^ phi) >> 30) = pre ^ phi, and the rest follows.
+// The same value as smix(base ^ phi), one 64-bit xorshift cheaper per column.
+__device__ __forceinline__ uint64_t smix_pre(uint64_t pre, uint32_t phi)
+{
+    uint64_t z = (pre ^ (uint64_t)phi) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
+__device__ __forceinline__ uint32_t shl32(uint32_t v, int s) { return s >= 32 ? 0u : v << s; }
+
+struct Decoded {
+    int side;
+    uint64_t qpack; // q_1 .. q_h, 8 bits each (q <= 255)
+};
+
+// mu (Sec. 2, the state is a concatenation of per-rotation codes): bit 0 is
+// the side; rotation j reads the ell-bit field at bit 1 + ell j and maps its
+// value v onto the xi non-identity Paulis as q_j = floor(v xi / 2^ell) + 1.
+__device__ __forceinline__ Decoded decode(uint64_t x, const LevelCtx &lv)
+{
+    Decoded d;
+    d.side = (int)(x & 1);
+    d.qpack = 0;
+    uint64_t f = x >> 1;
+    for (int j = 0; j < lv.h; j++) {
+        const uint32_t v = (uint32_t)f & lv.fmask;
+        d.qpack |= (uint64_t)(((v * lv.xi) >> lv.ell) + 1) << (8 * j);
+        f >>= lv.ell;
+    }
+    return d;
+}
+
+// starting state and chunk of trail (walk, seq) in the current version
+__device__ __forceinline__ uint64_t trail_start(const LevelCtx &lv, uint32_t walk, uint32_t seq)
+{
+    seq &= (1u << kRefSeqBits) - 1;
+    return smix(lv.seed ^ smix(((uint64_t)walk << 32) | seq) ^ ((uint64_t)lv.version << 40)) & lv.maskL;
+}
+__device__ __forceinline__ uint32_t trail_chunk(const LevelCtx &lv, uint64_t start)
+{
+    return lv.n_chunks ? 1u + (uint32_t)(smix(start ^ 0x5851F42D4C957F2Dull) % (uint64_t)lv.n_chunks) : 0u;
+}
+__device__ __forceinline__ uint64_t make_ref(uint32_t walk, uint32_t seq, uint32_t len)
+{
+    return (uint64_t)walk | ((uint64_t)(seq & ((1u << kRefSeqBits) - 1)) << kRefWalkBits) |
+           ((uint64_t)len << (kRefWalkBits + kRefSeqBits));
+}
+__device__ __forceinline__ void split_ref(uint64_t ref, uint32_t &walk, uint32_t &seq, uint32_t &len)
+{
+    walk = (uint32_t)(ref & ((1u << kRefWalkBits) - 1));
+    seq = (uint32_t)((ref >> kRefWalkBits) & ((1u << kRefSeqBits) - 1));
+    len = (uint32_t)(ref >> (kRefWalkBits + kRefSeqBits));
+}
+
+__device__ __forceinline__ void new_trail(WalkState &st, uint32_t walk, const LevelCtx &lv)
+{
+    st.seq++;
+    st.start = trail_start(lv, walk, st.seq);
+    st.cur = st.start;
+    st.len = 0;
+    st.chunk = trail_chunk(lv, st.start);
+}
+
+// per-walk-group tallies, added to the job's counters by the group's first
+// lane (the tensor-core kernel keeps them in 32 bits and flushes them before
+// they could overflow)
+template <typename T>
+struct TallyOf {
+    T steps = 0, w = 0, dp = 0, ab = 0, evicted = 0, duplicate = 0, pairs = 0;
+};
+using Tally = TallyOf<unsigned long long>;
+
+// Store the distinguished point (Sec. 3: the triple start, end, length) in
+// the slot its value hashes to, keeping the newest trail there (one 128-bit
+// atomic exchange, never a wait).  If the slot held the same point from
+// another trail the two trails merged: queue them for the re-walk.
+template <typename WL, typename T>
+__device__ void dp_insert(const WL &w, uint64_t dp, uint64_t ref, TallyOf<T> &c)
+{
+    if (w.outbox) {
+        // DP-owner sharding: the point goes to its owner's table after the exchange
+        const uint32_t idx = atomicAdd(w.ohead, 1u);
+        if (idx < w.ocap) {
+            Slot o;
+            o.key = dp;
+            o.ref = ref;
+            w.outbox[idx] = o;
+        }
+        return;
+    }
+    Slot nv;
+    nv.key = dp;
+    nv.ref = ref;
+    Slot *s = &w.table[smix(dp) & w.table_mask];
+    const Slot old = atomicExch(s, nv);
+    if (old.key == dp) {
+        if (old.ref == ref) {
+            c.duplicate++;
+            return;
+        }
+        c.pairs++;
+        const uint32_t idx = atomicAdd(w.qhead, 1u);
+        if (idx < w.qcap) {
+            Pair p;
+            p.ref_a = old.ref;
+            p.ref_b = ref;
+            p.dp = dp;
+            w.queue[idx] = p;
+        }
+    } else if (old.key != kEmptyKey) {
+        c.evicted++;
+    }
+}
+
+} // namespace
+} // namespace qcs

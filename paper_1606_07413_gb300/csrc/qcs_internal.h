@@ -28,6 +28,20 @@ constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
 constexpr uint64_t kSeedU = 0x6A09E667F3BCC908ull;
 constexpr uint64_t kSeedH = 0xBB67AE8584CAA73Bull;
 
+// The n = 4 engine's rows (qcs_engine4.cu): lane l (5 bits: z0 z1 z2 x0 x1 of
+// the row's Pauli index) and t (3 bits: z3 x3 x2) to the row, and a Pauli
+// index to its code, the same eight bits in that order (t above l).
+constexpr uint32_t row4(uint32_t l, uint32_t t)
+{
+    return (l & 7u) | (t & 1u) << 3 | ((l >> 3) & 3u) << 4 | ((t >> 2) & 1u) << 6 | ((t >> 1) & 1u) << 7;
+}
+// A column of C^ suits the engine's f32 sums when the absolute values of its
+// entries add up to at most this: a partial sum of the product is below
+// (1279 + 1024) * 1821 < 2^22 (weights up to 1024 + 255, and the offset's
+// correction).  By orthogonality a column's squares a^2 + 2 b^2 add up to
+// 2^E, so the sum is at most 16 sqrt(1.5 * 2^E), 1773 at E = 13.
+constexpr int kMaxColumnSum = 1821;
+
 // Everything a warp needs to evaluate one step f of the walk at one level.
 struct LevelCtx {
     // C^ numerators mod 2^32 as (a, b), 4^n x 4^n.  With W = lanes_per_walk(n)
@@ -40,15 +54,16 @@ struct LevelCtx {
     // Q0 = sub + 2 W j and Q1 = Q0 + W, the words (a-quad Q0, b-quad Q0,
     // a-quad Q1, b-quad Q1) (W, R as above).
     const uint4 *Cq;
-    // n = 4, when every entry of C^ fits in int8: C^ for the tensor-core
-    // contraction (launch shape 3 of k_walks<4>), else null.  K = 512 rows
-    // (the a-parts of the 256 rows, then the b-parts; within a part, K index
-    // 8 l + t is row 32 t + l), N = 256 columns, each entry stored as the
-    // byte entry + 128.  Column n takes 512 bytes at
-    // n * 512: 16-byte chunk c = 4 s + q (s = K-block of 64, q = 0..3),
-    // stored at chunk c ^ (4 (n & 1)), holds for the four 16-row K-blocks
-    // kb = 4 s .. 4 s + 3 the bytes of rows 16 kb + 2q, 2q + 1, 2q + 8, 2q + 9.
+    // n = 4, when C^ suits the tensor-core engine (qcs_engine4.cu), else null:
+    // every entry as the byte entry + 128, 512 bytes a column.  Byte
+    // part * 256 + 8 l + t of column Q is the a (part 0) or b (part 1) of row
+    // row4(l, t).  Csum[Q]: the sum of the column's entries.
     const uint4 *Cm;
+    const int16_t *Csum;
+    // n = 4: the weights after the first adjoint stage (as T1), for the
+    // engine: word (code * 32 + l) * 8 + t is row row4(l, t)'s Ua | Ub << 16
+    // after the Pauli of that code (code4); code 0 holds the weights themselves.
+    const uint4 *T4[2];
     const uint2 *U;    // fingerprint weights (Ua, Ub) per row, 4^n
     // The weights after the first adjoint stage of a side (index 0: V, 1: W),
     // mod 2^16, for every Pauli: entry e = q_a - 1, where q_a is the side's
@@ -254,6 +269,9 @@ cudaError_t launch_walk_step(const LevelCtx &lv, int chunk, const uint64_t *in, 
                              uint8_t *is_dp, size_t count, cudaStream_t s);
 cudaError_t launch_init_walks(const WalkLaunch &w, cudaStream_t s);
 cudaError_t launch_walks(const WalkLaunch &w, cudaStream_t s);
+// n = 4 with lv.Cm set: the level walk on the tensor-core engine (qcs_engine4.cu)
+cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s);
+int engine4_warps(); // warps of its CTA
 // DP-owner sharding: insert `count` distinguished points {dp, trail ref}
 // into w's table (merges queued as by the walk), and bin points by owner
 // rank (owner_of in qcs_walk.cu): out gets the points grouped by owner in
@@ -299,7 +317,8 @@ int pauli_phase(int n, uint32_t p, uint32_t q); // P(p)P(q) = i^lambda P(p^q)
 // device tables of the first adjoint stage (LevelCtx::T1), built once per
 // device and qubit count and kept for the life of the process
 // (*uploaded, when given, grows by the bytes this call copied to the device)
-int stage_tables(int n, const uint32_t *t1[2], int64_t *uploaded = nullptr);
+// (t4: LevelCtx::T4, null unless n = 4)
+int stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64_t *uploaded = nullptr);
 
 // How a level is walked (Sec. 3 and Appendix): theta, the launch shape, the
 // function-version period and the level's step budget.
@@ -336,8 +355,9 @@ struct qcs_problem {
     // device data
     uint2 *dC32 = nullptr, *dU = nullptr;
     uint32_t *dCq = nullptr; // n >= 3, when every entry of C^ fits in int8
-    uint32_t *dCm = nullptr; // n = 4, when every entry fits in int8: the tensor-core layout (LevelCtx::Cm)
+    uint32_t *dCm = nullptr; // n = 4, when C^ suits the tensor-core engine: LevelCtx::Cm, then Csum
     const uint32_t *dT1[2] = {nullptr, nullptr}; // shared stage tables
+    const uint32_t *dT4[2] = {nullptr, nullptr}; // and their n = 4 engine form (LevelCtx::T4)
     uint32_t *dCoef = nullptr;
     qcs::Slot *dTable = nullptr;
     qcs::Pair *dQueue = nullptr;

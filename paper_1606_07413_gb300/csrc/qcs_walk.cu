@@ -22,21 +22,20 @@
 // stages) instead of pushing all 4^n - 1 columns through them.  The V side is
 // then read off directly (its right factor is the identity), and the W side is
 // one contraction of the transformed weights with C^, staged in shared memory
-// as signed byte quads and contracted by byte-plane dp4a, or, at n = 4 in
-// launch shape 3, by f16 tensor-core MMAs in warps of their own, beside the
-// warps that run the stages of another set of walks (k_walks_mma4).  The
-// result is bit-identical to hashing the explicitly formed product.
+// as signed byte quads and contracted by byte-plane dp4a (the n = 4 engine
+// of qcs_engine4.cu contracts on the tensor cores instead).  The result is
+// bit-identical to hashing the explicitly formed product.
 //
 // Also here: the distinguished-point table insert and the re-walk of merged
 // trails (Sec. 3, Fig. 2), the batched forms of both, the exhaustive level
 // pass (Eq. mitm), and the owner binning and insertion of distinguished
 // points for a level sharded across ranks.
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
 
+#include "qcs_device.cuh"
 #include "qcs_internal.h"
 
 namespace qcs {
@@ -79,10 +78,9 @@ constexpr int kGemvUnroll = QCS_GEMV_UNROLL;
 //   n <= 2: 8 warps
 //   n = 3 : (16, 2) (8, 4) (32, 1) (16, 1)
 //   n = 4 : (16, 1) (24, 1) (32, 1)   (one CTA per SM: C^ takes 128 KB)
-//           and shape 3: the W side's contraction on the tensor cores
-//           (k_walks_mma4, 12 stage and 8 MMA warps; the level walk only,
-//           and only when C^ is held in int8; elsewhere shape 3 runs shape
-//           0, whose figures shape_warps gives for it)
+//           and shape 3: the tensor-core engine (qcs_engine4.cu; when C^
+//           suits it, LevelCtx::Cm; elsewhere shape 3 runs shape 0, whose
+//           figures shape_warps gives for it)
 __host__ __device__ constexpr int shape_count(int nq) { return nq <= 2 ? 1 : 4; }
 __host__ __device__ constexpr int shape_warps(int nq, int s)
 {
@@ -93,24 +91,6 @@ __host__ __device__ constexpr int shape_min_blocks(int nq, int s)
     return nq <= 2 ? 1 : nq == 3 ? (s == 1 ? 4 : s >= 2 ? 1 : QCS_MIN_BLOCKS3) : 1;
 }
 constexpr uint32_t kMaxRewalkLen = 1u << 20; // longer trails are reported as no merge
-
-__device__ __forceinline__ uint64_t smix(uint64_t z)
-{
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// smix(base ^ phi) for phi < 2^30, given pre = base ^ (base >> 30): the
-// first xorshift of the finaliser cannot see phi (it shifts by 30), so
-// (base ^ phi) ^ ((base ^ phi) >> 30) = pre ^ phi, and the rest follows.
-// The same value as smix(base ^ phi), one 64-bit xorshift cheaper per column.
-__device__ __forceinline__ uint64_t smix_pre(uint64_t pre, uint32_t phi)
-{
-    uint64_t z = (pre ^ (uint64_t)phi) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
 
 template <int NQ>
 struct Geo {
@@ -168,8 +148,6 @@ struct Smem {
     uint64_t *base;
     uint2 *xchg; // this lane group's exchange buffer
 };
-
-__device__ __forceinline__ uint32_t shl32(uint32_t v, int s) { return s >= 32 ? 0u : v << s; }
 
 // The lanes evaluating one walk: sub is the lane's index in its group of
 // LPW lanes, mask the group's lanes (every shuffle, reduction and warp
@@ -268,28 +246,6 @@ __device__ __forceinline__ void weight_planes(uint2 *su, Lanes g)
 #pragma unroll
     for (int r = 0; r < JOBS; r++) w2[lane + G::LPW * r] = pl[r];
     __syncwarp(g.mask);
-}
-
-struct Decoded {
-    int side;
-    uint64_t qpack; // q_1 .. q_h, 8 bits each (q <= 255)
-};
-
-// mu (Sec. 2, the state is a concatenation of per-rotation codes): bit 0 is
-// the side; rotation j reads the ell-bit field at bit 1 + ell j and maps its
-// value v onto the xi non-identity Paulis as q_j = floor(v xi / 2^ell) + 1.
-__device__ __forceinline__ Decoded decode(uint64_t x, const LevelCtx &lv)
-{
-    Decoded d;
-    d.side = (int)(x & 1);
-    d.qpack = 0;
-    uint64_t f = x >> 1;
-    for (int j = 0; j < lv.h; j++) {
-        const uint32_t v = (uint32_t)f & lv.fmask;
-        d.qpack |= (uint64_t)(((v * lv.xi) >> lv.ell) + 1) << (8 * j);
-        f >>= lv.ell;
-    }
-    return d;
 }
 
 // The fingerprint weights of one decoded point pushed through its side's
@@ -547,46 +503,6 @@ __global__ void __launch_bounds__(Geo<NQ>::THREADS) k_walk_step(LevelCtx lv, uin
     }
 }
 
-// starting state and chunk of trail (walk, seq) in the current version
-__device__ __forceinline__ uint64_t trail_start(const LevelCtx &lv, uint32_t walk, uint32_t seq)
-{
-    seq &= (1u << kRefSeqBits) - 1;
-    return smix(lv.seed ^ smix(((uint64_t)walk << 32) | seq) ^ ((uint64_t)lv.version << 40)) & lv.maskL;
-}
-__device__ __forceinline__ uint32_t trail_chunk(const LevelCtx &lv, uint64_t start)
-{
-    return lv.n_chunks ? 1u + (uint32_t)(smix(start ^ 0x5851F42D4C957F2Dull) % (uint64_t)lv.n_chunks) : 0u;
-}
-__device__ __forceinline__ uint64_t make_ref(uint32_t walk, uint32_t seq, uint32_t len)
-{
-    return (uint64_t)walk | ((uint64_t)(seq & ((1u << kRefSeqBits) - 1)) << kRefWalkBits) |
-           ((uint64_t)len << (kRefWalkBits + kRefSeqBits));
-}
-__device__ __forceinline__ void split_ref(uint64_t ref, uint32_t &walk, uint32_t &seq, uint32_t &len)
-{
-    walk = (uint32_t)(ref & ((1u << kRefWalkBits) - 1));
-    seq = (uint32_t)((ref >> kRefWalkBits) & ((1u << kRefSeqBits) - 1));
-    len = (uint32_t)(ref >> (kRefWalkBits + kRefSeqBits));
-}
-
-__device__ __forceinline__ void new_trail(WalkState &st, uint32_t walk, const LevelCtx &lv)
-{
-    st.seq++;
-    st.start = trail_start(lv, walk, st.seq);
-    st.cur = st.start;
-    st.len = 0;
-    st.chunk = trail_chunk(lv, st.start);
-}
-
-// per-walk-group tallies, added to the job's counters by the group's first
-// lane (the tensor-core kernel keeps them in 32 bits and flushes them before
-// they could overflow)
-template <typename T>
-struct TallyOf {
-    T steps = 0, w = 0, dp = 0, ab = 0, evicted = 0, duplicate = 0, pairs = 0;
-};
-using Tally = TallyOf<unsigned long long>;
-
 template <typename T>
 __device__ __forceinline__ void flush_tally(unsigned long long *counters, TallyOf<T> &t, Lanes g)
 {
@@ -600,48 +516,6 @@ __device__ __forceinline__ void flush_tally(unsigned long long *counters, TallyO
         if (t.pairs) atomicAdd(&counters[C_PAIRS], t.pairs);
     }
     t = TallyOf<T>();
-}
-
-// Store the distinguished point (Sec. 3: the triple start, end, length) in
-// the slot its value hashes to, keeping the newest trail there (one 128-bit
-// atomic exchange, never a wait).  If the slot held the same point from
-// another trail the two trails merged: queue them for the re-walk.
-template <typename WL, typename T>
-__device__ void dp_insert(const WL &w, uint64_t dp, uint64_t ref, TallyOf<T> &c)
-{
-    if (w.outbox) {
-        // DP-owner sharding: the point goes to its owner's table after the exchange
-        const uint32_t idx = atomicAdd(w.ohead, 1u);
-        if (idx < w.ocap) {
-            Slot o;
-            o.key = dp;
-            o.ref = ref;
-            w.outbox[idx] = o;
-        }
-        return;
-    }
-    Slot nv;
-    nv.key = dp;
-    nv.ref = ref;
-    Slot *s = &w.table[smix(dp) & w.table_mask];
-    const Slot old = atomicExch(s, nv);
-    if (old.key == dp) {
-        if (old.ref == ref) {
-            c.duplicate++;
-            return;
-        }
-        c.pairs++;
-        const uint32_t idx = atomicAdd(w.qhead, 1u);
-        if (idx < w.qcap) {
-            Pair p;
-            p.ref_a = old.ref;
-            p.ref_b = ref;
-            p.dp = dp;
-            w.queue[idx] = p;
-        }
-    } else if (old.key != kEmptyKey) {
-        c.evicted++;
-    }
 }
 
 // Advance one walk by w.steps steps (Sec. 3 trails): a trail that reaches a
@@ -720,685 +594,6 @@ __global__ void __launch_bounds__(Shape<NQ, S>::THREADS, Shape<NQ, S>::MIN_BLOCK
         if (walk < sw.n_walks) walk_one<NQ>(sw, sm, walk, g, t);
     }
     if (cur >= 0) flush_tally(sw.counters, t, g);
-}
-
-// ---- n = 4, launch shape 3: the W side's contraction on the tensor cores ----
-//
-// Warp-specialised: 12 stage warps and 8 MMA warps per CTA, one CTA per SM.
-// A CTA steps 48 walks as two sets of 24; each stage warp owns two walks of
-// each set.  For set X, step s:
-//  A. the stage warps evaluate the set's adjoint stages (side_weights).  A V
-//     walk's weights are already its column fingerprints: it hashes them into
-//     its shared sum at once.  A W walk writes its weights as two byte planes
-//     in f16 (bytes 0..255 are exact in f16) into its row buffer and flags
-//     its slot; then every stage warp signals "rows of X ready";
-//  B. the MMA warps multiply the flagged rows (compacted, up to 24: one M
-//     tile, rarely two) by C^ with mma.sync m16n8k16 (f16 x f16, f32
-//     accumulation), 32 columns per warp (8 accumulator chains; two MMA
-//     warps per scheduler keep the tensor pipe busy), hash those columns of
-//     every W walk into the walk's shared sum and signal "sums of X ready";
-//  C. the stage warps finish each walk's hash and take its step.
-// The stage warps run C and A of one set while the MMA warps run B of the
-// other (C_0(s) A_0(s+1) beside B_1(s); C_1(s) A_1(s+1) beside B_0(s+1)), so
-// the stages' integer work and the contraction overlap.  The hand-offs are
-// four mbarriers; every wait on them is bounded, and a wait that runs out
-// stops its warp and is counted in *w.stall (the results are then invalid).
-// C^'s entries are small integers, exact in f16.  In f16 C^ is 256 KB: more
-// than a CTA's shared memory, and exactly an SM's tensor memory (128 lanes x
-// 512 columns of 32 bits).  So at the start each MMA warp converts the MMA
-// fragments of its columns once and stores them in tensor memory
-// (tcgen05.st); it reloads them with tcgen05.ld, two K-blocks at a time.
-// Where theta is large the MMA warps also store the distinguished points the
-// stage warps find (the instantiation COLLECT; see Rings below).
-// Exactness: every product is an integer of magnitude below 2^15 (a byte
-// times an int8 entry), and every partial sum of a 512-term dot product is
-// below 512 x 255 x 128 < 2^24, so the f32 accumulation is exact and the
-// result converts back to the integer dot product; the fingerprint is then
-// L = P0 + 2^8 P1 (mod 2^16) from the two planes, as in the dp4a path.
-namespace mma4 {
-
-#ifndef QCS_WS_STAGE
-#define QCS_WS_STAGE 12 // stage warps
-#endif
-#ifndef QCS_WS_MMA
-#define QCS_WS_MMA 8 // MMA warps (two per scheduler keep the legacy tensor pipe busy)
-#endif
-#ifndef QCS_WS_WPW
-#define QCS_WS_WPW 2 // walks of each set per stage warp
-#endif
-constexpr int kStageWarps = QCS_WS_STAGE, kMmaWarps = QCS_WS_MMA, kWPW = QCS_WS_WPW;
-constexpr int kCtaWarps = kStageWarps + kMmaWarps, kThreads = kCtaWarps * 32;
-static_assert(kStageWarps % 4 == 0, "MMA warp m must be warp m % 4 of its warpgroup (tensor-memory lanes 32 (m % 4) ..)");
-static_assert(kMmaWarps == 4 || kMmaWarps == 8, "C^'s 256 columns split over 4 or 8 MMA warps");
-constexpr int kSets = 2, kWalks = kWPW * kStageWarps; // walks per set
-static_assert(kWalks <= 32, "a set's rows are compacted by one warp ballot");
-constexpr int kCT = 32 / kMmaWarps; // column tiles of 8 per MMA warp
-constexpr int kDim = 256, kK = 2 * kDim;
-// shared memory: weights | rotation masks | chunk bases | 2 x 24 row buffers
-// (2 KB each: a W walk's two f16 planes, and its stage exchanges) | per set,
-// the bookkeeping | the walks' states | the MMA warps' row lists | mbarriers
-// | tensor-memory address
-constexpr size_t off_coef = sizeof(uint2) * kDim;
-constexpr size_t off_base = off_coef + sizeof(uint32_t) * Geo<4>::COEF_WORDS;
-constexpr size_t off_xchg = off_base + sizeof(uint64_t) * Geo<4>::MAX_CHUNKS;
-static_assert(off_coef == Geo<4>::off_coef_v && off_base == Geo<4>::off_base_v, "layout of stage<4, false>");
-constexpr size_t off_book = off_xchg + (size_t)2048 * kWalks * kSets;
-struct Book {
-    unsigned long long sum[kWalks]; // per walk slot: the multiset hash's sum
-    uint64_t wbase[kWalks];         // per walk slot: the hash base (W walks)
-    uint32_t isw[kWalks];           // per walk slot: 1 if it is a W walk with a row this step
-};
-constexpr size_t off_wst = off_book + kSets * sizeof(Book);              // WalkState [set][slot]
-constexpr size_t off_rows = off_wst + sizeof(WalkState) * kSets * kWalks; // per MMA warp: slots of the compacted rows
-constexpr size_t off_bar = (off_rows + kMmaWarps * kWalks + 7) & ~(size_t)7;
-// The MMA warps are also the CTA's collectors (Sec. 4.2's role): they store
-// the distinguished points the stage warps hand them, while they wait for a
-// set's rows and after their last product, so that no stage warp waits on
-// the table's atomics.  One ring per stage warp (its lane 0 the only
-// producer; lane r / 8 of MMA warp r % 8 the only consumer of ring r); a
-// full ring makes the producer store the point itself.
-constexpr uint32_t kRing = 64;
-constexpr int kCollectBits = 8;
-struct Rings {
-    uint64_t dp[kStageWarps][kRing], ref[kStageWarps][kRing];
-    uint32_t tail[kStageWarps]; // points pushed (producer)
-    uint32_t head[kStageWarps]; // points stored (collector)
-    uint32_t done[kStageWarps]; // the stage warp has pushed its last point
-};
-constexpr size_t off_rings = off_bar + 4 * sizeof(uint64_t); // after: rows ready [2], sums ready [2]
-constexpr size_t off_tmem = off_rings + sizeof(Rings);
-constexpr size_t smem_bytes = off_tmem + 16;
-static_assert(smem_bytes <= 227 * 1024, "shared memory of the tensor-core walk kernel");
-// tensor memory: MMA warp m (the warp m % 4 of its warpgroup, so lanes
-// 32 (m % 4) .. + 31 are the ones it may access) holds C^'s columns
-// 8 kCT m .. 8 kCT (m + 1) - 1 in columns 64 kCT (m / 4) .. of those lanes;
-// column 2 kCT kb + 2 ct + h there is the B fragment register h of K-block
-// kb and column tile ct (columns 8 kCT m + 8 ct ..).
-constexpr uint32_t kTmemCols = 512;
-// a bounded wait gives up after this many SM clock cycles (about two seconds)
-constexpr long long kWaitCycles = 1ll << 32;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// Two bytes of `word` to an f16 pair, exactly: the byte permute `sel` puts
-// them in the low bytes of the two halves under 0x64 (0x64b = 1024 + b in
-// f16), then `bias` is subtracted (1024 for an unsigned byte; 1152 for a
-// signed byte stored with 128 added).
-__device__ __forceinline__ uint32_t bytes_to_f16x2(uint32_t word, uint32_t sel, float bias)
-{
-    const uint32_t v = __byte_perm(word, 0x64646464u, sel);
-    __half2 h = *reinterpret_cast<const __half2 *>(&v);
-    h = __hsub2(h, __float2half2_rn(bias));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&a)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
-                 : "r"(addr));
-}
-
-// Tensor memory (whole-warp instructions).  A load is asynchronous: its
-// registers are valid after tmem_wait_ld, which takes them as operands so
-// that no use can be scheduled before it.
-__device__ __forceinline__ void tmem_alloc(uint32_t *dst, uint32_t ncols)
-{
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
-{
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
-__device__ __forceinline__ void tmem_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tmem_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
-                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                 : "memory");
-}
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-                 "%15,%16};" ::"r"(taddr),
-                 "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
-                 "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-                 : "memory");
-}
-
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void tmem_ld16(uint32_t (&v)[16], uint32_t taddr)
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                 "[%16];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                   "=r"(v[15])
-                 : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t (&v)[8], uint32_t taddr)
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(taddr));
-}
-
-[[maybe_unused]] __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[8])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])
-                 :
-                 : "memory");
-}
-
-// (the 16-register forms serve 4 MMA warps, the 8-register ones 8)
-[[maybe_unused]] __device__ __forceinline__ void tmem_ld(uint32_t (&v)[16], uint32_t taddr) { tmem_ld16(v, taddr); }
-[[maybe_unused]] __device__ __forceinline__ void tmem_ld(uint32_t (&v)[8], uint32_t taddr) { tmem_ld8(v, taddr); }
-[[maybe_unused]] __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&v)[16]) { tmem_st16(taddr, v); }
-[[maybe_unused]] __device__ __forceinline__ void tmem_st(uint32_t taddr, const uint32_t (&v)[8]) { tmem_st8(taddr, v); }
-
-[[maybe_unused]] __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16])
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]),
-                   "+r"(v[15])
-                 :
-                 : "memory");
-}
-
-
-// mbarriers (shared memory): arrive has release and try_wait acquire
-// semantics at CTA scope.
-__device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *b)
-{
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(b))
-                 : "memory");
-}
-
-// Whether the phase of parity `ph` has completed (no waiting).
-__device__ __forceinline__ bool mbar_test(uint64_t *b, uint32_t ph)
-{
-    uint32_t done;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(done)
-                 : "r"(smem_u32(b)), "r"(ph)
-                 : "memory");
-    return done != 0;
-}
-
-// One bounded try: whether the phase of parity `ph` has completed, waiting
-// (suspended) for at most a system-dependent time.
-__device__ __forceinline__ bool mbar_try(uint64_t *b, uint32_t ph)
-{
-    uint32_t done;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(done)
-                 : "r"(smem_u32(b)), "r"(ph)
-                 : "memory");
-    return done != 0;
-}
-
-// Wait until the phase of parity `ph` has completed; false if the wait ran
-// out (kWaitCycles).
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t ph)
-{
-    const uint32_t a = smem_u32(b);
-    const long long t0 = clock64();
-    for (;;) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(a), "r"(ph)
-                     : "memory");
-        if (done) return true;
-        if (clock64() - t0 > kWaitCycles) return false;
-    }
-}
-
-// The bounded wait, made warp-uniform: true only if every lane saw the phase
-// complete (lanes that time out at different moments must not leave the warp
-// split before its next warp-wide operation).
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, uint32_t ph)
-{
-    return __all_sync(0xFFFFFFFFu, mbar_wait(b, ph));
-}
-
-} // namespace mma4
-
-// COLLECT: the MMA warps store the distinguished points (launched where
-// theta >= 2^-kCollectBits); otherwise the stage warps store their own and
-// the collecting code is not compiled in.
-template <bool COLLECT>
-__global__ void __launch_bounds__(mma4::kThreads, 1) k_walks_mma4(WalkLaunch w)
-{
-    using mma4::Book;
-    using mma4::kWalks;
-    using mma4::kK;
-    using G = Geo<4>;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    // weights, rotation masks and chunk bases as the other walk kernels stage them
-    Smem<4> sm = stage<4, false>(w.lv, smem_raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    Book *books = reinterpret_cast<Book *>(smem_raw + mma4::off_book);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem_raw + mma4::off_bar); // rows ready [2], sums ready [2]
-    uint32_t *tmem_addr = reinterpret_cast<uint32_t *>(smem_raw + mma4::off_tmem);
-    const Lanes g{lane, 0xFFFFFFFFu};
-    const int gq = lane >> 2, q = lane & 3; // MMA fragment coordinates
-    for (int i = threadIdx.x; i < mma4::kSets * kWalks; i += blockDim.x) {
-        books[i / kWalks].sum[i % kWalks] = 0;
-        books[i / kWalks].isw[i % kWalks] = 0;
-    }
-    mma4::Rings &rings = *reinterpret_cast<mma4::Rings *>(smem_raw + mma4::off_rings);
-    if (threadIdx.x < mma4::kStageWarps) {
-        rings.tail[threadIdx.x] = 0;
-        rings.head[threadIdx.x] = 0;
-        rings.done[threadIdx.x] = 0;
-    }
-    if (threadIdx.x == 0) {
-        mma4::mbar_init(&bars[0], mma4::kStageWarps);
-        mma4::mbar_init(&bars[1], mma4::kStageWarps);
-        mma4::mbar_init(&bars[2], mma4::kMmaWarps);
-        mma4::mbar_init(&bars[3], mma4::kMmaWarps);
-    }
-    if (warp == 0) mma4::tmem_alloc(tmem_addr, mma4::kTmemCols);
-    mma4::tmem_fence_before();
-    __syncthreads();
-    mma4::tmem_fence_after();
-    const uint32_t tmem = *tmem_addr;
-    if (warp >= mma4::kStageWarps) {
-        // MMA warp m: the fragments of its C^ columns, from the biased int8
-        // layout: column `col` is 512 bytes, its 16-byte chunk
-        // (4 (kb / 4) + q) ^ (4 (col & 1)) holds in word kb % 4 the four
-        // entries of K-block kb that lane (., q) of an MMA fragment takes
-        using mma4::kCT;
-        const int m = warp - mma4::kStageWarps;
-        const uint32_t tq = tmem + ((uint32_t)(32 * (m & 3)) << 16) + (uint32_t)(64 * kCT * (m >> 2));
-        const uint32_t *cm = reinterpret_cast<const uint32_t *>(w.lv.Cm);
-#pragma unroll 1
-        for (int kb = 0; kb < kK / 16; kb++) {
-            uint32_t v[2 * kCT];
-#pragma unroll
-            for (int ct = 0; ct < kCT; ct++) {
-                const int ncol = 8 * kCT * m + 8 * ct + gq;
-                const int chunk = (4 * (kb >> 2) + q) ^ (4 * (ncol & 1));
-                const uint32_t wd = cm[((size_t)ncol * 32 + chunk) * 4 + (kb & 3)];
-                v[2 * ct] = mma4::bytes_to_f16x2(wd, 0x4140, 1152.f);     // rows 2q, 2q + 1
-                v[2 * ct + 1] = mma4::bytes_to_f16x2(wd, 0x4342, 1152.f); // rows 2q + 8, 2q + 9
-            }
-            mma4::tmem_st(tq + (uint32_t)(2 * kCT * kb), v);
-        }
-        mma4::tmem_wait_st();
-    }
-    mma4::tmem_fence_before();
-    __syncthreads(); // the fragments are in tensor memory; the barriers are initialised
-    mma4::tmem_fence_after();
-
-    const LevelCtx &lv = w.lv;
-    const uint32_t steps = w.steps, max_len = w.max_len;
-    const int dshift = lv.dshift;
-    const int n_groups = (w.n_walks + mma4::kSets * kWalks - 1) / (mma4::kSets * kWalks);
-    bool stalled = false;
-    constexpr bool collect = COLLECT;
-    if (warp < mma4::kStageWarps) {
-        // ---- stage warp: walks kWPW warp .. kWPW warp + kWPW - 1 of each set ----
-        using mma4::kWPW;
-        // The walks' states live in shared memory (lane 0 writes them);
-        // a trail's start is only written (at a new trail), never read.
-        WalkState *wst = reinterpret_cast<WalkState *>(smem_raw + mma4::off_wst); // [set][slot]
-        TallyOf<uint32_t> t; // 32-bit tallies (fewer registers), flushed before they could overflow
-        uint32_t ph[2] = {0, 0}; // parity of the next "sums ready" phase of each set
-        for (int grp = blockIdx.x; grp < n_groups && !stalled; grp += gridDim.x) {
-            const int local0 = grp * mma4::kSets * kWalks + kWPW * warp; // + X kWalks + i
-            uint32_t live = 0; // bit kWPW X + i: walk i of set X exists
-#pragma unroll
-            for (int X = 0; X < 2; X++)
-#pragma unroll
-                for (int i = 0; i < kWPW; i++) {
-                    const int local = local0 + X * kWalks + i;
-                    if (local < w.n_walks) {
-                        live |= 1u << (kWPW * X + i);
-                        if (lane == 0) wst[X * kWalks + kWPW * warp + i] = w.walks[local];
-                    }
-                }
-            __syncwarp();
-            // A of set X: stages; V walks hash, W walks become matrix rows
-            auto phase_a = [&](int X) {
-                Book &bk = books[X];
-#pragma unroll
-                for (int i = 0; i < kWPW; i++) {
-                    const int slot = kWPW * warp + i;
-                    unsigned char *region = smem_raw + mma4::off_xchg + (size_t)2048 * (X * kWalks + slot);
-                    uint32_t isw = 0;
-                    if ((live >> (kWPW * X + i)) & 1u) {
-                        const uint64_t cur = wst[X * kWalks + slot].cur;
-                        const uint32_t chunk = wst[X * kWalks + slot].chunk;
-                        sm.xchg = reinterpret_cast<uint2 *>(region);
-                        const Decoded dx = decode(cur, lv);
-                        const uint64_t base = sm.base[chunk];
-                        uint32_t ua[G::RPL], ub[G::RPL];
-                        side_weights<4>(dx.side, dx.qpack, chunk, lv, sm, g, ua, ub);
-                        if (dx.side == 0) {
-                            const uint64_t sum = group_sum64(lane_column_sum<4>(ua, base, lane), 0xFFFFFFFFu);
-                            if (lane == 0) bk.sum[slot] = sum;
-                        } else {
-                            isw = 1;
-                            if (lane == 0) bk.wbase[slot] = base;
-                            // The K order of the product (as C^ is stored for it)
-                            // makes the lane's own rows j = lane + 32 t, t = 0..7,
-                            // the 16-byte chunk `lane` of each part (a: chunk lane,
-                            // b: chunk 32 + lane) and plane; chunk c is stored at
-                            // c ^ (slot & 7).  The region's stage exchange is done
-                            // (side_weights ends with a warp sync).
-                            uint4 out[4]; // (plane 0, a), (plane 1, a), (plane 0, b), (plane 1, b)
-                            uint32_t *o = reinterpret_cast<uint32_t *>(out);
-#pragma unroll
-                            for (int e = 0; e < 4; e++) {
-                                const uint32_t wa = (ua[2 * e] & 0xFFFFu) | (ua[2 * e + 1] << 16);
-                                const uint32_t wb = (ub[2 * e] & 0xFFFFu) | (ub[2 * e + 1] << 16);
-                                o[0 * 4 + e] = mma4::bytes_to_f16x2(wa, 0x7240, 1024.f);
-                                o[1 * 4 + e] = mma4::bytes_to_f16x2(wa, 0x7341, 1024.f);
-                                o[2 * 4 + e] = mma4::bytes_to_f16x2(wb, 0x7240, 1024.f);
-                                o[3 * 4 + e] = mma4::bytes_to_f16x2(wb, 0x7341, 1024.f);
-                            }
-                            const uint32_t swz = (uint32_t)slot & 7;
-                            uint4 *d4 = reinterpret_cast<uint4 *>(region);
-                            d4[0 * 64 + ((uint32_t)lane ^ swz)] = out[0];
-                            d4[1 * 64 + ((uint32_t)lane ^ swz)] = out[1];
-                            d4[0 * 64 + ((uint32_t)(32 + lane) ^ swz)] = out[2];
-                            d4[1 * 64 + ((uint32_t)(32 + lane) ^ swz)] = out[3];
-                        }
-                    }
-                    if (lane == 0) bk.isw[slot] = isw;
-                }
-                __syncwarp();
-                if (lane == 0) mma4::mbar_arrive(&bars[X]); // rows of X ready (this warp's part)
-            };
-            // C of set X: each walk's step
-            auto phase_c = [&](int X) {
-                Book &bk = books[X];
-#pragma unroll
-                for (int i = 0; i < kWPW; i++) {
-                    if (!((live >> (kWPW * X + i)) & 1u)) continue;
-                    const int slot = kWPW * warp + i;
-                    const uint64_t y = smix(bk.sum[slot]) & lv.maskL;
-                    WalkState S = wst[X * kWalks + slot];
-                    const int local = local0 + X * kWalks + i;
-                    const uint32_t gw = w.walk_base + (uint32_t)local;
-                    t.steps++;
-                    t.w += (uint32_t)(S.cur & 1);
-                    S.len++;
-                    if ((y >> dshift) == 0) {
-                        t.dp++;
-                        if (lane == 0) {
-                            // to the collector, or stored here if its ring is full
-                            volatile uint32_t *vt = rings.tail, *vh = rings.head;
-                            const uint32_t tl = vt[warp];
-                            if (collect && tl - vh[warp] < mma4::kRing) {
-                                rings.dp[warp][tl % mma4::kRing] = y;
-                                rings.ref[warp][tl % mma4::kRing] = make_ref(gw, S.seq, S.len);
-                                __threadfence_block();
-                                vt[warp] = tl + 1;
-                            } else {
-                                dp_insert(w, y, make_ref(gw, S.seq, S.len), t);
-                            }
-                        }
-                        __syncwarp();
-                        new_trail(S, gw, lv);
-                        if (lane == 0) w.walks[local].start = S.start;
-                    } else if (S.len >= max_len) {
-                        t.ab++;
-                        new_trail(S, gw, lv);
-                        if (lane == 0) w.walks[local].start = S.start;
-                    } else {
-                        S.cur = y;
-                    }
-                    __syncwarp(); // every lane has read the old state
-                    if (lane == 0) wst[X * kWalks + slot] = S;
-                }
-                // the sums start again from zero for the set's next products
-                __syncwarp();
-                if (lane < kWPW) bk.sum[kWPW * warp + lane] = 0;
-                __syncwarp();
-            };
-            if (steps > 0) {
-                phase_a(0);
-                phase_a(1);
-            }
-            for (uint32_t step = 0; step < steps && !stalled; step++) {
-#pragma unroll
-                for (int X = 0; X < 2; X++) {
-                    if (stalled) break;
-                    if (!mma4::mbar_wait_warp(&bars[2 + X], ph[X])) {
-                        stalled = true;
-                        break;
-                    }
-                    ph[X] ^= 1u;
-                    phase_c(X);
-                    if (step + 1 < steps) phase_a(X);
-                }
-                if (t.steps >= 0x40000000u) flush_tally(w.counters, t, g); // every tally is at most t.steps
-            }
-            // the states back to global memory (every lane has written its last update)
-#pragma unroll
-            for (int X = 0; X < 2; X++)
-#pragma unroll
-                for (int i = 0; i < kWPW; i++)
-                    if (((live >> (kWPW * X + i)) & 1u) && lane == 0) {
-                        const WalkState &S = wst[X * kWalks + kWPW * warp + i];
-                        WalkState *d = &w.walks[local0 + X * kWalks + i];
-                        d->cur = S.cur;
-                        d->len = S.len;
-                        d->chunk = S.chunk;
-                        d->seq = S.seq;
-                    }
-            __syncwarp();
-        }
-        flush_tally(w.counters, t, g);
-        // every point this warp pushed is in its ring: the collector may stop once they are stored
-        __syncwarp();
-        if (lane == 0) {
-            __threadfence_block();
-            reinterpret_cast<volatile uint32_t *>(rings.done)[warp] = 1;
-        }
-    } else {
-        // ---- MMA warp m: C^'s columns 8 kCT m .. 8 kCT (m + 1) - 1 ----
-        using mma4::kCT;
-        const int m = warp - mma4::kStageWarps;
-        const uint32_t tq = tmem + ((uint32_t)(32 * (m & 3)) << 16) + (uint32_t)(64 * kCT * (m >> 2));
-        uint8_t *rows = smem_raw + mma4::off_rows + kWalks * m; // slots of the compacted rows
-        uint32_t ph[2] = {0, 0}; // parity of the next "rows ready" phase of each set
-        // collecting: lane c < 2 consumes ring m + kMmaWarps c (if there is one)
-        TallyOf<uint32_t> tc;
-        volatile uint32_t *vt = rings.tail, *vd = rings.done;
-        const int ring = m + mma4::kMmaWarps * lane;
-        const bool owner = lane < 2 && ring < mma4::kStageWarps;
-        uint32_t rhead = 0;
-        // store up to `most` pushed points of the owned ring (one at a time
-        // while rows may become ready)
-        auto drain = [&](uint32_t most) -> bool {
-            bool moved = false;
-            if (owner) {
-                volatile uint32_t *vh = rings.head;
-                const uint32_t tl = vt[ring];
-                if (tl != rhead) {
-                    __threadfence_block(); // the entries before tail are written
-                    const uint32_t stop = tl - rhead > most ? rhead + most : tl;
-                    for (; rhead != stop; rhead++)
-                        dp_insert(w, rings.dp[ring][rhead % mma4::kRing], rings.ref[ring][rhead % mma4::kRing], tc);
-                    __threadfence_block();
-                    vh[ring] = rhead; // their slots may be reused
-                    moved = true;
-                }
-            }
-            return __any_sync(0xFFFFFFFFu, moved);
-        };
-        // wait for a set's rows, storing distinguished points meanwhile (with
-        // nothing to store, the warp sleeps on the barrier itself)
-        auto wait_rows = [&](int X) -> bool {
-            const long long t0 = clock64();
-            for (;;) {
-                if (__all_sync(0xFFFFFFFFu, mma4::mbar_test(&bars[X], ph[X]))) return true;
-                if (!drain(1)) {
-                    if (__all_sync(0xFFFFFFFFu, mma4::mbar_try(&bars[X], ph[X]))) return true;
-                    if (clock64() - t0 > mma4::kWaitCycles) return false;
-                }
-            }
-        };
-        const int mrow = (lane & 7) + 8 * ((lane >> 3) & 1), mkof = lane >> 4; // ldmatrix row, K offset
-        for (int grp = blockIdx.x; grp < n_groups && !stalled; grp += gridDim.x)
-            for (uint32_t step = 0; step < steps && !stalled; step++)
-#pragma unroll 1
-                for (int X = 0; X < 2; X++) {
-                    if (!(collect ? wait_rows(X) : mma4::mbar_wait_warp(&bars[X], ph[X]))) {
-                        stalled = true;
-                        break;
-                    }
-                    ph[X] ^= 1u;
-                    Book &bk = books[X];
-                    // the W rows, compacted in slot order
-                    const bool flagged = lane < kWalks && bk.isw[lane < kWalks ? lane : 0] != 0;
-                    const uint32_t mask = __ballot_sync(0xFFFFFFFFu, flagged);
-                    const uint32_t nrows = (uint32_t)__popc(mask);
-                    if (flagged) rows[__popc(mask & ((1u << lane) - 1u))] = (uint8_t)lane;
-                    __syncwarp();
-#pragma unroll 1
-                    for (int tile = 0; tile < (int)(nrows + 15) / 16; tile++) {
-                        const uint32_t r0 = (uint32_t)(16 * tile + mrow);
-                        const uint32_t sl0 = rows[r0 < nrows ? r0 : 0]; // rows past the W walks read row 0 (unused)
-                        const uint32_t arow =
-                            mma4::smem_u32(smem_raw + mma4::off_xchg + (size_t)2048 * (X * kWalks + sl0));
-                        const uint32_t aswz = sl0 & 7;
-                        float acc[2][kCT][4]; // [plane][column tile][fragment]
-#pragma unroll
-                        for (int b = 0; b < 2; b++)
-#pragma unroll
-                            for (int c = 0; c < kCT; c++)
-#pragma unroll
-                                for (int d = 0; d < 4; d++) acc[b][c][d] = 0.f;
-                        // one K-block: both planes' A fragments times the 8 column tiles
-                        auto kblock = [&](int kb, const uint32_t(&f)[2 * kCT]) {
-#pragma unroll
-                            for (int p = 0; p < 2; p++) {
-                                uint32_t af[4];
-                                mma4::ldmatrix_x4(af, arow + 1024 * p + 16 * (((uint32_t)(2 * kb + mkof)) ^ aswz));
-#pragma unroll
-                                for (int ct = 0; ct < kCT; ct++) mma4::mma16816(acc[p][ct], af, f[2 * ct], f[2 * ct + 1]);
-                            }
-                        };
-                        // C^'s fragments from tensor memory, two K-blocks (16
-                        // registers) at a time, the next two loading while these are used
-                        static_assert(kCT == 4, "two K-blocks per 16-register load");
-                        uint32_t f0[16], f1[16];
-                        auto half = [](const uint32_t(&f)[16], int i) -> const uint32_t(&)[8] {
-                            return *reinterpret_cast<const uint32_t(*)[8]>(&f[8 * i]);
-                        };
-                        mma4::tmem_ld16(f0, tq);
-#pragma unroll 1
-                        for (int kb4 = 0; kb4 < kK / 64; kb4++) {
-                            mma4::tmem_wait_ld(f0);
-                            mma4::tmem_ld16(f1, tq + 16u * (uint32_t)(2 * kb4 + 1));
-                            kblock(4 * kb4, half(f0, 0));
-                            kblock(4 * kb4 + 1, half(f0, 1));
-                            mma4::tmem_wait_ld(f1);
-                            if (kb4 + 1 < kK / 64) mma4::tmem_ld16(f0, tq + 16u * (uint32_t)(2 * kb4 + 2));
-                            kblock(4 * kb4 + 2, half(f1, 0));
-                            kblock(4 * kb4 + 3, half(f1, 1));
-                        }
-                        // fingerprints of the warp's columns for the tile's rows gq
-                        // and gq + 8, hashed into each row's walk
-#pragma unroll
-                        for (int hh = 0; hh < 2; hh++) {
-                            const uint32_t r = (uint32_t)(16 * tile + gq + 8 * hh);
-                            const bool valid = r < nrows;
-                            const uint32_t sl = rows[valid ? r : 0];
-                            const uint64_t base = valid ? bk.wbase[sl] : 0;
-                            const uint64_t pre = base ^ (base >> 30);
-                            uint64_t part = 0;
-#pragma unroll
-                            for (int ct = 0; ct < kCT; ct++)
-#pragma unroll
-                                for (int c = 0; c < 2; c++) {
-                                    const int Q = 8 * kCT * m + 8 * ct + 2 * q + c;
-                                    const int p0 = __float2int_rn(acc[0][ct][2 * hh + c]);
-                                    const int p1 = __float2int_rn(acc[1][ct][2 * hh + c]);
-                                    const uint32_t l = ((uint32_t)p0 + ((uint32_t)p1 << 8)) & 0xFFFFu;
-                                    const uint32_t nl = (0u - l) & 0xFFFFu;
-                                    const uint64_t e = smix_pre(pre, min(l, nl));
-                                    part += (Q >= 1) ? e : 0ull;
-                                }
-                            part += __shfl_xor_sync(0xFFFFFFFFu, part, 1);
-                            part += __shfl_xor_sync(0xFFFFFFFFu, part, 2);
-                            if (valid && q == 0) atomicAdd(&bk.sum[sl], part);
-                        }
-                    }
-                    __syncwarp();
-                    if (lane == 0) mma4::mbar_arrive(&bars[2 + X]); // sums of X ready (this warp's part)
-                }
-        // the stage warps' last steps come after the last product: store
-        // their points until each owned ring's producer is done and drained
-        long long last = clock64();
-        for (; collect;) {
-            const bool moved = drain(mma4::kRing);
-            bool fin = true;
-            if (owner) {
-                const bool d = vd[ring] != 0;
-                __threadfence_block(); // the final tail, read after its done flag
-                fin = d && vt[ring] == rhead;
-            }
-            if (__all_sync(0xFFFFFFFFu, fin)) break;
-            if (moved) {
-                last = clock64();
-            } else {
-                if (clock64() - last > mma4::kWaitCycles) {
-                    stalled = true; // a stage warp neither pushed nor finished for too long
-                    break;
-                }
-                __nanosleep(256);
-            }
-        }
-        tc.evicted = __reduce_add_sync(0xFFFFFFFFu, tc.evicted);
-        tc.duplicate = __reduce_add_sync(0xFFFFFFFFu, tc.duplicate);
-        tc.pairs = __reduce_add_sync(0xFFFFFFFFu, tc.pairs);
-        flush_tally(w.counters, tc, g);
-    }
-    if (stalled && lane == 0) atomicAdd(w.stall, 1u);
-    // every warp's tensor-memory loads have completed (each was waited for)
-    mma4::tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        mma4::tmem_fence_after();
-        mma4::tmem_dealloc(tmem, mma4::kTmemCols);
-    }
 }
 
 __global__ void k_init_walks(WalkLaunch w)
@@ -1846,31 +1041,6 @@ cudaError_t walks_ns(const WalkLaunch &w, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// the tensor-core level walk (n = 4, launch shape 3): one CTA per SM
-cudaError_t walks_mma4(const WalkLaunch &w, cudaStream_t s)
-{
-    static int per_sm = 0;
-    if (!per_sm) {
-        cudaFuncSetAttribute(k_walks_mma4<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma4::smem_bytes);
-        cudaFuncSetAttribute(k_walks_mma4<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mma4::smem_bytes);
-        int b = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_walks_mma4<false>, mma4::kThreads, mma4::smem_bytes);
-        per_sm = b > 0 ? b : 1;
-    }
-    if (!w.stall) return cudaErrorInvalidValue; // a stalled wait must have somewhere to be counted
-    const size_t groups = ((size_t)w.n_walks + mma4::kSets * mma4::kWalks - 1) / (mma4::kSets * mma4::kWalks);
-    size_t grid = (size_t)num_sms() * (size_t)per_sm;
-    if (grid > groups) grid = groups;
-    if (grid == 0) grid = 1;
-    // d_theta = L - dshift: the MMA warps collect where theta >= 2^-kCollectBits
-    const int dtheta = __builtin_popcountll(w.lv.maskL) - w.lv.dshift;
-    if (dtheta <= mma4::kCollectBits)
-        k_walks_mma4<true><<<(unsigned)grid, mma4::kThreads, mma4::smem_bytes, s>>>(w);
-    else
-        k_walks_mma4<false><<<(unsigned)grid, mma4::kThreads, mma4::smem_bytes, s>>>(w);
-    return cudaGetLastError();
-}
-
 template <int NQ>
 cudaError_t walks_n(const WalkLaunch &w, cudaStream_t s)
 {
@@ -1879,7 +1049,7 @@ cudaError_t walks_n(const WalkLaunch &w, cudaStream_t s)
     case 1: if constexpr (shape_count(NQ) > 1) return walks_ns<NQ, 1>(w, s); break;
     case 2: if constexpr (shape_count(NQ) > 2) return walks_ns<NQ, 2>(w, s); break;
     case 3:
-        if constexpr (NQ == 4) return w.lv.Cm ? walks_mma4(w, s) : walks_ns<4, 0>(w, s);
+        if constexpr (NQ == 4) return w.lv.Cm ? launch_walks_e4(w, s) : walks_ns<4, 0>(w, s);
         else if constexpr (shape_count(NQ) > 3) return walks_ns<NQ, 3>(w, s);
         break;
     }
@@ -2013,7 +1183,7 @@ int lanes_per_walk(int n) { return n == 4 ? Geo<4>::LPW : n == 3 ? Geo<3>::LPW :
 
 int launch_shapes(int n) { return n == 4 ? shape_count(4) : n == 3 ? shape_count(3) : shape_count(2); }
 
-int shape_warps_of(int n, int shape) { return n == 4 && shape == 3 ? mma4::kCtaWarps : shape_warps(n, shape); }
+int shape_warps_of(int n, int shape) { return n == 4 && shape == 3 ? engine4_warps() : shape_warps(n, shape); }
 
 int shape_min_blocks_of(int n, int shape) { return shape_min_blocks(n, shape); }
 
