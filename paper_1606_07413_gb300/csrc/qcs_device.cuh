@@ -62,7 +62,12 @@ __device__ __forceinline__ uint64_t trail_start(const LevelCtx &lv, uint32_t wal
 }
 __device__ __forceinline__ uint32_t trail_chunk(const LevelCtx &lv, uint64_t start)
 {
-    return lv.n_chunks ? 1u + (uint32_t)(smix(start ^ 0x5851F42D4C957F2Dull) % (uint64_t)lv.n_chunks) : 0u;
+    if (!lv.n_chunks) return 0u;
+    // n_chunks = xi = 4^n - 1: with v = hi 2^32 + lo and 2^32 = 1 (mod xi)
+    // for n = 1, 2, 4 (4^n's powers reach 2^32) and 4 (mod 63) for n = 3
+    const uint64_t v = smix(start ^ 0x5851F42D4C957F2Dull);
+    const uint32_t xi = (uint32_t)lv.n_chunks, r32 = lv.n == 3 ? 4u : 1u;
+    return 1u + ((uint32_t)(v >> 32) % xi * r32 + (uint32_t)v % xi) % xi;
 }
 __device__ __forceinline__ uint64_t make_ref(uint32_t walk, uint32_t seq, uint32_t len)
 {

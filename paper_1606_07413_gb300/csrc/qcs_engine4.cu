@@ -1,36 +1,39 @@
 // qcs_engine4.cu -- n = 4: the coset hash of many points at once, with the W
 // side's contraction on the fifth-generation tensor cores (tcgen05.mma).
 //
-// The engine.  A CTA (one per SM) evaluates the hash of 48 points in flight,
-// two sets of 24.  Its 19 warps have three roles:
-//  - 16 workers, each owning three points (one or two of each set).  Phase A
-//    of a set: a point's fingerprint weights go through its adjoint stages
-//    (one warp per point); a V point's weights are its column fingerprints,
-//    hashed at once; a W point writes its weights as two f16 byte planes, two
-//    rows of the set's B operand.  Phase E: the set's product D = C^^T B is
-//    read back from tensor memory and hashed, column sums of every W point.
+// The engine.  A CTA (one per SM) evaluates the hash of 72 points in flight,
+// three sets of 24.  Its 28 warps have three roles:
+//  - 24 workers, each owning one slot of every set.  Phase A of a set: a
+//    point's fingerprint weights go through its adjoint stages (one warp per
+//    point); a V point's weights are its column fingerprints, hashed at once;
+//    a W point writes its weights as two f16 byte planes, two rows of the
+//    set's B operand.  Phase E: the set's product D = C^^T B is read back from
+//    tensor memory and hashed, column sums of every W point.
 //  - one MMA warp: when all rows of a set are written it issues the product,
 //    64 tcgen05.mma (128 x N x 16 each, N = twice the set's W points).
-//  - one control warp per set: lane i is what uses slot i's hash (a walk, a
-//    re-walked merge, ...).  It takes the set's hashes, decides the slots'
-//    next points and publishes them; table inserts and the like follow after
-//    that, off the critical path.  All that a walk does besides f runs here
-//    on 24 lanes at once instead of once per walk on 32.
-// The workers run A(0) A(1) E(0) E(1) in turn: MMA(X) runs beside the other
-// set's A, control(X) beside the other set's E.
+//  - one control warp per set: lane i is what uses slot i's hash (a walk).  It
+//    takes the set's hashes, decides the slots' next points and publishes
+//    them; table inserts and the like follow after that, off the critical
+//    path.  All that a walk does besides f runs here on 24 lanes at once
+//    instead of once per walk on 32.
 //
-// What bounds it.  A point costs 618 warp instructions; half of them are the
-// 255 column finalisers.  Issue is 59 % active, the ALU pipe 59 %, the tensor
-// pipe 16 %: fixed-latency and load stalls between the phases take the rest.
-// 2^20 walks x 16 steps at level 7: 14.95 ms (1.12 G steps/s), against 26.7 ms
-// with mma.sync (12 stage and 8 MMA warps, C^'s fragments through
-// tcgen05.ld, the rows through ldmatrix: 1073 instructions a step).
+// What bounds it.  A set's round is a chain: its points through A (about 3000
+// cycles, the SM shared with the other sets), the product (1600: 16 cycles a
+// tcgen05.mma with A in tensor memory, 40 in shared memory, whatever N), E
+// (700), control (800).  With 48 points in flight (two sets of 24, or three
+// of 16) that chain was the bound; with 72 it is issue: 75 % active at 588
+// warp instructions a point, half of them the 255 column finalisers.
+// 2^20 walks x 16 steps at level 7: 11.1 ms (1.51 G steps/s); two sets and
+// 16 workers 14.9 ms; with mma.sync (12 stage and 8 MMA warps, C^'s fragments
+// through tcgen05.ld, the rows through ldmatrix, 1073 instructions) 26.7 ms.
+// B has room for 16 W points of a set's 24; more than 16 turn up in 3 % of
+// the rounds, and those past 16 wait for the next round.
 //
 // Where C^ sits.  In f16 it is 256 KB.  As the A operand (M = columns of C^,
 // K = its 512 numerator rows) its first 128 columns and K-blocks 0-7 of the
 // other 128 are in tensor memory (320 of 512 columns), the rest (96 KB) in
-// shared memory; that leaves 192 tensor-memory columns for two sets' D (2 x
-// 2 x 48 f32 columns) and 96 KB of shared memory for two sets' B.
+// shared memory; that leaves 192 tensor-memory columns for three sets' D (3 x
+// 2 x 32 f32 columns) and 96 KB of shared memory for three sets' B.
 //
 // Exactness.  B holds 1024 + byte (the f16 bits 0x6400 | byte, so no
 // conversion), and every sum is an integer below 2^24 in magnitude, so f32
@@ -55,10 +58,12 @@ namespace {
 
 namespace e4 {
 
-constexpr int kWorkers = 16, kSet = 24, kSets = 2;
-constexpr int kMmaWarp = kWorkers, kCtlWarp = kWorkers + 1; // control warps kCtlWarp, kCtlWarp + 1
+constexpr int kSet = 24, kSets = 3, kWorkers = kSet; // a worker owns one slot of each set
+constexpr int kPairs = 16;                            // W points of a set that fit one product
+static_assert(kWorkers % 4 == 0 && kPairs % 4 == 0 && kPairs / 4 < kWorkers / 4 && kSet <= 32, "units and slots");
+constexpr int kMmaWarp = kWorkers, kCtlWarp = kWorkers + 1; // control warps kCtlWarp + set
 constexpr int kWarps = kWorkers + 1 + kSets, kThreads = 32 * kWarps;
-constexpr int kN = 2 * kSet;                // columns of D per set and half
+constexpr int kN = 2 * kPairs;              // columns of D per set and half
 constexpr int kTmemK = 8;                   // K-blocks of C^'s second half held in tensor memory
 constexpr int kDcol = 256 + 8 * kTmemK;     // tensor-memory column of D (set X, half h: + 96 X + 48 h)
 static_assert(kDcol + kSets * 2 * kN <= 512, "tensor memory");
@@ -82,13 +87,14 @@ constexpr size_t off_A = 0;                                        // C^, second
 constexpr size_t off_B = off_A + 6 * 16384;                        // [set]: 8 chunks of 64 K x 48 rows
 constexpr size_t off_job = off_B + (size_t)kSets * 8 * kN * 128;   // Job [set][slot]
 constexpr size_t off_wb = off_job + sizeof(Job) * kSets * kSet;    // HashBase [set][row pair]
-constexpr size_t off_part = off_wb + sizeof(HashBase) * kSets * kSet;   // u64 [set][quadrant and half][row pair]
-constexpr size_t off_vsum = off_part + 8 * sizeof(uint64_t) * kSets * kSet; // u64 [set][slot]
+constexpr int kParts = 16; // partial column sums of a W point
+constexpr size_t off_part = off_wb + sizeof(HashBase) * kSets * kPairs; // u64 [set][part][row pair]
+constexpr size_t off_vsum = off_part + kParts * sizeof(uint64_t) * kSets * kPairs; // u64 [set][slot]
 constexpr size_t off_chunk = off_vsum + sizeof(uint64_t) * kSets * kSet; // HashBase [chunk]
-constexpr size_t off_stage = off_chunk + sizeof(HashBase) * 256;   // stage table: byte [code][lane]
-constexpr size_t off_nw = off_stage + 256 * 32;                    // u32 [set]: W points; [2 + set]: the set is done
-constexpr size_t off_bar = off_nw + 16;                            // mbarriers: jobs, rows, product, sums [set]
-constexpr size_t off_tmem = off_bar + 8 * sizeof(uint64_t);
+constexpr size_t off_stage = off_chunk + sizeof(HashBase) * 256;   // stage table: u32 [side][code % 64][lane]
+constexpr size_t off_nw = off_stage + 2 * 64 * 32 * sizeof(uint32_t);                  // u32 [set]: W points; [2 + set]: the set is done
+constexpr size_t off_bar = off_nw + 32;                            // mbarriers: jobs, rows, product, sums [set]
+constexpr size_t off_tmem = off_bar + 4 * kSets * sizeof(uint64_t);
 constexpr size_t smem_bytes = off_tmem + 16;
 static_assert(smem_bytes <= 227 * 1024, "shared memory of the n = 4 engine");
 
@@ -110,27 +116,31 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *b)
     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(b)) : "memory");
 }
 
+// One try: whether the phase of parity `ph` has completed, waiting
+// (suspended) for at most a system-dependent time.
+__device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t ph)
+{
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "selp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done)
+                 : "r"(a), "r"(ph)
+                 : "memory");
+    return done != 0;
+}
+
 // Wait until the phase of parity `ph` has completed; false if the wait ran
-// out.  Warp-uniform: true only if every lane saw the phase complete.
+// out.  Warp-uniform: true only once every lane saw the phase complete.
 __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t ph)
 {
     const uint32_t a = smem_u32(b);
+    if (__all_sync(0xFFFFFFFFu, mbar_try(a, ph))) return true;
     const long long t0 = clock64();
-    bool ok = false;
     for (;;) {
-        uint32_t done;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(a), "r"(ph)
-                     : "memory");
-        if (done) {
-            ok = true;
-            break;
-        }
-        if (clock64() - t0 > kWaitCycles) break;
+        if (__all_sync(0xFFFFFFFFu, mbar_try(a, ph))) return true;
+        // one lane's clock decides for the warp
+        if (__shfl_sync(0xFFFFFFFFu, clock64() - t0, 0) > kWaitCycles) return false;
     }
-    return __all_sync(0xFFFFFFFFu, ok);
 }
 
 // ---- tensor memory and products
@@ -166,10 +176,12 @@ __device__ __forceinline__ void tmem_ld16x256(uint32_t (&v)[4], uint32_t taddr)
 
 // the loads' registers are valid after this; it takes them as operands so
 // that no use is scheduled before it
-__device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[4], uint32_t (&b)[4])
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[4][4])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3])
+                 : "+r"(v[0][0]), "+r"(v[0][1]), "+r"(v[0][2]), "+r"(v[0][3]), "+r"(v[1][0]), "+r"(v[1][1]),
+                   "+r"(v[1][2]), "+r"(v[1][3]), "+r"(v[2][0]), "+r"(v[2][1]), "+r"(v[2][2]), "+r"(v[2][3]),
+                   "+r"(v[3][0]), "+r"(v[3][1]), "+r"(v[3][2]), "+r"(v[3][3])
                  :
                  : "memory");
 }
@@ -214,83 +226,101 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar)
 // ---- one point on one warp
 //
 // Lane l holds the eight weight rows row4(l, t) (qcs_internal.h): t carries
-// qubit 3's two bits and qubit 2's x bit, the lane the rest, and a Pauli's
-// code (code4) is laid out the same way: its low five bits are its lane part,
-// its high three its t part.  A stage takes row j to u_j +- u_{j^p} or to
-// sqrt2 u_j, by lambda(p, j) in P(p) P(j) = i^lambda P(p^j), which is a sum
-// over the qubits.  So with the t part of p known at compile time (a switch
-// over its eight values) the partner's register and qubit 3's share of lambda
-// are constants, and what is left of lambda is one value per lane and x bit of
-// qubit 2: a byte of the stage table per code and lane.
+// qubit 2's x bit and qubit 3, the lane the rest, and a Pauli's code (code_of)
+// is laid out the same way: its low five bits are its lane part, its high
+// three its t part.  A stage takes row j to u_j +- u_{j^p} or to sqrt2 u_j, by
+// lambda(p, j) in P(p) P(j) = i^lambda P(p^j), which is a sum over the qubits.
+// So with the t part of p known at compile time (a switch over its eight
+// values) the partner's register and qubit 3's share of lambda are constants,
+// and what is left of lambda is one value per lane and x bit of qubit 2: a
+// word of the stage table, which does not depend on p's qubit 3.  About 85
+// instructions a stage; with the signs and selections looked up row by row it
+// was 106.
 
 __host__ __device__ constexpr int lambda1(int px, int pz, int x, int z)
 {
     return (px * pz + x * z + 2 * pz * x - (px ^ x) * (pz ^ z)) & 3;
 }
 
-// lambda of the lane's rows but for qubit 3's share, for x bit 0 (bits 0-1)
-// and 1 (bits 2-3) of qubit 2
-__device__ __forceinline__ uint32_t stage_byte(uint32_t code, uint32_t l)
+// lambda of the lane's rows but for qubit 3's share, for x bit x2 = 0, 1 of
+// qubit 2: byte x2 is the sign (lambda 0 or 1: +1, 2 or 3: -1; for W the
+// other way round), byte 2 + x2 whether lambda is odd
+__device__ __forceinline__ uint32_t stage_word(uint32_t side, uint32_t code, uint32_t l)
 {
-    // lane bits: z0 z1 z2 x0 x1; code bits: the same, then z3 x3 x2
-    uint32_t v = 0;
+    // lane bits: z0 z1 z2 x0 x1; code bits: the same, then x2
+    int v = 0;
 #pragma unroll
     for (int q = 0; q < 2; q++)
         v += lambda1((code >> (3 + q)) & 1, (code >> q) & 1, (l >> (3 + q)) & 1, (l >> q) & 1);
-    const int px2 = (code >> 7) & 1, pz2 = (code >> 2) & 1, z2 = (l >> 2) & 1;
-    return ((v + lambda1(px2, pz2, 0, z2)) & 3) | ((v + lambda1(px2, pz2, 1, z2)) & 3) << 2;
-}
-
-// m: the multipliers of the partner row, per x bit of qubit 2 (second index)
-// for rows whose qubit-3 share of lambda is 0 (m[0]), 1 (m[1]) or 3 (m[2])
-template <int PT>
-__device__ __forceinline__ void stage_rows(uint32_t (&ua)[8], uint32_t (&ub)[8], int pl, const int (&m)[3][2],
-                                           const bool (&odd)[2])
-{
-    uint32_t na[8], nb[8];
-#pragma unroll
-    for (int t = 0; t < 8; t++) {
-        const int x2 = t >> 2, c = lambda1((PT >> 1) & 1, PT & 1, (t >> 1) & 1, t & 1);
-        const uint32_t va = __shfl_xor_sync(0xFFFFFFFFu, ua[t ^ PT], pl);
-        const uint32_t vb = __shfl_xor_sync(0xFFFFFFFFu, ub[t ^ PT], pl);
-        const bool anti = odd[x2] != ((c & 1) != 0);
-        const uint32_t mul = (uint32_t)m[c == 0 ? 0 : c == 1 ? 1 : 2][x2];
-        // anticommuting rows: u + s v; commuting rows (multiplier 0): (ub, 2 ua)
-        na[t] = va * mul + (anti ? ua[t] : ub[t]);
-        nb[t] = vb * mul + (anti ? ub[t] : ua[t] << 1);
-    }
-#pragma unroll
-    for (int t = 0; t < 8; t++) {
-        ua[t] = na[t];
-        ub[t] = nb[t];
-    }
-}
-
-// tr: 0 for V (adjoint of R^), 1 for W (adjoint of R^T)
-__device__ __forceinline__ void stage(uint32_t code, uint32_t tr, const uint8_t *tab, int lane, uint32_t (&ua)[8],
-                                      uint32_t (&ub)[8])
-{
-    const uint32_t v = tab[code * 32 + lane];
-    const int pl = (int)(code & 31);
-    int m[3][2];
-    bool odd[2];
+    uint32_t w = 0;
 #pragma unroll
     for (int x = 0; x < 2; x++) {
-        odd[x] = ((v >> (2 * x)) & 1u) != 0;
-        const int s = 1 - 2 * (int)(((v >> (2 * x + 1)) ^ tr) & 1u); // lambda 0 or 1: +, 2 or 3: - (V)
-        m[0][x] = odd[x] ? s : 0;
-        m[1][x] = odd[x] ? 0 : s;
-        m[2][x] = odd[x] ? 0 : -s;
+        const uint32_t a = (uint32_t)(v + lambda1((code >> 5) & 1, (code >> 2) & 1, x, (l >> 2) & 1)) & 3u;
+        w |= (((a >> 1) ^ side) ? 0xFFu : 1u) << (8 * x) | (a & 1u) << (16 + 8 * x);
     }
+    return w;
+}
+
+// (na, nb) = ODD == (odd != 0) ? (ub, 2 ua) : (ua + s va, ub + s vb)
+template <bool ODD>
+__device__ __forceinline__ void row_update(uint32_t &ua, uint32_t &ub, uint32_t va, uint32_t vb, uint32_t s,
+                                           uint32_t odd)
+{
+    uint32_t na, nb;
+    if (ODD)
+        asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %7, 0;\n\tmov.b32 %0, %5;\n\tadd.u32 %1, %4, %4;\n\t"
+            "@p mad.lo.u32 %0, %2, %6, %4;\n\t@p mad.lo.u32 %1, %3, %6, %5;\n\t}"
+            : "=&r"(na), "=&r"(nb)
+            : "r"(va), "r"(vb), "r"(ua), "r"(ub), "r"(s), "r"(odd));
+    else
+        asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %7, 0;\n\tmov.b32 %0, %5;\n\tadd.u32 %1, %4, %4;\n\t"
+            "@p mad.lo.u32 %0, %2, %6, %4;\n\t@p mad.lo.u32 %1, %3, %6, %5;\n\t}"
+            : "=&r"(na), "=&r"(nb)
+            : "r"(va), "r"(vb), "r"(ua), "r"(ub), "r"(s), "r"(odd));
+    ua = na;
+    ub = nb;
+}
+
+// the stage of a Pauli whose t part is PT; s, odd: the lane's sign and parity
+// of lambda per x bit of qubit 2, without qubit 3's share
+template <int PT>
+__device__ __forceinline__ void stage_rows(uint32_t (&ua)[8], uint32_t (&ub)[8], int pl, const int (&s)[2],
+                                           const uint32_t (&odd)[2])
+{
+    uint32_t va[8], vb[8];
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+        va[t] = __shfl_xor_sync(0xFFFFFFFFu, ua[t ^ PT], pl);
+        vb[t] = __shfl_xor_sync(0xFFFFFFFFu, ub[t ^ PT], pl);
+    }
+    const int neg[2] = {-s[0], -s[1]};
+#pragma unroll
+    for (int t = 0; t < 8; t++) {
+        // qubit 3's share of lambda: 0, 1 or 3 (3: the sign turns)
+        const int x2 = t & 1, c = lambda1((PT >> 2) & 1, (PT >> 1) & 1, (t >> 2) & 1, (t >> 1) & 1);
+        const uint32_t sg = (uint32_t)(c == 3 ? neg[x2] : s[x2]);
+        if (c & 1) row_update<true>(ua[t], ub[t], va[t], vb[t], sg, odd[x2]);
+        else row_update<false>(ua[t], ub[t], va[t], vb[t], sg, odd[x2]);
+    }
+}
+
+// side: 0 for V (adjoint of R^), 1 for W (adjoint of R^T)
+__device__ __forceinline__ void stage(uint32_t code, uint32_t side, const uint32_t *tab, int lane, uint32_t (&ua)[8],
+                                      uint32_t (&ub)[8])
+{
+    const uint32_t w = tab[(side << 6 | (code & 63u)) * 32 + lane];
+    const int pl = (int)(code & 31u);
+    const int s[2] = {(int)(int8_t)w, (int)(int8_t)(w >> 8)};
+    const uint32_t odd[2] = {w & 0xFF0000u, w & 0xFF000000u};
     switch (code >> 5) {
-    case 0: stage_rows<0>(ua, ub, pl, m, odd); break;
-    case 1: stage_rows<1>(ua, ub, pl, m, odd); break;
-    case 2: stage_rows<2>(ua, ub, pl, m, odd); break;
-    case 3: stage_rows<3>(ua, ub, pl, m, odd); break;
-    case 4: stage_rows<4>(ua, ub, pl, m, odd); break;
-    case 5: stage_rows<5>(ua, ub, pl, m, odd); break;
-    case 6: stage_rows<6>(ua, ub, pl, m, odd); break;
-    default: stage_rows<7>(ua, ub, pl, m, odd); break;
+    case 0: stage_rows<0>(ua, ub, pl, s, odd); break;
+    case 1: stage_rows<1>(ua, ub, pl, s, odd); break;
+    case 2: stage_rows<2>(ua, ub, pl, s, odd); break;
+    case 3: stage_rows<3>(ua, ub, pl, s, odd); break;
+    case 4: stage_rows<4>(ua, ub, pl, s, odd); break;
+    case 5: stage_rows<5>(ua, ub, pl, s, odd); break;
+    case 6: stage_rows<6>(ua, ub, pl, s, odd); break;
+    default: stage_rows<7>(ua, ub, pl, s, odd); break;
     }
 }
 
@@ -342,59 +372,75 @@ __device__ __forceinline__ void first_stage(const uint4 *tab, uint32_t code, int
 __device__ __forceinline__ uint64_t v_column_sum(const uint32_t (&ua)[8], const uint32_t (&ub)[8], int ev,
                                                  uint64_t PH, uint32_t pre16, int lane)
 {
-    const bool odd = (ev & 1) != 0;
     const int sh = (ev >> 1) < 31 ? ev >> 1 : 31;
     uint64_t acc = 0;
+    auto columns = [&](const uint32_t (&u)[8]) {
 #pragma unroll
-    for (int t = 0; t < 8; t++) {
-        const uint64_t e = column_hash((odd ? ub[t] : ua[t]) << sh, PH, pre16);
-        acc += (t == 0 && lane == 0) ? 0ull : e; // column 0, the identity, does not enter
-    }
+        for (int t = 0; t < 8; t++) {
+            const uint64_t e = column_hash(u[t] << sh, PH, pre16);
+            acc += (t == 0 && lane == 0) ? 0ull : e; // column 0, the identity, does not enter
+        }
+    };
+    if (ev & 1) columns(ub);
+    else columns(ua);
     return warp_sum64(acc);
 }
 
-// Pauli code of index q (row4's bit order)
-__device__ __forceinline__ uint32_t code_of(uint32_t q)
+// Pauli codes (row4's bit order) of four Pauli indices, one per byte
+__device__ __forceinline__ uint32_t codes_of(uint32_t q)
 {
-    return (q & 7u) | ((q >> 4) & 3u) << 3 | ((q >> 3) & 1u) << 5 | ((q >> 7) & 1u) << 6 | ((q >> 6) & 1u) << 7;
+    return (q & 0x87878787u) | ((q >> 1) & 0x38383838u) | ((q << 3) & 0x40404040u);
 }
 
-// The stages of a point: V takes q_h first and goes down to q_1; W takes q_1
-// .. q_h, then the chunk.  A product of no rotations starts from code 0, the
-// untouched weights; so does V's single rotation (its half product then is
-// not one lookup).  Returns the number of stages.
-__device__ __forceinline__ int stage_seq(int side, uint64_t qpack, uint32_t chunk, int h, uint64_t *out)
-{
-    uint64_t seq = 0;
-    int ns = 0;
-    if (side == 0) {
-        if (h <= 1) ns = 1;
-        for (int j = h - 1; j >= 0; j--) seq |= (uint64_t)code_of((uint32_t)(qpack >> (8 * j)) & 0xFFu) << (8 * ns++);
-    } else {
-        if (h == 0) ns = 1;
-        for (int j = 0; j < h; j++) seq |= (uint64_t)code_of((uint32_t)(qpack >> (8 * j)) & 0xFFu) << (8 * ns++);
-        if (chunk) seq |= (uint64_t)code_of(chunk) << (8 * ns++);
+// The stages of a point in order, a code per byte: V takes q_h first and goes
+// down to q_1; W takes q_1 .. q_h, then the chunk.  A product of no rotations
+// starts from code 0, the untouched weights; so does V's single rotation (its
+// half product then is not one lookup).  What depends on the level alone is
+// kept here; the control warps' time from a set's sums to its next points is
+// on the sets' critical path.
+struct Stages {
+    int h, sh_v, sh_rev; // sh_v: shift that puts code 0 first; sh_rev: of the reversed bytes
+    uint32_t ns_v, ns_w, sh_c; // stages of a side; shift of the chunk's code
+    __device__ __forceinline__ explicit Stages(const LevelCtx &lv)
+    {
+        h = lv.h;
+        sh_v = h == 1 ? 8 : 0;
+        sh_rev = 64 - 8 * h;
+        ns_v = (uint32_t)(h <= 1 ? h + 1 : h);
+        sh_c = (uint32_t)(8 * (h == 0 ? 1 : h));
+        ns_w = (uint32_t)(h == 0 ? 1 : h) + (uint32_t)(lv.k & 1);
     }
-    *out = seq;
-    return ns;
-}
+    __device__ __forceinline__ uint64_t chunk_code(uint32_t chunk) const
+    {
+        return (uint64_t)codes_of(chunk) << sh_c; // chunk < 256
+    }
+    // q: the indices, q_1 in the lowest byte; cc: chunk_code
+    __device__ __forceinline__ uint64_t seq(int side, uint64_t q, uint64_t cc) const
+    {
+        const uint32_t lo = codes_of((uint32_t)q), hi = codes_of((uint32_t)(q >> 32));
+        if (side) return (((uint64_t)hi << 32) | lo) | cc;
+        if (h == 0) return 0;
+        const uint64_t rev = ((uint64_t)__byte_perm(lo, 0, 0x0123) << 32) | __byte_perm(hi, 0, 0x0123);
+        return (rev >> sh_rev) << sh_v;
+    }
+};
 
 // ---- roles
 
 struct Cta {
     unsigned char *raw;
-    uint64_t *bars; // jobs [2], rows [2], product [2], sums [2]
-    uint32_t *nw;   // [2] W points, [2] set done
+    uint64_t *bars; // per set: jobs, rows, product, sums
+    uint32_t *nw;   // [set] W points, [4 + set] set done
     uint32_t tmem;
     __device__ Job *jobs(int X) const { return reinterpret_cast<Job *>(raw + off_job) + X * kSet; }
-    __device__ HashBase *wb(int X) const { return reinterpret_cast<HashBase *>(raw + off_wb) + X * kSet; }
-    __device__ uint64_t *part(int X) const { return reinterpret_cast<uint64_t *>(raw + off_part) + X * 8 * kSet; }
+    __device__ HashBase *wb(int X) const { return reinterpret_cast<HashBase *>(raw + off_wb) + X * kPairs; }
+    __device__ uint64_t *part(int X) const { return reinterpret_cast<uint64_t *>(raw + off_part) + X * kParts * kPairs; }
     __device__ uint64_t *vsum(int X) const { return reinterpret_cast<uint64_t *>(raw + off_vsum) + X * kSet; }
     __device__ const HashBase *chunk_base() const { return reinterpret_cast<const HashBase *>(raw + off_chunk); }
-    __device__ uint64_t *bar_jobs(int X) const { return bars + X; }
-    __device__ uint64_t *bar_rows(int X) const { return bars + 2 + X; }
-    __device__ uint64_t *bar_prod(int X) const { return bars + 4 + X; }
-    __device__ uint64_t *bar_sums(int X) const { return bars + 6 + X; }
+    __device__ uint64_t *bar_jobs(int X) const { return bars + 4 * X; }
+    __device__ uint64_t *bar_rows(int X) const { return bars + 4 * X + 1; }
+    __device__ uint64_t *bar_prod(int X) const { return bars + 4 * X + 2; }
+    __device__ uint64_t *bar_sums(int X) const { return bars + 4 * X + 3; }
 };
 
 // stage table, chunk bases, barriers, tensor memory and C^: every thread calls it
@@ -413,10 +459,11 @@ __device__ __forceinline__ Cta cta_begin(const LevelCtx &lv, unsigned char *raw,
             mbar_init(c.bar_prod(X), 1);
             mbar_init(c.bar_sums(X), kWorkers);
         }
-        c.nw[0] = c.nw[1] = c.nw[2] = c.nw[3] = 0;
+        for (int i = 0; i < 8; i++) c.nw[i] = 0;
     }
-    uint8_t *tab = raw + off_stage;
-    for (int i = threadIdx.x; i < 256 * 32; i += kThreads) tab[i] = (uint8_t)stage_byte(i >> 5, i & 31);
+    uint32_t *tab = reinterpret_cast<uint32_t *>(raw + off_stage);
+    for (int i = threadIdx.x; i < 2 * 64 * 32; i += kThreads)
+        tab[i] = stage_word((uint32_t)i >> 11, ((uint32_t)i >> 5) & 63u, (uint32_t)i & 31u);
     if (with_chunks) {
         // base(chunk) = smix(smix(seed_H ^ version) ^ (n | k << 8 | chunk << 16 | K << 32))
         const uint64_t vmix = smix(kSeedH ^ (uint64_t)lv.version);
@@ -488,7 +535,7 @@ __device__ __forceinline__ void point_a(const LevelCtx &lv, const Cta &c, int X,
     if (info & kInvalid) return;
     const uint64_t seq = jp->seq;
     const uint32_t side = (info >> 8) & 1u, ns = info & 0xFFu;
-    const uint8_t *tab = c.raw + off_stage;
+    const uint32_t *tab = reinterpret_cast<const uint32_t *>(c.raw + off_stage);
     uint32_t ua[8], ub[8];
     first_stage(lv.T4[side], (uint32_t)seq & 0xFFu, lane, ua, ub);
 #pragma unroll 1
@@ -523,89 +570,80 @@ __device__ __forceinline__ void point_a(const LevelCtx &lv, const Cta &c, int X,
     }
 }
 
-// Phase E, one unit: the 32 columns of C^ that quadrant qd holds of half h,
-// for row pairs 4 g .. 4 g + 3 (lane % 4)
-__device__ __forceinline__ void unit_e(const Cta &c, int X, int g, int h, int qd, int lane)
+// Phase E, one unit: the 64 columns of C^ that quadrant qd holds (32 of each
+// half), for row pairs 4 g .. 4 g + 3 (lane % 4).  Each lane sums eight
+// columns, lanes 16 apart are added, and the control warp adds the rest.
+__device__ __forceinline__ void unit_e(const Cta &c, int X, int g, int qd, int lane)
 {
-    const uint32_t t = c.tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(kDcol + X * 2 * kN + h * kN + 8 * g);
-    uint32_t v[2][4];
-    tmem_ld16x256(v[0], t);
-    tmem_ld16x256(v[1], t + (16u << 16));
+    const uint32_t t = c.tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(kDcol + X * 2 * kN + 8 * g);
+    uint32_t v[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) tmem_ld16x256(v[i], t + (uint32_t)(kN * (i >> 1)) + ((uint32_t)(16 * (i & 1)) << 16));
     const HashBase hb = c.wb(X)[4 * g + (lane & 3)];
-    tmem_wait_ld(v[0], v[1]);
+    tmem_wait_ld(v);
     uint64_t acc = 0;
 #pragma unroll
-    for (int s = 0; s < 2; s++)
+    for (int i = 0; i < 4; i++)
 #pragma unroll
         for (int e = 0; e < 2; e++) {
             // the two planes' dot products (their low 16 bits are exact)
-            const uint64_t z = column_hash(v[s][2 * e] + v[s][2 * e + 1] * 256u, hb.PH, hb.pre16);
-            acc += (s == 0 && e == 0 && h == 0 && qd == 0 && lane < 4) ? 0ull : z; // column 0 does not enter
+            const uint64_t z = column_hash(v[i][2 * e] + v[i][2 * e + 1] * 256u, hb.PH, hb.pre16);
+            acc += (i == 0 && e == 0 && qd == 0 && lane < 4) ? 0ull : z; // column 0 does not enter
         }
-    acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 4);
-    acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 8);
     acc += __shfl_xor_sync(0xFFFFFFFFu, acc, 16);
-    if (lane < 4) c.part(X)[(2 * qd + h) * kSet + 4 * g + lane] = acc;
+    if (lane < 16) c.part(X)[(4 * qd + (lane >> 2)) * kPairs + 4 * g + (lane & 3)] = acc;
 }
 
-// worker warp w; false if a wait ran out
+// worker warp w: slot w of every set; false if a wait ran out.  The phases run A(0) E(2) A(1) E(0) A(2) E(1): between a set's
+// A and its E (the product) and between its E and its next A (the control
+// warp) lie another set's A and E.
 __device__ __forceinline__ bool worker(const LevelCtx &lv, const Cta &c, int w, int lane)
 {
-    bool done[2] = {false, false};
+    uint32_t live = (1u << kSets) - 1; // sets that are not done
     uint32_t ph = 0;
-    const bool low = w < kWorkers / 2;
-    // set 0: slots 2w, 2w + 1 (w < 8) or 8 + w; set 1: the other way round
-    while (!(done[0] && done[1])) {
-#pragma unroll
-        for (int X = 0; X < 2; X++) {
-            if (done[X]) continue;
-            if (!mbar_wait(c.bar_jobs(X), ph)) return false;
-            if (c.nw[2 + X]) {
-                done[X] = true;
-                continue;
+    int u = w >> 2; // units of all sets in turn over the quadrant's warps
+    for (bool first = true;; first = false) {
+#pragma unroll 1
+        for (int X = 0; X < kSets; X++) {
+            if ((live >> X) & 1u) {
+                if (!mbar_wait(c.bar_jobs(X), ph)) return false;
+                if (c.nw[4 + X]) live &= ~(1u << X);
             }
-            const bool two = low == (X == 0);
-            const int v = low ? w : w - kWorkers / 2;
-            const int s0 = two ? 2 * v : kWorkers + v, s1 = two ? s0 + 1 : s0;
-#pragma unroll 1
-            for (int s = s0; s <= s1; s++) point_a(lv, c, X, s, lane);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(c.bar_rows(X));
-        }
-        int u0 = w >> 2; // units of both sets in turn over the quadrant's four warps
-#pragma unroll
-        for (int X = 0; X < 2; X++) {
-            if (done[X]) continue;
-            if (!mbar_wait(c.bar_prod(X), ph)) return false;
+            if ((live >> X) & 1u) {
+                point_a(lv, c, X, w, lane);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(c.bar_rows(X));
+            }
+            const int Y = X == 0 ? kSets - 1 : X - 1; // set 2's E is the last iteration's
+            if (!((live >> Y) & 1u) || (X == 0 && first)) continue;
+            if (!mbar_wait(c.bar_prod(Y), X == 0 ? ph ^ 1u : ph)) return false;
             tmem_fence_after();
-            const int units = 2 * ((int)(c.nw[X] + 3) >> 2);
-#pragma unroll 1
-            for (; u0 < units; u0 += kWorkers / 4) unit_e(c, X, u0 >> 1, u0 & 1, w & 3, lane);
-            u0 -= units;
+            const int units = (int)(c.nw[Y] + 3) >> 2; // at most kPairs / 4, fewer than the quadrant's warps
+            if (u < units) unit_e(c, Y, u, w & 3, lane);
+            u = u < units ? u + kWorkers / 4 - units : u - units;
             tmem_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(c.bar_sums(X));
+            if (lane == 0) mbar_arrive(c.bar_sums(Y));
         }
+        if (!live) return true;
         ph ^= 1u;
     }
-    return true;
 }
 
 // the MMA warp (the whole warp calls it); false if a wait ran out
 __device__ __forceinline__ bool mma_warp(const Cta &c)
 {
-    bool done[2] = {false, false};
+    uint32_t live = (1u << kSets) - 1;
     uint32_t ph = 0;
     const uint64_t a0 = smem_desc(smem_u32(c.raw + off_A));
-    while (!(done[0] && done[1])) {
+    while (live) {
 #pragma unroll 1
-        for (int X = 0; X < 2; X++) {
-            if (X ? done[1] : done[0]) continue;
+        for (int X = 0; X < kSets; X++) {
+            if (!((live >> X) & 1u)) continue;
             if (!mbar_wait(c.bar_jobs(X), ph)) return false;
-            if (c.nw[2 + X]) {
-                if (X) done[1] = true;
-                else done[0] = true;
+            if (c.nw[4 + X]) {
+                live &= ~(1u << X);
                 continue;
             }
             if (!mbar_wait(c.bar_rows(X), ph)) return false;
@@ -646,118 +684,148 @@ __device__ __forceinline__ bool mma_warp(const Cta &c)
     return true;
 }
 
-// Publish the set's next points: lane i < kSet passes slot i's (valid or
-// not).  The row pairs of the W points are numbered here.  Whole warp.
-// Returns the lane's row pair.
-__device__ __forceinline__ uint32_t publish(const Cta &c, int X, int lane, bool valid, int side, uint64_t qpack,
-                                            uint32_t chunk, int h, HashBase hb)
+// the rotations of a state, as decode's, q_1 in the lowest byte
+__device__ __forceinline__ uint64_t rotations(uint64_t x, const LevelCtx &lv)
 {
-    const uint32_t wm = __ballot_sync(0xFFFFFFFFu, valid && side == 1);
-    const uint32_t pos = (uint32_t)__popc(wm & ((1u << lane) - 1u));
-    if (lane < kSet) {
-        Job j;
-        j.PH = hb.PH;
-        j.pre16 = hb.pre16;
-        j.pad = 0;
-        j.seq = 0;
-        if (valid) {
-            const int ns = stage_seq(side, qpack, chunk, h, &j.seq);
-            j.info = (uint32_t)ns | (uint32_t)side << 8 | pos << 16;
-        } else {
-            j.info = kInvalid;
+    uint64_t q = 0, f = x >> 1;
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+        if (j < lv.h) {
+            q |= (uint64_t)((((uint32_t)f & lv.fmask) * 255u >> lv.ell) + 1u) << (8 * j);
+            f >>= lv.ell;
         }
-        c.jobs(X)[lane] = j;
-        if (valid && side == 1) c.wb(X)[pos] = hb;
+    return q;
+}
+
+// Publish the set's next points: lane i < kSet passes slot i's (valid or
+// not).  The W points are numbered here; those past kPairs (3 % of a set's
+// rounds have any) wait for the next round, where `late` puts them first.
+// Whole warp.  Returns whether the lane's point is evaluated this round, and
+// its number.
+__device__ __forceinline__ bool publish(const Cta &c, int X, int lane, bool valid, bool late, int side, uint64_t seq,
+                                        uint32_t ns, HashBase hb, uint32_t *pos_out)
+{
+    const bool isw = valid && side == 1;
+    const uint32_t before = (1u << lane) - 1u;
+    const uint32_t all = __ballot_sync(0xFFFFFFFFu, isw), first = __ballot_sync(0xFFFFFFFFu, isw && late);
+    const uint32_t pos = (uint32_t)(late ? __popc(first & before) : __popc(first) + __popc(all & ~first & before));
+    const bool go = valid && (!isw || pos < (uint32_t)kPairs);
+    if (lane < kSet) {
+        Job *j = c.jobs(X) + lane;
+        const uint32_t info = go ? ns | (uint32_t)side << 8 | pos << 16 : kInvalid;
+        *reinterpret_cast<uint4 *>(j) =
+            make_uint4((uint32_t)seq, (uint32_t)(seq >> 32), (uint32_t)hb.PH, (uint32_t)(hb.PH >> 32));
+        *(reinterpret_cast<uint2 *>(j) + 2) = make_uint2(hb.pre16, info);
+        if (go && isw)
+            *reinterpret_cast<uint4 *>(c.wb(X) + pos) =
+                make_uint4((uint32_t)hb.PH, (uint32_t)(hb.PH >> 32), hb.pre16, 0);
     }
-    if (lane == 0) c.nw[X] = (uint32_t)__popc(wm);
+    if (lane == 0) c.nw[X] = min((uint32_t)__popc(all), (uint32_t)kPairs);
     __syncwarp();
     if (lane == 0) mbar_arrive(c.bar_jobs(X));
-    return pos;
+    *pos_out = pos;
+    return go;
 }
 
 __device__ __forceinline__ void publish_done(const Cta &c, int X, int lane)
 {
     if (lane == 0) {
-        c.nw[2 + X] = 1;
+        c.nw[4 + X] = 1;
         mbar_arrive(c.bar_jobs(X));
     }
     __syncwarp();
 }
 
 // the hash of the lane's slot, after the set's sums are complete
-__device__ __forceinline__ uint64_t slot_hash(const Cta &c, int X, int lane, bool valid, int side, uint32_t pos)
+__device__ __forceinline__ uint64_t slot_hash(const Cta &c, int X, int lane, int side, uint32_t pos)
 {
-    uint64_t acc = 0;
-    if (valid) {
-        if (side == 0) {
-            acc = c.vsum(X)[lane];
-        } else {
+    uint64_t acc = c.vsum(X)[lane < kSet ? lane : 0];
+    if (side) {
+        uint64_t v[kParts];
 #pragma unroll
-            for (int i = 0; i < 8; i++) acc += c.part(X)[i * kSet + pos];
-        }
+        for (int i = 0; i < kParts; i++) v[i] = c.part(X)[i * kPairs + pos];
+#pragma unroll
+        for (int o = kParts / 2; o; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < o; i++) v[i] += v[i + o];
+        acc = v[0];
     }
     return smix(acc);
 }
 
 } // namespace e4
 
-// The level walk.  gsz walks (at most 48, chosen by the host so that every
-// CTA steps the same number of groups, as nearly full as that allows) per
-// group; a CTA steps its groups one after the other.
+// The level walk: slot lane * kSets + X of the CTA steps walk slot + gsz *
+// blockIdx.x and every gsz * gridDim.x-th after it, one after the other.  gsz
+// (at most kSets * kSet) is chosen by the host so that every slot has the
+// same number of walks, as nearly as that allows.
 __device__ __forceinline__ bool walk_control(const WalkLaunch &w, uint32_t gsz, const e4::Cta &c, int X, int lane)
 {
     using namespace e4;
     const LevelCtx &lv = w.lv;
-    const uint32_t n_groups = ((uint32_t)w.n_walks + gsz - 1) / gsz;
-    const uint32_t slot = (uint32_t)(X * kSet + lane);
+    const Stages sg(lv);
+    const uint32_t slot = (uint32_t)(lane * kSets + X), stride = gsz * gridDim.x, n = (uint32_t)w.n_walks;
+    uint32_t local = blockIdx.x * gsz + slot; // below 2^25: n <= 2^24, and a slot stops past n
+    bool valid = lane < kSet && slot < gsz && local < n, late = false, ok = true;
+    WalkState st{}, nx{};
+    if (valid) st = w.walks[local];
+    uint32_t left = w.steps, ph = 0;
     Tally t;
-    uint32_t ph = 0;
-    bool ok = true;
-    for (uint32_t grp = blockIdx.x; grp < n_groups && ok; grp += gridDim.x) {
-        const uint32_t local = grp * gsz + slot;
-        const bool valid = lane < kSet && slot < gsz && local < (uint32_t)w.n_walks;
-        WalkState st{};
-        if (valid) st = w.walks[local];
+    HashBase hb = c.chunk_base()[st.chunk];
+    uint64_t cc = sg.chunk_code(st.chunk), dp = 0, ref = 0;
+    bool store = false;
+    while (__any_sync(0xFFFFFFFFu, valid)) {
+        const int side = (int)(st.cur & 1);
+        uint32_t pos;
+        const bool go = publish(c, X, lane, valid, late, side, sg.seq(side, rotations(st.cur, lv), cc),
+                                side ? sg.ns_w : sg.ns_v, hb, &pos);
+        // while the workers run: the last step's distinguished points, and
+        // the slot's next walk if this is its walk's last step
+        if (store) dp_insert(w, dp, ref, t);
+        store = false;
+        late = valid && !go;
+        const bool last = st.len + 1 >= w.max_len; // this step ends the trail in any case
         const uint32_t walk = w.walk_base + local; // index among all ranks' walks
-        uint64_t dp = 0, ref = 0;
-        bool store = false;
-        for (uint32_t s = 0; s < w.steps; s++) {
-            const Decoded d = decode(st.cur, lv);
-            const uint32_t pos =
-                publish(c, X, lane, valid, d.side, d.qpack, st.chunk, lv.h, c.chunk_base()[valid ? st.chunk : 0]);
-            // the last step's distinguished points, while the workers run
-            if (store) dp_insert(w, dp, ref, t);
-            __syncwarp();
-            if (!mbar_wait(c.bar_sums(X), ph)) {
-                ok = false;
-                break;
-            }
-            ph ^= 1u;
-            const uint64_t y = slot_hash(c, X, lane, valid, d.side, pos) & lv.maskL;
-            store = false;
-            if (valid) {
-                t.steps++;
-                t.w += (uint32_t)d.side;
-                st.len++;
-                if ((y >> lv.dshift) == 0) {
+        if (go && left == 1 && local + stride < n) nx = w.walks[local + stride];
+        __syncwarp();
+        if (!mbar_wait(c.bar_sums(X), ph)) {
+            ok = false;
+            break;
+        }
+        ph ^= 1u;
+        const uint64_t y = slot_hash(c, X, lane, go ? side : 0, pos) & lv.maskL;
+        if (go) {
+            st.cur = y;
+            st.len++;
+            left--;
+            t.steps++;
+            t.w += side;
+            const bool is_dp = (y >> lv.dshift) == 0;
+            if (is_dp || last || left == 0) {
+                if (is_dp) {
                     t.dp++;
                     store = true;
                     dp = y;
                     ref = make_ref(walk, st.seq, st.len);
-                    new_trail(st, walk, lv);
-                } else if (st.len >= w.max_len) {
+                } else if (last) {
                     t.ab++;
-                    new_trail(st, walk, lv);
-                } else {
-                    st.cur = y;
                 }
+                if (is_dp || last) new_trail(st, walk, lv);
+                if (left == 0) {
+                    w.walks[local] = st;
+                    local += stride;
+                    valid = local < n;
+                    st = nx;
+                    left = w.steps;
+                }
+                hb = c.chunk_base()[st.chunk];
+                cc = sg.chunk_code(st.chunk);
             }
-            __syncwarp();
         }
-        if (store) dp_insert(w, dp, ref, t);
-        if (valid) w.walks[local] = st;
         __syncwarp();
     }
+    if (ok && store) dp_insert(w, dp, ref, t);
+    __syncwarp();
     if (ok) publish_done(c, X, lane);
     unsigned long long v[7] = {t.steps, t.w, t.dp, t.ab, t.evicted, t.duplicate, t.pairs};
     const int idx[7] = {C_STEPS, C_WSTEPS, C_DPS, C_ABANDONED, C_EVICTED, C_DUPLICATE, C_PAIRS};
@@ -799,12 +867,13 @@ cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s)
     const cudaError_t e =
         cudaFuncSetAttribute(k_walks_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
     if (e != cudaSuccess) return e;
+    if (w.n_walks <= 0) return cudaSuccess;
+    // every slot the same number of walks, as few as the slots allow
     const uint32_t sms = (uint32_t)num_sms(), full = sms * e4::kSets * e4::kSet, n = (uint32_t)w.n_walks;
-    if (n == 0) return cudaSuccess;
     const uint32_t rounds = (n + full - 1) / full;
     const uint32_t gsz = (n + rounds * sms - 1) / (rounds * sms);
-    const uint32_t groups = (n + gsz - 1) / gsz;
-    k_walks_e4<<<groups < sms ? groups : sms, e4::kThreads, e4::smem_bytes, s>>>(w, gsz);
+    const uint32_t ctas = (n + gsz - 1) / gsz;
+    k_walks_e4<<<ctas < sms ? ctas : sms, e4::kThreads, e4::smem_bytes, s>>>(w, gsz);
     return cudaGetLastError();
 }
 

@@ -29,11 +29,11 @@ constexpr uint64_t kSeedU = 0x6A09E667F3BCC908ull;
 constexpr uint64_t kSeedH = 0xBB67AE8584CAA73Bull;
 
 // The n = 4 engine's rows (qcs_engine4.cu): lane l (5 bits: z0 z1 z2 x0 x1 of
-// the row's Pauli index) and t (3 bits: z3 x3 x2) to the row, and a Pauli
+// the row's Pauli index) and t (3 bits: x2 z3 x3) to the row, and a Pauli
 // index to its code, the same eight bits in that order (t above l).
 constexpr uint32_t row4(uint32_t l, uint32_t t)
 {
-    return (l & 7u) | (t & 1u) << 3 | ((l >> 3) & 3u) << 4 | ((t >> 2) & 1u) << 6 | ((t >> 1) & 1u) << 7;
+    return (l & 7u) | ((t >> 1) & 1u) << 3 | ((l >> 3) & 3u) << 4 | (t & 1u) << 6 | ((t >> 2) & 1u) << 7;
 }
 // A column of C^ suits the engine's f32 sums when the absolute values of its
 // entries add up to at most this: a partial sum of the product is below

@@ -1,5 +1,5 @@
 """The n = 4 engine (qcs_engine4.cu) against the dp4a kernels, bit for bit:
-group sizes around one and two rounds of every SM, levels with none to three
+walk counts around one and two rounds of every SM, levels with none to three
 stages beside the first and with and without the chunk's, targets whose C^ is
 sparse or near the largest column sums that the engine takes, and one beyond
 them, which the engine leaves to the dp4a kernels."""
@@ -36,10 +36,11 @@ def walk(dev, shape, t, k, walks, steps, dpb):
         return ws.cpu().numpy(), c[:4].tolist()
 
 
-# 48 walks to a group and one CTA per SM: 152 x 48 = 7296 walks are one full
-# round, 7297 two rounds of smaller groups
+# 72 slots (three sets of 24, 16 W points each at most) and one CTA per SM:
+# 152 x 72 = 10944 walks fill every slot, 10945 are two walks to most slots.
+# About 3 % of a full set's rounds have a point that waits for the next one.
 @pytest.mark.parametrize("t,k,walks,steps,dpb", [
-    (7, 7, 7296, 2, 3), (7, 7, 7297, 2, 12), (7, 7, 14593, 3, 1), (7, 7, 151, 2, 3), (7, 7, 3800, 2, 3),
+    (7, 7, 10944, 9, 3), (7, 7, 10945, 2, 12), (7, 7, 21889, 3, 1), (7, 7, 151, 2, 3), (7, 7, 3800, 2, 3),
     (0, 2, 100, 6, 2), (3, 3, 100, 6, 2), (5, 4, 100, 6, 2), (5, 5, 100, 6, 2), (7, 6, 100, 6, 2), (9, 8, 100, 6, 2),
     (9, 9, 100, 6, 2), (7, 15, 100, 4, 2), (13, 7, 500, 8, 2), (12, 13, 500, 8, 2), (15, 7, 500, 4, 2),
 ])
