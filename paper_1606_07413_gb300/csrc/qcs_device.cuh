@@ -141,5 +141,71 @@ __device__ void dp_insert(const WL &w, uint64_t dp, uint64_t ref, TallyOf<T> &c)
     }
 }
 
+constexpr uint32_t kMaxRewalkLen = 1u << 20; // longer trails are reported as no merge
+
+// A merge of a launch's work list: first the re-walks carried from the
+// previous launch or round, then this launch's queued merges.  The two states
+// with the steps each still has to the shared point, and their trails' chunks
+// (different ones: the same value reached in two chunks' functions, no merge).
+struct Merge {
+    uint64_t a, b;
+    uint32_t la, lb, ca, cb;
+};
+template <typename WL>
+__device__ __forceinline__ Merge load_merge(const WL &w, uint32_t p)
+{
+    Merge m;
+    if (p < w.pend_in_n) {
+        const Pending q = w.pend_in[p];
+        m.a = q.a;
+        m.b = q.b;
+        m.la = q.la;
+        m.lb = q.lb;
+        m.ca = m.cb = q.chunk;
+    } else {
+        const Pair P = w.queue[p - w.pend_in_n];
+        uint32_t wa, sa, wb, sb;
+        split_ref(P.ref_a, wa, sa, m.la);
+        split_ref(P.ref_b, wb, sb, m.lb);
+        m.a = trail_start(w.lv, wa, sa);
+        m.b = trail_start(w.lv, wb, sb);
+        m.ca = trail_chunk(w.lv, m.a);
+        m.cb = trail_chunk(w.lv, m.b);
+    }
+    return m;
+}
+
+// budget spent: carry the re-walk to the next launch or round (if there is room)
+template <typename WL>
+__device__ __forceinline__ void carry_merge(const WL &w, uint64_t a, uint32_t la, uint64_t b, uint32_t lb,
+                                            uint32_t chunk)
+{
+    const uint32_t idx = atomicAdd(w.pend_out_n, 1u);
+    if (idx < w.pend_cap) {
+        Pending q;
+        q.a = a;
+        q.b = b;
+        q.la = la;
+        q.lb = lb;
+        q.chunk = chunk;
+        q.pad = 0;
+        w.pend_out[idx] = q;
+    }
+}
+
+template <typename WL>
+__device__ __forceinline__ void append_claw(const WL &w, uint64_t a, uint64_t b, uint32_t chunk)
+{
+    const uint32_t idx = atomicAdd(w.ccount, 1u);
+    if (idx < w.ccap) {
+        Cand c;
+        c.a = a;
+        c.b = b;
+        c.chunk = chunk;
+        c.pad = 0;
+        w.cands[idx] = c;
+    }
+}
+
 } // namespace
 } // namespace qcs

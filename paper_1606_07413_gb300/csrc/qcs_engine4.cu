@@ -859,6 +859,183 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_e4(WalkLaunch w, uint
     }
 }
 
+// The re-walk of a level's merges (Sec. 3, Fig. 2; the same steps and classes
+// as rewalk_resume in qcs_walk.cu): slot lane * kSets + X re-walks merges
+// claimed one after the other from the device cursor, evaluating f at one
+// state a round: the longer trail until both are aligned, then a and b in
+// turn.  The next merge is claimed and its starts computed while the workers
+// run.  cnt: merges in the work list; slots: slots that take merges (a short
+// list is spread over all CTAs).  A merge to a warp with the dp4a step, a
+// search at level 6 (theta 1/2, 2^26 steps) took 240 ms; so it takes 109.
+__device__ __forceinline__ bool rewalk_control(const WalkLaunch &w, uint32_t cnt, uint32_t slots, const e4::Cta &c,
+                                               int X, int lane)
+{
+    using namespace e4;
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const LevelCtx &lv = w.lv;
+    const Stages sg(lv);
+    const bool mine = lane < kSet && (uint32_t)(lane * kSets + X) < slots;
+    uint32_t cls[6] = {0, 0, 0, 0, 0, 0}, ph = 0;
+    unsigned long long nf = 0;
+    uint64_t a = 0, b = 0, fa = 0, na = 0, nb = 0, cc = 0;
+    uint32_t la = 0, lb = 0, chunk = 0, nla = 0, nlb = 0, nchunk = 0, used = 0;
+    bool active = false, second = false, checked = false, have = false, more = mine, late = false, ok = true;
+    HashBase hb{};
+
+    // give every slot without a next merge one that needs an evaluation, as
+    // far as the list goes; the others are classified at once
+    auto fetch = [&]() {
+        for (;;) {
+            const bool need = more && !have;
+            const uint32_t m = __ballot_sync(kAll, need);
+            if (!m) break;
+            uint32_t base = 0;
+            if (lane == __ffs((int)m) - 1) base = atomicAdd(w.rw_next, (uint32_t)__popc(m));
+            base = __shfl_sync(kAll, base, __ffs((int)m) - 1);
+            if (need) {
+                const uint32_t p = base + (uint32_t)__popc(m & ((1u << lane) - 1u));
+                if (p >= cnt) {
+                    more = false;
+                } else {
+                    const Merge q = load_merge(w, p);
+                    const bool bad = q.ca != q.cb || q.la > kMaxRewalkLen || q.lb > kMaxRewalkLen;
+                    const bool hood = !bad && q.la == q.lb && q.a == q.b, none = bad || (!hood && (q.la | q.lb) == 0);
+                    cls[0] += hood;
+                    cls[5] += none;
+                    if (!hood && !none) {
+                        const bool sw = q.la < q.lb; // a is the longer trail
+                        na = sw ? q.b : q.a;
+                        nb = sw ? q.a : q.b;
+                        nla = sw ? q.lb : q.la;
+                        nlb = sw ? q.la : q.lb;
+                        nchunk = q.ca;
+                        have = true;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    };
+    // whether the merge goes on; if not it is classified or carried
+    auto settle = [&]() {
+        if (la == lb) {
+            if (second) return;
+            if (!checked) {
+                checked = true;
+                if (a == b) {
+                    cls[0]++; // Robin Hood
+                    active = false;
+                    return;
+                }
+            }
+            if (lb == 0) {
+                cls[5]++; // no merge
+                active = false;
+                return;
+            }
+        }
+        if (w.rewalk_budget && used + (la > lb ? 0u : 1u) >= w.rewalk_budget) {
+            carry_merge(w, a, la, b, lb, chunk);
+            active = false;
+        }
+    };
+    auto take = [&]() {
+        if (active || !have) return;
+        a = na;
+        b = nb;
+        la = nla;
+        lb = nlb;
+        chunk = nchunk;
+        hb = c.chunk_base()[chunk];
+        cc = sg.chunk_code(chunk);
+        used = 0;
+        second = checked = have = false;
+        active = true;
+        settle();
+    };
+    fetch();
+    take();
+    __syncwarp();
+    while (__any_sync(kAll, active || have)) {
+        const uint64_t x = second ? b : a;
+        const int side = (int)(x & 1);
+        uint32_t pos;
+        const bool go = publish(c, X, lane, active, late, side, sg.seq(side, rotations(x, lv), cc),
+                                side ? sg.ns_w : sg.ns_v, hb, &pos);
+        late = active && !go;
+        fetch();
+        if (!mbar_wait(c.bar_sums(X), ph)) {
+            ok = false;
+            break;
+        }
+        ph ^= 1u;
+        const uint64_t y = slot_hash(c, X, lane, go ? side : 0, pos) & lv.maskL;
+        if (go) {
+            used++;
+            nf++;
+            if (la > lb) {
+                a = y;
+                la--;
+                settle();
+            } else if (!second) {
+                fa = y;
+                second = true;
+            } else {
+                second = false;
+                if (fa == y) {
+                    const bool claw = ((a ^ b) & 1) != 0, same = rotations(a, lv) == rotations(b, lv);
+                    if (claw) append_claw(w, a, b, chunk);
+                    cls[1] += !claw && same; // trivial
+                    cls[2] += !claw && !same; // same side
+                    cls[3] += claw;
+                    active = false;
+                } else {
+                    a = fa;
+                    b = y;
+                    la--;
+                    lb--;
+                    settle();
+                }
+            }
+        }
+        take();
+        __syncwarp();
+    }
+    if (ok) publish_done(c, X, lane);
+    unsigned long long v[8] = {cls[0], cls[1], cls[2], cls[3], cls[4], cls[5], cls[3], nf};
+    const int idx[8] = {C_CLS0, C_CLS0 + 1, C_CLS0 + 2, C_CLS0 + 3, C_CLS0 + 4, C_CLS0 + 5, C_CANDS, C_RSTEPS};
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) v[i] += __shfl_xor_sync(kAll, v[i], o);
+        if (lane == 0 && v[i]) atomicAdd(&w.counters[idx[i]], v[i]);
+    }
+    return ok;
+}
+
+__global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_e4(WalkLaunch w)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const uint32_t cnt = w.pend_in_n + min(*w.qhead, w.qcap);
+    if (cnt <= blockIdx.x) return; // no merge for this CTA
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const e4::Cta c = e4::cta_begin(w.lv, smem_raw, true);
+    e4::load_c(w.lv, c);
+    __syncthreads();
+    e4::tmem_fence_after();
+    bool ok;
+    if (warp < e4::kWorkers) ok = e4::worker(w.lv, c, warp, lane);
+    else if (warp == e4::kMmaWarp) ok = e4::mma_warp(c);
+    else ok = rewalk_control(w, cnt, (cnt + gridDim.x - 1) / gridDim.x, c, warp - e4::kCtlWarp, lane);
+    if (!ok && lane == 0) atomicAdd(w.stall, 1u);
+    e4::tmem_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        e4::tmem_fence_after();
+        e4::tmem_dealloc(c.tmem);
+    }
+}
+
 } // namespace
 
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s)
@@ -874,6 +1051,16 @@ cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s)
     const uint32_t gsz = (n + rounds * sms - 1) / (rounds * sms);
     const uint32_t ctas = (n + gsz - 1) / gsz;
     k_walks_e4<<<ctas < sms ? ctas : sms, e4::kThreads, e4::smem_bytes, s>>>(w, gsz);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rewalk_e4(const WalkLaunch &w, cudaStream_t s)
+{
+    if (!w.stall || !w.rw_next) return cudaErrorInvalidValue;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_rewalk_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
+    if (e != cudaSuccess) return e;
+    k_rewalk_e4<<<(unsigned)num_sms(), e4::kThreads, e4::smem_bytes, s>>>(w);
     return cudaGetLastError();
 }
 

@@ -271,6 +271,8 @@ cudaError_t launch_init_walks(const WalkLaunch &w, cudaStream_t s);
 cudaError_t launch_walks(const WalkLaunch &w, cudaStream_t s);
 // n = 4 with lv.Cm set: the level walk on the tensor-core engine (qcs_engine4.cu)
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s);
+// the re-walk of a level's merges on the engine
+cudaError_t launch_rewalk_e4(const WalkLaunch &w, cudaStream_t s);
 int engine4_warps(); // warps of its CTA
 // DP-owner sharding: insert `count` distinguished points {dp, trail ref}
 // into w's table (merges queued as by the walk), and bin points by owner

@@ -90,7 +90,6 @@ __host__ __device__ constexpr int shape_min_blocks(int nq, int s)
 {
     return nq <= 2 ? 1 : nq == 3 ? (s == 1 ? 4 : s >= 2 ? 1 : QCS_MIN_BLOCKS3) : 1;
 }
-constexpr uint32_t kMaxRewalkLen = 1u << 20; // longer trails are reported as no merge
 
 template <int NQ>
 struct Geo {
@@ -771,43 +770,16 @@ __device__ __forceinline__ void rewalk_job(const WL &w, const Smem<NQ> &sm, uint
     for (uint32_t p = cursor ? claim() : p_begin; p < p_end; p = cursor ? claim() : p + p_stride) {
         // the job's work list: first the re-walks carried from the previous
         // round (batched search), then this launch's queued merges
-        uint64_t xa, xb;
-        uint32_t la, lb, ca, cb;
-        if (p < w.pend_in_n) {
-            const Pending q = w.pend_in[p];
-            xa = q.a;
-            xb = q.b;
-            la = q.la;
-            lb = q.lb;
-            ca = cb = q.chunk;
-        } else {
-            const Pair P = w.queue[p - w.pend_in_n];
-            uint32_t wa, sa, wb, sb;
-            split_ref(P.ref_a, wa, sa, la);
-            split_ref(P.ref_b, wb, sb, lb);
-            xa = trail_start(w.lv, wa, sa);
-            xb = trail_start(w.lv, wb, sb);
-            ca = trail_chunk(w.lv, xa);
-            cb = trail_chunk(w.lv, xb);
-        }
+        const Merge m = load_merge(w, p);
+        uint64_t xa = m.a, xb = m.b;
+        uint32_t la = m.la, lb = m.lb;
+        const uint32_t ca = m.ca;
         RewalkOut r;
-        if (ca != cb) { // the same value reached in two chunks' functions: no merge
+        if (ca != m.cb) { // the same value reached in two chunks' functions: no merge
             r.cls = 5;
         } else if (!rewalk_resume<NQ>(w.lv, ca, xa, la, xb, lb, w.rewalk_budget, sm, g, fev, r)) {
             // budget spent: carry the re-walk to the next round (if there is room)
-            if (g.sub == 0) {
-                const uint32_t idx = atomicAdd(w.pend_out_n, 1u);
-                if (idx < w.pend_cap) {
-                    Pending q;
-                    q.a = xa;
-                    q.b = xb;
-                    q.la = la;
-                    q.lb = lb;
-                    q.chunk = ca;
-                    q.pad = 0;
-                    w.pend_out[idx] = q;
-                }
-            }
+            if (g.sub == 0) carry_merge(w, xa, la, xb, lb, ca);
             continue;
         }
         c0 += r.cls == 0;
@@ -817,15 +789,7 @@ __device__ __forceinline__ void rewalk_job(const WL &w, const Smem<NQ> &sm, uint
         c4 += r.cls == 4;
         c5 += r.cls == 5;
         if (r.cls == 3 && g.sub == 0) {
-            const uint32_t idx = atomicAdd(w.ccount, 1u);
-            if (idx < w.ccap) {
-                Cand c;
-                c.a = r.a;
-                c.b = r.b;
-                c.chunk = ca;
-                c.pad = 0;
-                w.cands[idx] = c;
-            }
+            append_claw(w, r.a, r.b, ca);
         }
     }
     if (g.sub == 0) {
@@ -1112,6 +1076,10 @@ cudaError_t rewalk_batch_n(const BatchArgs &a, cudaStream_t s)
 template <int NQ>
 cudaError_t rewalk_pairs_n(const WalkLaunch &w, cudaStream_t s)
 {
+    // the engine is the faster one from a list of 32 merges on (6 merges: 51
+    // against 47 us; 130: 54 / 66; 17320: 115 / 193; 116090: 311 / 869 us at
+    // theta 1/2, 431 at 2^-8: 1.25 / 1.42 ms)
+    if (NQ == 4 && w.lv.Cm) return launch_rewalk_e4(w, s);
     cudaFuncSetAttribute(k_rewalk_pairs<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)Geo<NQ>::smem_bytes);
     k_rewalk_pairs<NQ><<<grid_for<NQ>(w.qcap), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(w);

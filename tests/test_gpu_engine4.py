@@ -49,3 +49,76 @@ def test_engine_walk_equals_the_dp4a_walk(dev, t, k, walks, steps, dpb):
     assert a[1][0] == walks * steps
     assert np.array_equal(a[0], b[0])
     assert a[1] == b[1]
+
+
+M64 = (1 << 64) - 1
+
+
+def smix(z):
+    z &= M64
+    z = ((z ^ (z >> 30)) * 0xBF58476D1CE4E5B9) & M64
+    z = ((z ^ (z >> 27)) * 0x94D049BB133111EB) & M64
+    return z ^ (z >> 31)
+
+
+def trail(ref, seed, version, n_chunks):
+    walk, seq, length = ref & ((1 << 24) - 1), (ref >> 24) & ((1 << 23) - 1), ref >> 47
+    start = smix(seed ^ smix((walk << 32) | seq) ^ (version << 40))
+    return start, (1 + smix(start ^ 0x5851F42D4C957F2D) % n_chunks if n_chunks else 0), length
+
+
+def classes(r):
+    return np.array([r["robin_hood"], r["trivial"], r["same_side"], r["claws"] + r["false_hash"], r["no_merge"]])
+
+
+# lists shorter than the CTAs, around one merge per slot and far longer, with
+# and without chunks, and an evaluation budget; levels below the target's
+# T-count, so no claw ends the host's check of candidates
+@pytest.mark.parametrize("k,dpb,walks,steps,budget", [
+    (4, 4, 400, 30, 0), (4, 4, 3000, 24, 0), (4, 1, 20000, 24, 0), (4, 7, 20000, 60, 0), (5, 3, 12000, 60, 0),
+    (2, 2, 5000, 8, 0), (4, 3, 6000, 24, 5),
+])
+def test_engine_rewalk_classes_equal_the_array_rewalk(dev, k, dpb, walks, steps, budget):
+    """Every merge of a launch, classified by the level's re-walk and, from its
+    two trails' recomputed starts, by qcs_rewalk (one lane group per pair)."""
+    gates, _ = W.seeded_target(4, 7, 4007)
+    version = 2
+    p = Q.default_params(4, walks=walks, table_log2=16, rewalk_budget=budget)
+    with Q.Problem.from_circuit(4, gates, 7, p) as prob:
+        prob.level_begin(k, version, dpb)
+        prob.level_walk(steps)
+        m = prob.level_merges()
+        prob.level_rewalk()
+        r = prob.level_collect()
+        launches = 1
+        while r["rewalk_carried"]:  # resumed first in the next launch
+            prob.level_walk(1)
+            m = np.concatenate([m, prob.level_merges()])
+            prob.level_rewalk()
+            r = prob.level_collect()
+            launches += 1
+            if launches == 6:
+                break
+        got, carried = classes(r), r["rewalk_carried"]
+        assert len(m) > (1000 if walks > 400 else 10) and r["queue_overflow"] == 0
+        assert got.sum() + carried == len(m)
+        if carried:
+            return
+        want = np.zeros(6, np.int64)
+        trails = [[trail(int(ref), p.seed, version, 255 if k & 1 else 0) for ref in row[:2]] for row in m]
+        by_chunk = {}
+        for ta, tb in trails:
+            if ta[1] != tb[1]:
+                want[5] += 1
+            else:
+                by_chunk.setdefault(ta[1], []).append((ta[0], ta[2], tb[0], tb[2]))
+        for chunk, rows in by_chunk.items():
+            x = np.array(rows, np.uint64)
+            sa, sb = (torch.from_numpy(np.ascontiguousarray(x[:, i]).view(np.int64)).to(dev) for i in (0, 2))
+            la, lb = (torch.from_numpy(x[:, i].astype(np.int32)).to(dev) for i in (1, 3))
+            cls = torch.empty(len(rows), dtype=torch.int32, device=dev)
+            ab = torch.empty(2 * len(rows), dtype=torch.int64, device=dev)
+            prob.rewalk(k, chunk, version, sa, la, sb, lb, cls, ab)
+            torch.cuda.synchronize()
+            want += np.bincount(cls.cpu().numpy(), minlength=6)
+        assert np.array_equal(got, [want[0], want[1], want[2], want[3] + want[4], want[5]])
