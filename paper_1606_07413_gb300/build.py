@@ -18,7 +18,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libqcs.so")
 
-SOURCES = ["qcs_walk.cu", "qcs_engine4.cu", "qcs_api.cpp", "qcs_exact.cpp", "qcs_noalloc.cu", "qcs_batch.cpp"]
+SOURCES = ["qcs_walk.cu", "qcs_engine4.cu", "qcs_certify.cu", "qcs_api.cpp", "qcs_exact.cpp", "qcs_noalloc.cu", "qcs_batch.cpp"]
 PEAK_SRC = "qcs_peak.cu"
 PEAK_LIB = os.path.join(BUILD, "libqcs_peak.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -33,7 +33,8 @@ def nvcc() -> str:
 
 def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
-    files += [os.path.join(CSRC, "qcs_internal.h"), os.path.join(CSRC, "qcs_device.cuh"), os.path.join(INCLUDE, "qcs.h"), __file__,
+    files += [os.path.join(CSRC, "qcs_internal.h"), os.path.join(CSRC, "qcs_device.cuh"),
+              os.path.join(CSRC, "qcs_rows.cuh"), os.path.join(INCLUDE, "qcs.h"), __file__,
               os.path.join(CSRC, PEAK_SRC), os.path.join(INCLUDE, "qcs_peak.h")]
     return files
 

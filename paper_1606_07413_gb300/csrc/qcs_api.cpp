@@ -184,13 +184,13 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64
                 for (uint32_t j = 0; j < D; j++) t1[(size_t)(qa - 1) * D + j] = ua[j] | (ub[j] << 16);
             }
             CK(upload(&tabs[side], t1));
-            if (n == 4) {
-                // the Pauli of code t << 5 | l is row4(l, t)
+            if (n >= 3) {
+                // the Pauli of code t << (2n - 3) | l is row_of(n, l, t)
                 std::vector<uint32_t> t4v((size_t)D * D);
                 for (uint32_t code = 0; code < D; code++) {
-                    const uint32_t q = row4(code & 31, code >> 5);
+                    const uint32_t q = row_of(n, code & (D / 8 - 1), code / (D / 8));
                     for (uint32_t i = 0; i < D; i++) {
-                        const uint32_t j = row4(i >> 3, i & 7);
+                        const uint32_t j = row_of(n, i >> 3, i & 7);
                         t4v[(size_t)code * D + i] = q ? t1[(size_t)(q - 1) * D + j] : (u0a[j] | u0b[j] << 16);
                     }
                 }
@@ -281,7 +281,7 @@ int upload_problem(qcs_problem *P)
                 for (int Q = 0; Q < D; Q++) {
                     int64_t sum = 0, abs_sum = 0;
                     for (int i = 0; i < D; i++) {
-                        const uint32_t j = row4((uint32_t)i >> 3, (uint32_t)i & 7);
+                        const uint32_t j = row_of(4, (uint32_t)i >> 3, (uint32_t)i & 7);
                         const int64_t a = P->C.a[(size_t)j * D + Q], b = P->C.b[(size_t)j * D + Q];
                         bytes[(size_t)Q * 2 * D + i] = (uint8_t)(a + 128);
                         bytes[(size_t)Q * 2 * D + D + i] = (uint8_t)(b + 128);
@@ -692,8 +692,9 @@ int qcs::cert_begin(qcs_problem *P, int k, cudaStream_t s, CertPass *c)
     c->slice = CertPass::kSliceMin;
     cudaError_t e = cudaMalloc(&a.table, sizeof(CertSlot) * slots);
     if (e == cudaSuccess) e = cudaMalloc(&a.pairs, sizeof(uint64_t) * 2 * CertPass::kCap);
-    if (e == cudaSuccess) e = cudaMalloc(&a.n_pairs, sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMallocHost(&c->hN, sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMalloc(&a.n_pairs, 2 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMallocHost(&c->hN, 2 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.n_pairs, 0, 2 * sizeof(uint32_t), s);
     if (e == cudaSuccess) e = cudaMallocHost(&c->hPairs, sizeof(uint64_t) * 2 * CertPass::kCap);
     if (e == cudaSuccess) e = cudaMemsetAsync(a.table, 0xFF, sizeof(CertSlot) * slots, s);
     if (e != cudaSuccess) {
@@ -746,9 +747,11 @@ int qcs::cert_advance(qcs_problem *P, CertPass *c, cudaStream_t s, uint64_t budg
         a.count = n;
         if ((e = cudaMemsetAsync(a.n_pairs, 0, sizeof(uint32_t), s)) != cudaSuccess) break;
         if ((e = launch_certify(a, s)) != cudaSuccess) break;
-        if ((e = cudaMemcpyAsync(c->hN, a.n_pairs, sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
+        if ((e = cudaMemcpyAsync(c->hN, a.n_pairs, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+            break;
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-        c->d2h += (int64_t)sizeof(uint32_t);
+        c->d2h += (int64_t)(2 * sizeof(uint32_t));
+        if (c->hN[1]) return QCS_ERR_DEVICE; // a bounded wait ran out (in this launch or in the stored side's)
         c->probed += n;
         *used += n * cost;
         if (n == c->slice) c->slice = std::min(2 * c->slice, CertPass::kSliceMax);

@@ -207,5 +207,116 @@ __device__ __forceinline__ void append_claw(const WL &w, uint64_t a, uint64_t b,
     }
 }
 
+// The nd low base-xi digits of v, digit j in byte j (xi <= 255).
+__device__ __forceinline__ uint64_t base_xi_digits(uint64_t v, uint32_t xi, int nd)
+{
+    uint64_t r = 0;
+    for (int j = 0; j < nd; j++) {
+        r |= (v % xi) << (8 * j);
+        v /= xi;
+    }
+    return r;
+}
+
+// (d + s) mod xi^nd on packed base-xi digits (digit j in byte j, nd <= 8).
+__device__ __forceinline__ uint64_t add_base_xi(uint64_t d, uint64_t s, uint32_t xi, int nd)
+{
+    uint64_t r = 0;
+    uint32_t carry = 0;
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        if (j < nd) {
+            uint32_t t = (uint32_t)((d >> (8 * j)) & 0xFFu) + (uint32_t)((s >> (8 * j)) & 0xFFu) + carry;
+            carry = t >= xi ? 1u : 0u;
+            t -= carry * xi;
+            r |= (uint64_t)t << (8 * j);
+        }
+    }
+    return r;
+}
+
+// Exhaustive pass: the key table.  A key's slots are s, s + d, s + 2d, .. with
+// a step d of its own (odd, so the sequence meets every slot); it goes to the
+// first empty one, and at most half of the table is full, so there is one.
+// The step matters: a point with two equal neighbouring rotations is in the
+// coset of the rest, so at h = 3 each single rotation's key is stored some 640
+// times.  In one run of slots they held up every probe that met the run
+// (16.6 M probes of a 2^25-slot table: 110 ms on the n = 4 engine, 12 ms with
+// steps).
+struct CertProbe {
+    uint64_t s, d;
+    __device__ __forceinline__ CertProbe(uint64_t key, uint64_t mask)
+    {
+        const uint64_t z = smix(key);
+        s = z & mask;
+        d = (z >> 32) | 1u;
+    }
+};
+
+__device__ __forceinline__ bool cert_put(const CertArgs &a, uint64_t slot, uint64_t key, uint64_t idx)
+{
+    if (atomicCAS(reinterpret_cast<unsigned long long *>(&a.table[slot].key), ~0ull, (unsigned long long)key) != ~0ull)
+        return false;
+    a.table[slot].idx = idx;
+    return true;
+}
+
+__device__ __forceinline__ void cert_insert(const CertArgs &a, uint64_t key, uint64_t idx)
+{
+    CertProbe p(key, a.mask);
+    for (uint64_t probe = 0; probe <= a.mask; probe++, p.s = (p.s + p.d) & a.mask)
+        if (cert_put(a, p.s, key, idx)) return;
+}
+
+// The same for a whole warp, a point to a valid lane: after a few tries the
+// warp looks for each remaining lane's empty slot together, 32 slots at a
+// time (the 640th copy of a key alone: as many dependent exchanges; 16.6 M
+// points at n = 4: 35 ms lane by lane, 7 ms so).
+__device__ __forceinline__ void cert_insert_warp(const CertArgs &a, bool valid, uint64_t key, uint64_t idx, int lane)
+{
+    CertProbe p(key, a.mask);
+    bool left = valid;
+    for (int probe = 0; probe < 6 && left; probe++, p.s = (p.s + p.d) & a.mask) left = !cert_put(a, p.s, key, idx);
+    __syncwarp();
+    uint32_t todo;
+    while ((todo = __ballot_sync(0xFFFFFFFFu, left)) != 0) {
+        const int src = __ffs((int)todo) - 1;
+        const uint64_t d = __shfl_sync(0xFFFFFFFFu, p.d, src);
+        uint64_t at = __shfl_sync(0xFFFFFFFFu, p.s, src);
+        for (uint64_t probe = 0; probe <= a.mask; probe += 32) {
+            const uint64_t k =
+                *reinterpret_cast<volatile const uint64_t *>(&a.table[(at + d * (uint64_t)lane) & a.mask].key);
+            uint32_t empty = __ballot_sync(0xFFFFFFFFu, k == ~0ull);
+            bool done = false;
+            while (empty && !done) { // another warp may take the slot first
+                const uint64_t slot = (at + d * (uint64_t)(__ffs((int)empty) - 1)) & a.mask;
+                if (lane == src) done = cert_put(a, slot, key, idx);
+                done = __shfl_sync(0xFFFFFFFFu, done, src);
+                empty &= empty - 1;
+            }
+            if (done) break;
+            at = (at + 32 * d) & a.mask;
+        }
+        if (lane == src) left = false;
+    }
+}
+
+// a probing point's matches are queued
+__device__ __forceinline__ void cert_probe(const CertArgs &a, uint64_t key, uint64_t idx)
+{
+    CertProbe p(key, a.mask);
+    for (uint64_t probe = 0; probe <= a.mask; probe++, p.s = (p.s + p.d) & a.mask) {
+        const uint64_t k2 = a.table[p.s].key;
+        if (k2 == ~0ull) return;
+        if (k2 == key) {
+            const uint32_t n = atomicAdd(a.n_pairs, 1u);
+            if (n < a.cap) {
+                a.pairs[2 * (size_t)n] = a.table[p.s].idx;
+                a.pairs[2 * (size_t)n + 1] = idx;
+            }
+        }
+    }
+}
+
 } // namespace
 } // namespace qcs

@@ -52,6 +52,7 @@
 
 #include "qcs_device.cuh"
 #include "qcs_internal.h"
+#include "qcs_rows.cuh"
 
 namespace qcs {
 namespace {
@@ -77,11 +78,6 @@ struct alignas(16) Job {
     uint32_t info;  // stages | side << 8 | row pair << 16, or kInvalid
     uint64_t pad;
 };
-struct alignas(16) HashBase { // the hash base of a W row pair, for phase E
-    uint64_t PH;
-    uint32_t pre16, pad;
-};
-
 // shared memory
 constexpr size_t off_A = 0;                                        // C^, second half, K-blocks 8..31: 6 chunks of 64 K
 constexpr size_t off_B = off_A + 6 * 16384;                        // [set]: 8 chunks of 64 K x 48 rows
@@ -100,8 +96,6 @@ static_assert(smem_bytes <= 227 * 1024, "shared memory of the n = 4 engine");
 
 // a bounded wait gives up after this many SM clock cycles (about two seconds)
 constexpr long long kWaitCycles = 1ll << 32;
-
-constexpr uint64_t kC1 = 0xBF58476D1CE4E5B9ull, kC2 = 0x94D049BB133111EBull; // SplitMix64's finaliser
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -223,126 +217,7 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar)
                  : "memory");
 }
 
-// ---- one point on one warp
-//
-// Lane l holds the eight weight rows row4(l, t) (qcs_internal.h): t carries
-// qubit 2's x bit and qubit 3, the lane the rest, and a Pauli's code (code_of)
-// is laid out the same way: its low five bits are its lane part, its high
-// three its t part.  A stage takes row j to u_j +- u_{j^p} or to sqrt2 u_j, by
-// lambda(p, j) in P(p) P(j) = i^lambda P(p^j), which is a sum over the qubits.
-// So with the t part of p known at compile time (a switch over its eight
-// values) the partner's register and qubit 3's share of lambda are constants,
-// and what is left of lambda is one value per lane and x bit of qubit 2: a
-// word of the stage table, which does not depend on p's qubit 3.  About 85
-// instructions a stage; with the signs and selections looked up row by row it
-// was 106.
-
-__host__ __device__ constexpr int lambda1(int px, int pz, int x, int z)
-{
-    return (px * pz + x * z + 2 * pz * x - (px ^ x) * (pz ^ z)) & 3;
-}
-
-// lambda of the lane's rows but for qubit 3's share, for x bit x2 = 0, 1 of
-// qubit 2: byte x2 is the sign (lambda 0 or 1: +1, 2 or 3: -1; for W the
-// other way round), byte 2 + x2 whether lambda is odd
-__device__ __forceinline__ uint32_t stage_word(uint32_t side, uint32_t code, uint32_t l)
-{
-    // lane bits: z0 z1 z2 x0 x1; code bits: the same, then x2
-    int v = 0;
-#pragma unroll
-    for (int q = 0; q < 2; q++)
-        v += lambda1((code >> (3 + q)) & 1, (code >> q) & 1, (l >> (3 + q)) & 1, (l >> q) & 1);
-    uint32_t w = 0;
-#pragma unroll
-    for (int x = 0; x < 2; x++) {
-        const uint32_t a = (uint32_t)(v + lambda1((code >> 5) & 1, (code >> 2) & 1, x, (l >> 2) & 1)) & 3u;
-        w |= (((a >> 1) ^ side) ? 0xFFu : 1u) << (8 * x) | (a & 1u) << (16 + 8 * x);
-    }
-    return w;
-}
-
-// (na, nb) = ODD == (odd != 0) ? (ub, 2 ua) : (ua + s va, ub + s vb)
-template <bool ODD>
-__device__ __forceinline__ void row_update(uint32_t &ua, uint32_t &ub, uint32_t va, uint32_t vb, uint32_t s,
-                                           uint32_t odd)
-{
-    uint32_t na, nb;
-    if (ODD)
-        asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %7, 0;\n\tmov.b32 %0, %5;\n\tadd.u32 %1, %4, %4;\n\t"
-            "@p mad.lo.u32 %0, %2, %6, %4;\n\t@p mad.lo.u32 %1, %3, %6, %5;\n\t}"
-            : "=&r"(na), "=&r"(nb)
-            : "r"(va), "r"(vb), "r"(ua), "r"(ub), "r"(s), "r"(odd));
-    else
-        asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %7, 0;\n\tmov.b32 %0, %5;\n\tadd.u32 %1, %4, %4;\n\t"
-            "@p mad.lo.u32 %0, %2, %6, %4;\n\t@p mad.lo.u32 %1, %3, %6, %5;\n\t}"
-            : "=&r"(na), "=&r"(nb)
-            : "r"(va), "r"(vb), "r"(ua), "r"(ub), "r"(s), "r"(odd));
-    ua = na;
-    ub = nb;
-}
-
-// the stage of a Pauli whose t part is PT; s, odd: the lane's sign and parity
-// of lambda per x bit of qubit 2, without qubit 3's share
-template <int PT>
-__device__ __forceinline__ void stage_rows(uint32_t (&ua)[8], uint32_t (&ub)[8], int pl, const int (&s)[2],
-                                           const uint32_t (&odd)[2])
-{
-    uint32_t va[8], vb[8];
-#pragma unroll
-    for (int t = 0; t < 8; t++) {
-        va[t] = __shfl_xor_sync(0xFFFFFFFFu, ua[t ^ PT], pl);
-        vb[t] = __shfl_xor_sync(0xFFFFFFFFu, ub[t ^ PT], pl);
-    }
-    const int neg[2] = {-s[0], -s[1]};
-#pragma unroll
-    for (int t = 0; t < 8; t++) {
-        // qubit 3's share of lambda: 0, 1 or 3 (3: the sign turns)
-        const int x2 = t & 1, c = lambda1((PT >> 2) & 1, (PT >> 1) & 1, (t >> 2) & 1, (t >> 1) & 1);
-        const uint32_t sg = (uint32_t)(c == 3 ? neg[x2] : s[x2]);
-        if (c & 1) row_update<true>(ua[t], ub[t], va[t], vb[t], sg, odd[x2]);
-        else row_update<false>(ua[t], ub[t], va[t], vb[t], sg, odd[x2]);
-    }
-}
-
-// side: 0 for V (adjoint of R^), 1 for W (adjoint of R^T)
-__device__ __forceinline__ void stage(uint32_t code, uint32_t side, const uint32_t *tab, int lane, uint32_t (&ua)[8],
-                                      uint32_t (&ub)[8])
-{
-    const uint32_t w = tab[(side << 6 | (code & 63u)) * 32 + lane];
-    const int pl = (int)(code & 31u);
-    const int s[2] = {(int)(int8_t)w, (int)(int8_t)(w >> 8)};
-    const uint32_t odd[2] = {w & 0xFF0000u, w & 0xFF000000u};
-    switch (code >> 5) {
-    case 0: stage_rows<0>(ua, ub, pl, s, odd); break;
-    case 1: stage_rows<1>(ua, ub, pl, s, odd); break;
-    case 2: stage_rows<2>(ua, ub, pl, s, odd); break;
-    case 3: stage_rows<3>(ua, ub, pl, s, odd); break;
-    case 4: stage_rows<4>(ua, ub, pl, s, odd); break;
-    case 5: stage_rows<5>(ua, ub, pl, s, odd); break;
-    case 6: stage_rows<6>(ua, ub, pl, s, odd); break;
-    default: stage_rows<7>(ua, ub, pl, s, odd); break;
-    }
-}
-
-// smix(base ^ phi) of one column, phi the sign-folded low 16 bits of l, given
-// pre = base ^ (base >> 30) as PH = (pre & ~0xFFFF) * kC1 and pre16 = pre &
-// 0xFFFF: (pre ^ phi) * kC1 = PH + (pre16 ^ phi) * kC1, and the second
-// product has a 16-bit factor.
-__device__ __forceinline__ uint64_t column_hash(uint32_t l, uint64_t PH, uint32_t pre16)
-{
-    const int s = (int)(int16_t)(uint16_t)l;
-    const uint32_t x = (uint32_t)abs(s) ^ pre16;
-    uint64_t z = (uint64_t)x * (uint32_t)kC1 + PH;
-    z += (uint64_t)(x * (uint32_t)(kC1 >> 32)) << 32;
-    z = (z ^ (z >> 27)) * kC2;
-    return z ^ (z >> 31);
-}
-
-__device__ __forceinline__ HashBase hash_base(uint64_t base)
-{
-    const uint64_t pre = base ^ (base >> 30);
-    return HashBase{(pre & ~0xFFFFull) * kC1, (uint32_t)pre & 0xFFFFu, 0};
-}
+// ---- one point on one warp (the rows and stages of qcs_rows.cuh, n = 4)
 
 // sum mod 2^64 over the warp from three 32-bit reductions (see group_sum64 in qcs_walk.cu)
 __device__ __forceinline__ uint64_t warp_sum64(uint64_t acc)
@@ -352,18 +227,6 @@ __device__ __forceinline__ uint64_t warp_sum64(uint64_t acc)
     const uint32_t s_l0 = __reduce_add_sync(0xFFFFFFFFu, lo & 0xFFFFu);
     const uint32_t s_l1 = __reduce_add_sync(0xFFFFFFFFu, lo >> 16);
     return ((uint64_t)s_hi << 32) + ((uint64_t)s_l1 << 16) + (uint64_t)s_l0;
-}
-
-// the weights after the first stage of a point (LevelCtx::T4), as two 16-byte
-// loads; the upper halves of ua are never looked at (every sum is mod 2^16)
-__device__ __forceinline__ void first_stage(const uint4 *tab, uint32_t code, int lane, uint32_t (&ua)[8],
-                                            uint32_t (&ub)[8])
-{
-    const uint4 w0 = __ldg(tab + (code * 32 + lane) * 2), w1 = __ldg(tab + (code * 32 + lane) * 2 + 1);
-    ua[0] = w0.x; ua[1] = w0.y; ua[2] = w0.z; ua[3] = w0.w;
-    ua[4] = w1.x; ua[5] = w1.y; ua[6] = w1.z; ua[7] = w1.w;
-#pragma unroll
-    for (int t = 0; t < 8; t++) ub[t] = ua[t] >> 16;
 }
 
 // The multiset sum of a V point: its weights, scaled by sqrt2^ev, are its
@@ -386,12 +249,6 @@ __device__ __forceinline__ uint64_t v_column_sum(const uint32_t (&ua)[8], const 
     return warp_sum64(acc);
 }
 
-// Pauli codes (row4's bit order) of four Pauli indices, one per byte
-__device__ __forceinline__ uint32_t codes_of(uint32_t q)
-{
-    return (q & 0x87878787u) | ((q >> 1) & 0x38383838u) | ((q << 3) & 0x40404040u);
-}
-
 // The stages of a point in order, a code per byte: V takes q_h first and goes
 // down to q_1; W takes q_1 .. q_h, then the chunk.  A product of no rotations
 // starts from code 0, the untouched weights; so does V's single rotation (its
@@ -412,12 +269,12 @@ struct Stages {
     }
     __device__ __forceinline__ uint64_t chunk_code(uint32_t chunk) const
     {
-        return (uint64_t)codes_of(chunk) << sh_c; // chunk < 256
+        return (uint64_t)codes_of<4>(chunk) << sh_c; // chunk < 256
     }
     // q: the indices, q_1 in the lowest byte; cc: chunk_code
     __device__ __forceinline__ uint64_t seq(int side, uint64_t q, uint64_t cc) const
     {
-        const uint32_t lo = codes_of((uint32_t)q), hi = codes_of((uint32_t)(q >> 32));
+        const uint32_t lo = codes_of<4>((uint32_t)q), hi = codes_of<4>((uint32_t)(q >> 32));
         if (side) return (((uint64_t)hi << 32) | lo) | cc;
         if (h == 0) return 0;
         const uint64_t rev = ((uint64_t)__byte_perm(lo, 0, 0x0123) << 32) | __byte_perm(hi, 0, 0x0123);
@@ -463,7 +320,7 @@ __device__ __forceinline__ Cta cta_begin(const LevelCtx &lv, unsigned char *raw,
     }
     uint32_t *tab = reinterpret_cast<uint32_t *>(raw + off_stage);
     for (int i = threadIdx.x; i < 2 * 64 * 32; i += kThreads)
-        tab[i] = stage_word((uint32_t)i >> 11, ((uint32_t)i >> 5) & 63u, (uint32_t)i & 31u);
+        tab[i] = stage_word<4>((uint32_t)i >> 11, ((uint32_t)i >> 5) & 63u, (uint32_t)i & 31u);
     if (with_chunks) {
         // base(chunk) = smix(smix(seed_H ^ version) ^ (n | k << 8 | chunk << 16 | K << 32))
         const uint64_t vmix = smix(kSeedH ^ (uint64_t)lv.version);
@@ -537,10 +394,10 @@ __device__ __forceinline__ void point_a(const LevelCtx &lv, const Cta &c, int X,
     const uint32_t side = (info >> 8) & 1u, ns = info & 0xFFu;
     const uint32_t *tab = reinterpret_cast<const uint32_t *>(c.raw + off_stage);
     uint32_t ua[8], ub[8];
-    first_stage(lv.T4[side], (uint32_t)seq & 0xFFu, lane, ua, ub);
+    first_stage<4>(lv.T4[side], (uint32_t)seq & 0xFFu, lane, ua, ub);
 #pragma unroll 1
     for (uint32_t i = 1; i < ns; i++)
-        stage(__shfl_sync(0xFFFFFFFFu, (uint32_t)(seq >> (8 * i)) & 0xFFu, 0), side, tab, lane, ua, ub);
+        stage<4>(__shfl_sync(0xFFFFFFFFu, (uint32_t)(seq >> (8 * i)) & 0xFFu, 0), side, tab, lane, ua, ub);
     if (side == 0) {
         const uint64_t sum = v_column_sum(ua, ub, lv.ev, jp->PH, jp->pre16, lane);
         if (lane == 0) c.vsum(X)[slot] = sum;
@@ -1036,6 +893,79 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_e4(WalkLaunch w)
     }
 }
 
+// W points of the exhaustive pass: the set takes kPairs points a round (all
+// of them need a row pair; which of its slots they sit on turns with the set,
+// so that every worker has two points a round), inserts or probes the last
+// round's keys and counts its indices on while the workers run.
+__device__ __forceinline__ bool certify_control(const CertArgs &a, const e4::Cta &c, int X, int lane)
+{
+    using namespace e4;
+    const Stages sg(a.lv);
+    const int my = (lane + kSet - (kSet - kPairs) * X) % kSet, h = a.lv.h;
+    const bool mine = lane < kSet && my < kPairs, has_chunk = (a.lv.k & 1) != 0;
+    const int nd = h + (has_chunk ? 1 : 0);
+    const uint64_t hmask = h >= 8 ? ~0ull : (1ull << (8 * h)) - 1;
+    const uint64_t stride = (uint64_t)gridDim.x * kSets * kPairs;
+    uint64_t i = ((uint64_t)blockIdx.x * kSets + (uint64_t)X) * kPairs + (uint64_t)my;
+    // While i + stride < count, the stride is below xi^nd and its nd digits
+    // are exact; otherwise the slot ends before the sum is used.
+    const uint64_t sdig = base_xi_digits(stride, 255, nd);
+    uint64_t dig = mine && i < a.count ? base_xi_digits(a.first + i, 255, nd) : 0;
+    const HashBase hb = hash_base(a.base);
+    uint64_t key = 0, idx = 0;
+    uint32_t ph = 0;
+    bool have = false, valid = mine && i < a.count, ok = true;
+    while (__any_sync(0xFFFFFFFFu, valid)) {
+        const uint64_t q = (dig & hmask) + (0x0101010101010101ull & hmask);
+        const uint32_t chunk = has_chunk ? (uint32_t)((dig >> (8 * h)) & 0xFFu) + 1 : 0u;
+        uint32_t pos;
+        publish(c, X, lane, valid, false, 1, sg.seq(1, q, has_chunk ? sg.chunk_code(chunk) : 0), sg.ns_w, hb, &pos);
+        if (a.insert) cert_insert_warp(a, have, key, idx, lane);
+        else if (have) cert_probe(a, key, idx);
+        __syncwarp();
+        have = valid;
+        idx = a.first + i;
+        i += stride;
+        valid = mine && i < a.count;
+        dig = add_base_xi(dig, sdig, 255, nd);
+        if (!mbar_wait(c.bar_sums(X), ph)) {
+            ok = false;
+            break;
+        }
+        ph ^= 1u;
+        key = slot_hash(c, X, lane, have ? 1 : 0, pos);
+        if (key == ~0ull) key = ~0ull - 1; // ~0 marks an empty slot
+    }
+    if (ok) {
+        if (a.insert) cert_insert_warp(a, have, key, idx, lane);
+        else if (have) cert_probe(a, key, idx);
+        __syncwarp();
+        publish_done(c, X, lane);
+    }
+    return ok;
+}
+
+__global__ void __launch_bounds__(e4::kThreads, 1) k_certify_e4(CertArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const e4::Cta c = e4::cta_begin(a.lv, smem_raw, false);
+    e4::load_c(a.lv, c);
+    __syncthreads();
+    e4::tmem_fence_after();
+    bool ok;
+    if (warp < e4::kWorkers) ok = e4::worker(a.lv, c, warp, lane);
+    else if (warp == e4::kMmaWarp) ok = e4::mma_warp(c);
+    else ok = certify_control(a, c, warp - e4::kCtlWarp, lane);
+    if (!ok && lane == 0) atomicAdd(a.n_pairs + 1, 1u);
+    e4::tmem_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        e4::tmem_fence_after();
+        e4::tmem_dealloc(c.tmem);
+    }
+}
+
 } // namespace
 
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s)
@@ -1061,6 +991,17 @@ cudaError_t launch_rewalk_e4(const WalkLaunch &w, cudaStream_t s)
         cudaFuncSetAttribute(k_rewalk_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
     if (e != cudaSuccess) return e;
     k_rewalk_e4<<<(unsigned)num_sms(), e4::kThreads, e4::smem_bytes, s>>>(w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_certify_e4(const CertArgs &a, cudaStream_t s)
+{
+    if (a.count == 0) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_certify_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
+    if (e != cudaSuccess) return e;
+    const uint64_t ctas = (a.count + e4::kSets * e4::kPairs - 1) / (e4::kSets * e4::kPairs), sms = (uint64_t)num_sms();
+    k_certify_e4<<<(unsigned)(ctas < sms ? ctas : sms), e4::kThreads, e4::smem_bytes, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -28,12 +28,15 @@ constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
 constexpr uint64_t kSeedU = 0x6A09E667F3BCC908ull;
 constexpr uint64_t kSeedH = 0xBB67AE8584CAA73Bull;
 
-// The n = 4 engine's rows (qcs_engine4.cu): lane l (5 bits: z0 z1 z2 x0 x1 of
-// the row's Pauli index) and t (3 bits: x2 z3 x3) to the row, and a Pauli
-// index to its code, the same eight bits in that order (t above l).
-constexpr uint32_t row4(uint32_t l, uint32_t t)
+// Rows on lanes (qcs_rows.cuh): lane l (2n - 3 bits: z_0 .. z_(n-2), then x_0
+// .. x_(n-3) of the row's Pauli index) and t (3 bits: x_(n-2), z_(n-1),
+// x_(n-1)) to the row, and a Pauli's code, the same bits in that order (t
+// above l).  n >= 2.
+__host__ __device__ constexpr uint32_t row_of(int n, uint32_t l, uint32_t t)
 {
-    return (l & 7u) | ((t >> 1) & 1u) << 3 | ((l >> 3) & 3u) << 4 | (t & 1u) << 6 | ((t >> 2) & 1u) << 7;
+    const uint32_t z = (l & ((1u << (n - 1)) - 1u)) | ((t >> 1) & 1u) << (n - 1);
+    const uint32_t x = (l >> (n - 1)) | (t & 1u) << (n - 2) | ((t >> 2) & 1u) << (n - 1);
+    return x << n | z;
 }
 // A column of C^ suits the engine's f32 sums when the absolute values of its
 // entries add up to at most this: a partial sum of the product is below
@@ -57,12 +60,12 @@ struct LevelCtx {
     // n = 4, when C^ suits the tensor-core engine (qcs_engine4.cu), else null:
     // every entry as the byte entry + 128, 512 bytes a column.  Byte
     // part * 256 + 8 l + t of column Q is the a (part 0) or b (part 1) of row
-    // row4(l, t).  Csum[Q]: the sum of the column's entries.
+    // row_of(4, l, t).  Csum[Q]: the sum of the column's entries.
     const uint4 *Cm;
     const int16_t *Csum;
-    // n = 4: the weights after the first adjoint stage (as T1), for the
-    // engine: word (code * 32 + l) * 8 + t is row row4(l, t)'s Ua | Ub << 16
-    // after the Pauli of that code (code4); code 0 holds the weights themselves.
+    // n >= 3: the weights after the first adjoint stage, as T1, by code: word
+    // code * 4^n + 8 l + t is row row_of(n, l, t)'s Ua | Ub << 16 after the
+    // Pauli of that code; code 0 holds the weights themselves.
     const uint4 *T4[2];
     const uint2 *U;    // fingerprint weights (Ua, Ub) per row, 4^n
     // The weights after the first adjoint stage of a side (index 0: V, 1: W),
@@ -222,10 +225,13 @@ struct CertArgs {
     CertSlot *table;
     uint64_t mask;     // table slots - 1 (a power of two, at least twice the stored points)
     uint64_t *pairs;   // key matches (stored index, probing index)
-    uint32_t *n_pairs; // matches found (may exceed cap; only cap are stored)
+    uint32_t *n_pairs; // [0] matches found (may exceed cap; only cap are stored); [1] the engine's bounded
+                       // waits that ran out (the points are then not all evaluated)
     uint32_t cap;
 };
 cudaError_t launch_certify(const CertArgs &a, cudaStream_t s);
+cudaError_t launch_certify_v(const CertArgs &a, cudaStream_t s); // V points at n >= 3 (qcs_certify.cu)
+cudaError_t launch_certify_e4(const CertArgs &a, cudaStream_t s); // W points at n = 4 with lv.Cm set (qcs_engine4.cu)
 // Host driver of the exhaustive pass (qcs_certify_level); *got = verified claw.
 int certify_level(::qcs_problem *P, int k, cudaStream_t s, bool *got);
 
@@ -319,7 +325,7 @@ int pauli_phase(int n, uint32_t p, uint32_t q); // P(p)P(q) = i^lambda P(p^q)
 // device tables of the first adjoint stage (LevelCtx::T1), built once per
 // device and qubit count and kept for the life of the process
 // (*uploaded, when given, grows by the bytes this call copied to the device)
-// (t4: LevelCtx::T4, null unless n = 4)
+// (t4: LevelCtx::T4, null below n = 3)
 int stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64_t *uploaded = nullptr);
 
 // How a level is walked (Sec. 3 and Appendix): theta, the launch shape, the
@@ -359,7 +365,7 @@ struct qcs_problem {
     uint32_t *dCq = nullptr; // n >= 3, when every entry of C^ fits in int8
     uint32_t *dCm = nullptr; // n = 4, when C^ suits the tensor-core engine: LevelCtx::Cm, then Csum
     const uint32_t *dT1[2] = {nullptr, nullptr}; // shared stage tables
-    const uint32_t *dT4[2] = {nullptr, nullptr}; // and their n = 4 engine form (LevelCtx::T4)
+    const uint32_t *dT4[2] = {nullptr, nullptr}; // and their form by code (LevelCtx::T4)
     uint32_t *dCoef = nullptr;
     qcs::Slot *dTable = nullptr;
     qcs::Pair *dQueue = nullptr;

@@ -867,34 +867,6 @@ __global__ void __launch_bounds__(Geo<NQ>::THREADS) k_rewalk_arrays(LevelCtx lv,
     }
 }
 
-// The nd low base-xi digits of v, digit j in byte j (xi <= 255).
-__device__ __forceinline__ uint64_t base_xi_digits(uint64_t v, uint32_t xi, int nd)
-{
-    uint64_t r = 0;
-    for (int j = 0; j < nd; j++) {
-        r |= (v % xi) << (8 * j);
-        v /= xi;
-    }
-    return r;
-}
-
-// (d + s) mod xi^nd on packed base-xi digits (digit j in byte j, nd <= 8).
-__device__ __forceinline__ uint64_t add_base_xi(uint64_t d, uint64_t s, uint32_t xi, int nd)
-{
-    uint64_t r = 0;
-    uint32_t carry = 0;
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-        if (j < nd) {
-            uint32_t t = (uint32_t)((d >> (8 * j)) & 0xFFu) + (uint32_t)((s >> (8 * j)) & 0xFFu) + carry;
-            carry = t >= xi ? 1u : 0u;
-            t -= carry * xi;
-            r |= (uint64_t)t << (8 * j);
-        }
-    }
-    return r;
-}
-
 // Exhaustive level pass (CertArgs): one lane group per point, grid-stride.
 // VONLY: the points are V products (a.side == 0), which never touch C^, so
 // the CTA stages the smaller layout without it.  A point index is nd base-xi
@@ -929,32 +901,8 @@ __global__ void __launch_bounds__(Geo<NQ>::THREADS) k_certify(CertArgs a)
         uint64_t key = coset_hash<NQ>(side, qpack, chunk, a.base, a.lv, sm, g);
         if (key == ~0ull) key = ~0ull - 1; // ~0 marks an empty slot
         if (g.sub == 0) {
-            uint64_t s = smix(key) & a.mask;
-            if (a.insert) {
-                // the table is at most half full, so an empty slot is always found
-                for (uint64_t probe = 0; probe <= a.mask; probe++) {
-                    const unsigned long long prev = atomicCAS(
-                        reinterpret_cast<unsigned long long *>(&a.table[s].key), ~0ull, (unsigned long long)key);
-                    if (prev == ~0ull) {
-                        a.table[s].idx = idx;
-                        break;
-                    }
-                    s = (s + 1) & a.mask;
-                }
-            } else {
-                for (uint64_t probe = 0; probe <= a.mask; probe++) {
-                    const uint64_t k2 = a.table[s].key;
-                    if (k2 == ~0ull) break;
-                    if (k2 == key) {
-                        const uint32_t n = atomicAdd(a.n_pairs, 1u);
-                        if (n < a.cap) {
-                            a.pairs[2 * (size_t)n] = a.table[s].idx;
-                            a.pairs[2 * (size_t)n + 1] = idx;
-                        }
-                    }
-                    s = (s + 1) & a.mask;
-                }
-            }
+            if (a.insert) cert_insert(a, key, idx);
+            else cert_probe(a, key, idx);
         }
         __syncwarp(g.mask);
     }
@@ -1119,7 +1067,12 @@ cudaError_t certify_nv(const CertArgs &a, cudaStream_t s)
 template <int NQ>
 cudaError_t certify_n(const CertArgs &a, cudaStream_t s)
 {
-    return a.side == 0 ? certify_nv<NQ, true>(a, s) : certify_nv<NQ, false>(a, s);
+    if constexpr (NQ == 4)
+        if (a.side == 1 && a.lv.Cm) return launch_certify_e4(a, s);
+    if constexpr (NQ >= 3)
+        return a.side == 0 ? launch_certify_v(a, s) : certify_nv<NQ, false>(a, s);
+    else
+        return a.side == 0 ? certify_nv<NQ, true>(a, s) : certify_nv<NQ, false>(a, s);
 }
 
 } // namespace
