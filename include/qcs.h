@@ -115,10 +115,10 @@ typedef struct qcs_params {
                                  without walking them (0: walk first) */
     int32_t launch_shape;     /* launch shape of the level-walk kernel, 0 .. qcs_launch_shapes(n) - 1
                                  (default 3 at n = 4, else 0); the walks and results do not depend on
-                                 it.  n = 4, shape 3: the W side's contraction on the tensor cores
-                                 (f16 byte planes, exact f32 sums) in warps of its own, beside the
-                                 warps that evaluate the stages, when C^ is held in int8 (c_layout
-                                 0); otherwise, and in a batch, it runs shape 0 */
+                                 it.  n = 4, shape 3: the tensor-core engine (the W side's
+                                 contraction as f16 byte planes with exact f32 sums), when C^ is held
+                                 in int8 (c_layout 0) and its columns' absolute sums are at most
+                                 1821; otherwise it runs shape 0 */
     int32_t c_layout;         /* device layout of C^ for the W side's contraction (n >= 3): 0 = signed
                                  byte quads when every entry fits in int8 (dp4a), else 32-bit words;
                                  1 = 32-bit words always (IMAD).  Results do not depend on it */
@@ -169,8 +169,8 @@ typedef struct qcs_problem qcs_problem;
  * a passage of the paper: how walks map onto the GPU).  Returns the number
  * of shapes (>= 1) and fills, for shape i < max_shapes, warps[i] (warps per
  * CTA of the level walk, each warp evaluating 32 / min(32, 4^n) walks; at
- * n = 4, shape 3 is the tensor-core walk: 12 warps evaluating two walks of
- * each of two sets, and 8 warps doing the contraction) and min_blocks[i] (the
+ * n = 4, shape 3 is the tensor-core engine: 24 warps evaluating one walk of
+ * each of three sets, and 4 warps for the products and the walks' bookkeeping) and min_blocks[i] (the
  * resident CTAs per SM the kernel is compiled for, capping its registers at
  * 65536 / (32 warps[i] min_blocks[i])).  Either pointer may be NULL.
  * QCS_ERR_ARG if n is not in 1..4. */
@@ -401,7 +401,8 @@ typedef struct qcs_batch_params {
     int32_t rewalk_budget;   /* evaluations of f one re-walk may take per round; an unfinished
                                 re-walk resumes in the next round (0: no bound) */
     int32_t launch_shape[4];  /* launch shape of the batched walk kernel for n = 1..4 qubits
-                                 (index n - 1; 0 = default; see qcs_launch_shapes) */
+                                 (index n - 1; 0 = default; see qcs_launch_shapes).  n = 4: with 0 and
+                                3 the jobs that the tensor-core engine takes run on it */
     int32_t cert_points_log2; /* a round runs at most 2^cert_points_log2 points' worth of exhaustive-pass
                                  work (a point with the contraction against C^ counts four), the job
                                  with the least pass work left first (ties: the oldest); a job whose

@@ -24,7 +24,8 @@ using namespace qcs;
 namespace {
 
 constexpr uint32_t kBatchCandCap = 1024; // claw candidates kept per job per round
-constexpr int kClasses = 5;              // qubit counts 1..4 (index 0 unused)
+constexpr int kClasses = 6;              // qubit counts 1..4 (index 0 unused), and n = 4 on the engine
+constexpr int kEngineClass = 5;
 constexpr int kHeads = 4;                // per slot: merge queue, candidates, carried re-walks, unused
 
 struct Job {
@@ -66,10 +67,10 @@ struct qcs_batch {
     unsigned long long *dCounters = nullptr, *hCounters = nullptr; // [slot][C_NCOUNTERS]
     uint32_t *dHeads = nullptr, *hHeads = nullptr;                 // [slot][kHeads]
     Cand *dCands = nullptr, *hCands = nullptr;                     // [slot][kBatchCandCap]
-    uint32_t *dTasks = nullptr, *hTasks = nullptr;                 // [class][2 * max_tasks]
+    uint32_t *dTasks = nullptr, *hTasks = nullptr;                 // from task_off[class]: (job, first walk) pairs
     uint32_t *dIds = nullptr, *hIds = nullptr;                     // [class][max_jobs]
     uint32_t *dCounts = nullptr, *hCounts = nullptr;               // [class][2]: tasks, jobs
-    uint32_t max_tasks = 0;
+    size_t task_off[kClasses + 1] = {}; // each class has room for every job's tasks; [kClasses]: the end
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int64_t rounds = 0;
@@ -267,6 +268,7 @@ int begin_level(qcs_batch *B, Job &j, int slot)
     w.ccount = B->dHeads + kHeads * slot + 1;
     w.ccap = kBatchCandCap;
     w.counters = B->dCounters + (size_t)slot * C_NCOUNTERS;
+    w.stall = reinterpret_cast<uint32_t *>(w.counters + C_STALLED); // its low word
     cudaError_t e = cudaMemsetAsync(j.table, 0xFF, sizeof(Slot) << j.jp.table_log2, B->s);
     if (e == cudaSuccess) e = launch_init_walks(w, B->s);
     if (e != cudaSuccess) return fail(e);
@@ -280,6 +282,19 @@ int begin_level(qcs_batch *B, Job &j, int slot)
     return QCS_OK;
 }
 
+// the kernels a job runs in: n = 4 jobs whose C^ suits it go to the engine
+// (qcs_engine4.cu) unless the batch asks for a dp4a shape (1 or 2)
+int job_class(const qcs_batch *B, const Job &j)
+{
+    const int n = j.P->n, shape = B->bp.launch_shape[n - 1];
+    return n == 4 && j.w.lv.Cm && (shape == 0 || shape == 3) ? kEngineClass : n;
+}
+
+int class_walks_per_task(const qcs_batch_params &bp, int c)
+{
+    return c == kEngineClass ? engine4_walks_per_task() : walks_per_task(c, bp.launch_shape[c - 1]);
+}
+
 // rebuild the per-class task and job lists of the active jobs
 void build_tasks(qcs_batch *B)
 {
@@ -287,11 +302,11 @@ void build_tasks(qcs_batch *B)
     for (size_t slot = 0; slot < B->jobs.size(); slot++) {
         const Job &j = B->jobs[slot];
         if (!j.active || j.parked) continue;
-        const int c = j.P->n;
+        const int c = job_class(B, j);
         B->hIds[(size_t)c * B->bp.max_jobs + nj[c]++] = (uint32_t)slot;
-        const int per = walks_per_task(c, B->bp.launch_shape[c - 1]);
+        const int per = class_walks_per_task(B->bp, c);
         for (int first = 0; first < j.w.n_walks; first += per) {
-            uint32_t *t = B->hTasks + (size_t)c * 2 * B->max_tasks + 2 * nt[c]++;
+            uint32_t *t = B->hTasks + B->task_off[c] + 2 * (size_t)nt[c]++;
             t[0] = (uint32_t)slot;
             t[1] = (uint32_t)first;
         }
@@ -308,7 +323,7 @@ int enqueue_round(qcs_batch *B)
     cudaStream_t s = B->s;
     const size_t J = (size_t)B->bp.max_jobs;
     cudaError_t e = cudaMemcpyAsync(B->dJobs, B->hJobs, sizeof(WalkLaunch) * J, cudaMemcpyHostToDevice, s);
-    if (!e) e = cudaMemcpyAsync(B->dTasks, B->hTasks, sizeof(uint32_t) * kClasses * 2 * B->max_tasks,
+    if (!e) e = cudaMemcpyAsync(B->dTasks, B->hTasks, sizeof(uint32_t) * B->task_off[kClasses],
                                 cudaMemcpyHostToDevice, s);
     if (!e) e = cudaMemcpyAsync(B->dIds, B->hIds, sizeof(uint32_t) * kClasses * J, cudaMemcpyHostToDevice, s);
     if (!e) e = cudaMemcpyAsync(B->dCounts, B->hCounts, sizeof(uint32_t) * kClasses * 2, cudaMemcpyHostToDevice, s);
@@ -316,11 +331,16 @@ int enqueue_round(qcs_batch *B)
     if (!e) e = cudaMemsetAsync(B->dCounters, 0, sizeof(unsigned long long) * C_NCOUNTERS * J, s);
     if (!e) e = cudaEventRecord(B->fork, s);
     for (int c = 1; c < kClasses && !e; c++) {
-        BatchArgs a{B->dJobs, B->dTasks + (size_t)c * 2 * B->max_tasks, B->dCounts + 2 * c, B->dIds + (size_t)c * J,
+        BatchArgs a{B->dJobs, B->dTasks + B->task_off[c], B->dCounts + 2 * c, B->dIds + (size_t)c * J,
                     B->dCounts + 2 * c + 1};
         e = cudaStreamWaitEvent(B->cs[c], B->fork, 0);
-        if (!e) e = launch_walks_batch(c, B->bp.launch_shape[c - 1], a, B->cs[c]);
-        if (!e) e = launch_rewalk_batch(c, a, B->cs[c]);
+        if (c == kEngineClass) {
+            if (!e) e = launch_walks_batch_e4(a, B->cs[c]);
+            if (!e) e = launch_rewalk_batch_e4(a, B->cs[c]);
+        } else {
+            if (!e) e = launch_walks_batch(c, B->bp.launch_shape[c - 1], a, B->cs[c]);
+            if (!e) e = launch_rewalk_batch(c, a, B->cs[c]);
+        }
         if (!e) e = cudaEventRecord(B->join[c], B->cs[c]);
         if (!e) e = cudaStreamWaitEvent(s, B->join[c], 0);
     }
@@ -335,6 +355,10 @@ int enqueue_round(qcs_batch *B)
 void collect_job(Job &j, const unsigned long long *c, const uint32_t *heads, const Cand *cands)
 {
     qcs_problem *P = j.P;
+    if (c[C_STALLED]) { // a bounded wait of the engine ran out: nothing of the round is valid
+        job_error(j, QCS_ERR_DEVICE);
+        return;
+    }
     const int k = j.k, h = k / 2;
     const uint32_t npairs = std::min(heads[0], (uint32_t)j.jp.queue_capacity);
     // re-walks that ran out of budget resume from the other buffer next round
@@ -460,7 +484,10 @@ int qcs_batch_create(const qcs_batch_params *pin, void *stream, qcs_batch **out)
         return QCS_ERR_CUDA;
     }
     B->jobs.resize((size_t)bp.max_jobs);
-    B->max_tasks = (uint32_t)bp.max_jobs * ((uint32_t)bp.walks_per_job / 8); // at least 8 walks per task
+    for (int c = 1; c < kClasses; c++) {
+        const size_t per = (size_t)class_walks_per_task(bp, c);
+        B->task_off[c + 1] = B->task_off[c] + 2 * (size_t)bp.max_jobs * (((size_t)bp.walks_per_job + per - 1) / per);
+    }
     const size_t J = (size_t)bp.max_jobs;
     cudaError_t e = cudaSuccess;
     auto dev = [&](void **p, size_t bytes) { if (!e) e = cudaMalloc(p, bytes); };
@@ -476,8 +503,8 @@ int qcs_batch_create(const qcs_batch_params *pin, void *stream, qcs_batch **out)
     pin_((void **)&B->hHeads, sizeof(uint32_t) * kHeads * J);
     dev((void **)&B->dCands, sizeof(Cand) * kBatchCandCap * J);
     pin_((void **)&B->hCands, sizeof(Cand) * kBatchCandCap * J);
-    dev((void **)&B->dTasks, sizeof(uint32_t) * kClasses * 2 * B->max_tasks);
-    pin_((void **)&B->hTasks, sizeof(uint32_t) * kClasses * 2 * B->max_tasks);
+    dev((void **)&B->dTasks, sizeof(uint32_t) * B->task_off[kClasses]);
+    pin_((void **)&B->hTasks, sizeof(uint32_t) * B->task_off[kClasses]);
     dev((void **)&B->dIds, sizeof(uint32_t) * kClasses * J);
     pin_((void **)&B->hIds, sizeof(uint32_t) * kClasses * J);
     dev((void **)&B->dCounts, sizeof(uint32_t) * kClasses * 2);

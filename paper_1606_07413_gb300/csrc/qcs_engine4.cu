@@ -92,7 +92,7 @@ constexpr size_t off_nw = off_stage + 2 * 64 * 32 * sizeof(uint32_t);           
 constexpr size_t off_bar = off_nw + 32;                            // mbarriers: jobs, rows, product, sums [set]
 constexpr size_t off_tmem = off_bar + 4 * kSets * sizeof(uint64_t);
 constexpr size_t smem_bytes = off_tmem + 16;
-static_assert(smem_bytes <= 227 * 1024, "shared memory of the n = 4 engine");
+static_assert(smem_bytes + sizeof(WalkLaunch) + 64 <= 227 * 1024, "shared memory of the n = 4 engine");
 
 // a bounded wait gives up after this many SM clock cycles (about two seconds)
 constexpr long long kWaitCycles = 1ll << 32;
@@ -103,6 +103,11 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 __device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void mbar_inval(uint64_t *b)
+{
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(b)) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *b)
@@ -300,8 +305,8 @@ struct Cta {
     __device__ uint64_t *bar_sums(int X) const { return bars + 4 * X + 3; }
 };
 
-// stage table, chunk bases, barriers, tensor memory and C^: every thread calls it
-__device__ __forceinline__ Cta cta_begin(const LevelCtx &lv, unsigned char *raw, bool with_chunks)
+// tensor memory and the stage table, once per launch; every thread calls it
+__device__ __forceinline__ Cta cta_open(unsigned char *raw)
 {
     Cta c;
     c.raw = raw;
@@ -309,8 +314,32 @@ __device__ __forceinline__ Cta cta_begin(const LevelCtx &lv, unsigned char *raw,
     c.nw = reinterpret_cast<uint32_t *>(raw + off_nw);
     uint32_t *taddr = reinterpret_cast<uint32_t *>(raw + off_tmem);
     if (threadIdx.x < 32) tmem_alloc(taddr);
-    if (threadIdx.x == 32) {
+    uint32_t *tab = reinterpret_cast<uint32_t *>(raw + off_stage);
+    for (int i = threadIdx.x; i < 2 * 64 * 32; i += kThreads)
+        tab[i] = stage_word<4>((uint32_t)i >> 11, ((uint32_t)i >> 5) & 63u, (uint32_t)i & 31u);
+    tmem_fence_before();
+    __syncthreads();
+    tmem_fence_after();
+    c.tmem = *taddr;
+    return c;
+}
+
+__device__ __forceinline__ void cta_close(const Cta &c)
+{
+    if (threadIdx.x < 32) tmem_dealloc(c.tmem); // after cta_run's last barrier
+}
+
+// the barriers and the chunks' hash bases of a level
+__device__ __forceinline__ void level_begin(const LevelCtx &lv, const Cta &c, bool again)
+{
+    if (threadIdx.x == 0) {
         for (int X = 0; X < kSets; X++) {
+            if (again) {
+                mbar_inval(c.bar_jobs(X));
+                mbar_inval(c.bar_rows(X));
+                mbar_inval(c.bar_prod(X));
+                mbar_inval(c.bar_sums(X));
+            }
             mbar_init(c.bar_jobs(X), 1);
             mbar_init(c.bar_rows(X), kWorkers);
             mbar_init(c.bar_prod(X), 1);
@@ -318,23 +347,13 @@ __device__ __forceinline__ Cta cta_begin(const LevelCtx &lv, unsigned char *raw,
         }
         for (int i = 0; i < 8; i++) c.nw[i] = 0;
     }
-    uint32_t *tab = reinterpret_cast<uint32_t *>(raw + off_stage);
-    for (int i = threadIdx.x; i < 2 * 64 * 32; i += kThreads)
-        tab[i] = stage_word<4>((uint32_t)i >> 11, ((uint32_t)i >> 5) & 63u, (uint32_t)i & 31u);
-    if (with_chunks) {
-        // base(chunk) = smix(smix(seed_H ^ version) ^ (n | k << 8 | chunk << 16 | K << 32))
-        const uint64_t vmix = smix(kSeedH ^ (uint64_t)lv.version);
-        for (int i = threadIdx.x; i < 256; i += kThreads) {
-            const uint64_t tag = (uint64_t)lv.n | ((uint64_t)lv.k << 8) | ((uint64_t)i << 16) |
-                                 ((uint64_t)(uint32_t)lv.K << 32);
-            reinterpret_cast<HashBase *>(raw + off_chunk)[i] = hash_base(smix(vmix ^ tag));
-        }
+    // base(chunk) = smix(smix(seed_H ^ version) ^ (n | k << 8 | chunk << 16 | K << 32))
+    const uint64_t vmix = smix(kSeedH ^ (uint64_t)lv.version);
+    for (int i = threadIdx.x; i < 256; i += kThreads) {
+        const uint64_t tag =
+            (uint64_t)lv.n | ((uint64_t)lv.k << 8) | ((uint64_t)i << 16) | ((uint64_t)(uint32_t)lv.K << 32);
+        reinterpret_cast<HashBase *>(c.raw + off_chunk)[i] = hash_base(smix(vmix ^ tag));
     }
-    tmem_fence_before();
-    __syncthreads();
-    tmem_fence_after();
-    c.tmem = *taddr;
-    return c;
 }
 
 // two biased bytes of a word of LevelCtx::Cm as an f16 pair: the byte permute
@@ -498,12 +517,18 @@ __device__ __forceinline__ bool mma_warp(const Cta &c)
 #pragma unroll 1
         for (int X = 0; X < kSets; X++) {
             if (!((live >> X) & 1u)) continue;
-            if (!mbar_wait(c.bar_jobs(X), ph)) return false;
-            if (c.nw[4 + X]) {
+            bool ok = mbar_wait(c.bar_jobs(X), ph);
+            if (ok && c.nw[4 + X]) {
                 live &= ~(1u << X);
                 continue;
             }
-            if (!mbar_wait(c.bar_rows(X), ph)) return false;
+            ok = ok && mbar_wait(c.bar_rows(X), ph);
+            if (!ok) {
+                // the products in flight (sets before X: this round's, the others': the last)
+                for (int Y = 0; Y < kSets; Y++)
+                    if ((live >> Y) & 1u) mbar_wait(c.bar_prod(Y), Y < X ? ph : ph ^ 1u);
+                return false;
+            }
             tmem_fence_after();
             const uint32_t nw = c.nw[X];
             if (elect_one()) {
@@ -610,20 +635,41 @@ __device__ __forceinline__ uint64_t slot_hash(const Cta &c, int X, int lane, int
     return smix(acc);
 }
 
+// Run the roles over one level's points: ctl(X) is control warp X's part.
+// Every thread calls it; false (for all) if a wait ran out.
+template <class Ctl>
+__device__ __forceinline__ bool cta_run(const LevelCtx &lv, const Cta &c, bool again, Ctl ctl)
+{
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    level_begin(lv, c, again);
+    load_c(lv, c);
+    __syncthreads();
+    tmem_fence_after();
+    bool ok;
+    if (warp < kWorkers) ok = worker(lv, c, warp, lane);
+    else if (warp == kMmaWarp) ok = mma_warp(c);
+    else ok = ctl(warp - kCtlWarp, lane);
+    // every product has completed: its sums were taken, or the MMA warp waited for it
+    tmem_fence_before();
+    ok = __syncthreads_and(ok) != 0;
+    tmem_fence_after();
+    return ok;
+}
+
 } // namespace e4
 
-// The level walk: slot lane * kSets + X of the CTA steps walk slot + gsz *
-// blockIdx.x and every gsz * gridDim.x-th after it, one after the other.  gsz
-// (at most kSets * kSet) is chosen by the host so that every slot has the
-// same number of walks, as nearly as that allows.
-__device__ __forceinline__ bool walk_control(const WalkLaunch &w, uint32_t gsz, const e4::Cta &c, int X, int lane)
+// The level walk: the CTA's slot i (lane * kSets + X) < slots steps walk
+// first + i and every stride-th after it below n, one after the other.
+template <typename WL>
+__device__ __forceinline__ bool walk_control(const WL &w, uint32_t first, uint32_t slots, uint32_t stride, uint32_t n,
+                                             const e4::Cta &c, int X, int lane)
 {
     using namespace e4;
     const LevelCtx &lv = w.lv;
     const Stages sg(lv);
-    const uint32_t slot = (uint32_t)(lane * kSets + X), stride = gsz * gridDim.x, n = (uint32_t)w.n_walks;
-    uint32_t local = blockIdx.x * gsz + slot; // below 2^25: n <= 2^24, and a slot stops past n
-    bool valid = lane < kSet && slot < gsz && local < n, late = false, ok = true;
+    const uint32_t slot = (uint32_t)(lane * kSets + X);
+    uint32_t local = first + slot; // below 2^25: n <= 2^24, and a slot stops past n
+    bool valid = lane < kSet && slot < slots && local < n, late = false, ok = true;
     WalkState st{}, nx{};
     if (valid) st = w.walks[local];
     uint32_t left = w.steps, ph = 0;
@@ -694,26 +740,52 @@ __device__ __forceinline__ bool walk_control(const WalkLaunch &w, uint32_t gsz, 
     return ok;
 }
 
+// gsz (at most kSets * kSet) is chosen by the host so that every slot has the
+// same number of walks, as nearly as that allows
 __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_e4(WalkLaunch w, uint32_t gsz)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const e4::Cta c = e4::cta_begin(w.lv, smem_raw, true);
-    e4::load_c(w.lv, c);
-    __syncthreads();
-    e4::tmem_fence_after();
-    bool ok;
-    if (warp < e4::kWorkers) ok = e4::worker(w.lv, c, warp, lane);
-    else if (warp == e4::kMmaWarp) ok = e4::mma_warp(c);
-    else ok = walk_control(w, gsz, c, warp - e4::kCtlWarp, lane);
-    if (!ok && lane == 0) atomicAdd(w.stall, 1u);
-    // every product has completed (its sums were taken) unless a wait ran out
-    e4::tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        e4::tmem_fence_after();
-        e4::tmem_dealloc(c.tmem);
+    const e4::Cta c = e4::cta_open(smem_raw);
+    const bool ok = e4::cta_run(w.lv, c, false, [&](int X, int lane) {
+        return walk_control(w, blockIdx.x * gsz, gsz, gsz * gridDim.x, (uint32_t)w.n_walks, c, X, lane);
+    });
+    if (!ok && threadIdx.x == 0) atomicAdd(w.stall, 1u);
+    e4::cta_close(c);
+}
+
+// Many jobs in one launch: the CTA takes a contiguous range of tasks (job,
+// first walk of kSets * kSet); neighbouring tasks of one job are one run of
+// the engine, so C^ is reloaded only where the job changes.
+__global__ void __launch_bounds__(e4::kThreads, 1) k_walks_batch_e4(BatchArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    __shared__ WalkLaunch sw;
+    constexpr uint32_t per = e4::kSets * e4::kSet;
+    const uint32_t nt = *a.n_tasks;
+    const uint32_t t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
+    uint32_t task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
+    if (task >= t_end) return;
+    const e4::Cta c = e4::cta_open(smem_raw);
+    bool ok = true, again = false;
+    while (task < t_end && ok) {
+        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
+        uint32_t last = task + 1;
+        while (last < t_end && a.tasks[2 * last] == job) last++;
+        if (threadIdx.x == 0) sw = a.jobs[job];
+        __syncthreads();
+        const uint32_t end = min((uint32_t)sw.n_walks, first + (last - task) * per);
+        // the slots' shares as even as they can be
+        const uint32_t cnt = end > first ? end - first : 0, rounds = (cnt + per - 1) / per;
+        const uint32_t slots = rounds ? (cnt + rounds - 1) / rounds : 0;
+        ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
+            return walk_control(sw, first, slots, slots, end, c, X, lane);
+        });
+        if (!ok && threadIdx.x == 0) atomicAdd(sw.stall, 1u);
+        __syncthreads(); // before sw changes
+        again = true;
+        task = last;
     }
+    e4::cta_close(c);
 }
 
 // The re-walk of a level's merges (Sec. 3, Fig. 2; the same steps and classes
@@ -721,11 +793,12 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_e4(WalkLaunch w, uint
 // claimed one after the other from the device cursor, evaluating f at one
 // state a round: the longer trail until both are aligned, then a and b in
 // turn.  The next merge is claimed and its starts computed while the workers
-// run.  cnt: merges in the work list; slots: slots that take merges (a short
-// list is spread over all CTAs).  A merge to a warp with the dp4a step, a
+// run.  cursor (device or shared memory): the next merge; cnt: the list's end;
+// slots: slots that take merges (a short list is spread over all CTAs).  A merge to a warp with the dp4a step, a
 // search at level 6 (theta 1/2, 2^26 steps) took 240 ms; so it takes 109.
-__device__ __forceinline__ bool rewalk_control(const WalkLaunch &w, uint32_t cnt, uint32_t slots, const e4::Cta &c,
-                                               int X, int lane)
+template <typename WL>
+__device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, uint32_t cnt, uint32_t slots,
+                                               const e4::Cta &c, int X, int lane)
 {
     using namespace e4;
     constexpr unsigned kAll = 0xFFFFFFFFu;
@@ -747,7 +820,7 @@ __device__ __forceinline__ bool rewalk_control(const WalkLaunch &w, uint32_t cnt
             const uint32_t m = __ballot_sync(kAll, need);
             if (!m) break;
             uint32_t base = 0;
-            if (lane == __ffs((int)m) - 1) base = atomicAdd(w.rw_next, (uint32_t)__popc(m));
+            if (lane == __ffs((int)m) - 1) base = atomicAdd(cursor, (uint32_t)__popc(m));
             base = __shfl_sync(kAll, base, __ffs((int)m) - 1);
             if (need) {
                 const uint32_t p = base + (uint32_t)__popc(m & ((1u << lane) - 1u));
@@ -875,22 +948,55 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_e4(WalkLaunch w)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const uint32_t cnt = w.pend_in_n + min(*w.qhead, w.qcap);
     if (cnt <= blockIdx.x) return; // no merge for this CTA
-    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const e4::Cta c = e4::cta_begin(w.lv, smem_raw, true);
-    e4::load_c(w.lv, c);
-    __syncthreads();
-    e4::tmem_fence_after();
-    bool ok;
-    if (warp < e4::kWorkers) ok = e4::worker(w.lv, c, warp, lane);
-    else if (warp == e4::kMmaWarp) ok = e4::mma_warp(c);
-    else ok = rewalk_control(w, cnt, (cnt + gridDim.x - 1) / gridDim.x, c, warp - e4::kCtlWarp, lane);
-    if (!ok && lane == 0) atomicAdd(w.stall, 1u);
-    e4::tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        e4::tmem_fence_after();
-        e4::tmem_dealloc(c.tmem);
+    const e4::Cta c = e4::cta_open(smem_raw);
+    const bool ok = e4::cta_run(w.lv, c, false, [&](int X, int lane) {
+        return rewalk_control(w, w.rw_next, cnt, (cnt + gridDim.x - 1) / gridDim.x, c, X, lane);
+    });
+    if (!ok && threadIdx.x == 0) atomicAdd(w.stall, 1u);
+    e4::cta_close(c);
+}
+
+// The batched re-walk: the work lists of all jobs form one index space; each
+// CTA takes a contiguous range of it and reloads C^ where its range enters
+// another job.
+__global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_batch_e4(BatchArgs a)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    __shared__ WalkLaunch sw;
+    __shared__ uint32_t cursor;
+    const uint32_t nj = *a.n_jobs;
+    uint64_t total = 0;
+    for (uint32_t j = 0; j < nj; j++) {
+        const WalkLaunch &w = a.jobs[a.job_ids[j]];
+        total += w.pend_in_n + min(*w.qhead, w.qcap);
     }
+    const uint64_t lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
+    if (lo >= hi) return;
+    const e4::Cta c = e4::cta_open(smem_raw);
+    bool ok = true, again = false;
+    uint64_t base = 0;
+    for (uint32_t j = 0; j < nj && base < hi && ok; j++) {
+        const WalkLaunch &wj = a.jobs[a.job_ids[j]];
+        const uint32_t cnt = wj.pend_in_n + min(*wj.qhead, wj.qcap);
+        if (base + cnt <= lo) {
+            base += cnt;
+            continue;
+        }
+        const uint32_t p0 = (uint32_t)(max(lo, base) - base), p1 = (uint32_t)(min(hi, base + cnt) - base);
+        base += cnt;
+        if (p0 >= p1) continue;
+        if (threadIdx.x == 0) {
+            sw = wj;
+            cursor = p0;
+        }
+        __syncthreads();
+        ok = e4::cta_run(sw.lv, c, again,
+                         [&](int X, int lane) { return rewalk_control(sw, &cursor, p1, p1 - p0, c, X, lane); });
+        if (!ok && threadIdx.x == 0) atomicAdd(sw.stall, 1u);
+        __syncthreads(); // before sw and cursor change
+        again = true;
+    }
+    e4::cta_close(c);
 }
 
 // W points of the exhaustive pass: the set takes kPairs points a round (all
@@ -948,22 +1054,10 @@ __device__ __forceinline__ bool certify_control(const CertArgs &a, const e4::Cta
 __global__ void __launch_bounds__(e4::kThreads, 1) k_certify_e4(CertArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const e4::Cta c = e4::cta_begin(a.lv, smem_raw, false);
-    e4::load_c(a.lv, c);
-    __syncthreads();
-    e4::tmem_fence_after();
-    bool ok;
-    if (warp < e4::kWorkers) ok = e4::worker(a.lv, c, warp, lane);
-    else if (warp == e4::kMmaWarp) ok = e4::mma_warp(c);
-    else ok = certify_control(a, c, warp - e4::kCtlWarp, lane);
-    if (!ok && lane == 0) atomicAdd(a.n_pairs + 1, 1u);
-    e4::tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        e4::tmem_fence_after();
-        e4::tmem_dealloc(c.tmem);
-    }
+    const e4::Cta c = e4::cta_open(smem_raw);
+    const bool ok = e4::cta_run(a.lv, c, false, [&](int X, int lane) { return certify_control(a, c, X, lane); });
+    if (!ok && threadIdx.x == 0) atomicAdd(a.n_pairs + 1, 1u);
+    e4::cta_close(c);
 }
 
 } // namespace
@@ -1005,6 +1099,26 @@ cudaError_t launch_certify_e4(const CertArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+cudaError_t launch_walks_batch_e4(const BatchArgs &a, cudaStream_t s)
+{
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_walks_batch_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
+    if (e != cudaSuccess) return e;
+    k_walks_batch_e4<<<(unsigned)num_sms(), e4::kThreads, e4::smem_bytes, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rewalk_batch_e4(const BatchArgs &a, cudaStream_t s)
+{
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_rewalk_batch_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
+    if (e != cudaSuccess) return e;
+    k_rewalk_batch_e4<<<(unsigned)num_sms(), e4::kThreads, e4::smem_bytes, s>>>(a);
+    return cudaGetLastError();
+}
+
 int engine4_warps() { return e4::kWarps; }
+
+int engine4_walks_per_task() { return e4::kSets * e4::kSet; }
 
 } // namespace qcs

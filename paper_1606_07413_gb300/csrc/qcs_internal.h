@@ -279,7 +279,11 @@ cudaError_t launch_walks(const WalkLaunch &w, cudaStream_t s);
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s);
 // the re-walk of a level's merges on the engine
 cudaError_t launch_rewalk_e4(const WalkLaunch &w, cudaStream_t s);
+// jobs of a batch on the engine: tasks of engine4_walks_per_task() walks, and the jobs' re-walks
+cudaError_t launch_walks_batch_e4(const BatchArgs &a, cudaStream_t s);
+cudaError_t launch_rewalk_batch_e4(const BatchArgs &a, cudaStream_t s);
 int engine4_warps(); // warps of its CTA
+int engine4_walks_per_task();
 // DP-owner sharding: insert `count` distinguished points {dp, trail ref}
 // into w's table (merges queued as by the walk), and bin points by owner
 // rank (owner_of in qcs_walk.cu): out gets the points grouped by owner in

@@ -122,3 +122,31 @@ def test_engine_rewalk_classes_equal_the_array_rewalk(dev, k, dpb, walks, steps,
             torch.cuda.synchronize()
             want += np.bincount(cls.cpu().numpy(), minlength=6)
         assert np.array_equal(got, [want[0], want[1], want[2], want[3] + want[4], want[5]])
+
+
+# walks per job around a task (72 walks) and far above; one job whose C^ the
+# engine does not take runs beside the others
+@pytest.mark.parametrize("walks,targets", [(16, (7, 7, 7)), (64, (7, 6)), (80, (7,) * 5), (2048, (7, 15, 6)),
+                                           (144, (7,) * 40)])
+def test_batched_jobs_on_the_engine_walk_as_on_dp4a(walks, targets):
+    """Walk counters of every job and round, engine (shape 0) against dp4a (shape 1)."""
+    hist = {}
+    for shape in (0, 1):
+        bp = Q.default_batch_params(max_jobs=len(targets), walks_per_job=walks, steps_per_round=24, table_log2=14,
+                                    queue_capacity=1 << 12, rewalk_budget=7, launch_shape={4: shape})
+        probs = [Q.Problem.from_circuit(4, W.seeded_target(4, t, 4000 + t + 100 * i)[0], min(t, 9), Q.default_params(
+            4, state_bits=64, seed=77 + i)) for i, t in enumerate(targets)]
+        rows = []
+        with Q.Batch(bp) as batch:
+            ids = [batch.add(p) for p in probs]
+            for _ in range(4):
+                batch.round()
+                rs = [batch.poll(j) for j in ids]
+                rows.append([(r["k"], r["steps"], r["w_steps"], r["dps"], r["abandoned"]) for r in rs])
+                for r in rs:
+                    assert r["status"] in (Q.SEARCHING, Q.FOUND, Q.BUDGET_EXHAUSTED)
+        hist[shape] = rows
+        for p in probs:
+            p.close()
+    assert hist[0] == hist[1]
+    assert sum(r[1] for r in hist[0][-1]) > 0
