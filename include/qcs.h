@@ -118,7 +118,7 @@ typedef struct qcs_params {
                                  it.  n = 4, shape 3: the tensor-core engine (the W side's
                                  contraction as f16 byte planes with exact f32 sums), when C^ is held
                                  in int8 (c_layout 0) and its columns' absolute sums are at most
-                                 1821; otherwise it runs shape 0 */
+                                 1820; otherwise it runs shape 0 */
     int32_t c_layout;         /* device layout of C^ for the W side's contraction (n >= 3): 0 = signed
                                  byte quads when every entry fits in int8 (dp4a), else 32-bit words;
                                  1 = 32-bit words always (IMAD).  Results do not depend on it */

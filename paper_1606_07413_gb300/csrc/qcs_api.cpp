@@ -101,6 +101,8 @@ LevelCtx qcs::make_level(const qcs_problem *P, int k, uint32_t version, int dp_b
     lv.Cq = reinterpret_cast<const uint4 *>(P->dCq);
     lv.Cm = reinterpret_cast<const uint4 *>(P->dCm);
     lv.Csum = P->dCm ? reinterpret_cast<const int16_t *>(P->dCm + (size_t)P->D * P->D / 2) : nullptr;
+    lv.q8 = P->q8 ? 1 : 0;
+    lv.quad = reinterpret_cast<const uint4 *>(P->dQuad);
     lv.U = P->dU;
     for (int side = 0; side < 2; side++) {
         lv.T1[side] = P->dT1[side];
@@ -152,11 +154,11 @@ void host_adj_stage(int n, uint32_t p, bool adj_of_transpose, std::vector<uint32
 }
 
 std::mutex g_tab_mu;
-std::map<std::pair<int, int>, std::array<uint32_t *, 4>> g_tabs; // (device, n) -> T1v, T1w, T4v, T4w
+std::map<std::pair<int, int>, std::array<uint32_t *, 5>> g_tabs; // (device, n) -> T1v, T1w, T4v, T4w, quad
 
 } // namespace
 
-int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64_t *uploaded)
+int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], const uint32_t **quad, int64_t *uploaded)
 {
     int dev = 0;
     CK(cudaGetDevice(&dev));
@@ -169,7 +171,8 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64
             u0a[i] = (uint32_t)smix_host(kSeedU + (2ull * i + 1) * kGamma) & 0xFFFFu;
             u0b[i] = (uint32_t)smix_host(kSeedU + (2ull * i + 2) * kGamma) & 0xFFFFu;
         }
-        std::array<uint32_t *, 4> tabs{nullptr, nullptr, nullptr, nullptr};
+        std::array<uint32_t *, 5> tabs{nullptr, nullptr, nullptr, nullptr, nullptr};
+        std::vector<uint32_t> quad_t; // the quad kernels' T, both sides
         auto upload = [&](uint32_t **d, const std::vector<uint32_t> &h) {
             cudaError_t e = cudaMalloc(d, sizeof(uint32_t) * h.size());
             if (e == cudaSuccess) e = cudaMemcpy(*d, h.data(), sizeof(uint32_t) * h.size(), cudaMemcpyHostToDevice);
@@ -184,7 +187,7 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64
                 for (uint32_t j = 0; j < D; j++) t1[(size_t)(qa - 1) * D + j] = ua[j] | (ub[j] << 16);
             }
             CK(upload(&tabs[side], t1));
-            if (n >= 3) {
+            if (n >= 2) {
                 // the Pauli of code t << (2n - 3) | l is row_of(n, l, t)
                 std::vector<uint32_t> t4v((size_t)D * D);
                 for (uint32_t code = 0; code < D; code++) {
@@ -196,6 +199,34 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64
                 }
                 CK(upload(&tabs[2 + side], t4v));
             }
+            if (n == 2 || n == 3)
+                for (uint32_t code = 0; code < D; code++)
+                    for (uint32_t i = 0; i < D; i++) { // row / 4, lane, row % 4
+                        const uint32_t q = code_pauli(n, code), j = quad_row(n, (i >> 2) & 3, (i >> 4) * 4 + (i & 3));
+                        quad_t.push_back(q ? t1[(size_t)(q - 1) * D + j] : (u0a[j] | u0b[j] << 16));
+                    }
+        }
+        if (n == 2 || n == 3) {
+            const uint32_t R = D / 4, m = (1u << n) - 1;
+            std::vector<uint32_t> anti((size_t)D * 4, 0);
+            std::vector<uint8_t> sign((size_t)2 * D * 4 * R);
+            for (uint32_t code = 0; code < D; code++)
+                for (uint32_t i = 0; i < D; i++) { // lane, row
+                    const uint32_t p = code_pauli(n, code), j = quad_row(n, i / R, i % R);
+                    if (!(__builtin_popcount(((p >> n) & (j & m)) ^ ((p & m) & (j >> n))) & 1)) {
+                        sign[(size_t)code * D + i] = sign[((size_t)D + code) * D + i] = 1;
+                        continue;
+                    }
+                    const bool plus = pauli_phase(n, p, j) == 1; // V adds, W subtracts the partner
+                    anti[(size_t)code * 4 + i / R] |= 1u << (i % R);
+                    sign[(size_t)code * D + i] = plus ? 1 : 0xFF;
+                    sign[((size_t)D + code) * D + i] = plus ? 0xFF : 1;
+                }
+            const size_t words = sign.size() / 4;
+            quad_t.resize(quad_t.size() + words);
+            memcpy(quad_t.data() + quad_t.size() - words, sign.data(), sign.size());
+            quad_t.insert(quad_t.end(), anti.begin(), anti.end());
+            CK(upload(&tabs[4], quad_t));
         }
         it = g_tabs.emplace(std::make_pair(dev, n), tabs).first;
     }
@@ -203,6 +234,7 @@ int qcs::stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64
     t1[1] = it->second[1];
     t4[0] = it->second[2];
     t4[1] = it->second[3];
+    *quad = it->second[4];
     return QCS_OK;
 }
 
@@ -244,6 +276,19 @@ int upload_problem(qcs_problem *P)
         }
     std::vector<uint32_t> coef(coef16.size() / 2);
     memcpy(coef.data(), coef16.data(), sizeof(uint32_t) * coef.size());
+    // n = 2, 3: do the entries fit int8 and the columns the f32 sums of the
+    // quad kernels (the identity's row is not part of a product)
+    if ((n == 2 || n == 3) && P->p.c_layout == 0) {
+        bool fits = true;
+        for (size_t i = 0; i < P->C.a.size() && fits; i++)
+            fits = P->C.a[i] >= -128 && P->C.a[i] <= 127 && P->C.b[i] >= -128 && P->C.b[i] <= 127;
+        for (int Q = 0; Q < D && fits; Q++) {
+            int64_t sum = 0;
+            for (int i = 1; i < D; i++) sum += std::abs(P->C.a[(size_t)i * D + Q]) + std::abs(P->C.b[(size_t)i * D + Q]);
+            fits = sum <= kMaxColumnSum;
+        }
+        P->q8 = fits;
+    }
     // n >= 3: also C^ as signed byte quads (rows 4q .. 4q+3 of a column in
     // one word) when every entry fits in int8, laid out for the walk
     // kernel's byte-plane contraction (LevelCtx::Cq)
@@ -298,7 +343,7 @@ int upload_problem(qcs_problem *P)
     }
     CK(cudaGetDevice(&P->device));
     int64_t h2d = 0;
-    if (int rc = stage_tables(n, P->dT1, P->dT4, &h2d)) return rc;
+    if (int rc = stage_tables(n, P->dT1, P->dT4, &P->dQuad, &h2d)) return rc;
     if (!cq.empty()) {
         CK(cudaMalloc(&P->dCq, sizeof(uint32_t) * cq.size()));
         CK(cudaMemcpy(P->dCq, cq.data(), sizeof(uint32_t) * cq.size(), cudaMemcpyHostToDevice));

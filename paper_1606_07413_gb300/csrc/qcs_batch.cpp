@@ -24,8 +24,10 @@ using namespace qcs;
 namespace {
 
 constexpr uint32_t kBatchCandCap = 1024; // claw candidates kept per job per round
-constexpr int kClasses = 6;              // qubit counts 1..4 (index 0 unused), and n = 4 on the engine
-constexpr int kEngineClass = 5;
+// kernel classes: 1..4, the qubit counts; kTensor + n for n = 2..4, the jobs of
+// n qubits on the tensor-core kernels (qcs_quad.cu, qcs_engine4.cu)
+constexpr int kTensor = 4, kClasses = kTensor + 5;
+constexpr bool class_used(int c) { return c >= 1 && c != kTensor + 1; }
 constexpr int kHeads = 4;                // per slot: merge queue, candidates, carried re-walks, unused
 
 struct Job {
@@ -282,27 +284,37 @@ int begin_level(qcs_batch *B, Job &j, int slot)
     return QCS_OK;
 }
 
-// the kernels a job runs in: n = 4 jobs whose C^ suits it go to the engine
-// (qcs_engine4.cu) unless the batch asks for a dp4a shape (1 or 2)
-int job_class(const qcs_batch *B, const Job &j)
+// The kernels a job runs in: the tensor-core ones where C^ suits them and the
+// batch asks for its qubit count's default shape (or, n = 4, for theirs).  Few
+// n = 3 walks (walks3: of all jobs this round) are left to the others.
+int job_class(const qcs_batch *B, const Job &j, uint64_t walks3)
 {
     const int n = j.P->n, shape = B->bp.launch_shape[n - 1];
-    return n == 4 && j.w.lv.Cm && (shape == 0 || shape == 3) ? kEngineClass : n;
+    bool tensor = false;
+    if (n == 4) tensor = j.w.lv.Cm && (shape == 0 || shape == 3);
+    else if (n == 3) tensor = j.w.lv.q8 && shape == 0 && walks3 >= kQuadWalks3;
+    else if (n == 2) tensor = j.w.lv.q8 != 0;
+    return tensor ? kTensor + n : n;
 }
 
 int class_walks_per_task(const qcs_batch_params &bp, int c)
 {
-    return c == kEngineClass ? engine4_walks_per_task() : walks_per_task(c, bp.launch_shape[c - 1]);
+    return c == kTensor + 4 ? engine4_walks_per_task()
+           : c > kTensor    ? quad_walks_per_task()
+                            : walks_per_task(c, bp.launch_shape[c - 1]);
 }
 
 // rebuild the per-class task and job lists of the active jobs
 void build_tasks(qcs_batch *B)
 {
     uint32_t nt[kClasses] = {0}, nj[kClasses] = {0};
+    uint64_t walks3 = 0;
+    for (const Job &j : B->jobs)
+        if (j.active && !j.parked && j.P->n == 3) walks3 += (uint64_t)j.w.n_walks;
     for (size_t slot = 0; slot < B->jobs.size(); slot++) {
         const Job &j = B->jobs[slot];
         if (!j.active || j.parked) continue;
-        const int c = job_class(B, j);
+        const int c = job_class(B, j, walks3);
         B->hIds[(size_t)c * B->bp.max_jobs + nj[c]++] = (uint32_t)slot;
         const int per = class_walks_per_task(B->bp, c);
         for (int first = 0; first < j.w.n_walks; first += per) {
@@ -331,12 +343,16 @@ int enqueue_round(qcs_batch *B)
     if (!e) e = cudaMemsetAsync(B->dCounters, 0, sizeof(unsigned long long) * C_NCOUNTERS * J, s);
     if (!e) e = cudaEventRecord(B->fork, s);
     for (int c = 1; c < kClasses && !e; c++) {
+        if (!class_used(c)) continue;
         BatchArgs a{B->dJobs, B->dTasks + B->task_off[c], B->dCounts + 2 * c, B->dIds + (size_t)c * J,
                     B->dCounts + 2 * c + 1};
         e = cudaStreamWaitEvent(B->cs[c], B->fork, 0);
-        if (c == kEngineClass) {
+        if (c == kTensor + 4) {
             if (!e) e = launch_walks_batch_e4(a, B->cs[c]);
             if (!e) e = launch_rewalk_batch_e4(a, B->cs[c]);
+        } else if (c > kTensor) {
+            if (!e) e = launch_walks_batch_q(c - kTensor, a, B->cs[c]);
+            if (!e) e = launch_rewalk_batch_q(c - kTensor, a, B->cs[c]);
         } else {
             if (!e) e = launch_walks_batch(c, B->bp.launch_shape[c - 1], a, B->cs[c]);
             if (!e) e = launch_rewalk_batch(c, a, B->cs[c]);
@@ -485,8 +501,8 @@ int qcs_batch_create(const qcs_batch_params *pin, void *stream, qcs_batch **out)
     }
     B->jobs.resize((size_t)bp.max_jobs);
     for (int c = 1; c < kClasses; c++) {
-        const size_t per = (size_t)class_walks_per_task(bp, c);
-        B->task_off[c + 1] = B->task_off[c] + 2 * (size_t)bp.max_jobs * (((size_t)bp.walks_per_job + per - 1) / per);
+        const size_t per = class_used(c) ? (size_t)class_walks_per_task(bp, c) : 1;
+        B->task_off[c + 1] = B->task_off[c] + (class_used(c) ? 2 * (size_t)bp.max_jobs * (((size_t)bp.walks_per_job + per - 1) / per) : 0);
     }
     const size_t J = (size_t)bp.max_jobs;
     cudaError_t e = cudaSuccess;

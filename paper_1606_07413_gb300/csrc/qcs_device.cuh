@@ -60,13 +60,17 @@ __device__ __forceinline__ uint64_t trail_start(const LevelCtx &lv, uint32_t wal
     seq &= (1u << kRefSeqBits) - 1;
     return smix(lv.seed ^ smix(((uint64_t)walk << 32) | seq) ^ ((uint64_t)lv.version << 40)) & lv.maskL;
 }
+// NQ: the qubit count where the kernel knows it (the divisions are then by a
+// constant), else 0
+template <int NQ = 0>
 __device__ __forceinline__ uint32_t trail_chunk(const LevelCtx &lv, uint64_t start)
 {
     if (!lv.n_chunks) return 0u;
     // n_chunks = xi = 4^n - 1: with v = hi 2^32 + lo and 2^32 = 1 (mod xi)
     // for n = 1, 2, 4 (4^n's powers reach 2^32) and 4 (mod 63) for n = 3
     const uint64_t v = smix(start ^ 0x5851F42D4C957F2Dull);
-    const uint32_t xi = (uint32_t)lv.n_chunks, r32 = lv.n == 3 ? 4u : 1u;
+    const uint32_t xi = NQ ? (1u << (2 * NQ)) - 1u : (uint32_t)lv.n_chunks;
+    const uint32_t r32 = (NQ ? NQ : lv.n) == 3 ? 4u : 1u;
     return 1u + ((uint32_t)(v >> 32) % xi * r32 + (uint32_t)v % xi) % xi;
 }
 __device__ __forceinline__ uint64_t make_ref(uint32_t walk, uint32_t seq, uint32_t len)
@@ -81,13 +85,14 @@ __device__ __forceinline__ void split_ref(uint64_t ref, uint32_t &walk, uint32_t
     len = (uint32_t)(ref >> (kRefWalkBits + kRefSeqBits));
 }
 
+template <int NQ = 0>
 __device__ __forceinline__ void new_trail(WalkState &st, uint32_t walk, const LevelCtx &lv)
 {
     st.seq++;
     st.start = trail_start(lv, walk, st.seq);
     st.cur = st.start;
     st.len = 0;
-    st.chunk = trail_chunk(lv, st.start);
+    st.chunk = trail_chunk<NQ>(lv, st.start);
 }
 
 // per-walk-group tallies, added to the job's counters by the group's first
@@ -151,7 +156,7 @@ struct Merge {
     uint64_t a, b;
     uint32_t la, lb, ca, cb;
 };
-template <typename WL>
+template <int NQ = 0, typename WL>
 __device__ __forceinline__ Merge load_merge(const WL &w, uint32_t p)
 {
     Merge m;
@@ -169,8 +174,8 @@ __device__ __forceinline__ Merge load_merge(const WL &w, uint32_t p)
         split_ref(P.ref_b, wb, sb, m.lb);
         m.a = trail_start(w.lv, wa, sa);
         m.b = trail_start(w.lv, wb, sb);
-        m.ca = trail_chunk(w.lv, m.a);
-        m.cb = trail_chunk(w.lv, m.b);
+        m.ca = trail_chunk<NQ>(w.lv, m.a);
+        m.cb = trail_chunk<NQ>(w.lv, m.b);
     }
     return m;
 }
@@ -233,6 +238,44 @@ __device__ __forceinline__ uint64_t add_base_xi(uint64_t d, uint64_t s, uint32_t
         }
     }
     return r;
+}
+
+// A batched re-walk's shares: the CTAs take equal parts of all jobs' work, a
+// merge of a job counting about its evaluations of f: three trail lengths, or
+// the budget.  (By merges alone the CTAs that met the jobs of small theta, 64
+// evaluations to a merge, took three times as long as the others.)
+template <typename WL>
+__device__ __forceinline__ uint64_t merge_weight(const WL &w)
+{
+    const int d = __popcll(w.lv.maskL) - w.lv.dshift; // theta = 2^-d
+    const uint64_t len = 3ull << min(d, 20);
+    return w.rewalk_budget && w.rewalk_budget < len ? (uint64_t)w.rewalk_budget : len;
+}
+
+// Walk a CTA's share: body(job index, its first merge, the end of its merges)
+// for every job that the share meets, in order, until body returns false.
+template <class Body>
+__device__ __forceinline__ void merge_shares(const BatchArgs &a, Body body)
+{
+    const uint32_t nj = *a.n_jobs;
+    uint64_t total = 0;
+    for (uint32_t j = 0; j < nj; j++) {
+        const WalkLaunch &w = a.jobs[a.job_ids[j]];
+        total += (uint64_t)(w.pend_in_n + min(*w.qhead, w.qcap)) * merge_weight(w);
+    }
+    const uint64_t lo = total / gridDim.x * blockIdx.x + total % gridDim.x * blockIdx.x / gridDim.x;
+    const uint64_t hi = total / gridDim.x * (blockIdx.x + 1) + total % gridDim.x * (blockIdx.x + 1) / gridDim.x;
+    uint64_t base = 0;
+    for (uint32_t j = 0; j < nj && base < hi; j++) {
+        const uint32_t job = a.job_ids[j];
+        const WalkLaunch &w = a.jobs[job];
+        const uint64_t cnt = w.pend_in_n + min(*w.qhead, w.qcap), wt = merge_weight(w), at = base;
+        base += cnt * wt;
+        if (base <= lo) continue;
+        // a merge belongs to the share its first unit lies in
+        const uint64_t p0 = lo > at ? (lo - at + wt - 1) / wt : 0, p1 = hi < base ? (hi - at + wt - 1) / wt : cnt;
+        if (p0 < p1 && !body(job, (uint32_t)p0, (uint32_t)p1)) return;
+    }
 }
 
 // Exhaustive pass: the key table.  A key's slots are s, s + d, s + 2d, .. with

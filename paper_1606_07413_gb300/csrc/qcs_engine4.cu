@@ -69,6 +69,7 @@ constexpr int kTmemK = 8;                   // K-blocks of C^'s second half held
 constexpr int kDcol = 256 + 8 * kTmemK;     // tensor-memory column of D (set X, half h: + 96 X + 48 h)
 static_assert(kDcol + kSets * 2 * kN <= 512, "tensor memory");
 constexpr uint32_t kInvalid = 1u << 31;
+constexpr int kTaskWalks = 24; // of a batch: a third of the slots, for even shares
 
 // one point to evaluate, published by the set's control warp
 struct alignas(16) Job {
@@ -713,7 +714,7 @@ __device__ __forceinline__ bool walk_control(const WL &w, uint32_t first, uint32
                 } else if (last) {
                     t.ab++;
                 }
-                if (is_dp || last) new_trail(st, walk, lv);
+                if (is_dp || last) new_trail<4>(st, walk, lv);
                 if (left == 0) {
                     w.walks[local] = st;
                     local += stride;
@@ -754,13 +755,13 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_e4(WalkLaunch w, uint
 }
 
 // Many jobs in one launch: the CTA takes a contiguous range of tasks (job,
-// first walk of kSets * kSet); neighbouring tasks of one job are one run of
+// first walk of kTaskWalks); neighbouring tasks of one job are one run of
 // the engine, so C^ is reloaded only where the job changes.
 __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_batch_e4(BatchArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ WalkLaunch sw;
-    constexpr uint32_t per = e4::kSets * e4::kSet;
+    constexpr uint32_t per = e4::kSets * e4::kSet; // slots
     const uint32_t nt = *a.n_tasks;
     const uint32_t t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
     uint32_t task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
@@ -773,7 +774,7 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_batch_e4(BatchArgs a)
         while (last < t_end && a.tasks[2 * last] == job) last++;
         if (threadIdx.x == 0) sw = a.jobs[job];
         __syncthreads();
-        const uint32_t end = min((uint32_t)sw.n_walks, first + (last - task) * per);
+        const uint32_t end = min((uint32_t)sw.n_walks, first + (last - task) * e4::kTaskWalks);
         // the slots' shares as even as they can be
         const uint32_t cnt = end > first ? end - first : 0, rounds = (cnt + per - 1) / per;
         const uint32_t slots = rounds ? (cnt + rounds - 1) / rounds : 0;
@@ -827,7 +828,7 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
                 if (p >= cnt) {
                     more = false;
                 } else {
-                    const Merge q = load_merge(w, p);
+                    const Merge q = load_merge<4>(w, p);
                     const bool bad = q.ca != q.cb || q.la > kMaxRewalkLen || q.lb > kMaxRewalkLen;
                     const bool hood = !bad && q.la == q.lb && q.a == q.b, none = bad || (!hood && (q.la | q.lb) == 0);
                     cls[0] += hood;
@@ -956,47 +957,31 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_e4(WalkLaunch w)
     e4::cta_close(c);
 }
 
-// The batched re-walk: the work lists of all jobs form one index space; each
-// CTA takes a contiguous range of it and reloads C^ where its range enters
-// another job.
+// The batched re-walk: each CTA takes its share of all jobs' merges (see
+// merge_shares) and reloads C^ where the share enters another job.
 __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_batch_e4(BatchArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ WalkLaunch sw;
     __shared__ uint32_t cursor;
-    const uint32_t nj = *a.n_jobs;
-    uint64_t total = 0;
-    for (uint32_t j = 0; j < nj; j++) {
-        const WalkLaunch &w = a.jobs[a.job_ids[j]];
-        total += w.pend_in_n + min(*w.qhead, w.qcap);
-    }
-    const uint64_t lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
-    if (lo >= hi) return;
-    const e4::Cta c = e4::cta_open(smem_raw);
-    bool ok = true, again = false;
-    uint64_t base = 0;
-    for (uint32_t j = 0; j < nj && base < hi && ok; j++) {
-        const WalkLaunch &wj = a.jobs[a.job_ids[j]];
-        const uint32_t cnt = wj.pend_in_n + min(*wj.qhead, wj.qcap);
-        if (base + cnt <= lo) {
-            base += cnt;
-            continue;
-        }
-        const uint32_t p0 = (uint32_t)(max(lo, base) - base), p1 = (uint32_t)(min(hi, base + cnt) - base);
-        base += cnt;
-        if (p0 >= p1) continue;
+    e4::Cta c;
+    bool again = false;
+    merge_shares(a, [&](uint32_t job, uint32_t p0, uint32_t p1) {
+        if (!again) c = e4::cta_open(smem_raw);
         if (threadIdx.x == 0) {
-            sw = wj;
+            sw = a.jobs[job];
             cursor = p0;
         }
         __syncthreads();
-        ok = e4::cta_run(sw.lv, c, again,
-                         [&](int X, int lane) { return rewalk_control(sw, &cursor, p1, p1 - p0, c, X, lane); });
+        const bool ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
+            return rewalk_control(sw, &cursor, p1, p1 - p0, c, X, lane);
+        });
         if (!ok && threadIdx.x == 0) atomicAdd(sw.stall, 1u);
         __syncthreads(); // before sw and cursor change
         again = true;
-    }
-    e4::cta_close(c);
+        return ok;
+    });
+    if (again) e4::cta_close(c);
 }
 
 // W points of the exhaustive pass: the set takes kPairs points a round (all
@@ -1119,6 +1104,6 @@ cudaError_t launch_rewalk_batch_e4(const BatchArgs &a, cudaStream_t s)
 
 int engine4_warps() { return e4::kWarps; }
 
-int engine4_walks_per_task() { return e4::kSets * e4::kSet; }
+int engine4_walks_per_task() { return e4::kTaskWalks; }
 
 } // namespace qcs

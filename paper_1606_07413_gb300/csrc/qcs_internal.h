@@ -38,12 +38,24 @@ __host__ __device__ constexpr uint32_t row_of(int n, uint32_t l, uint32_t t)
     const uint32_t x = (l >> (n - 1)) | (t & 1u) << (n - 2) | ((t >> 2) & 1u) << (n - 1);
     return x << n | z;
 }
-// A column of C^ suits the engine's f32 sums when the absolute values of its
+// Rows on quads (qcs_quad.cu, n = 2 and 3): lane q is qubit 0 (z0 | x0 << 1),
+// row t the other qubits: z1 above t8 = (x1 z2 x2) at n = 3, (z1 x1) at n = 2.
+// The Pauli index, and the Pauli of a code (row_of's order).
+__host__ __device__ constexpr uint32_t quad_row(int n, uint32_t q, uint32_t t)
+{
+    return n == 2 ? (q & 1u) | (t & 1u) << 1 | (q >> 1) << 2 | (t >> 1) << 3
+                  : row_of(3, (q & 1u) | (t >> 3) << 1 | (q >> 1) << 2, t & 7u);
+}
+__host__ __device__ constexpr uint32_t code_pauli(int n, uint32_t code)
+{
+    return row_of(n, code & ((1u << (2 * n - 3)) - 1u), code >> (2 * n - 3));
+}
+// A column of C^ suits the tensor-core kernels' f32 sums when the absolute values of its
 // entries add up to at most this: a partial sum of the product is below
-// (1279 + 1024) * 1821 < 2^22 (weights up to 1024 + 255, and the offset's
-// correction).  By orthogonality a column's squares a^2 + 2 b^2 add up to
+// (1279 + 1024) * 1820 + 1279 < 2^22 (weights up to 1024 + 255, the offset's
+// correction, and V's own k-step in qcs_quad.cu).  By orthogonality a column's squares a^2 + 2 b^2 add up to
 // 2^E, so the sum is at most 16 sqrt(1.5 * 2^E), 1773 at E = 13.
-constexpr int kMaxColumnSum = 1821;
+constexpr int kMaxColumnSum = 1820;
 
 // Everything a warp needs to evaluate one step f of the walk at one level.
 struct LevelCtx {
@@ -63,10 +75,16 @@ struct LevelCtx {
     // row_of(4, l, t).  Csum[Q]: the sum of the column's entries.
     const uint4 *Cm;
     const int16_t *Csum;
-    // n >= 3: the weights after the first adjoint stage, as T1, by code: word
+    // n >= 2: the weights after the first adjoint stage, as T1, by code: word
     // code * 4^n + 8 l + t is row row_of(n, l, t)'s Ua | Ub << 16 after the
     // Pauli of that code; code 0 holds the weights themselves.
     const uint4 *T4[2];
+    int32_t q8;        // n = 2, 3: C^ suits the quad kernels (qcs_quad.cu): int8 entries, small column sums
+    // n = 2, 3: the quad kernels' tables (stage_tables): T, uint4 [side][code]
+    // [row / 4][lane], the weights after the first stage of a code, Ua | Ub <<
+    // 16 of four rows; then the signs, i8 [side][code][lane][row], 1 where the
+    // row commutes; then the anticommuting rows, u32 [code][lane], a bit per row
+    const uint4 *quad;
     const uint2 *U;    // fingerprint weights (Ua, Ub) per row, 4^n
     // The weights after the first adjoint stage of a side (index 0: V, 1: W),
     // mod 2^16, for every Pauli: entry e = q_a - 1, where q_a is the side's
@@ -284,6 +302,21 @@ cudaError_t launch_walks_batch_e4(const BatchArgs &a, cudaStream_t s);
 cudaError_t launch_rewalk_batch_e4(const BatchArgs &a, cudaStream_t s);
 int engine4_warps(); // warps of its CTA
 int engine4_walks_per_task();
+// n = 2, 3 with lv.q8: eight walks to a warp (qcs_quad.cu)
+cudaError_t launch_walks_q(const WalkLaunch &w, cudaStream_t s);
+cudaError_t launch_rewalk_q(const WalkLaunch &w, cudaStream_t s);
+// jobs of a batch: tasks of quad_walks_per_task() walks, and the jobs' re-walks
+cudaError_t launch_walks_batch_q(int n, const BatchArgs &a, cudaStream_t s);
+cudaError_t launch_rewalk_batch_q(int n, const BatchArgs &a, cudaStream_t s);
+int quad_walks_per_task();
+// below this many n = 3 walks in a launch the warp-per-walk kernels are the
+// faster ones (us a launch of 64 steps at theta 2^-8 and 2^-2, quads / them:
+// 1000 walks 127 / 94 and 179 / 109, 3000 129 / 144 and 185 / 168, 10000 208 /
+// 318 and 257 / 364; 4566 walks x 55 steps at theta 1/2 167 / 164).  At n = 2
+// quads always win (200 walks: 53 / 88 and 86 / 112).
+constexpr uint32_t kQuadWalks3 = 6144;
+cudaError_t launch_walk_step_q(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
+                               size_t count, cudaStream_t s);
 // DP-owner sharding: insert `count` distinguished points {dp, trail ref}
 // into w's table (merges queued as by the walk), and bin points by owner
 // rank (owner_of in qcs_walk.cu): out gets the points grouped by owner in
@@ -329,8 +362,10 @@ int pauli_phase(int n, uint32_t p, uint32_t q); // P(p)P(q) = i^lambda P(p^q)
 // device tables of the first adjoint stage (LevelCtx::T1), built once per
 // device and qubit count and kept for the life of the process
 // (*uploaded, when given, grows by the bytes this call copied to the device)
-// (t4: LevelCtx::T4, null below n = 3)
-int stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], int64_t *uploaded = nullptr);
+// (t4: LevelCtx::T4, null at n = 1)
+// (quad: LevelCtx::quad, null unless n is 2 or 3)
+int stage_tables(int n, const uint32_t *t1[2], const uint32_t *t4[2], const uint32_t **quad,
+                 int64_t *uploaded = nullptr);
 
 // How a level is walked (Sec. 3 and Appendix): theta, the launch shape, the
 // function-version period and the level's step budget.
@@ -368,8 +403,10 @@ struct qcs_problem {
     uint2 *dC32 = nullptr, *dU = nullptr;
     uint32_t *dCq = nullptr; // n >= 3, when every entry of C^ fits in int8
     uint32_t *dCm = nullptr; // n = 4, when C^ suits the tensor-core engine: LevelCtx::Cm, then Csum
+    bool q8 = false;         // LevelCtx::q8
     const uint32_t *dT1[2] = {nullptr, nullptr}; // shared stage tables
     const uint32_t *dT4[2] = {nullptr, nullptr}; // and their form by code (LevelCtx::T4)
+    const uint32_t *dQuad = nullptr;             // LevelCtx::quad
     uint32_t *dCoef = nullptr;
     qcs::Slot *dTable = nullptr;
     qcs::Pair *dQueue = nullptr;

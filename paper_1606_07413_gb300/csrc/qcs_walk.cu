@@ -939,6 +939,11 @@ template <int NQ>
 cudaError_t walk_step_n(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
                         size_t count, cudaStream_t s)
 {
+    // quads, but for short n = 3 lists, whose one step does not make up for
+    // the larger set-up (us a launch: 4096 states 9.3 against 8.2, 16384 12.0
+    // / 14.2, 50021 19 / 28; n = 2: 64 5.2 / 6.3, 50021 8 / 17)
+    if ((NQ == 2 || (NQ == 3 && count >= 8192)) && lv.q8)
+        return launch_walk_step_q(lv, chunk, in, out, is_dp, count, s);
     cudaFuncSetAttribute(k_walk_step<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<NQ>::smem_bytes);
     k_walk_step<NQ><<<grid_for<NQ>(count), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(lv, (uint32_t)chunk, in, out, is_dp,
                                                                                count);
@@ -957,7 +962,9 @@ template <int NQ>
 cudaError_t walks_n(const WalkLaunch &w, cudaStream_t s)
 {
     switch (w.shape) {
-    case 0: return walks_ns<NQ, 0>(w, s);
+    case 0:
+        if ((NQ == 2 || (NQ == 3 && (uint32_t)w.n_walks >= kQuadWalks3)) && w.lv.q8) return launch_walks_q(w, s);
+        return walks_ns<NQ, 0>(w, s);
     case 1: if constexpr (shape_count(NQ) > 1) return walks_ns<NQ, 1>(w, s); break;
     case 2: if constexpr (shape_count(NQ) > 2) return walks_ns<NQ, 2>(w, s); break;
     case 3:
@@ -1028,6 +1035,7 @@ cudaError_t rewalk_pairs_n(const WalkLaunch &w, cudaStream_t s)
     // against 47 us; 130: 54 / 66; 17320: 115 / 193; 116090: 311 / 869 us at
     // theta 1/2, 431 at 2^-8: 1.25 / 1.42 ms)
     if (NQ == 4 && w.lv.Cm) return launch_rewalk_e4(w, s);
+    if ((NQ == 2 || NQ == 3) && w.lv.q8) return launch_rewalk_q(w, s);
     cudaFuncSetAttribute(k_rewalk_pairs<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)Geo<NQ>::smem_bytes);
     k_rewalk_pairs<NQ><<<grid_for<NQ>(w.qcap), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(w);
