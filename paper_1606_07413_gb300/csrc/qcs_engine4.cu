@@ -1045,6 +1045,124 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_certify_e4(CertArgs a)
     e4::cta_close(c);
 }
 
+// f of a list of states: slot lane * kSets + X of the CTA takes the state of
+// that index among the CTA's and every stride-th after it; a state is loaded
+// a round before it is published and its image stored a round after.  us a
+// launch at level 7 against the dp4a warp-per-state kernel: 16 states 15.5 /
+// 19.4 (C^ is read once a CTA here too), 2500 19 / 30, 10000 24 / 53, 50021
+// 51 / 164; 33 of the last are the engine's rate and 15 its set-up.
+__device__ __forceinline__ bool list_control(const LevelCtx &lv, uint32_t chunk, const uint64_t *in, uint64_t *out,
+                                             uint8_t *is_dp, size_t count, uint32_t slots, const e4::Cta &c,
+                                             uint64_t *next, int X, int lane)
+{
+    using namespace e4;
+    const Stages sg(lv);
+    const uint32_t slot = (uint32_t)(lane * kSets + X);
+    const size_t stride = (size_t)slots * gridDim.x;
+    const uint64_t cc = (lv.k & 1) ? sg.chunk_code(chunk) : 0ull;
+    const HashBase hb = c.chunk_base()[chunk];
+    size_t i = (size_t)blockIdx.x * slots + slot, at = 0;
+    bool valid = lane < kSet && slot < slots && i < count, late = false, have = false, ok = true;
+    uint64_t x = valid ? in[i] : 0ull, nx = 0, y = 0;
+    uint32_t ph = 0;
+    while (__any_sync(0xFFFFFFFFu, valid)) {
+        const int side = (int)(x & 1);
+        uint32_t pos;
+        const bool go = publish(c, X, lane, valid, late, side, sg.seq(side, rotations(x, lv), cc),
+                                side ? sg.ns_w : sg.ns_v, hb, &pos);
+        if (have) {
+            out[at] = y;
+            if (is_dp) is_dp[at] = (uint8_t)((y >> lv.dshift) == 0);
+        }
+        if (go && i + stride < count) nx = in[i + stride];
+        late = valid && !go;
+        __syncwarp();
+        if (!mbar_wait(c.bar_sums(X), ph)) {
+            ok = false;
+            break;
+        }
+        ph ^= 1u;
+        y = slot_hash(c, X, lane, go ? side : 0, pos) & lv.maskL;
+        have = go;
+        at = i;
+        if (go) {
+            i += stride;
+            valid = i < count;
+            x = nx;
+        }
+    }
+    if (ok && have) {
+        out[at] = y;
+        if (is_dp) is_dp[at] = (uint8_t)((y >> lv.dshift) == 0);
+    }
+    if (lane < kSet) next[slot] = i; // the slot's first state not stored
+    __syncwarp();
+    if (ok) publish_done(c, X, lane);
+    return ok;
+}
+
+// The full hash of one point by one warp alone, no barrier but its own: what
+// is left when a bounded wait ran out and the caller has no status to report
+// it by.  buf: 512 words of shared memory of the warp's own.
+__device__ __noinline__ uint64_t hash_alone(const LevelCtx &lv, const uint32_t *tab, int side, uint64_t seq, int ns,
+                                            HashBase hb, uint32_t *buf, int lane)
+{
+    using namespace e4;
+    uint32_t ua[8], ub[8];
+    first_stage<4>(lv.T4[side], (uint32_t)seq & 0xFFu, lane, ua, ub);
+    for (int i = 1; i < ns; i++) stage<4>((uint32_t)(seq >> (8 * i)) & 0xFFu, (uint32_t)side, tab, lane, ua, ub);
+    if (side == 0) return smix(v_column_sum(ua, ub, lv.ev, hb.PH, hb.pre16, lane));
+    for (int t = 0; t < 8; t++) {
+        buf[8 * lane + t] = ua[t];
+        buf[256 + 8 * lane + t] = ub[t];
+    }
+    __syncwarp();
+    uint64_t acc = 0;
+    for (int t = 0; t < 8; t++) {
+        const int Q = lane + 32 * t;
+        const uint8_t *col = reinterpret_cast<const uint8_t *>(lv.Cm) + Q * 512;
+        uint32_t l = 0;
+        for (int k = 0; k < 512; k++) l += buf[k] * (uint32_t)((int)col[k] - 128);
+        if (Q) acc += column_hash(l, hb.PH, hb.pre16);
+    }
+    __syncwarp();
+    return smix(warp_sum64(acc));
+}
+
+__global__ void __launch_bounds__(e4::kThreads, 1) k_walk_step_e4(LevelCtx lv, uint32_t chunk, const uint64_t *in,
+                                                                  uint64_t *out, uint8_t *is_dp, size_t count,
+                                                                  uint32_t slots)
+{
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    using namespace e4;
+    __shared__ uint64_t next[kSets * kSet];
+    const Cta c = cta_open(smem_raw);
+    const bool ok = cta_run(lv, c, false, [&](int X, int lane) {
+        return list_control(lv, chunk, in, out, is_dp, count, slots, c, next, X, lane);
+    });
+    if (!ok) { // the call has no status: what is left is evaluated without the engine
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const uint32_t *tab = reinterpret_cast<const uint32_t *>(smem_raw + off_stage);
+        uint32_t *buf = reinterpret_cast<uint32_t *>(smem_raw + off_B) + 512 * warp;
+        const Stages sg(lv);
+        const uint64_t cc = (lv.k & 1) ? sg.chunk_code(chunk) : 0ull;
+        for (uint32_t j = (uint32_t)warp; j < slots; j += kWarps)
+            for (size_t i = next[j]; i < count; i += (size_t)slots * gridDim.x) {
+                const uint64_t x = in[i];
+                const int side = (int)(x & 1);
+                const uint64_t y = hash_alone(lv, tab, side, sg.seq(side, rotations(x, lv), cc),
+                                              (int)(side ? sg.ns_w : sg.ns_v), c.chunk_base()[chunk], buf, lane) &
+                                   lv.maskL;
+                __syncwarp();
+                if (lane == 0) {
+                    out[i] = y;
+                    if (is_dp) is_dp[i] = (uint8_t)((y >> lv.dshift) == 0);
+                }
+            }
+    }
+    cta_close(c);
+}
+
 } // namespace
 
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s)
@@ -1081,6 +1199,20 @@ cudaError_t launch_certify_e4(const CertArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const uint64_t ctas = (a.count + e4::kSets * e4::kPairs - 1) / (e4::kSets * e4::kPairs), sms = (uint64_t)num_sms();
     k_certify_e4<<<(unsigned)(ctas < sms ? ctas : sms), e4::kThreads, e4::smem_bytes, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_walk_step_e4(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
+                                size_t count, cudaStream_t s)
+{
+    if (count == 0) return cudaSuccess;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_walk_step_e4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e4::smem_bytes);
+    if (e != cudaSuccess) return e;
+    const size_t sms = (size_t)num_sms(), full = sms * e4::kSets * e4::kSet, rounds = (count + full - 1) / full;
+    const size_t slots = (count + rounds * sms - 1) / (rounds * sms), ctas = (count + slots - 1) / slots;
+    k_walk_step_e4<<<(unsigned)(ctas < sms ? ctas : sms), e4::kThreads, e4::smem_bytes, s>>>(
+        lv, (uint32_t)chunk, in, out, is_dp, count, (uint32_t)slots);
     return cudaGetLastError();
 }
 

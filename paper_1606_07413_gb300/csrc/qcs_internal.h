@@ -297,6 +297,9 @@ cudaError_t launch_walks(const WalkLaunch &w, cudaStream_t s);
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s);
 // the re-walk of a level's merges on the engine
 cudaError_t launch_rewalk_e4(const WalkLaunch &w, cudaStream_t s);
+// f of a list of states on the engine
+cudaError_t launch_walk_step_e4(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
+                                size_t count, cudaStream_t s);
 // jobs of a batch on the engine: tasks of engine4_walks_per_task() walks, and the jobs' re-walks
 cudaError_t launch_walks_batch_e4(const BatchArgs &a, cudaStream_t s);
 cudaError_t launch_rewalk_batch_e4(const BatchArgs &a, cudaStream_t s);

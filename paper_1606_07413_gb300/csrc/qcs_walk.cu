@@ -944,6 +944,7 @@ cudaError_t walk_step_n(const LevelCtx &lv, int chunk, const uint64_t *in, uint6
     // / 14.2, 50021 19 / 28; n = 2: 64 5.2 / 6.3, 50021 8 / 17)
     if ((NQ == 2 || (NQ == 3 && count >= 8192)) && lv.q8)
         return launch_walk_step_q(lv, chunk, in, out, is_dp, count, s);
+    if (NQ == 4 && lv.Cm) return launch_walk_step_e4(lv, chunk, in, out, is_dp, count, s);
     cudaFuncSetAttribute(k_walk_step<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<NQ>::smem_bytes);
     k_walk_step<NQ><<<grid_for<NQ>(count), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(lv, (uint32_t)chunk, in, out, is_dp,
                                                                                count);

@@ -51,6 +51,25 @@ def test_engine_walk_equals_the_dp4a_walk(dev, t, k, walks, steps, dpb):
     assert a[1] == b[1]
 
 
+# lists of one state, around a state to a slot and two, and in place: the
+# images are stored a round after they are known
+@pytest.mark.parametrize("t", [0, 7, 13])
+def test_engine_step_equals_the_dp4a_step(dev, t):
+    gates, _ = W.seeded_target(4, t, 4100 + t)
+    with Q.Problem.from_circuit(4, gates, 15, Q.default_params(4)) as a, \
+            Q.Problem.from_circuit(4, gates, 15, Q.default_params(4, c_layout=1)) as b:
+        for k in range(16):
+            for count in ((1, 153, 10944, 10945, 32833) if k in (4, 7) else (305,)):
+                x = torch.from_numpy(W.seeded_states(count, 64, 9 * k + count).view(np.int64)).to(dev)
+                chunk = (255 if count == 153 else 1 + (7 * k) % 255) if k & 1 else 0
+                got = []
+                for prob in (a, b):
+                    y, dp = x.clone(), torch.empty(count, dtype=torch.uint8, device=dev)
+                    prob.walk_step(k, chunk, 4, y, y, dp)
+                    got.append((y.cpu().numpy(), dp.cpu().numpy()))
+                assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1]), (k, count)
+
+
 M64 = (1 << 64) - 1
 
 
