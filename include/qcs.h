@@ -116,9 +116,10 @@ typedef struct qcs_params {
     int32_t launch_shape;     /* launch shape of the level-walk kernel, 0 .. qcs_launch_shapes(n) - 1
                                  (default 3 at n = 4, else 0); the walks and results do not depend on
                                  it.  n = 4, shape 3: the tensor-core engine (the W side's
-                                 contraction as f16 byte planes with exact f32 sums), when C^ is held
-                                 in int8 (c_layout 0) and its columns' absolute sums are at most
-                                 1820; otherwise it runs shape 0 */
+                                 contraction as f16 byte planes with exact f32 sums), when c_layout is
+                                 0, C^'s numerators are at most 2048 and its columns' absolute sums
+                                 at most 16448 (any C^ up to denominator exponent 19); otherwise it
+                                 runs shape 0 */
     int32_t c_layout;         /* device layout of C^ for the W side's contraction (n >= 3): 0 = signed
                                  byte quads when every entry fits in int8 (dp4a), else 32-bit words;
                                  1 = 32-bit words always (IMAD).  Results do not depend on it */

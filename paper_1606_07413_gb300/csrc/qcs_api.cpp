@@ -100,7 +100,6 @@ LevelCtx qcs::make_level(const qcs_problem *P, int k, uint32_t version, int dp_b
     lv.C32 = P->dC32;
     lv.Cq = reinterpret_cast<const uint4 *>(P->dCq);
     lv.Cm = reinterpret_cast<const uint4 *>(P->dCm);
-    lv.Csum = P->dCm ? reinterpret_cast<const int16_t *>(P->dCm + (size_t)P->D * P->D / 2) : nullptr;
     lv.q8 = P->q8 ? 1 : 0;
     lv.quad = reinterpret_cast<const uint4 *>(P->dQuad);
     lv.U = P->dU;
@@ -315,29 +314,38 @@ int upload_problem(qcs_problem *P)
                             cq[o] = wa;
                             cq[o + 1] = wb;
                         }
-            if (n == 4) {
-                // the engine's layout (LevelCtx::Cm, Csum): biased bytes by
-                // column, then each column's sum, if the sums suit its f32
-                // accumulation
-                cm.assign((size_t)D * D / 2 + (size_t)D / 2, 0);
-                uint8_t *bytes = reinterpret_cast<uint8_t *>(cm.data());
-                int16_t *sums = reinterpret_cast<int16_t *>(cm.data() + (size_t)D * D / 2);
-                int64_t most = 0;
+        }
+    }
+    // n = 4: C^ as the tensor-core engine's f16 operand (LevelCtx::Cm), if
+    // its entries are exact there and its column sums in the f32 product
+    if (n == 4 && P->p.c_layout == 0) {
+        int64_t most = 0, entry = 0;
+        for (int Q = 0; Q < D; Q++) {
+            int64_t abs_sum = 0;
+            for (int j = 1; j < D; j++) { // the identity's row is not part of the product
+                const int64_t a = std::abs(P->C.a[(size_t)j * D + Q]), b = std::abs(P->C.b[(size_t)j * D + Q]);
+                abs_sum += a + b;
+                entry = std::max(entry, std::max(a, b));
+            }
+            most = std::max(most, abs_sum);
+        }
+        if (most <= kMaxColumnSum4 && entry <= kMaxEntry4) {
+            // |v| <= 2048 as f16 bits
+            const auto f16 = [](int64_t v) {
+                const uint32_t m = (uint32_t)(v < 0 ? -v : v);
+                if (m == 0) return (uint16_t)0;
+                const int e = 31 - __builtin_clz(m);
+                const uint32_t frac = e <= 10 ? m << (10 - e) : m >> (e - 10);
+                return (uint16_t)((v < 0 ? 0x8000u : 0u) | (uint32_t)(e + 15) << 10 | (frac & 0x3FFu));
+            };
+            cm.assign((size_t)D * D, 0);
+            uint16_t *w = reinterpret_cast<uint16_t *>(cm.data());
+            for (int i = 0; i < D; i++) {
+                const uint32_t j = row_of(4, (uint32_t)i >> 3, (uint32_t)i & 7);
                 for (int Q = 0; Q < D; Q++) {
-                    int64_t sum = 0, abs_sum = 0;
-                    for (int i = 0; i < D; i++) {
-                        const uint32_t j = row_of(4, (uint32_t)i >> 3, (uint32_t)i & 7);
-                        const int64_t a = P->C.a[(size_t)j * D + Q], b = P->C.b[(size_t)j * D + Q];
-                        bytes[(size_t)Q * 2 * D + i] = (uint8_t)(a + 128);
-                        bytes[(size_t)Q * 2 * D + D + i] = (uint8_t)(b + 128);
-                        if (j == 0) continue; // the identity's row is not part of the product
-                        sum += a + b;
-                        abs_sum += std::abs(a) + std::abs(b);
-                    }
-                    sums[Q] = (int16_t)sum;
-                    most = std::max(most, abs_sum);
+                    w[cm_index((uint32_t)Q, (uint32_t)i)] = j ? f16(P->C.a[(size_t)j * D + Q]) : kCmBias;
+                    w[cm_index((uint32_t)Q, (uint32_t)(D + i))] = j ? f16(P->C.b[(size_t)j * D + Q]) : (uint16_t)0;
                 }
-                if (most > kMaxColumnSum) cm.clear();
             }
         }
     }
@@ -1012,7 +1020,7 @@ void qcs_default_params(int n_qubits, qcs_params *p)
     case 3: p->state_bits = 48; p->dp_bits = 10; p->walks = 1 << 16; p->table_log2 = 22; break;
     default:
         p->state_bits = 64; p->dp_bits = 12; p->walks = 1 << 20; p->table_log2 = 26;
-        p->launch_shape = 3; // the tensor-core walk (shape 0 where C^ does not fit int8)
+        p->launch_shape = 3; // the tensor-core walk (shape 0 where C^ does not suit it)
         break;
     }
     p->steps_per_launch = 64;

@@ -35,16 +35,18 @@
 // shared memory; that leaves 192 tensor-memory columns for three sets' D (3 x
 // 2 x 32 f32 columns) and 96 KB of shared memory for three sets' B.
 //
-// Exactness.  B holds 1024 + byte (the f16 bits 0x6400 | byte, so no
-// conversion), and every sum is an integer below 2^24 in magnitude, so f32
-// accumulation is exact.  Row 0 (the identity) has zero weight on both parts,
-// so its two K slots are free; their B values are 1024 and their A values are
-// 12288 and -sum(c), which adds 1.5 x 2^23 and takes the offset's 1024 sum(c)
-// away again: the bits of the f32 result are 0x4B400000 + P, P the integer
-// dot product, and its low 16 bits are those of P.  |P| and every partial sum
-// stay below 2^22 when a column's absolute sum is at most kMaxColumnSum
-// (qcs_internal.h), which the host checks (columns of an orthogonal C^ in
-// int8 obey it up to denominator exponent 13).
+// Exactness.  B holds a weight's byte as the f16 with those bits, a subnormal
+// (byte x 2^-24): no conversion.  C^'s entries are f16 integers (up to 2048),
+// so every sum is a multiple of 2^-24.  Row 0 (the identity) has zero weight
+// on both parts, so its K slots are free; the first one's B value is 1024 and
+// its A value 0.75 / 1024 puts 0.75 on every sum.  While |P| (the integer dot
+// product) and its partial sums stay below 2^22, a sum lies in [0.5, 1], whose
+// f32 spacing is 2^-24: the accumulation is exact and the result's bits are
+// 0x3F400000 + P, its low 16 bits those of P.  That holds when a column's
+// absolute sum is at most kMaxColumnSum4 (qcs_internal.h), which the host
+// checks.  (With 1024 + byte in B and 1.5 x 2^23 as the offset the bound was
+// 1820, and C^ of 15 rotations went to the 32-bit-word kernels: 2^15 walks x
+// 16 steps 15.4 ms there, 0.37 ms here.)
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -357,49 +359,27 @@ __device__ __forceinline__ void level_begin(const LevelCtx &lv, const Cta &c, bo
     }
 }
 
-// two biased bytes of a word of LevelCtx::Cm as an f16 pair: the byte permute
-// puts them under 0x64 (1024 + byte in f16), then 1152 is subtracted
-__device__ __forceinline__ uint32_t bytes_to_f16x2(uint32_t word, uint32_t sel)
-{
-    const uint32_t v = __byte_perm(word, 0x64646464u, sel);
-    __half2 h = *reinterpret_cast<const __half2 *>(&v);
-    h = __hsub2(h, __float2half2_rn(1152.f));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
 // C^ into tensor and shared memory; every thread calls it, and a barrier follows
 __device__ __forceinline__ void load_c(const LevelCtx &lv, const Cta &c)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr uint32_t kBias = 0x7200u; // 12288 in f16: 1024 * 12288 = 1.5 * 2^23
     if (warp < kWorkers) {
         // warp w writes the tensor-memory lanes 32 (w % 4) ..: K-blocks
         // w / 4, w / 4 + 4, .. of its 32 columns of either half
         const uint32_t tq = c.tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         for (int b = warp >> 2; b < 32 + kTmemK; b += kWorkers / 4) {
-            const int half = b >= 32, kb = half ? b - 32 : b, Q = 128 * half + 32 * (warp & 3) + lane;
-            const uint4 w = __ldg(lv.Cm + Q * 32 + kb);
-            uint32_t v[8] = {bytes_to_f16x2(w.x, 0x4140), bytes_to_f16x2(w.x, 0x4342), bytes_to_f16x2(w.y, 0x4140),
-                             bytes_to_f16x2(w.y, 0x4342), bytes_to_f16x2(w.z, 0x4140), bytes_to_f16x2(w.z, 0x4342),
-                             bytes_to_f16x2(w.w, 0x4140), bytes_to_f16x2(w.w, 0x4342)};
-            if (kb == 0) v[0] = (v[0] & 0xFFFF0000u) | kBias;
-            if (kb == 16)
-                v[0] = (v[0] & 0xFFFF0000u) | __half_as_ushort(__float2half_rn(-(float)lv.Csum[Q]));
-            tmem_st8(tq + (half ? 256u : 0u) + 8u * (uint32_t)kb, v);
+            const uint4 *src = lv.Cm + (size_t)(b * 128 + 32 * (warp & 3) + lane) * 2;
+            const uint4 w0 = __ldg(src), w1 = __ldg(src + 1);
+            const uint32_t v[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+            tmem_st8(tq + 8u * (uint32_t)b, v);
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
-    // second half, K-blocks kTmemK ..: 16-byte units (8 K) of 128 rows
-    constexpr int U0 = 2 * kTmemK, UN = 64 - U0;
-    for (int i = threadIdx.x; i < 128 * UN; i += kThreads) {
-        const int r = i / UN, u = U0 + i % UN, Q = 128 + r;
-        const uint2 w = __ldg(reinterpret_cast<const uint2 *>(lv.Cm + Q * 32) + u);
-        uint4 v = make_uint4(bytes_to_f16x2(w.x, 0x4140), bytes_to_f16x2(w.x, 0x4342), bytes_to_f16x2(w.y, 0x4140),
-                             bytes_to_f16x2(w.y, 0x4342));
-        if (u == 32) v.x = (v.x & 0xFFFF0000u) | __half_as_ushort(__float2half_rn(-(float)lv.Csum[Q]));
-        *reinterpret_cast<uint4 *>(c.raw + off_A + (size_t)((u >> 3) - U0 / 8) * 16384 + (r >> 3) * 1024 +
-                                   (r & 7) * 128 + (((u & 7) ^ (r & 7)) * 16)) = v;
-    }
+    // the rest of the second half, as it lies in shared memory
+    static_assert(kTmemK == 8, "cm_index");
+    const uint4 *src = lv.Cm + (32 + kTmemK) * 256;
+    uint4 *dst = reinterpret_cast<uint4 *>(c.raw + off_A);
+    for (int i = threadIdx.x; i < 6 * 1024; i += kThreads) dst[i] = __ldg(src + i);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tmem_fence_before();
 }
@@ -426,7 +406,7 @@ __device__ __forceinline__ void point_a(const LevelCtx &lv, const Cta &c, int X,
         // lane's eight rows are the K indices 8 lane .. of each part, one
         // 16-byte unit; unit u of row r is at unit u ^ (r & 7) of its 128
         // bytes in chunk u / 8.
-        const uint32_t r = 2 * (info >> 16);
+        const uint32_t r = 2 * (info >> 16), one = lane == 0 ? 0x6400u : 0u; // K slot 0
         unsigned char *b = c.raw + off_B + (size_t)X * 8 * kN * 128 + (size_t)(lane >> 3) * (kN * 128) + (r >> 3) * 1024;
 #pragma unroll
         for (int p = 0; p < 2; p++) { // a, b part
@@ -435,8 +415,12 @@ __device__ __forceinline__ void point_a(const LevelCtx &lv, const Cta &c, int X,
             for (int e = 0; e < 4; e++) {
                 const uint32_t w = p ? __byte_perm(ub[2 * e], ub[2 * e + 1], 0x5410)
                                      : __byte_perm(ua[2 * e], ua[2 * e + 1], 0x5410);
-                lo[e] = (w & 0x00FF00FFu) | 0x64006400u;
-                hi[e] = __byte_perm(w, 0x64646464u, 0x4341);
+                lo[e] = w & 0x00FF00FFu;
+                hi[e] = __byte_perm(w, 0, 0x4341);
+                if (p == 0 && e == 0) {
+                    lo[e] |= one;
+                    hi[e] |= one;
+                }
             }
             unsigned char *d = b + (size_t)p * 4 * (kN * 128);
             const uint32_t u = (uint32_t)lane & 7u, r0 = r & 7u;
@@ -1050,7 +1034,7 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_certify_e4(CertArgs a)
 // a round before it is published and its image stored a round after.  us a
 // launch at level 7 against the dp4a warp-per-state kernel: 16 states 15.5 /
 // 19.4 (C^ is read once a CTA here too), 2500 19 / 30, 10000 24 / 53, 50021
-// 51 / 164; 33 of the last are the engine's rate and 15 its set-up.
+// 48 / 164; 33 of the last are the engine's rate and 15 its set-up.
 __device__ __forceinline__ bool list_control(const LevelCtx &lv, uint32_t chunk, const uint64_t *in, uint64_t *out,
                                              uint8_t *is_dp, size_t count, uint32_t slots, const e4::Cta &c,
                                              uint64_t *next, int X, int lane)
@@ -1120,9 +1104,11 @@ __device__ __noinline__ uint64_t hash_alone(const LevelCtx &lv, const uint32_t *
     uint64_t acc = 0;
     for (int t = 0; t < 8; t++) {
         const int Q = lane + 32 * t;
-        const uint8_t *col = reinterpret_cast<const uint8_t *>(lv.Cm) + Q * 512;
+        const unsigned short *col = reinterpret_cast<const unsigned short *>(lv.Cm);
         uint32_t l = 0;
-        for (int k = 0; k < 512; k++) l += buf[k] * (uint32_t)((int)col[k] - 128);
+        for (uint32_t k = 0; k < 512; k++)
+            if (k & 255u) // the identity's weights are zero
+                l += buf[k] * (uint32_t)(int)__half2float(__ushort_as_half(col[cm_index((uint32_t)Q, k)]));
         if (Q) acc += column_hash(l, hb.PH, hb.pre16);
     }
     __syncwarp();

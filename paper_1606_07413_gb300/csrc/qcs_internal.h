@@ -50,12 +50,29 @@ __host__ __device__ constexpr uint32_t code_pauli(int n, uint32_t code)
 {
     return row_of(n, code & ((1u << (2 * n - 3)) - 1u), code >> (2 * n - 3));
 }
-// A column of C^ suits the tensor-core kernels' f32 sums when the absolute values of its
-// entries add up to at most this: a partial sum of the product is below
-// (1279 + 1024) * 1820 + 1279 < 2^22 (weights up to 1024 + 255, the offset's
-// correction, and V's own k-step in qcs_quad.cu).  By orthogonality a column's squares a^2 + 2 b^2 add up to
-// 2^E, so the sum is at most 16 sqrt(1.5 * 2^E), 1773 at E = 13.
+// A column of C^ suits the quad kernels' f32 sums (qcs_quad.cu) when the
+// absolute values of its entries add up to at most this: a partial sum of the
+// product is below (1279 + 1024) * 1820 + 1279 < 2^22 (weights up to 1024 +
+// 255, the offset's correction, and V's own k-step).
 constexpr int kMaxColumnSum = 1820;
+// And the n = 4 engine (qcs_engine4.cu), whose weights are bytes: 255 * 16448
+// < 2^22, and entries up to 2048 are exact in f16.  By orthogonality a
+// column's squares a^2 + 2 b^2 add up to 2^E, so its sum is at most 16
+// sqrt(1.5 * 2^E), 14189 at E = 19, and an entry at most 2^(E / 2).
+constexpr int kMaxColumnSum4 = 16448, kMaxEntry4 = 2048;
+constexpr uint16_t kCmBias = 0x1200; // 0.75 / 1024 in f16
+// f16 index in LevelCtx::Cm of column Q, K index k (part * 256 + 8 l + t).
+// First what goes to tensor memory, columns 0 .. 127 and then K-blocks 0 .. 7
+// of the others, 16 K of one column together; then K-blocks 8 .. 31 of columns
+// 128 .. 255 as they lie in shared memory (chunks of 64 K x 128 columns, 128
+// bytes a column, its 16-byte units exchanged by the 128-byte swizzle).
+__host__ __device__ constexpr uint32_t cm_index(uint32_t Q, uint32_t k)
+{
+    const uint32_t r = Q & 127u;
+    return Q < 128 || k < 128
+               ? (((Q >> 7) * 32 + (k >> 4)) * 128 + r) * 16 + (k & 15u)
+               : 40 * 2048 + ((k >> 6) - 2) * 8192 + (r >> 3) * 512 + (r & 7u) * 64 + ((((k >> 3) ^ r) & 7u) * 8) + (k & 7u);
+}
 
 // Everything a warp needs to evaluate one step f of the walk at one level.
 struct LevelCtx {
@@ -70,11 +87,10 @@ struct LevelCtx {
     // a-quad Q1, b-quad Q1) (W, R as above).
     const uint4 *Cq;
     // n = 4, when C^ suits the tensor-core engine (qcs_engine4.cu), else null:
-    // every entry as the byte entry + 128, 512 bytes a column.  Byte
-    // part * 256 + 8 l + t of column Q is the a (part 0) or b (part 1) of row
-    // row_of(4, l, t).  Csum[Q]: the sum of the column's entries.
+    // C^ as its f16 operand, 512 K by 256 columns, ordered by cm_index.  K
+    // index part * 256 + 8 l + t is the a (part 0) or b (part 1) of row
+    // row_of(4, l, t); the identity's are kCmBias and 0.
     const uint4 *Cm;
-    const int16_t *Csum;
     // n >= 2: the weights after the first adjoint stage, as T1, by code: word
     // code * 4^n + 8 l + t is row row_of(n, l, t)'s Ua | Ub << 16 after the
     // Pauli of that code; code 0 holds the weights themselves.
@@ -405,7 +421,7 @@ struct qcs_problem {
     // device data
     uint2 *dC32 = nullptr, *dU = nullptr;
     uint32_t *dCq = nullptr; // n >= 3, when every entry of C^ fits in int8
-    uint32_t *dCm = nullptr; // n = 4, when C^ suits the tensor-core engine: LevelCtx::Cm, then Csum
+    uint32_t *dCm = nullptr; // n = 4, when C^ suits the tensor-core engine: LevelCtx::Cm
     bool q8 = false;         // LevelCtx::q8
     const uint32_t *dT1[2] = {nullptr, nullptr}; // shared stage tables
     const uint32_t *dT4[2] = {nullptr, nullptr}; // and their form by code (LevelCtx::T4)

@@ -1,8 +1,8 @@
 """The n = 4 engine (qcs_engine4.cu) against the dp4a kernels, bit for bit:
 walk counts around one and two rounds of every SM, levels with none to three
 stages beside the first and with and without the chunk's, targets whose C^ is
-sparse or near the largest column sums that the engine takes, and one beyond
-them, which the engine leaves to the dp4a kernels."""
+sparse, beyond int8, near the largest column sums that the engine takes and
+beyond them, where it leaves them to the 32-bit-word kernels."""
 import numpy as np
 import pytest
 
@@ -42,7 +42,8 @@ def walk(dev, shape, t, k, walks, steps, dpb):
 @pytest.mark.parametrize("t,k,walks,steps,dpb", [
     (7, 7, 10944, 9, 3), (7, 7, 10945, 2, 12), (7, 7, 21889, 3, 1), (7, 7, 151, 2, 3), (7, 7, 3800, 2, 3),
     (0, 2, 100, 6, 2), (3, 3, 100, 6, 2), (5, 4, 100, 6, 2), (5, 5, 100, 6, 2), (7, 6, 100, 6, 2), (9, 8, 100, 6, 2),
-    (9, 9, 100, 6, 2), (7, 15, 100, 4, 2), (13, 7, 500, 8, 2), (12, 13, 500, 8, 2), (15, 7, 500, 4, 2),
+    (9, 9, 100, 6, 2), (7, 15, 100, 4, 2), (13, 7, 500, 8, 2), (12, 13, 500, 8, 2), (15, 7, 10945, 4, 2),
+    (17, 6, 500, 4, 2), (19, 7, 3800, 4, 2), (22, 7, 500, 4, 2),
 ])
 def test_engine_walk_equals_the_dp4a_walk(dev, t, k, walks, steps, dpb):
     a, b = walk(dev, 0, t, k, walks, steps, dpb), walk(dev, 3, t, k, walks, steps, dpb)
@@ -53,7 +54,7 @@ def test_engine_walk_equals_the_dp4a_walk(dev, t, k, walks, steps, dpb):
 
 # lists of one state, around a state to a slot and two, and in place: the
 # images are stored a round after they are known
-@pytest.mark.parametrize("t", [0, 7, 13])
+@pytest.mark.parametrize("t", [0, 7, 13, 15, 18, 19])
 def test_engine_step_equals_the_dp4a_step(dev, t):
     gates, _ = W.seeded_target(4, t, 4100 + t)
     with Q.Problem.from_circuit(4, gates, 15, Q.default_params(4)) as a, \
