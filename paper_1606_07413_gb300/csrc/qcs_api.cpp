@@ -100,7 +100,6 @@ LevelCtx qcs::make_level(const qcs_problem *P, int k, uint32_t version, int dp_b
     lv.C32 = P->dC32;
     lv.Cq = reinterpret_cast<const uint4 *>(P->dCq);
     lv.Cm = reinterpret_cast<const uint4 *>(P->dCm);
-    lv.q8 = P->q8 ? 1 : 0;
     lv.quad = reinterpret_cast<const uint4 *>(P->dQuad);
     lv.U = P->dU;
     for (int side = 0; side < 2; side++) {
@@ -275,23 +274,10 @@ int upload_problem(qcs_problem *P)
         }
     std::vector<uint32_t> coef(coef16.size() / 2);
     memcpy(coef.data(), coef16.data(), sizeof(uint32_t) * coef.size());
-    // n = 2, 3: do the entries fit int8 and the columns the f32 sums of the
-    // quad kernels (the identity's row is not part of a product)
-    if ((n == 2 || n == 3) && P->p.c_layout == 0) {
-        bool fits = true;
-        for (size_t i = 0; i < P->C.a.size() && fits; i++)
-            fits = P->C.a[i] >= -128 && P->C.a[i] <= 127 && P->C.b[i] >= -128 && P->C.b[i] <= 127;
-        for (int Q = 0; Q < D && fits; Q++) {
-            int64_t sum = 0;
-            for (int i = 1; i < D; i++) sum += std::abs(P->C.a[(size_t)i * D + Q]) + std::abs(P->C.b[(size_t)i * D + Q]);
-            fits = sum <= kMaxColumnSum;
-        }
-        P->q8 = fits;
-    }
     // n >= 3: also C^ as signed byte quads (rows 4q .. 4q+3 of a column in
     // one word) when every entry fits in int8, laid out for the walk
     // kernel's byte-plane contraction (LevelCtx::Cq)
-    std::vector<uint32_t> cq, cm;
+    std::vector<uint32_t> cq;
     if (n >= 3 && P->p.c_layout == 0) {
         bool fits = true;
         for (size_t i = 0; i < P->C.a.size() && fits; i++)
@@ -316,9 +302,10 @@ int upload_problem(qcs_problem *P)
                         }
         }
     }
-    // n = 4: C^ as the tensor-core engine's f16 operand (LevelCtx::Cm), if
-    // its entries are exact there and its column sums in the f32 product
-    if (n == 4 && P->p.c_layout == 0) {
+    // n >= 2: does C^ suit the tensor-core kernels (LevelCtx::Cm), its entries
+    // as f16 and its column sums as f32
+    bool operand = false;
+    if (n >= 2 && P->p.c_layout == 0) {
         int64_t most = 0, entry = 0;
         for (int Q = 0; Q < D; Q++) {
             int64_t abs_sum = 0;
@@ -329,25 +316,7 @@ int upload_problem(qcs_problem *P)
             }
             most = std::max(most, abs_sum);
         }
-        if (most <= kMaxColumnSum4 && entry <= kMaxEntry4) {
-            // |v| <= 2048 as f16 bits
-            const auto f16 = [](int64_t v) {
-                const uint32_t m = (uint32_t)(v < 0 ? -v : v);
-                if (m == 0) return (uint16_t)0;
-                const int e = 31 - __builtin_clz(m);
-                const uint32_t frac = e <= 10 ? m << (10 - e) : m >> (e - 10);
-                return (uint16_t)((v < 0 ? 0x8000u : 0u) | (uint32_t)(e + 15) << 10 | (frac & 0x3FFu));
-            };
-            cm.assign((size_t)D * D, 0);
-            uint16_t *w = reinterpret_cast<uint16_t *>(cm.data());
-            for (int i = 0; i < D; i++) {
-                const uint32_t j = row_of(4, (uint32_t)i >> 3, (uint32_t)i & 7);
-                for (int Q = 0; Q < D; Q++) {
-                    w[cm_index((uint32_t)Q, (uint32_t)i)] = j ? f16(P->C.a[(size_t)j * D + Q]) : kCmBias;
-                    w[cm_index((uint32_t)Q, (uint32_t)(D + i))] = j ? f16(P->C.b[(size_t)j * D + Q]) : (uint16_t)0;
-                }
-            }
-        }
+        operand = most <= kMaxColumnSum && entry <= kMaxEntry;
     }
     CK(cudaGetDevice(&P->device));
     int64_t h2d = 0;
@@ -357,17 +326,17 @@ int upload_problem(qcs_problem *P)
         CK(cudaMemcpy(P->dCq, cq.data(), sizeof(uint32_t) * cq.size(), cudaMemcpyHostToDevice));
         h2d += (int64_t)(sizeof(uint32_t) * cq.size());
     }
-    if (!cm.empty()) {
-        CK(cudaMalloc(&P->dCm, sizeof(uint32_t) * cm.size()));
-        CK(cudaMemcpy(P->dCm, cm.data(), sizeof(uint32_t) * cm.size(), cudaMemcpyHostToDevice));
-        h2d += (int64_t)(sizeof(uint32_t) * cm.size());
-    }
     CK(cudaMalloc(&P->dC32, sizeof(uint2) * c32.size()));
     CK(cudaMalloc(&P->dU, sizeof(uint2) * D));
     CK(cudaMalloc(&P->dCoef, sizeof(uint32_t) * coef.size()));
     CK(cudaMemcpy(P->dC32, c32.data(), sizeof(uint2) * c32.size(), cudaMemcpyHostToDevice));
+    if (operand) {
+        CK(cudaMalloc(&P->dCm, sizeof(uint16_t) * 2 * D * D));
+        CK(launch_operand(n, P->dC32, P->dCm, 0));
+    }
     CK(cudaMemcpy(P->dU, u.data(), sizeof(uint2) * D, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(P->dCoef, coef.data(), sizeof(uint32_t) * coef.size(), cudaMemcpyHostToDevice));
+    if (operand) CK(cudaStreamSynchronize(0)); // the first launch may be on a stream that does not wait for this one
     h2d += (int64_t)(sizeof(uint2) * c32.size() + sizeof(uint2) * D + sizeof(uint32_t) * coef.size());
     P->res.h2d_bytes += h2d;
     return QCS_OK;

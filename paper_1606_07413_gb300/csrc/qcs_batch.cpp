@@ -292,8 +292,8 @@ int job_class(const qcs_batch *B, const Job &j, uint64_t walks3)
     const int n = j.P->n, shape = B->bp.launch_shape[n - 1];
     bool tensor = false;
     if (n == 4) tensor = j.w.lv.Cm && (shape == 0 || shape == 3);
-    else if (n == 3) tensor = j.w.lv.q8 && shape == 0 && walks3 >= kQuadWalks3;
-    else if (n == 2) tensor = j.w.lv.q8 != 0;
+    else if (n == 3) tensor = j.w.lv.Cm && shape == 0 && walks3 >= kQuadWalks3;
+    else if (n == 2) tensor = j.w.lv.Cm != nullptr;
     return tensor ? kTensor + n : n;
 }
 

@@ -43,7 +43,7 @@
 // product) and its partial sums stay below 2^22, a sum lies in [0.5, 1], whose
 // f32 spacing is 2^-24: the accumulation is exact and the result's bits are
 // 0x3F400000 + P, its low 16 bits those of P.  That holds when a column's
-// absolute sum is at most kMaxColumnSum4 (qcs_internal.h), which the host
+// absolute sum is at most kMaxColumnSum (qcs_internal.h), which the host
 // checks.  (With 1024 + byte in B and 1.5 x 2^23 as the offset the bound was
 // 1820, and C^ of 15 rotations went to the 32-bit-word kernels: 2^15 walks x
 // 16 steps 15.4 ms there, 0.37 ms here.)
@@ -416,11 +416,8 @@ __device__ __forceinline__ void point_a(const LevelCtx &lv, const Cta &c, int X,
                 const uint32_t w = p ? __byte_perm(ub[2 * e], ub[2 * e + 1], 0x5410)
                                      : __byte_perm(ua[2 * e], ua[2 * e + 1], 0x5410);
                 lo[e] = w & 0x00FF00FFu;
-                hi[e] = __byte_perm(w, 0, 0x4341);
-                if (p == 0 && e == 0) {
-                    lo[e] |= one;
-                    hi[e] |= one;
-                }
+                hi[e] = __byte_perm(w, p == 0 && e == 0 ? one : 0u, 0x7351);
+                if (p == 0 && e == 0) lo[e] |= one;
             }
             unsigned char *d = b + (size_t)p * 4 * (kN * 128);
             const uint32_t u = (uint32_t)lane & 7u, r0 = r & 7u;

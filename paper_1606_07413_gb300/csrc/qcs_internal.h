@@ -50,18 +50,15 @@ __host__ __device__ constexpr uint32_t code_pauli(int n, uint32_t code)
 {
     return row_of(n, code & ((1u << (2 * n - 3)) - 1u), code >> (2 * n - 3));
 }
-// A column of C^ suits the quad kernels' f32 sums (qcs_quad.cu) when the
-// absolute values of its entries add up to at most this: a partial sum of the
-// product is below (1279 + 1024) * 1820 + 1279 < 2^22 (weights up to 1024 +
-// 255, the offset's correction, and V's own k-step).
-constexpr int kMaxColumnSum = 1820;
-// And the n = 4 engine (qcs_engine4.cu), whose weights are bytes: 255 * 16448
-// < 2^22, and entries up to 2048 are exact in f16.  By orthogonality a
-// column's squares a^2 + 2 b^2 add up to 2^E, so its sum is at most 16
-// sqrt(1.5 * 2^E), 14189 at E = 19, and an entry at most 2^(E / 2).
-constexpr int kMaxColumnSum4 = 16448, kMaxEntry4 = 2048;
+// C^ suits the tensor-core kernels (qcs_engine4.cu, qcs_quad.cu) when the
+// absolute values of a column's entries add up to at most kMaxColumnSum (the
+// weights are bytes: 255 * 16448 < 2^22) and none is above 2048 (exact in
+// f16).  By orthogonality a column's squares a^2 + 2 b^2 add up to 2^E, so its
+// sum is at most 2^n sqrt(1.5 * 2^E), 14189 at n = 4, E = 19, and an entry at
+// most 2^(E / 2).
+constexpr int kMaxColumnSum = 16448, kMaxEntry = 2048;
 constexpr uint16_t kCmBias = 0x1200; // 0.75 / 1024 in f16
-// f16 index in LevelCtx::Cm of column Q, K index k (part * 256 + 8 l + t).
+// n = 4: f16 index in LevelCtx::Cm of column Q, K index k (part * 256 + 8 l + t).
 // First what goes to tensor memory, columns 0 .. 127 and then K-blocks 0 .. 7
 // of the others, 16 K of one column together; then K-blocks 8 .. 31 of columns
 // 128 .. 255 as they lie in shared memory (chunks of 64 K x 128 columns, 128
@@ -86,16 +83,17 @@ struct LevelCtx {
     // Q0 = sub + 2 W j and Q1 = Q0 + W, the words (a-quad Q0, b-quad Q0,
     // a-quad Q1, b-quad Q1) (W, R as above).
     const uint4 *Cq;
-    // n = 4, when C^ suits the tensor-core engine (qcs_engine4.cu), else null:
-    // C^ as its f16 operand, 512 K by 256 columns, ordered by cm_index.  K
-    // index part * 256 + 8 l + t is the a (part 0) or b (part 1) of row
-    // row_of(4, l, t); the identity's are kCmBias and 0.
+    // n >= 2, when C^ suits the tensor-core kernels, else null: C^ as their
+    // f16 operand, the a and then the b part of every row against every
+    // column; the identity's row holds kCmBias and 0.  n = 4
+    // (qcs_engine4.cu): ordered by cm_index, K index part * 256 + 8 l + t is
+    // row row_of(4, l, t).  n = 2, 3 (qcs_quad.cu): A's fragments, uint4
+    // [tile][part][k-step][lane].
     const uint4 *Cm;
     // n >= 2: the weights after the first adjoint stage, as T1, by code: word
     // code * 4^n + 8 l + t is row row_of(n, l, t)'s Ua | Ub << 16 after the
     // Pauli of that code; code 0 holds the weights themselves.
     const uint4 *T4[2];
-    int32_t q8;        // n = 2, 3: C^ suits the quad kernels (qcs_quad.cu): int8 entries, small column sums
     // n = 2, 3: the quad kernels' tables (stage_tables): T, uint4 [side][code]
     // [row / 4][lane], the weights after the first stage of a code, Ua | Ub <<
     // 16 of four rows; then the signs, i8 [side][code][lane][row], 1 where the
@@ -309,6 +307,8 @@ cudaError_t launch_walk_step(const LevelCtx &lv, int chunk, const uint64_t *in, 
                              uint8_t *is_dp, size_t count, cudaStream_t s);
 cudaError_t launch_init_walks(const WalkLaunch &w, cudaStream_t s);
 cudaError_t launch_walks(const WalkLaunch &w, cudaStream_t s);
+// C^ (LevelCtx::C32) as the tensor-core kernels' operand (LevelCtx::Cm), n >= 2
+cudaError_t launch_operand(int n, const uint2 *C32, uint16_t *Cm, cudaStream_t s);
 // n = 4 with lv.Cm set: the level walk on the tensor-core engine (qcs_engine4.cu)
 cudaError_t launch_walks_e4(const WalkLaunch &w, cudaStream_t s);
 // the re-walk of a level's merges on the engine
@@ -321,7 +321,7 @@ cudaError_t launch_walks_batch_e4(const BatchArgs &a, cudaStream_t s);
 cudaError_t launch_rewalk_batch_e4(const BatchArgs &a, cudaStream_t s);
 int engine4_warps(); // warps of its CTA
 int engine4_walks_per_task();
-// n = 2, 3 with lv.q8: eight walks to a warp (qcs_quad.cu)
+// n = 2, 3 with lv.Cm set: eight walks to a warp (qcs_quad.cu)
 cudaError_t launch_walks_q(const WalkLaunch &w, cudaStream_t s);
 cudaError_t launch_rewalk_q(const WalkLaunch &w, cudaStream_t s);
 // jobs of a batch: tasks of quad_walks_per_task() walks, and the jobs' re-walks
@@ -332,8 +332,10 @@ int quad_walks_per_task();
 // faster ones (us a launch of 64 steps at theta 2^-8 and 2^-2, quads / them:
 // 1000 walks 127 / 94 and 179 / 109, 3000 129 / 144 and 185 / 168, 10000 208 /
 // 318 and 257 / 364; 4566 walks x 55 steps at theta 1/2 167 / 164).  At n = 2
-// quads always win (200 walks: 53 / 88 and 86 / 112).
-constexpr uint32_t kQuadWalks3 = 6144;
+// quads always win (200 walks: 53 / 88 and 86 / 112).  Where C^ is not int8
+// those kernels take 32-bit words: 1000 walks 126 / 152 and 175 / 152, 3000
+// 127 / 228 and 182 / 240.
+constexpr uint32_t kQuadWalks3 = 6144, kQuadWalksWide3 = 2048;
 cudaError_t launch_walk_step_q(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
                                size_t count, cudaStream_t s);
 // DP-owner sharding: insert `count` distinguished points {dp, trail ref}
@@ -421,8 +423,7 @@ struct qcs_problem {
     // device data
     uint2 *dC32 = nullptr, *dU = nullptr;
     uint32_t *dCq = nullptr; // n >= 3, when every entry of C^ fits in int8
-    uint32_t *dCm = nullptr; // n = 4, when C^ suits the tensor-core engine: LevelCtx::Cm
-    bool q8 = false;         // LevelCtx::q8
+    uint16_t *dCm = nullptr; // n >= 2, when C^ suits the tensor-core kernels: LevelCtx::Cm
     const uint32_t *dT1[2] = {nullptr, nullptr}; // shared stage tables
     const uint32_t *dT4[2] = {nullptr, nullptr}; // and their form by code (LevelCtx::T4)
     const uint32_t *dQuad = nullptr;             // LevelCtx::quad

@@ -22,13 +22,13 @@
 //    the others;
 //  - each lane hashes the columns it holds of two walks, the sums are exchanged
 //    and the quad takes its walk's step.
-// The exactness argument is the engine's (qcs_engine4.cu): B holds 1024 +
-// byte, row 0's two k slots add 1.5 x 2^23 and take the offsets away again.
+// The exactness argument is the engine's (qcs_engine4.cu): a weight's byte is
+// the f16 subnormal with those bits, and row 0's first k slot puts 0.75 on
+// every sum.
 //
 // What bounds it: issue.  A step costs about 130 warp instructions at n = 3 and
 // 50 at n = 2 (379 and 325 with one and two walks to a warp, whose bookkeeping
 // ran on all lanes of each).
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -90,28 +90,18 @@ struct Sm {
     uint32_t *x; // this warp's exchange rows
 };
 
-__device__ __forceinline__ uint32_t half2_bits(int lo, int hi)
-{
-    const __half2 h = __halves2half2(__int2half_rn(lo), __int2half_rn(hi));
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
 // C^'s fragments, the first-stage and stage tables and the chunks' hash bases
 // of a level (scale: Level::scale); every thread calls it, a barrier at its
-// end.  The tables are copied from LevelCtx::quad; the fragments are put
-// together here, 3 us of a launch's 5 to 8 before the first step.
+// end.
 template <int NQ>
 __device__ __forceinline__ Sm<NQ> set_up(const LevelCtx &lv, int scale, unsigned char *raw)
 {
     using G = Geo<NQ>;
     uint4 *frag = reinterpret_cast<uint4 *>(raw), *T = reinterpret_cast<uint4 *>(raw + G::off_T);
     HashBase *base = reinterpret_cast<HashBase *>(raw + G::off_base);
-    // the exchange rows (of at least eight warps) are not in use yet: C^ as
-    // signed bytes [row][Q] (a, b), and its columns' sums
-    char2 *c8 = reinterpret_cast<char2 *>(raw + G::off_x);
-    int *sums = reinterpret_cast<int *>(raw + G::off_x + sizeof(char2) * G::D * G::D);
-    static_assert(sizeof(char2) * G::D * G::D + sizeof(int) * G::D <= 8 * G::x_warp, "room for C^");
-    for (int i = threadIdx.x; i < G::D; i += blockDim.x) sums[i] = 1; // V's identity
+    constexpr int nFrag = (int)(G::off_T / sizeof(uint4));
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nFrag; i += blockDim.x) frag[i] = __ldg(lv.Cm + i);
     constexpr int nT = 2 * G::D * G::KS * 4, nAll = (int)((G::off_base - G::off_T) / sizeof(uint4));
 #pragma unroll 4
     for (int i = threadIdx.x; i < nAll; i += blockDim.x) {
@@ -133,42 +123,6 @@ __device__ __forceinline__ Sm<NQ> set_up(const LevelCtx &lv, int scale, unsigned
         const uint64_t tag =
             (uint64_t)lv.n | ((uint64_t)lv.k << 8) | ((uint64_t)i << 16) | ((uint64_t)(uint32_t)lv.K << 32);
         base[i] = hash_base(smix(vmix ^ tag));
-    }
-    __syncthreads();
-    // numerators of C^ (LevelCtx::C32): row i's entry of column Q = l + W t at i D + l R + t
-    constexpr int W = G::D < 32 ? G::D : 32, CR = G::D / W;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < G::D * G::D / 2; i += blockDim.x) {
-        const uint4 c = __ldg(reinterpret_cast<const uint4 *>(lv.C32) + i);
-#pragma unroll
-        for (int j = 0; j < 2; j++) {
-            const int row = (2 * i + j) / G::D, at = (2 * i + j) % G::D, Q = at / CR + W * (at % CR);
-            const int ca = (int)(j ? c.z : c.x), cb = (int)(j ? c.w : c.y);
-            c8[row * G::D + Q] = make_char2((signed char)ca, (signed char)cb);
-            if (row) atomicAdd(&sums[Q], ca + cb); // row 0 is not part of the product
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < G::MT * 2 * G::KS * 32; i += blockDim.x) {
-        const int lane = i & 31, g = lane >> 2, q = lane & 3, s = (i >> 5) % G::KS, part = (i >> 5) / G::KS & 1,
-                  mt = (i >> 5) / (2 * G::KS);
-        uint32_t v[4];
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            // register r: column g (+ 8 for odd r) of the tile, k 2q (+ 8 for r >= 2) and one more
-            const int m = g + 8 * (r & 1);
-            const uint32_t Q = quad_row(NQ, (uint32_t)(m & 7) >> 1, (uint32_t)(4 * mt + (m & 1) + 2 * (m >> 3)));
-            int e[2];
-#pragma unroll
-            for (int b = 0; b < 2; b++) {
-                const uint32_t row = quad_row(NQ, (uint32_t)q, (uint32_t)(4 * s + 2 * (r >> 1) + b));
-                const char2 c = c8[row * G::D + Q];
-                // row 0's places: the bias and the offsets' correction
-                e[b] = row == 0 ? (part ? -sums[Q] : 12288) : part ? (int)c.y : (int)c.x;
-            }
-            v[r] = half2_bits(e[0], e[1]);
-        }
-        frag[i] = make_uint4(v[0], v[1], v[2], v[3]);
     }
     __syncthreads();
     return Sm<NQ>{frag,
@@ -314,6 +268,7 @@ __device__ __forceinline__ uint64_t step(uint64_t seq, int side, uint32_t chunk,
     const uint32_t one = g == 2 * q ? 0x00003C00u : g == 2 * q + 1 ? 0x3C000000u : 0u;
     const uint4 ident = make_uint4(one, 0, 0, one);
     // the weights as pairs of 16-bit words; V's a parts are its fingerprints
+    const uint32_t bias = q == 0 ? 0x6400u : 0u; // row 0's slot of the first k-step
     const uint32_t mw = side ? 0x00FF00FFu : 0u, mv = ~mw & 0x00FF00FFu; // low bytes, or none
     const uint32_t sw = side ? 0x7351u : 0x7454u, sv = side ? 0x7454u : 0x7351u; // high bytes, or none
     uint32_t pa[G::R / 2], pb[G::R / 2];
@@ -331,8 +286,8 @@ __device__ __forceinline__ uint64_t step(uint64_t seq, int side, uint32_t chunk,
     for (int s = 0; s < 2 * G::KS; s++) {
         const uint32_t w0 = s < G::KS ? pa[2 * s] : pb[2 * (s - G::KS)];
         const uint32_t w1 = s < G::KS ? pa[2 * s + 1] : pb[2 * (s - G::KS) + 1];
-        const uint32_t l0 = (w0 & mw) | 0x64006400u, l1 = (w1 & mw) | 0x64006400u;
-        const uint32_t u0 = __byte_perm(w0, 0x64006400u, sw), u1 = __byte_perm(w1, 0x64006400u, sw);
+        const uint32_t l0 = s == 0 ? (w0 & mw) | bias : w0 & mw, l1 = w1 & mw;
+        const uint32_t u0 = __byte_perm(w0, s == 0 ? bias : 0u, sw), u1 = __byte_perm(w1, 0, sw);
 #pragma unroll
         for (int mt = 0; mt < G::MT; mt++) {
             const uint4 a = sm.frag[(mt * 2 * G::KS + s) * 32 + lane];
@@ -343,8 +298,8 @@ __device__ __forceinline__ uint64_t step(uint64_t seq, int side, uint32_t chunk,
 #pragma unroll
     for (int mt = 0; mt < G::MT; mt++) {
         const uint32_t w0 = pa[2 * mt], w1 = pa[2 * mt + 1];
-        mma16816(d[mt][0], ident, (w0 & mv) | 0x64006400u, (w1 & mv) | 0x64006400u);
-        mma16816(d[mt][1], ident, __byte_perm(w0, 0x64006400u, sv), __byte_perm(w1, 0x64006400u, sv));
+        mma16816(d[mt][0], ident, w0 & mv, w1 & mv);
+        mma16816(d[mt][1], ident, __byte_perm(w0, 0, sv), __byte_perm(w1, 0, sv));
     }
     uint64_t s0 = 0, s1 = 0;
 #pragma unroll

@@ -30,6 +30,7 @@
 // trails (Sec. 3, Fig. 2), the batched forms of both, the exhaustive level
 // pass (Eq. mitm), and the owner binning and insertion of distinguished
 // points for a level sharded across ranks.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -935,14 +936,44 @@ unsigned grid_for(size_t units)
     return (unsigned)g;
 }
 
+// One entry of LevelCtx::Cm a thread, once per problem: 2 D^2 threads.
+template <int NQ>
+__global__ void k_operand(const uint2 *__restrict__ C32, uint16_t *__restrict__ Cm)
+{
+    constexpr uint32_t D = 1u << (2 * NQ), W = D < 32 ? D : 32, R = D / W;
+    const uint32_t i = blockIdx.x * 256 + threadIdx.x;
+    uint32_t at, part, row, Q;
+    if constexpr (NQ == 4) {
+        Q = i & (D - 1);
+        part = i >> 16;
+        const uint32_t k = (i >> 8) & 255u;
+        row = row_of(4, k >> 3, k & 7u);
+        at = cm_index(Q, part * D + k);
+    } else {
+        // fragments of m16n8k16's A, [tile][part][k-step][lane][register][half]:
+        // register r holds column lane / 4 (+ 8 for odd r) of the tile, k
+        // 2 (lane % 4) (+ 8 for r >= 2) and one more
+        constexpr uint32_t T = D / 16;
+        const uint32_t half = i & 1u, r = (i >> 1) & 3u, lane = (i >> 3) & 31u, ks = (i >> 8) % T, mt = (i >> 8) / (2 * T);
+        const uint32_t m = (lane >> 2) + 8 * (r & 1u);
+        part = ((i >> 8) / T) & 1u;
+        Q = quad_row(NQ, (m & 7u) >> 1, 4 * mt + (m & 1u) + 2 * (m >> 3));
+        row = quad_row(NQ, lane & 3u, 4 * ks + 2 * (r >> 1) + half);
+        at = i;
+    }
+    const uint2 c = C32[row * D + (Q % W) * R + Q / W];
+    Cm[at] = row == 0 ? (part ? (uint16_t)0 : kCmBias) : __half_as_ushort(__int2half_rn((int)(part ? c.y : c.x)));
+}
+
 template <int NQ>
 cudaError_t walk_step_n(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
                         size_t count, cudaStream_t s)
 {
-    // quads, but for short n = 3 lists, whose one step does not make up for
-    // the larger set-up (us a launch: 4096 states 9.3 against 8.2, 16384 12.0
-    // / 14.2, 50021 19 / 28; n = 2: 64 5.2 / 6.3, 50021 8 / 17)
-    if ((NQ == 2 || (NQ == 3 && count >= 8192)) && lv.q8)
+    // quads, but for short n = 3 lists with C^ in int8, whose one step does
+    // not make up for the larger set-up (us a launch: 4096 states 7.6 against
+    // 7.3, 16384 10.3 / 14.2, 50021 17.5 / 28; n = 3 with C^ in 32-bit words:
+    // 64 7.9 / 9.0, 50021 18 / 44; n = 2: 64 5.2 / 6.3, 50021 8 / 17)
+    if ((NQ == 2 || (NQ == 3 && (count >= 8192 || !lv.Cq))) && lv.Cm)
         return launch_walk_step_q(lv, chunk, in, out, is_dp, count, s);
     if (NQ == 4 && lv.Cm) return launch_walk_step_e4(lv, chunk, in, out, is_dp, count, s);
     cudaFuncSetAttribute(k_walk_step<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<NQ>::smem_bytes);
@@ -964,7 +995,7 @@ cudaError_t walks_n(const WalkLaunch &w, cudaStream_t s)
 {
     switch (w.shape) {
     case 0:
-        if ((NQ == 2 || (NQ == 3 && (uint32_t)w.n_walks >= kQuadWalks3)) && w.lv.q8) return launch_walks_q(w, s);
+        if ((NQ == 2 || (NQ == 3 && (uint32_t)w.n_walks >= (w.lv.Cq ? kQuadWalks3 : kQuadWalksWide3))) && w.lv.Cm) return launch_walks_q(w, s);
         return walks_ns<NQ, 0>(w, s);
     case 1: if constexpr (shape_count(NQ) > 1) return walks_ns<NQ, 1>(w, s); break;
     case 2: if constexpr (shape_count(NQ) > 2) return walks_ns<NQ, 2>(w, s); break;
@@ -1036,7 +1067,7 @@ cudaError_t rewalk_pairs_n(const WalkLaunch &w, cudaStream_t s)
     // against 47 us; 130: 54 / 66; 17320: 115 / 193; 116090: 311 / 869 us at
     // theta 1/2, 431 at 2^-8: 1.25 / 1.42 ms)
     if (NQ == 4 && w.lv.Cm) return launch_rewalk_e4(w, s);
-    if ((NQ == 2 || NQ == 3) && w.lv.q8) return launch_rewalk_q(w, s);
+    if ((NQ == 2 || NQ == 3) && w.lv.Cm) return launch_rewalk_q(w, s);
     cudaFuncSetAttribute(k_rewalk_pairs<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)Geo<NQ>::smem_bytes);
     k_rewalk_pairs<NQ><<<grid_for<NQ>(w.qcap), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(w);
@@ -1145,6 +1176,16 @@ cudaError_t launch_walk_step(const LevelCtx &lv, int chunk, const uint64_t *in, 
 cudaError_t launch_init_walks(const WalkLaunch &w, cudaStream_t s)
 {
     if (w.n_walks > 0) k_init_walks<<<(w.n_walks + 255) / 256, 256, 0, s>>>(w);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_operand(int n, const uint2 *C32, uint16_t *Cm, cudaStream_t s)
+{
+    const unsigned blocks = (2u << (4 * n)) / 256;
+    if (n == 2) k_operand<2><<<blocks, 256, 0, s>>>(C32, Cm);
+    else if (n == 3) k_operand<3><<<blocks, 256, 0, s>>>(C32, Cm);
+    else if (n == 4) k_operand<4><<<blocks, 256, 0, s>>>(C32, Cm);
+    else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 

@@ -1,8 +1,8 @@
 """The quad kernels (qcs_quad.cu: n = 2, 3, eight walks to a warp) against the
 32-bit-word kernels (c_layout 1), bit for bit: every level from 0 to 15 (no, one
 and more rotations per side, one word of stage codes and two), counts around a
-warp's eight walks and the least that n = 3 takes there, dense and sparse targets, and one whose C^ they
-do not take."""
+warp's eight walks and the least that n = 3 takes there, dense and sparse targets, and ones whose C^ is
+beyond int8 and beyond what the quads take."""
 import numpy as np
 import pytest
 
@@ -27,7 +27,8 @@ def problem(n, t, layout, k_max=15, **over):
     return Q.Problem.from_circuit(n, gates, k_max, Q.default_params(n, c_layout=layout, **over))
 
 
-@pytest.mark.parametrize("n,t", [(2, 0), (2, 3), (2, 7), (2, 13), (3, 0), (3, 5), (3, 12), (3, 19)])
+@pytest.mark.parametrize("n,t", [(2, 0), (2, 3), (2, 7), (2, 13), (2, 19), (3, 0), (3, 5), (3, 12), (3, 19),
+                                 (3, 24)])
 def test_walk_step_at_every_level(dev, n, t):
     bits = {2: 40, 3: 63}[n]
     with problem(n, t, 0, state_bits=bits) as a, problem(n, t, 1, state_bits=bits) as b:
@@ -47,7 +48,7 @@ def test_walk_step_at_every_level(dev, n, t):
 @pytest.mark.parametrize("n,t,k,walks,steps,dpb", [
     (2, 3, 3, 4096, 40, 6), (2, 3, 2, 1, 9, 2), (2, 5, 5, 8, 9, 2), (2, 7, 11, 9, 9, 2), (2, 5, 4, 40000, 5, 1),
     (3, 5, 5, 7001, 20, 3), (3, 5, 2, 6145, 9, 2), (3, 7, 3, 6144, 9, 2), (3, 9, 13, 6151, 9, 2), (3, 7, 6, 40000, 3, 1),
-    (3, 19, 5, 6300, 5, 2), (3, 5, 5, 6143, 5, 2),
+    (3, 19, 5, 2049, 5, 2), (3, 24, 5, 6300, 5, 2), (3, 5, 5, 6143, 5, 2), (2, 17, 5, 900, 9, 2),
 ])
 def test_level_walk(dev, n, t, k, walks, steps, dpb):
     got = []
@@ -138,7 +139,7 @@ def prob_seed(n):
 # one small job (its n = 3 walks stay with the warp-per-walk kernels) up to more jobs
 # than CTAs, walk counts of one task and of many, one job whose C^ the quads
 # do not take, two qubit counts together
-@pytest.mark.parametrize("walks,jobs", [(16, [(3, 7)]), (1024, [(3, 7), (3, 6), (3, 9), (3, 19)] * 2 + [(3, 8)]),
+@pytest.mark.parametrize("walks,jobs", [(16, [(3, 7)]), (1024, [(3, 7), (3, 6), (3, 9), (3, 24)] * 2 + [(3, 8)]),
                                         (48, [(2, 9)] * 3), (512, [(3, 7), (2, 9)] * 13), (64, [(3, 8)] * 170)])
 def test_batched_jobs_walk_the_same(walks, jobs):
     """Walk counters of every job and round against the 32-bit-word kernels."""
