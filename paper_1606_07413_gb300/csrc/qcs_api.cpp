@@ -712,18 +712,22 @@ int qcs::cert_begin(qcs_problem *P, int k, cudaStream_t s, CertPass *c)
         (uint64_t)P->n | ((uint64_t)k << 8) | (0xFFFFull << 16) | ((uint64_t)(uint32_t)c->lv_store.K << 32);
     a.base = smix_host(smix_host(kSeedH ^ 0xCE27u) ^ tag);
     c->slice = CertPass::kSliceMin;
-    cudaError_t e = cudaMalloc(&a.table, sizeof(CertSlot) * slots);
-    if (e == cudaSuccess) e = cudaMalloc(&a.pairs, sizeof(uint64_t) * 2 * CertPass::kCap);
-    if (e == cudaSuccess) e = cudaMalloc(&a.n_pairs, 2 * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMallocHost(&c->hN, 2 * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.n_pairs, 0, 2 * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMallocHost(&c->hPairs, sizeof(uint64_t) * 2 * CertPass::kCap);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.table, 0xFF, sizeof(CertSlot) * slots, s);
+    // one allocation: the key table, the matches, their number
+    const size_t table_bytes = sizeof(CertSlot) * slots, pair_bytes = sizeof(uint64_t) * 2 * CertPass::kCap;
+    cudaError_t e = cudaMalloc(&a.table, table_bytes + pair_bytes + 2 * sizeof(uint32_t));
+    if (e == cudaSuccess) {
+        a.pairs = reinterpret_cast<uint64_t *>(reinterpret_cast<char *>(a.table) + table_bytes);
+        a.n_pairs = reinterpret_cast<uint32_t *>(a.pairs + 2 * CertPass::kCap);
+        e = cudaMemsetAsync(a.n_pairs, 0, 2 * sizeof(uint32_t), s);
+    }
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.table, 0xFF, table_bytes, s);
+    c->hPairs = static_cast<uint64_t *>(malloc(pair_bytes));
+    if (e == cudaSuccess && !c->hPairs) e = cudaErrorMemoryAllocation;
     if (e != cudaSuccess) {
         cert_end(P, c, s);
         return e == cudaErrorMemoryAllocation ? QCS_ERR_NOMEM : cuda_fail(e);
     }
-    c->table_bytes = sizeof(CertSlot) * slots;
+    c->table_bytes = table_bytes;
     return QCS_OK;
 }
 
@@ -742,7 +746,7 @@ int qcs::cert_advance(qcs_problem *P, CertPass *c, cudaStream_t s, uint64_t budg
             // contraction with C^ when the extra rotation went on V)
             const uint64_t cost = c->v_heavy ? kStoreCost : 1;
             uint64_t n = std::min<uint64_t>(c->xi_h - c->stored, CertPass::kSliceMax);
-            n = std::max<uint64_t>(1, std::min<uint64_t>(n, (budget - *used + cost - 1) / cost));
+            n = std::max<uint64_t>(1, std::min<uint64_t>(n, (budget - *used - 1) / cost + 1));
             a.lv = c->lv_store;
             a.side = c->v_heavy ? 1 : 0;
             a.insert = 1;
@@ -761,7 +765,7 @@ int qcs::cert_advance(qcs_problem *P, CertPass *c, cudaStream_t s, uint64_t budg
         // matches of each slice are checked exactly on the host
         const uint64_t cost = c->v_heavy ? 1 : kStoreCost;
         uint64_t n = std::min(c->slice, c->n_probe - c->probed);
-        n = std::max<uint64_t>(1, std::min<uint64_t>(n, (budget - *used + cost - 1) / cost));
+        n = std::max<uint64_t>(1, std::min<uint64_t>(n, (budget - *used - 1) / cost + 1));
         a.lv = c->lv_probe;
         a.side = c->v_heavy ? 0 : 1;
         a.insert = 0;
@@ -777,8 +781,8 @@ int qcs::cert_advance(qcs_problem *P, CertPass *c, cudaStream_t s, uint64_t budg
         c->probed += n;
         *used += n * cost;
         if (n == c->slice) c->slice = std::min(2 * c->slice, CertPass::kSliceMax);
-        const uint32_t m = std::min(*c->hN, CertPass::kCap);
-        if (*c->hN > CertPass::kCap) c->overflow = true;
+        const uint32_t m = std::min(c->hN[0], CertPass::kCap);
+        if (c->hN[0] > CertPass::kCap) c->overflow = true;
         if (m > 0) {
             // read back only the matches the slice queued
             if ((e = cudaMemcpyAsync(c->hPairs, a.pairs, sizeof(uint64_t) * 2 * m, cudaMemcpyDeviceToHost, s)) !=
@@ -826,14 +830,10 @@ int qcs::cert_end(qcs_problem *P, CertPass *c, cudaStream_t s)
 {
     cudaStreamSynchronize(s);
     cudaFree(c->a.table);
-    cudaFree(c->a.pairs);
-    cudaFree(c->a.n_pairs);
-    cudaFreeHost(c->hN);
-    cudaFreeHost(c->hPairs);
     c->a.table = nullptr;
     c->a.pairs = nullptr;
     c->a.n_pairs = nullptr;
-    c->hN = nullptr;
+    free(c->hPairs);
     c->hPairs = nullptr;
     {
         std::lock_guard<std::mutex> g(P->mu);

@@ -285,7 +285,9 @@ struct CertPass {
     int64_t d2h = 0;
     LevelCtx lv_store{}, lv_probe{};
     CertArgs a{};
-    uint32_t *hN = nullptr;
+    // matches are few and seldom: read into pageable memory (pinning and
+    // unpinning 1 MB for each pass took longer than a small level's kernels)
+    uint32_t hN[2] = {0, 0};
     uint64_t *hPairs = nullptr;
 };
 int cert_begin(::qcs_problem *P, int k, cudaStream_t s, CertPass *c);
