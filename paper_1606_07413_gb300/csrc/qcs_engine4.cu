@@ -743,31 +743,41 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_batch_e4(BatchArgs a)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ WalkLaunch sw;
     constexpr uint32_t per = e4::kSets * e4::kSet; // slots
-    const uint32_t nt = *a.n_tasks;
-    const uint32_t t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
-    uint32_t task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
-    if (task >= t_end) return;
-    const e4::Cta c = e4::cta_open(smem_raw);
-    bool ok = true, again = false;
-    while (task < t_end && ok) {
-        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
-        uint32_t last = task + 1;
-        while (last < t_end && a.tasks[2 * last] == job) last++;
+    e4::Cta c;
+    bool again = false;
+    auto run = [&](uint32_t job, uint32_t first, uint32_t most) {
+        if (!again) c = e4::cta_open(smem_raw);
         if (threadIdx.x == 0) sw = a.jobs[job];
         __syncthreads();
-        const uint32_t end = min((uint32_t)sw.n_walks, first + (last - task) * e4::kTaskWalks);
+        const uint32_t end = min((uint32_t)sw.n_walks, first + most);
         // the slots' shares as even as they can be
         const uint32_t cnt = end > first ? end - first : 0, rounds = (cnt + per - 1) / per;
         const uint32_t slots = rounds ? (cnt + rounds - 1) / rounds : 0;
-        ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
+        const bool ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
             return walk_control(sw, first, slots, slots, end, c, X, lane);
         });
         if (!ok && threadIdx.x == 0) atomicAdd(sw.stall, 1u);
         __syncthreads(); // before sw changes
         again = true;
+        return ok;
+    };
+    JobShare s;
+    const uint32_t nt = *a.n_tasks;
+    uint32_t task = 0, t_end = 0;
+    if (own_job(a, 8, 1, job_walks, s)) {
+        if (s.job != ~0u) run(s.job, s.p0, s.p1 - s.p0);
+    } else {
+        t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
+        task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
+    }
+    while (task < t_end) {
+        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
+        uint32_t last = task + 1;
+        while (last < t_end && a.tasks[2 * last] == job) last++;
+        if (!run(job, first, (last - task) * e4::kTaskWalks)) break;
         task = last;
     }
-    e4::cta_close(c);
+    if (again) e4::cta_close(c);
 }
 
 // The re-walk of a level's merges (Sec. 3, Fig. 2; the same steps and classes

@@ -576,20 +576,29 @@ __global__ void __launch_bounds__(qd::kBatchThreads, 1) k_walks_batch_q(BatchArg
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ WalkLaunch sw;
     const uint32_t nt = *a.n_tasks, warps = blockDim.x >> 5;
-    const uint32_t t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
-    uint32_t task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
-    while (task < t_end) {
-        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
-        uint32_t last = task + 1;
-        while (last < t_end && a.tasks[2 * last] == job) last++;
+    auto run = [&](uint32_t job, uint32_t first, uint32_t most) {
         __syncthreads(); // every warp is done with the previous job
         if (threadIdx.x == 0) sw = a.jobs[job];
         __syncthreads();
         const qd::Level<NQ> L(sw.lv);
         const qd::Sm<NQ> sm = qd::set_up<NQ>(sw.lv, L.scale, smem_raw);
-        const uint32_t end = min((uint32_t)sw.n_walks, first + (last - task) * qd::kTaskWalks);
+        const uint32_t end = min((uint32_t)sw.n_walks, first + most);
         for (uint32_t base = first + 8 * (threadIdx.x >> 5); base < end; base += 8 * warps)
             walk_eight<NQ>(sw, base, end, L, sm, threadIdx.x & 31);
+    };
+    JobShare s;
+    uint32_t task = 0, t_end = 0;
+    if (own_job(a, 8, 8, job_walks, s)) {
+        if (s.job != ~0u) run(s.job, s.p0, s.p1 - s.p0);
+    } else {
+        t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
+        task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
+    }
+    while (task < t_end) {
+        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
+        uint32_t last = task + 1;
+        while (last < t_end && a.tasks[2 * last] == job) last++;
+        run(job, first, (last - task) * qd::kTaskWalks);
         task = last;
     }
 }
