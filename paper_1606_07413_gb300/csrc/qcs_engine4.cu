@@ -21,7 +21,7 @@
 // cycles, the SM shared with the other sets), the product (1600: 16 cycles a
 // tcgen05.mma with A in tensor memory, 40 in shared memory, whatever N), E
 // (700), control (800).  With 48 points in flight (two sets of 24, or three
-// of 16) that chain was the bound; with 72 it is issue: 75 % active at 588
+// of 16) that chain was the bound; with 72 it is issue: 75 % active at 582
 // warp instructions a point, half of them the 255 column finalisers.
 // 2^20 walks x 16 steps at level 7: 11.1 ms (1.51 G steps/s); two sets and
 // 16 workers 14.9 ms; with mma.sync (12 stage and 8 MMA warps, C^'s fragments
@@ -131,17 +131,32 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t ph)
     return done != 0;
 }
 
+// All lanes of a warp, as a mask whose value the compiler does not know, so
+// that every vote and shuffle under it first brings the warp's lanes together.
+// Under a constant full mask the compiled code did not: in the budgeted re-walk
+// the lanes whose merge was carried in the middle of a round ran on a round
+// behind the others, each group voting for itself, merges were lost and
+// bounded waits ran out.  It costs 1.5 % (2^20 walks x 16 steps 10.95 -> 11.1
+// ms); the workers' and the MMA warp's waits, which no lane reaches alone,
+// keep the constant (with the mask there too 11.9 ms).
+__device__ __forceinline__ uint32_t all_lanes()
+{
+    uint32_t lt, ge;
+    asm volatile("mov.u32 %0, %%lanemask_lt;\n\tmov.u32 %1, %%lanemask_ge;" : "=r"(lt), "=r"(ge));
+    return lt | ge;
+}
+
 // Wait until the phase of parity `ph` has completed; false if the wait ran
 // out.  Warp-uniform: true only once every lane saw the phase complete.
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t ph)
+__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t ph, uint32_t all = 0xFFFFFFFFu)
 {
     const uint32_t a = smem_u32(b);
-    if (__all_sync(0xFFFFFFFFu, mbar_try(a, ph))) return true;
+    if (__all_sync(all, mbar_try(a, ph))) return true;
     const long long t0 = clock64();
     for (;;) {
-        if (__all_sync(0xFFFFFFFFu, mbar_try(a, ph))) return true;
+        if (__all_sync(all, mbar_try(a, ph))) return true;
         // one lane's clock decides for the warp
-        if (__shfl_sync(0xFFFFFFFFu, clock64() - t0, 0) > kWaitCycles) return false;
+        if (__shfl_sync(all, clock64() - t0, 0) > kWaitCycles) return false;
     }
 }
 
@@ -297,6 +312,7 @@ struct Cta {
     uint64_t *bars; // per set: jobs, rows, product, sums
     uint32_t *nw;   // [set] W points, [4 + set] set done
     uint32_t tmem;
+    uint32_t all; // all_lanes, for the control warps
     __device__ Job *jobs(int X) const { return reinterpret_cast<Job *>(raw + off_job) + X * kSet; }
     __device__ HashBase *wb(int X) const { return reinterpret_cast<HashBase *>(raw + off_wb) + X * kPairs; }
     __device__ uint64_t *part(int X) const { return reinterpret_cast<uint64_t *>(raw + off_part) + X * kParts * kPairs; }
@@ -324,6 +340,7 @@ __device__ __forceinline__ Cta cta_open(unsigned char *raw)
     __syncthreads();
     tmem_fence_after();
     c.tmem = *taddr;
+    c.all = all_lanes();
     return c;
 }
 
@@ -571,7 +588,7 @@ __device__ __forceinline__ bool publish(const Cta &c, int X, int lane, bool vali
 {
     const bool isw = valid && side == 1;
     const uint32_t before = (1u << lane) - 1u;
-    const uint32_t all = __ballot_sync(0xFFFFFFFFu, isw), first = __ballot_sync(0xFFFFFFFFu, isw && late);
+    const uint32_t all = __ballot_sync(c.all, isw), first = __ballot_sync(c.all, isw && late);
     const uint32_t pos = (uint32_t)(late ? __popc(first & before) : __popc(first) + __popc(all & ~first & before));
     const bool go = valid && (!isw || pos < (uint32_t)kPairs);
     if (lane < kSet) {
@@ -585,7 +602,7 @@ __device__ __forceinline__ bool publish(const Cta &c, int X, int lane, bool vali
                 make_uint4((uint32_t)hb.PH, (uint32_t)(hb.PH >> 32), hb.pre16, 0);
     }
     if (lane == 0) c.nw[X] = min((uint32_t)__popc(all), (uint32_t)kPairs);
-    __syncwarp();
+    __syncwarp(c.all);
     if (lane == 0) mbar_arrive(c.bar_jobs(X));
     *pos_out = pos;
     return go;
@@ -597,7 +614,7 @@ __device__ __forceinline__ void publish_done(const Cta &c, int X, int lane)
         c.nw[4 + X] = 1;
         mbar_arrive(c.bar_jobs(X));
     }
-    __syncwarp();
+    __syncwarp(c.all);
 }
 
 // the hash of the lane's slot, after the set's sums are complete
@@ -659,7 +676,7 @@ __device__ __forceinline__ bool walk_control(const WL &w, uint32_t first, uint32
     HashBase hb = c.chunk_base()[st.chunk];
     uint64_t cc = sg.chunk_code(st.chunk), dp = 0, ref = 0;
     bool store = false;
-    while (__any_sync(0xFFFFFFFFu, valid)) {
+    while (__any_sync(c.all, valid)) {
         const int side = (int)(st.cur & 1);
         uint32_t pos;
         const bool go = publish(c, X, lane, valid, late, side, sg.seq(side, rotations(st.cur, lv), cc),
@@ -672,8 +689,8 @@ __device__ __forceinline__ bool walk_control(const WL &w, uint32_t first, uint32
         const bool last = st.len + 1 >= w.max_len; // this step ends the trail in any case
         const uint32_t walk = w.walk_base + local; // index among all ranks' walks
         if (go && left == 1 && local + stride < n) nx = w.walks[local + stride];
-        __syncwarp();
-        if (!mbar_wait(c.bar_sums(X), ph)) {
+        __syncwarp(c.all);
+        if (!mbar_wait(c.bar_sums(X), ph, c.all)) {
             ok = false;
             break;
         }
@@ -707,16 +724,16 @@ __device__ __forceinline__ bool walk_control(const WL &w, uint32_t first, uint32
                 cc = sg.chunk_code(st.chunk);
             }
         }
-        __syncwarp();
+        __syncwarp(c.all);
     }
     if (ok && store) dp_insert(w, dp, ref, t);
-    __syncwarp();
+    __syncwarp(c.all);
     if (ok) publish_done(c, X, lane);
     unsigned long long v[7] = {t.steps, t.w, t.dp, t.ab, t.evicted, t.duplicate, t.pairs};
     const int idx[7] = {C_STEPS, C_WSTEPS, C_DPS, C_ABANDONED, C_EVICTED, C_DUPLICATE, C_PAIRS};
     for (int i = 0; i < 7; i++) {
 #pragma unroll
-        for (int o = 16; o; o >>= 1) v[i] += __shfl_xor_sync(0xFFFFFFFFu, v[i], o);
+        for (int o = 16; o; o >>= 1) v[i] += __shfl_xor_sync(c.all, v[i], o);
         if (lane == 0 && v[i]) atomicAdd(&w.counters[idx[i]], v[i]);
     }
     return ok;
@@ -793,7 +810,7 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
                                                const e4::Cta &c, int X, int lane)
 {
     using namespace e4;
-    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const unsigned kAll = c.all;
     const LevelCtx &lv = w.lv;
     const Stages sg(lv);
     const bool mine = lane < kSet && (uint32_t)(lane * kSets + X) < slots;
@@ -835,7 +852,7 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
                     }
                 }
             }
-            __syncwarp();
+            __syncwarp(c.all);
         }
     };
     // whether the merge goes on; if not it is classified or carried
@@ -877,7 +894,7 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
     };
     fetch();
     take();
-    __syncwarp();
+    __syncwarp(c.all);
     while (__any_sync(kAll, active || have)) {
         const uint64_t x = second ? b : a;
         const int side = (int)(x & 1);
@@ -886,7 +903,7 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
                                 side ? sg.ns_w : sg.ns_v, hb, &pos);
         late = active && !go;
         fetch();
-        if (!mbar_wait(c.bar_sums(X), ph)) {
+        if (!mbar_wait(c.bar_sums(X), ph, c.all)) {
             ok = false;
             break;
         }
@@ -921,7 +938,7 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
             }
         }
         take();
-        __syncwarp();
+        __syncwarp(c.all);
     }
     if (ok) publish_done(c, X, lane);
     unsigned long long v[8] = {cls[0], cls[1], cls[2], cls[3], cls[4], cls[5], cls[3], nf};
@@ -997,20 +1014,20 @@ __device__ __forceinline__ bool certify_control(const CertArgs &a, const e4::Cta
     uint64_t key = 0, idx = 0;
     uint32_t ph = 0;
     bool have = false, valid = mine && i < a.count, ok = true;
-    while (__any_sync(0xFFFFFFFFu, valid)) {
+    while (__any_sync(c.all, valid)) {
         const uint64_t q = (dig & hmask) + (0x0101010101010101ull & hmask);
         const uint32_t chunk = has_chunk ? (uint32_t)((dig >> (8 * h)) & 0xFFu) + 1 : 0u;
         uint32_t pos;
         publish(c, X, lane, valid, false, 1, sg.seq(1, q, has_chunk ? sg.chunk_code(chunk) : 0), sg.ns_w, hb, &pos);
         if (a.insert) cert_insert_warp(a, have, key, idx, lane);
         else if (have) cert_probe(a, key, idx);
-        __syncwarp();
+        __syncwarp(c.all);
         have = valid;
         idx = a.first + i;
         i += stride;
         valid = mine && i < a.count;
         dig = add_base_xi(dig, sdig, 255, nd);
-        if (!mbar_wait(c.bar_sums(X), ph)) {
+        if (!mbar_wait(c.bar_sums(X), ph, c.all)) {
             ok = false;
             break;
         }
@@ -1021,7 +1038,7 @@ __device__ __forceinline__ bool certify_control(const CertArgs &a, const e4::Cta
     if (ok) {
         if (a.insert) cert_insert_warp(a, have, key, idx, lane);
         else if (have) cert_probe(a, key, idx);
-        __syncwarp();
+        __syncwarp(c.all);
         publish_done(c, X, lane);
     }
     return ok;
@@ -1056,7 +1073,7 @@ __device__ __forceinline__ bool list_control(const LevelCtx &lv, uint32_t chunk,
     bool valid = lane < kSet && slot < slots && i < count, late = false, have = false, ok = true;
     uint64_t x = valid ? in[i] : 0ull, nx = 0, y = 0;
     uint32_t ph = 0;
-    while (__any_sync(0xFFFFFFFFu, valid)) {
+    while (__any_sync(c.all, valid)) {
         const int side = (int)(x & 1);
         uint32_t pos;
         const bool go = publish(c, X, lane, valid, late, side, sg.seq(side, rotations(x, lv), cc),
@@ -1067,8 +1084,8 @@ __device__ __forceinline__ bool list_control(const LevelCtx &lv, uint32_t chunk,
         }
         if (go && i + stride < count) nx = in[i + stride];
         late = valid && !go;
-        __syncwarp();
-        if (!mbar_wait(c.bar_sums(X), ph)) {
+        __syncwarp(c.all);
+        if (!mbar_wait(c.bar_sums(X), ph, c.all)) {
             ok = false;
             break;
         }
@@ -1087,7 +1104,7 @@ __device__ __forceinline__ bool list_control(const LevelCtx &lv, uint32_t chunk,
         if (is_dp) is_dp[at] = (uint8_t)((y >> lv.dshift) == 0);
     }
     if (lane < kSet) next[slot] = i; // the slot's first state not stored
-    __syncwarp();
+    __syncwarp(c.all);
     if (ok) publish_done(c, X, lane);
     return ok;
 }

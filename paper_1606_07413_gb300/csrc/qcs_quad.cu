@@ -26,7 +26,7 @@
 // the f16 subnormal with those bits, and row 0's first k slot puts 0.75 on
 // every sum.
 //
-// What bounds it: issue.  A step costs about 130 warp instructions at n = 3 and
+// What bounds it: issue.  A step costs 145 warp instructions at n = 3 and about
 // 50 at n = 2 (379 and 325 with one and two walks to a warp, whose bookkeeping
 // ran on all lanes of each).
 #include <cuda_runtime.h>

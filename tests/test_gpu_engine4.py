@@ -91,6 +91,24 @@ def classes(r):
     return np.array([r["robin_hood"], r["trivial"], r["same_side"], r["claws"] + r["false_hash"], r["no_merge"]])
 
 
+# Slots whose merges end at different points of a round (classified, carried
+# for their budget, two chunks' functions): every merge is accounted for.
+@pytest.mark.parametrize("k,dpb,walks,steps,budget", [(5, 2, 1 << 16, 32, 5), (7, 4, 1 << 17, 32, 9), (6, 3, 1 << 17, 32, 7),
+                                                      (4, 1, 1 << 16, 16, 2), (6, 1, 1 << 17, 16, 0)])
+def test_engine_rewalk_loses_no_merge(dev, k, dpb, walks, steps, budget):
+    gates, _ = W.seeded_target(4, 9, 59)
+    p = Q.default_params(4, walks=walks, table_log2=20, rewalk_budget=budget)
+    with Q.Problem.from_circuit(4, gates, 15, p) as prob:
+        assert prob.sde > k
+        prob.level_begin(k, 1, dpb)
+        for _ in range(12):
+            prob.level_walk(steps)
+            prob.level_rewalk()
+            r = prob.level_collect()
+        assert r["merges"] > 10000 and r["queue_overflow"] == 0 and r["false_hash"] == 0
+        assert classes(r).sum() + r["rewalk_carried"] == r["merges"]
+
+
 # lists shorter than the CTAs, around one merge per slot and far longer, with
 # and without chunks, and an evaluation budget; levels below the target's
 # T-count, so no claw ends the host's check of candidates
