@@ -95,7 +95,7 @@ def workload_config(c, k=None, steps=None, rewalk_budget=None):
         "level_points": 2 * (4 ** c["n"] - 1) ** (k // 2) * ((4 ** c["n"] - 1) if k & 1 else 1),
         "steps_per_walk_per_step": steps, "state_bits": c["L"], "dp_bits": c["dtheta"],
         "rewalk_budget_per_step": rewalk_budget or "none (every merge re-walked in its own step)",
-        "table_slots": 1 << c["table_log2"], "coefficients": "exact: int64 on the host, C^ as int8 byte quads on the device; fingerprints mod 2^16",
+        "table_slots": 1 << c["table_log2"], "coefficients": "exact: int64 on the host, C^ as f16 integers on the device; fingerprints mod 2^16",
         "l2": f"flushed between steps ({FLUSH_BYTES >> 20} MiB write)",
         "parallelism": "one GPU (with N > 1: the level sharded over ranks by distinguished-point owner)",
     }
@@ -111,19 +111,19 @@ def workload_config(c, k=None, steps=None, rewalk_budget=None):
 # are reported as null.
 # Each n = 4 record: `ncu --set full` of `bench.py --level-only n4_level7
 # --steps 2 --shape S` (2^20 walks x 16 steps; profiles/k_walks_n4_level7_walks1048576.md
-# and profiles/k_walks_mma4_n4_level7_walks1048576.md).  The launch's DRAM
+# and profiles/k_walks_e4_n4_level7_walks1048576.md).  The launch's DRAM
 # traffic is the walk states and the staged tables, which do not grow with
 # the steps, plus 32 bytes per distinguished point (0.5 MB at the headline's
 # 64 steps), so the figure stands for the headline launch.
 WALK_NCU = {
-    "k_walks<4,3>": {"source_sha256_16": "80027283cc3dbf3c", "dram_bytes_per_launch": 34747136,
-                     "warp_inst_per_step": 1073.2},
-    "k_walks<4,0>": {"source_sha256_16": "80027283cc3dbf3c", "dram_bytes_per_launch": 35021312,
-                     "warp_inst_per_step": 1937.6},
+    "k_walks<4,3>": {"source_sha256_16": "9d7e516ae4b45619", "dram_bytes_per_launch": 34704640,
+                     "warp_inst_per_step": 582.3},
+    "k_walks<4,0>": {"source_sha256_16": "9d7e516ae4b45619", "dram_bytes_per_launch": 34991872,
+                     "warp_inst_per_step": 1935.6},
     # n = 3, level 5: `bench.py --level-only n3_level5 --steps 2`, one launch of 2^16 walks x 512 steps,
     # the launch of the n3_level5 record (profiles/k_walks_n3_level5_walks65536.md)
-    "k_walks<3,0>": {"source_sha256_16": "80027283cc3dbf3c", "dram_bytes_per_launch": 2178304,
-                     "warp_inst_per_step": 379.3},
+    "k_walks<3,0>": {"source_sha256_16": "9d7e516ae4b45619", "dram_bytes_per_launch": 2203392,
+                     "warp_inst_per_step": 145.2},
 }
 
 
@@ -134,7 +134,7 @@ def walk_source_hash() -> str:
     import re
 
     h = hashlib.sha256()
-    for f in ("qcs_walk.cu", "qcs_engine4.cu", "qcs_device.cuh", "qcs_internal.h"):
+    for f in ("qcs_walk.cu", "qcs_engine4.cu", "qcs_quad.cu", "qcs_device.cuh", "qcs_rows.cuh", "qcs_internal.h"):
         with open(os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_1606_07413_gb300", "csrc", f)) as fh:
             text = fh.read()
         if f == "qcs_internal.h":
@@ -209,14 +209,15 @@ def walk_roofline(kernel, n, w_steps, steps, walk_s, launches, dp4a_per_s, clock
         # The tensor-core shape: each 16-bit-weight multiply-add is two f16
         # byte-plane multiply-adds (4 flops) on the tensor cores, against the
         # measured dense f16/bf16 peak; beside it the same work against the
-        # legacy mma.sync rate this kernel issues on, and the issue slots.
+        # legacy mma.sync rate, and the issue slots.
         peak_tf, peak_src = measured_tensor_tflops(sustained=True)
         flops = 4 * achieved
         mma_sync = None
         if hmma_per_s:
             mma_sync = {"achieved_mac_per_s": 2 * achieved, "peak_mac_per_s": hmma_per_s,
                         "frac": 2 * achieved / hmma_per_s,
-                        "peak_source": "measured mma.sync m16n8k16 f16 -> f32 rate (qcs_peak_hmma, this run)"}
+                        "peak_source": "measured mma.sync m16n8k16 f16 -> f32 rate (qcs_peak_hmma, this run; the "
+                                       "kernel issues tcgen05.mma)"}
         return {"bound": "tensor", "unit": "TFLOP/s", "kernel": kernel,
                 "achieved": flops / 1e12, "peak": peak_tf, "frac": flops / 1e12 / peak_tf,
                 "peak_source": peak_src, "mma_sync": mma_sync,
@@ -231,7 +232,8 @@ def walk_roofline(kernel, n, w_steps, steps, walk_s, launches, dp4a_per_s, clock
             "peak_source": "2 x measured dp4a rate (qcs_peak_idp4a, this run: "
                            f"{dp4a_per_s / 1e9:.0f} G dp4a/s)",
             "algorithmic_ops": f"2*d^2 = {2 * d * d} 16-bit-weight multiply-adds per W-side walk step "
-                               "(executed as two byte-plane dp4a per four multiply-adds)"}
+                               + ("(by mma.sync, two f16 byte planes, where 6144 walks or more run)" if n == 3 else
+                                  "(executed as two byte-plane dp4a per four multiply-adds)")}
 
 
 # ------------------------------------------------------------------ ranks
@@ -877,12 +879,9 @@ def run_ours(args):
                 # the table at its busiest: half the points distinguished
                 "n3_level5_theta_half": level_throughput(Q, W, torch, 2, 5, 64, stream, alu_per_s=2 * dp4a_per_s,
                                                          dp_bits=1, table_log2=26),
-                # targets whose reduced C^ leaves int8: the 32-bit word contraction (IMAD; n = 4 reads C^
-                # through L2), against the measured IMAD rate
-                "c32_n3_level5": level_throughput(Q, W, torch, 2, 5, 512, stream, alu_per_s=imad_per_s,
-                                                  target=(3, 19, 4019)),
-                "c32_n4_level7": level_throughput(Q, W, torch, 3, 7, 16, stream, alu_per_s=imad_per_s,
-                                                  target=(4, 15, 4015)),
+                # targets whose reduced C^ leaves int8 (exact in f16 all the same)
+                "c32_n3_level5": level_throughput(Q, W, torch, 2, 5, 512, stream, target=(3, 19, 4019)),
+                "c32_n4_level7": level_throughput(Q, W, torch, 3, 7, 16, stream, target=(4, 15, 4015), shape=3),
             })
 
     if rank == 0:
