@@ -146,6 +146,22 @@ __device__ void dp_insert(const WL &w, uint64_t dp, uint64_t ref, TallyOf<T> &c)
     }
 }
 
+// All lanes of a warp, as a mask whose value the compiler does not know, so
+// that every vote and shuffle under it first brings the warp's lanes together.
+// Warps that run a re-walk or the like on every lane need that: under a
+// constant full mask the compiled code of the n = 4 engine's budgeted re-walk
+// did not, the lanes whose merge was carried in the middle of a round ran on a
+// round behind the others, each group voting for itself, merges were lost and
+// bounded waits ran out.  It costs the engine 1.5 % (2^20 walks x 16 steps
+// 10.95 -> 11.1 ms); its workers' and its MMA warp's waits, which no lane
+// reaches alone, keep the constant (with the mask there too 11.9 ms).
+__device__ __forceinline__ uint32_t all_lanes()
+{
+    uint32_t lt, ge;
+    asm volatile("mov.u32 %0, %%lanemask_lt;\n\tmov.u32 %1, %%lanemask_ge;" : "=r"(lt), "=r"(ge));
+    return lt | ge;
+}
+
 constexpr uint32_t kMaxRewalkLen = 1u << 20; // longer trails are reported as no merge
 
 // A merge of a launch's work list: first the re-walks carried from the

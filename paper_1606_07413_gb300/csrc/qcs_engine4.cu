@@ -131,21 +131,6 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t ph)
     return done != 0;
 }
 
-// All lanes of a warp, as a mask whose value the compiler does not know, so
-// that every vote and shuffle under it first brings the warp's lanes together.
-// Under a constant full mask the compiled code did not: in the budgeted re-walk
-// the lanes whose merge was carried in the middle of a round ran on a round
-// behind the others, each group voting for itself, merges were lost and
-// bounded waits ran out.  It costs 1.5 % (2^20 walks x 16 steps 10.95 -> 11.1
-// ms); the workers' and the MMA warp's waits, which no lane reaches alone,
-// keep the constant (with the mask there too 11.9 ms).
-__device__ __forceinline__ uint32_t all_lanes()
-{
-    uint32_t lt, ge;
-    asm volatile("mov.u32 %0, %%lanemask_lt;\n\tmov.u32 %1, %%lanemask_ge;" : "=r"(lt), "=r"(ge));
-    return lt | ge;
-}
-
 // Wait until the phase of parity `ph` has completed; false if the wait ran
 // out.  Warp-uniform: true only once every lane saw the phase complete.
 __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t ph, uint32_t all = 0xFFFFFFFFu)

@@ -424,7 +424,7 @@ template <int NQ, typename WL>
 __device__ __forceinline__ void rewalk_eight(const WL &w, uint32_t *cursor, uint32_t cnt, const qd::Level<NQ> &L,
                                              const qd::Sm<NQ> &sm, int lane)
 {
-    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const unsigned kAll = all_lanes(); // 2 % of an n = 3 search
     const LevelCtx &lv = w.lv;
     const bool head = (lane & 3) == 0;
     uint32_t cls[6] = {0, 0, 0, 0, 0, 0}, nf = 0, used = 0;
@@ -484,7 +484,7 @@ __device__ __forceinline__ void rewalk_eight(const WL &w, uint32_t *cursor, uint
                     cs = trail_chunk<NQ>(lv, s);
                 }
             }
-            __syncwarp();
+            __syncwarp(kAll);
             const uint64_t o = __shfl_xor_sync(kAll, s, 1);
             const uint32_t lo = __shfl_xor_sync(kAll, ls, 1), co = __shfl_xor_sync(kAll, cs, 1);
             if (got) {
@@ -505,7 +505,7 @@ __device__ __forceinline__ void rewalk_eight(const WL &w, uint32_t *cursor, uint
                     settle();
                 }
             }
-            __syncwarp();
+            __syncwarp(kAll);
         }
         if (!__any_sync(kAll, active)) break;
         const uint64_t x = second ? b : a;
@@ -539,7 +539,7 @@ __device__ __forceinline__ void rewalk_eight(const WL &w, uint32_t *cursor, uint
                 }
             }
         }
-        __syncwarp();
+        __syncwarp(kAll);
         if (nf >= 0x40000000u) { // tallies are in 32 bits
             if (head) atomicAdd(&w.counters[C_RSTEPS], (unsigned long long)nf);
             nf = 0;
