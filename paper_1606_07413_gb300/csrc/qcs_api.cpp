@@ -624,7 +624,9 @@ LevelPlan qcs::plan_level_n(int D, int k, const qcs_params &p)
     long double steps = (long double)p.steps_per_launch, walks = (long double)p.walks;
     const long double s_min = std::min<long double>(steps, 4.0L / theta);
     if (walks * steps > version_steps) steps = std::max(s_min, std::floor(version_steps / walks));
-    if (walks * steps > version_steps) walks = std::max(32.0L, std::floor(version_steps / steps));
+    // at least a warp's worth of walks, but never more than there is memory for
+    const long double few = std::min(32.0L, walks);
+    if (walks * steps > version_steps) walks = std::max(few, std::floor(version_steps / steps));
     // expected merges per launch (distinguished points that meet a stored
     // one, about the stored fraction of all distinguished points) fit half
     // the queue
@@ -636,7 +638,7 @@ LevelPlan qcs::plan_level_n(int D, int k, const qcs_params &p)
         const long double keep = std::max(1.0L, std::min(steps, s_min));
         walks = std::min(walks, std::max(std::min(walks, 8192.0L), std::floor(qroom / (keep * per_step))));
         steps = std::max(1.0L, std::min(steps, std::floor(qroom / (walks * per_step))));
-        if (walks * steps * per_step > qroom) walks = std::max(32.0L, std::floor(qroom / (steps * per_step)));
+        if (walks * steps * per_step > qroom) walks = std::max(few, std::floor(qroom / (steps * per_step)));
     }
     pl.walks = (uint32_t)walks;
     pl.steps = (uint32_t)std::max(1.0L, steps);

@@ -258,7 +258,8 @@ int begin_level(qcs_batch *B, Job &j, int slot)
     w = WalkLaunch{};
     w.lv = make_level(P, j.k, j.version, j.pl.dp_bits);
     w.walks = j.walks;
-    w.n_walks = (int32_t)j.pl.walks;
+    // the walk buffer and the task lists hold jp.walks walks
+    w.n_walks = (int32_t)std::min<uint32_t>(j.pl.walks, (uint32_t)j.jp.walks);
     w.steps = j.pl.steps;
     w.max_len = (uint32_t)std::min<uint64_t>((uint64_t)j.jp.max_trail_factor << j.pl.dp_bits, kMaxTrailLen);
     w.table = j.table;
