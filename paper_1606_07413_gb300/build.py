@@ -34,7 +34,7 @@ def nvcc() -> str:
 def _inputs():
     files = [os.path.join(CSRC, s) for s in SOURCES]
     files += [os.path.join(CSRC, "qcs_internal.h"), os.path.join(CSRC, "qcs_device.cuh"),
-              os.path.join(CSRC, "qcs_rows.cuh"), os.path.join(INCLUDE, "qcs.h"), __file__,
+              os.path.join(CSRC, "qcs_rows.cuh"), os.path.join(CSRC, "qcs_shares.h"), os.path.join(INCLUDE, "qcs.h"), __file__,
               os.path.join(CSRC, PEAK_SRC), os.path.join(INCLUDE, "qcs_peak.h")]
     return files
 

@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #include "qcs_internal.h"
+#include "qcs_shares.h"
 
 namespace qcs {
 namespace {
@@ -254,108 +255,6 @@ __device__ __forceinline__ uint64_t add_base_xi(uint64_t d, uint64_t s, uint32_t
         }
     }
     return r;
-}
-
-// A batched re-walk's shares: the CTAs take equal parts of all jobs' work, a
-// merge of a job counting about its evaluations of f: three trail lengths, or
-// the budget.  (By merges alone the CTAs that met the jobs of small theta, 64
-// evaluations to a merge, took three times as long as the others.)
-template <typename WL>
-__device__ __forceinline__ uint64_t merge_weight(const WL &w)
-{
-    const int d = __popcll(w.lv.maskL) - w.lv.dshift; // theta = 2^-d
-    const uint64_t len = 3ull << min(d, 20);
-    return w.rewalk_budget && w.rewalk_budget < len ? (uint64_t)w.rewalk_budget : len;
-}
-
-// Few jobs: every CTA works for one of them alone.  A job gets one CTA and of
-// the others a part in proportion to its weight, and its CTAs share its items
-// evenly, in units of `unit`.  A CTA that takes up two jobs runs them one after
-// the other, each as long as its longest chain (a re-walk: up to 64 dependent
-// evaluations) with its slots partly empty.  With fewer CTAs to a job the
-// one CTA more or less that a job gets would cost as much.  (13 n = 4 and 11
-// n = 3 jobs, ms a round: walks 1.42 -> 1.33 and 0.46 -> 0.31, re-walks 0.74 ->
-// 0.51 and 0.43 -> 0.36.)  job is ~0 if there is no item for this CTA; false:
-// more than a job to ctas_per_job CTAs.  items(w, count, weight) tells a job's
-// items.
-struct JobShare {
-    uint32_t job, p0, p1;
-};
-template <class Items>
-__device__ __forceinline__ bool own_job(const BatchArgs &a, uint32_t ctas_per_job, uint32_t unit, Items items,
-                                        JobShare &s)
-{
-    const uint32_t nj = *a.n_jobs;
-    uint64_t total = 0;
-    uint32_t n = 0;
-    for (uint32_t j = 0; j < nj; j++) {
-        uint64_t cnt, wt;
-        items(a.jobs[a.job_ids[j]], cnt, wt);
-        total += cnt * wt;
-        n += cnt != 0;
-    }
-    s.job = ~0u;
-    if (n * ctas_per_job > gridDim.x) return false;
-    const uint64_t spare = gridDim.x - n;
-    uint64_t base = 0;
-    uint32_t i = 0;
-    for (uint32_t j = 0; j < nj; j++) {
-        uint64_t cnt, wt;
-        items(a.jobs[a.job_ids[j]], cnt, wt);
-        if (cnt == 0) continue;
-        const uint32_t c0 = i + (uint32_t)(base * spare / total);
-        base += cnt * wt;
-        const uint32_t c1 = ++i + (uint32_t)(base * spare / total);
-        if (blockIdx.x < c0 || blockIdx.x >= c1) continue;
-        const uint64_t units = (cnt + unit - 1) / unit, r = blockIdx.x - c0, c = c1 - c0;
-        s.p0 = (uint32_t)(units * r / c) * unit;
-        s.p1 = (uint32_t)min(cnt, units * (r + 1) / c * unit);
-        if (s.p0 < s.p1) s.job = a.job_ids[j];
-    }
-    return true;
-}
-
-// own_job's items of a batched walk: the walks, of as many steps each
-__device__ __forceinline__ void job_walks(const WalkLaunch &w, uint64_t &cnt, uint64_t &wt)
-{
-    cnt = (uint64_t)w.n_walks;
-    wt = w.steps;
-}
-
-// Walk a CTA's share: body(job index, its first merge, the end of its merges)
-// for every job that the share meets, in order, until body returns false.
-template <class Body>
-__device__ __forceinline__ void merge_shares(const BatchArgs &a, Body body)
-{
-    JobShare s;
-    if (own_job(a, 4, 1,
-                [](const WalkLaunch &w, uint64_t &cnt, uint64_t &wt) {
-                    cnt = w.pend_in_n + min(*w.qhead, w.qcap);
-                    wt = merge_weight(w);
-                },
-                s)) {
-        if (s.job != ~0u) body(s.job, s.p0, s.p1);
-        return;
-    }
-    const uint32_t nj = *a.n_jobs;
-    uint64_t total = 0;
-    for (uint32_t j = 0; j < nj; j++) {
-        const WalkLaunch &w = a.jobs[a.job_ids[j]];
-        total += (uint64_t)(w.pend_in_n + min(*w.qhead, w.qcap)) * merge_weight(w);
-    }
-    const uint64_t lo = total / gridDim.x * blockIdx.x + total % gridDim.x * blockIdx.x / gridDim.x;
-    const uint64_t hi = total / gridDim.x * (blockIdx.x + 1) + total % gridDim.x * (blockIdx.x + 1) / gridDim.x;
-    uint64_t base = 0;
-    for (uint32_t j = 0; j < nj && base < hi; j++) {
-        const uint32_t job = a.job_ids[j];
-        const WalkLaunch &w = a.jobs[job];
-        const uint64_t cnt = w.pend_in_n + min(*w.qhead, w.qcap), wt = merge_weight(w), at = base;
-        base += cnt * wt;
-        if (base <= lo) continue;
-        // a merge belongs to the share its first unit lies in
-        const uint64_t p0 = lo > at ? (lo - at + wt - 1) / wt : 0, p1 = hi < base ? (hi - at + wt - 1) / wt : cnt;
-        if (p0 < p1 && !body(job, (uint32_t)p0, (uint32_t)p1)) return;
-    }
 }
 
 // Exhaustive pass: the key table.  A key's slots are s, s + d, s + 2d, .. with

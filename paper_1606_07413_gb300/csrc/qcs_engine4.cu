@@ -642,6 +642,12 @@ __device__ __forceinline__ bool cta_run(const LevelCtx &lv, const Cta &c, bool a
 
 } // namespace e4
 
+// of a batch: the job's round is not complete (the host reads the counter)
+__device__ __forceinline__ void count_stall(const BatchArgs &a, uint32_t job)
+{
+    if (threadIdx.x == 0) atomicAdd(a.jobs[job].stall, 1u);
+}
+
 // The level walk: the CTA's slot i (lane * kSets + X) < slots steps walk
 // first + i and every stride-th after it below n, one after the other.
 template <typename WL>
@@ -737,9 +743,8 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_e4(WalkLaunch w, uint
     e4::cta_close(c);
 }
 
-// Many jobs in one launch: the CTA takes a contiguous range of tasks (job,
-// first walk of kTaskWalks); neighbouring tasks of one job are one run of
-// the engine, so C^ is reloaded only where the job changes.
+// Many jobs in one launch (walk_shares): the CTA runs the engine once for each
+// job that its share meets, so C^ is reloaded only where the job changes.
 __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_batch_e4(BatchArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -747,38 +752,24 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_walks_batch_e4(BatchArgs a)
     constexpr uint32_t per = e4::kSets * e4::kSet; // slots
     e4::Cta c;
     bool again = false;
-    auto run = [&](uint32_t job, uint32_t first, uint32_t most) {
-        if (!again) c = e4::cta_open(smem_raw);
-        if (threadIdx.x == 0) sw = a.jobs[job];
-        __syncthreads();
-        const uint32_t end = min((uint32_t)sw.n_walks, first + most);
-        // the slots' shares as even as they can be
-        const uint32_t cnt = end > first ? end - first : 0, rounds = (cnt + per - 1) / per;
-        const uint32_t slots = rounds ? (cnt + rounds - 1) / rounds : 0;
-        const bool ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
-            return walk_control(sw, first, slots, slots, end, c, X, lane);
-        });
-        if (!ok && threadIdx.x == 0) atomicAdd(sw.stall, 1u);
-        __syncthreads(); // before sw changes
-        again = true;
-        return ok;
-    };
-    JobShare s;
-    const uint32_t nt = *a.n_tasks;
-    uint32_t task = 0, t_end = 0;
-    if (own_job(a, 8, 1, job_walks, s)) {
-        if (s.job != ~0u) run(s.job, s.p0, s.p1 - s.p0);
-    } else {
-        t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
-        task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
-    }
-    while (task < t_end) {
-        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
-        uint32_t last = task + 1;
-        while (last < t_end && a.tasks[2 * last] == job) last++;
-        if (!run(job, first, (last - task) * e4::kTaskWalks)) break;
-        task = last;
-    }
+    walk_shares(
+        a, blockIdx.x, gridDim.x, 1, e4::kTaskWalks,
+        [&](uint32_t job, uint32_t first, uint32_t most) {
+            if (!again) c = e4::cta_open(smem_raw);
+            if (threadIdx.x == 0) sw = a.jobs[job];
+            __syncthreads();
+            const uint32_t end = min((uint32_t)sw.n_walks, first + most);
+            // the slots' shares as even as they can be
+            const uint32_t cnt = end > first ? end - first : 0, rounds = (cnt + per - 1) / per;
+            const uint32_t slots = rounds ? (cnt + rounds - 1) / rounds : 0;
+            const bool ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
+                return walk_control(sw, first, slots, slots, end, c, X, lane);
+            });
+            __syncthreads(); // before sw changes
+            again = true;
+            return ok;
+        },
+        [&](uint32_t job) { count_stall(a, job); });
     if (again) e4::cta_close(c);
 }
 
@@ -950,8 +941,8 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_e4(WalkLaunch w)
     e4::cta_close(c);
 }
 
-// The batched re-walk: each CTA takes its share of all jobs' merges (see
-// merge_shares) and reloads C^ where the share enters another job.
+// The batched re-walk: each CTA takes its share of all jobs' merges
+// (merge_shares) and reloads C^ where the share enters another job.
 __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_batch_e4(BatchArgs a)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -959,21 +950,23 @@ __global__ void __launch_bounds__(e4::kThreads, 1) k_rewalk_batch_e4(BatchArgs a
     __shared__ uint32_t cursor;
     e4::Cta c;
     bool again = false;
-    merge_shares(a, [&](uint32_t job, uint32_t p0, uint32_t p1) {
-        if (!again) c = e4::cta_open(smem_raw);
-        if (threadIdx.x == 0) {
-            sw = a.jobs[job];
-            cursor = p0;
-        }
-        __syncthreads();
-        const bool ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
-            return rewalk_control(sw, &cursor, p1, p1 - p0, c, X, lane);
-        });
-        if (!ok && threadIdx.x == 0) atomicAdd(sw.stall, 1u);
-        __syncthreads(); // before sw and cursor change
-        again = true;
-        return ok;
-    });
+    merge_shares(
+        a, blockIdx.x, gridDim.x,
+        [&](uint32_t job, uint32_t p0, uint32_t p1) {
+            if (!again) c = e4::cta_open(smem_raw);
+            if (threadIdx.x == 0) {
+                sw = a.jobs[job];
+                cursor = p0;
+            }
+            __syncthreads();
+            const bool ok = e4::cta_run(sw.lv, c, again, [&](int X, int lane) {
+                return rewalk_control(sw, &cursor, p1, p1 - p0, c, X, lane);
+            });
+            __syncthreads(); // before sw and cursor change
+            again = true;
+            return ok;
+        },
+        [&](uint32_t job) { count_stall(a, job); });
     if (again) e4::cta_close(c);
 }
 

@@ -567,40 +567,29 @@ __global__ void __launch_bounds__(qd::Geo<NQ>::kThreads, 1) k_rewalk_q(WalkLaunc
     rewalk_eight<NQ>(w, w.rw_next, cnt, L, sm, threadIdx.x & 31);
 }
 
-// Many jobs in one launch (see k_walks_batch in qcs_walk.cu): contiguous tasks
-// of one job are walked together, eight walks to a warp, and the tables are
-// set up again where the job changes.
+// Many jobs in one launch (walk_shares): a job's walks of the CTA's share are
+// walked together, eight to a warp, and the tables are set up again where the
+// job changes.  No wait of these kernels can run out.
 template <int NQ>
 __global__ void __launch_bounds__(qd::kBatchThreads, 1) k_walks_batch_q(BatchArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ WalkLaunch sw;
-    const uint32_t nt = *a.n_tasks, warps = blockDim.x >> 5;
-    auto run = [&](uint32_t job, uint32_t first, uint32_t most) {
-        __syncthreads(); // every warp is done with the previous job
-        if (threadIdx.x == 0) sw = a.jobs[job];
-        __syncthreads();
-        const qd::Level<NQ> L(sw.lv);
-        const qd::Sm<NQ> sm = qd::set_up<NQ>(sw.lv, L.scale, smem_raw);
-        const uint32_t end = min((uint32_t)sw.n_walks, first + most);
-        for (uint32_t base = first + 8 * (threadIdx.x >> 5); base < end; base += 8 * warps)
-            walk_eight<NQ>(sw, base, end, L, sm, threadIdx.x & 31);
-    };
-    JobShare s;
-    uint32_t task = 0, t_end = 0;
-    if (own_job(a, 8, 8, job_walks, s)) {
-        if (s.job != ~0u) run(s.job, s.p0, s.p1 - s.p0);
-    } else {
-        t_end = (uint32_t)(((uint64_t)nt * (blockIdx.x + 1)) / gridDim.x);
-        task = (uint32_t)(((uint64_t)nt * blockIdx.x) / gridDim.x);
-    }
-    while (task < t_end) {
-        const uint32_t job = a.tasks[2 * task], first = a.tasks[2 * task + 1];
-        uint32_t last = task + 1;
-        while (last < t_end && a.tasks[2 * last] == job) last++;
-        run(job, first, (last - task) * qd::kTaskWalks);
-        task = last;
-    }
+    const uint32_t warps = blockDim.x >> 5;
+    walk_shares(
+        a, blockIdx.x, gridDim.x, 8, qd::kTaskWalks,
+        [&](uint32_t job, uint32_t first, uint32_t most) {
+            __syncthreads(); // every warp is done with the previous job
+            if (threadIdx.x == 0) sw = a.jobs[job];
+            __syncthreads();
+            const qd::Level<NQ> L(sw.lv);
+            const qd::Sm<NQ> sm = qd::set_up<NQ>(sw.lv, L.scale, smem_raw);
+            const uint32_t end = min((uint32_t)sw.n_walks, first + most);
+            for (uint32_t base = first + 8 * (threadIdx.x >> 5); base < end; base += 8 * warps)
+                walk_eight<NQ>(sw, base, end, L, sm, threadIdx.x & 31);
+            return true;
+        },
+        [](uint32_t) {});
 }
 
 template <int NQ>
@@ -609,18 +598,21 @@ __global__ void __launch_bounds__(qd::kBatchThreads, 1) k_rewalk_batch_q(BatchAr
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ WalkLaunch sw;
     __shared__ uint32_t cursor;
-    merge_shares(a, [&](uint32_t job, uint32_t p0, uint32_t p1) {
-        __syncthreads(); // every warp is done with the previous job
-        if (threadIdx.x == 0) {
-            sw = a.jobs[job];
-            cursor = p0;
-        }
-        __syncthreads();
-        const qd::Level<NQ> L(sw.lv);
-        const qd::Sm<NQ> sm = qd::set_up<NQ>(sw.lv, L.scale, smem_raw);
-        rewalk_eight<NQ>(sw, &cursor, p1, L, sm, threadIdx.x & 31);
-        return true;
-    });
+    merge_shares(
+        a, blockIdx.x, gridDim.x,
+        [&](uint32_t job, uint32_t p0, uint32_t p1) {
+            __syncthreads(); // every warp is done with the previous job
+            if (threadIdx.x == 0) {
+                sw = a.jobs[job];
+                cursor = p0;
+            }
+            __syncthreads();
+            const qd::Level<NQ> L(sw.lv);
+            const qd::Sm<NQ> sm = qd::set_up<NQ>(sw.lv, L.scale, smem_raw);
+            rewalk_eight<NQ>(sw, &cursor, p1, L, sm, threadIdx.x & 31);
+            return true;
+        },
+        [](uint32_t) {});
 }
 
 // Grid and warps of a CTA for `groups` warp-loads: warp w of CTA b takes loads
