@@ -871,7 +871,9 @@ __device__ __forceinline__ bool rewalk_control(const WL &w, uint32_t *cursor, ui
     fetch();
     take();
     __syncwarp(c.all);
-    while (__any_sync(kAll, active || have)) {
+    // `more` alone: every merge that was taken was carried at once (a budget of
+    // one evaluation and aligned trails), and the list goes on
+    while (__any_sync(kAll, active || have || more)) {
         const uint64_t x = second ? b : a;
         const int side = (int)(x & 1);
         uint32_t pos;
