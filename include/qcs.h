@@ -63,7 +63,8 @@ extern "C" {
 #define QCS_ERR_OVERFLOW (-6)    /* exact arithmetic would overflow int64 */
 #define QCS_ERR_BUSY (-7)        /* a search is already running on this problem */
 #define QCS_ERR_TIMEOUT (-8)     /* qcs_wait ran out of time */
-#define QCS_ERR_DEVICE (-9)      /* a device-side bounded wait gave up */
+#define QCS_ERR_DEVICE (-9)      /* a device-side bounded wait gave up, or an exhaustive pass's key table
+                                    does not hold every stored point */
 
 /* search status reported by qcs_poll_collisions */
 #define QCS_IDLE 0

@@ -714,13 +714,13 @@ int qcs::cert_begin(qcs_problem *P, int k, cudaStream_t s, CertPass *c)
         (uint64_t)P->n | ((uint64_t)k << 8) | (0xFFFFull << 16) | ((uint64_t)(uint32_t)c->lv_store.K << 32);
     a.base = smix_host(smix_host(kSeedH ^ 0xCE27u) ^ tag);
     c->slice = CertPass::kSliceMin;
-    // one allocation: the key table, the matches, their number
+    // one allocation: the key table, the matches, their number and the other counts (CertArgs::n_pairs)
     const size_t table_bytes = sizeof(CertSlot) * slots, pair_bytes = sizeof(uint64_t) * 2 * CertPass::kCap;
-    cudaError_t e = cudaMalloc(&a.table, table_bytes + pair_bytes + 2 * sizeof(uint32_t));
+    cudaError_t e = cudaMalloc(&a.table, table_bytes + pair_bytes + sizeof c->hN);
     if (e == cudaSuccess) {
         a.pairs = reinterpret_cast<uint64_t *>(reinterpret_cast<char *>(a.table) + table_bytes);
         a.n_pairs = reinterpret_cast<uint32_t *>(a.pairs + 2 * CertPass::kCap);
-        e = cudaMemsetAsync(a.n_pairs, 0, 2 * sizeof(uint32_t), s);
+        e = cudaMemsetAsync(a.n_pairs, 0, sizeof c->hN, s);
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(a.table, 0xFF, table_bytes, s);
     c->hPairs = static_cast<uint64_t *>(malloc(pair_bytes));
@@ -775,11 +775,12 @@ int qcs::cert_advance(qcs_problem *P, CertPass *c, cudaStream_t s, uint64_t budg
         a.count = n;
         if ((e = cudaMemsetAsync(a.n_pairs, 0, sizeof(uint32_t), s)) != cudaSuccess) break;
         if ((e = launch_certify(a, s)) != cudaSuccess) break;
-        if ((e = cudaMemcpyAsync(c->hN, a.n_pairs, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
-            break;
+        if ((e = cudaMemcpyAsync(c->hN, a.n_pairs, sizeof c->hN, cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) break;
-        c->d2h += (int64_t)(2 * sizeof(uint32_t));
+        c->d2h += (int64_t)sizeof c->hN;
         if (c->hN[1]) return QCS_ERR_DEVICE; // a bounded wait ran out (in this launch or in the stored side's)
+        // the whole stored side is in the table: a key short, and a level could pass for empty
+        if (((uint64_t)c->hN[3] << 32 | c->hN[2]) != c->xi_h) return QCS_ERR_DEVICE;
         c->probed += n;
         *used += n * cost;
         if (n == c->slice) c->slice = std::min(2 * c->slice, CertPass::kSliceMax);
@@ -1372,7 +1373,7 @@ const char *qcs_strerror(int code)
     case QCS_ERR_OVERFLOW: return "exact arithmetic overflow";
     case QCS_ERR_BUSY: return "a search is already running";
     case QCS_ERR_TIMEOUT: return "timed out";
-    case QCS_ERR_DEVICE: return "a device-side bounded wait gave up";
+    case QCS_ERR_DEVICE: return "a device-side bounded wait gave up or a key was lost";
     default: return "unknown status";
     }
 }

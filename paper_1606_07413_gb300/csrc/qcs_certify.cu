@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(cv::kThreads, 1) k_certify_v(CertArgs a)
     const uint64_t units = blocks * G::UNITS, warps = (uint64_t)gridDim.x * cv::kWarps;
     const uint64_t me = (uint64_t)blockIdx.x * cv::kWarps + (uint64_t)warp;
     const uint64_t end = units * (me + 1) / warps;
+    uint32_t stored = 0;
     for (uint64_t u = units * me / warps; u < end; u++) {
         const uint64_t block = b0 + u / G::UNITS;
         const uint32_t part = (uint32_t)(u % G::UNITS);
@@ -194,10 +195,13 @@ __global__ void __launch_bounds__(cv::kThreads, 1) k_certify_v(CertArgs a)
         const bool valid = q != 0 && idx >= a.first && idx - a.first < a.count;
         uint64_t key = smix(acc);
         if (key == ~0ull) key = ~0ull - 1; // ~0 marks an empty slot
-        if (a.insert) cert_insert_warp(a, valid, key, idx, lane);
+        const uint32_t all = all_lanes(); // not kept: a register less in the loops
+        if (a.insert) cert_insert_warp(a, all, valid, key, idx, lane, stored);
         else if (valid) cert_probe(a, key, idx);
-        __syncwarp();
+        __syncwarp(all);
     }
+    stored = __reduce_add_sync(all_lanes(), stored);
+    if (lane == 0) cert_count(a, stored);
 }
 
 template <int NQ>

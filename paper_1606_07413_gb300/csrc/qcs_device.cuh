@@ -283,37 +283,50 @@ __device__ __forceinline__ bool cert_put(const CertArgs &a, uint64_t slot, uint6
     return true;
 }
 
-__device__ __forceinline__ void cert_insert(const CertArgs &a, uint64_t key, uint64_t idx)
+// whether the key was stored (it is unless the table is full)
+__device__ __forceinline__ bool cert_insert(const CertArgs &a, uint64_t key, uint64_t idx)
 {
     CertProbe p(key, a.mask);
     for (uint64_t probe = 0; probe <= a.mask; probe++, p.s = (p.s + p.d) & a.mask)
-        if (cert_put(a, p.s, key, idx)) return;
+        if (cert_put(a, p.s, key, idx)) return true;
+    return false;
+}
+
+// keys stored by this launch, for the host's check that none was lost
+__device__ __forceinline__ void cert_count(const CertArgs &a, uint32_t stored)
+{
+    if (stored) atomicAdd(reinterpret_cast<unsigned long long *>(a.n_pairs + 2), (unsigned long long)stored);
 }
 
 // The same for a whole warp, a point to a valid lane: after a few tries the
 // warp looks for each remaining lane's empty slot together, 32 slots at a
 // time (the 640th copy of a key alone: as many dependent exchanges; 16.6 M
-// points at n = 4: 35 ms lane by lane, 7 ms so).
-__device__ __forceinline__ void cert_insert_warp(const CertArgs &a, bool valid, uint64_t key, uint64_t idx, int lane)
+// points at n = 4: 35 ms lane by lane, 7 ms so).  all: all_lanes(), which
+// brings the lanes back together after their tries; a vote that some of them
+// missed would lose their keys.  stored counts the lane's keys.
+__device__ __forceinline__ void cert_insert_warp(const CertArgs &a, uint32_t all, bool valid, uint64_t key,
+                                                 uint64_t idx, int lane, uint32_t &stored)
 {
     CertProbe p(key, a.mask);
     bool left = valid;
     for (int probe = 0; probe < 6 && left; probe++, p.s = (p.s + p.d) & a.mask) left = !cert_put(a, p.s, key, idx);
-    __syncwarp();
+    stored += valid && !left;
+    __syncwarp(all);
     uint32_t todo;
-    while ((todo = __ballot_sync(0xFFFFFFFFu, left)) != 0) {
+    while ((todo = __ballot_sync(all, left)) != 0) {
         const int src = __ffs((int)todo) - 1;
-        const uint64_t d = __shfl_sync(0xFFFFFFFFu, p.d, src);
-        uint64_t at = __shfl_sync(0xFFFFFFFFu, p.s, src);
+        const uint64_t d = __shfl_sync(all, p.d, src);
+        uint64_t at = __shfl_sync(all, p.s, src);
         for (uint64_t probe = 0; probe <= a.mask; probe += 32) {
             const uint64_t k =
                 *reinterpret_cast<volatile const uint64_t *>(&a.table[(at + d * (uint64_t)lane) & a.mask].key);
-            uint32_t empty = __ballot_sync(0xFFFFFFFFu, k == ~0ull);
+            uint32_t empty = __ballot_sync(all, k == ~0ull);
             bool done = false;
             while (empty && !done) { // another warp may take the slot first
                 const uint64_t slot = (at + d * (uint64_t)(__ffs((int)empty) - 1)) & a.mask;
                 if (lane == src) done = cert_put(a, slot, key, idx);
-                done = __shfl_sync(0xFFFFFFFFu, done, src);
+                stored += done;
+                done = __shfl_sync(all, done, src);
                 empty &= empty - 1;
             }
             if (done) break;

@@ -992,14 +992,14 @@ __device__ __forceinline__ bool certify_control(const CertArgs &a, const e4::Cta
     uint64_t dig = mine && i < a.count ? base_xi_digits(a.first + i, 255, nd) : 0;
     const HashBase hb = hash_base(a.base);
     uint64_t key = 0, idx = 0;
-    uint32_t ph = 0;
+    uint32_t ph = 0, stored = 0;
     bool have = false, valid = mine && i < a.count, ok = true;
     while (__any_sync(c.all, valid)) {
         const uint64_t q = (dig & hmask) + (0x0101010101010101ull & hmask);
         const uint32_t chunk = has_chunk ? (uint32_t)((dig >> (8 * h)) & 0xFFu) + 1 : 0u;
         uint32_t pos;
         publish(c, X, lane, valid, false, 1, sg.seq(1, q, has_chunk ? sg.chunk_code(chunk) : 0), sg.ns_w, hb, &pos);
-        if (a.insert) cert_insert_warp(a, have, key, idx, lane);
+        if (a.insert) cert_insert_warp(a, c.all, have, key, idx, lane, stored);
         else if (have) cert_probe(a, key, idx);
         __syncwarp(c.all);
         have = valid;
@@ -1016,11 +1016,13 @@ __device__ __forceinline__ bool certify_control(const CertArgs &a, const e4::Cta
         if (key == ~0ull) key = ~0ull - 1; // ~0 marks an empty slot
     }
     if (ok) {
-        if (a.insert) cert_insert_warp(a, have, key, idx, lane);
+        if (a.insert) cert_insert_warp(a, c.all, have, key, idx, lane, stored);
         else if (have) cert_probe(a, key, idx);
         __syncwarp(c.all);
         publish_done(c, X, lane);
     }
+    stored = __reduce_add_sync(c.all, stored);
+    if (lane == 0) cert_count(a, stored);
     return ok;
 }
 

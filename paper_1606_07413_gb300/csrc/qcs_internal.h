@@ -258,7 +258,8 @@ struct CertArgs {
     uint64_t mask;     // table slots - 1 (a power of two, at least twice the stored points)
     uint64_t *pairs;   // key matches (stored index, probing index)
     uint32_t *n_pairs; // [0] matches found (may exceed cap; only cap are stored); [1] the engine's bounded
-                       // waits that ran out (the points are then not all evaluated)
+                       // waits that ran out (the points are then not all evaluated); [2, 3] as one word,
+                       // keys stored
     uint32_t cap;
 };
 cudaError_t launch_certify(const CertArgs &a, cudaStream_t s);
@@ -287,7 +288,7 @@ struct CertPass {
     CertArgs a{};
     // matches are few and seldom: read into pageable memory (pinning and
     // unpinning 1 MB for each pass took longer than a small level's kernels)
-    uint32_t hN[2] = {0, 0};
+    uint32_t hN[4] = {0, 0, 0, 0};
     uint64_t *hPairs = nullptr;
 };
 int cert_begin(::qcs_problem *P, int k, cudaStream_t s, CertPass *c);

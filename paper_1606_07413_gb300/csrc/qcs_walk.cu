@@ -891,6 +891,7 @@ __global__ void __launch_bounds__(Geo<NQ>::THREADS) k_certify(CertArgs a)
     // While i + stride < count, the stride is below xi^nd and its nd digits
     // are exact; otherwise the loop ends before the sum is used.
     uint64_t dig = 0, sdig = 0;
+    uint32_t stored = 0;
     if (i < a.count) {
         dig = base_xi_digits(a.first + i, xi, nd);
         sdig = base_xi_digits(stride, xi, nd);
@@ -902,11 +903,12 @@ __global__ void __launch_bounds__(Geo<NQ>::THREADS) k_certify(CertArgs a)
         uint64_t key = coset_hash<NQ>(side, qpack, chunk, a.base, a.lv, sm, g);
         if (key == ~0ull) key = ~0ull - 1; // ~0 marks an empty slot
         if (g.sub == 0) {
-            if (a.insert) cert_insert(a, key, idx);
+            if (a.insert) stored += cert_insert(a, key, idx);
             else cert_probe(a, key, idx);
         }
         __syncwarp(g.mask);
     }
+    cert_count(a, stored);
 }
 
 int g_num_sms = 0;
