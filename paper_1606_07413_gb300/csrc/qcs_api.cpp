@@ -455,6 +455,7 @@ int level_begin(qcs_problem *P, int k, uint32_t version, int dp_bits, uint32_t n
     int rc = ensure_search_buffers(P);
     if (rc) return rc;
     auto &L = P->lvl;
+    if (L.k != k || L.dp_bits != dp_bits) L.rw_last = 0; // a new version's lists are about as long as the last one's
     L.k = k;
     L.h = k / 2;
     L.dp_bits = dp_bits;
@@ -516,6 +517,7 @@ int level_rewalk(qcs_problem *P, cudaStream_t s)
         CK(cudaMemsetAsync(P->dQhead + 2, 0, sizeof(uint32_t), s));
     }
     w.rw_next = P->dQhead + 3;
+    w.rw_last = L.rw_last;
     CK(cudaMemsetAsync(P->dQhead + 3, 0, sizeof(uint32_t), s));
     CK(launch_rewalk_pairs(w, s));
     CK(cudaMemcpyAsync(P->hCounters, P->dCounters, sizeof(unsigned long long) * C_NCOUNTERS,
@@ -536,6 +538,7 @@ int level_collect(qcs_problem *P, cudaStream_t s, bool *got, uint64_t *steps)
     if (c[C_STALLED]) return QCS_ERR_DEVICE; // a bounded wait of the walk kernel ran out: nothing here is valid
     const uint32_t npairs = std::min(P->hQhead[0], L.w.qcap);
     const uint32_t ncand = std::min(P->hQhead[1], kCandCap);
+    P->lvl.rw_last = npairs + P->lvl.pend_n;
     int64_t d2h = (int64_t)(sizeof(unsigned long long) * C_NCOUNTERS + 3 * sizeof(uint32_t));
     int64_t carried_lost = 0;
     if (P->p.rewalk_budget > 0) {

@@ -219,6 +219,7 @@ struct WalkLaunch {
     // single-target re-walk: merges are claimed from this device counter
     // (zeroed before the launch); null: a fixed stride (the batched re-walk)
     uint32_t *rw_next;
+    uint32_t rw_last; // merges of the level's last re-walk (0: unknown), for the choice of this one's kernels
     // the tensor-core walk (n = 4, launch shape 3) counts here the warps
     // whose bounded wait ran out (the launch's results are then invalid);
     // it refuses to launch without it
@@ -326,7 +327,8 @@ int engine4_warps(); // warps of its CTA
 int engine4_walks_per_task();
 // n = 2, 3 with lv.Cm set: eight walks to a warp (qcs_quad.cu)
 cudaError_t launch_walks_q(const WalkLaunch &w, cudaStream_t s);
-cudaError_t launch_rewalk_q(const WalkLaunch &w, cudaStream_t s);
+// (least: the kernel leaves shorter merge lists alone; their length is known on the device only)
+cudaError_t launch_rewalk_q(const WalkLaunch &w, uint32_t least, cudaStream_t s);
 // jobs of a batch: tasks of quad_walks_per_task() walks, and the jobs' re-walks
 cudaError_t launch_walks_batch_q(int n, const BatchArgs &a, cudaStream_t s);
 cudaError_t launch_rewalk_batch_q(int n, const BatchArgs &a, cudaStream_t s);
@@ -339,6 +341,16 @@ int quad_walks_per_task();
 // those kernels take 32-bit words: 1000 walks 126 / 152 and 175 / 152, 3000
 // 127 / 228 and 182 / 240.
 constexpr uint32_t kQuadWalks3 = 6144, kQuadWalksWide3 = 2048;
+// An n = 3 re-walk of fewer merges than this is left to the lane-group kernel:
+// a merge is a chain of evaluations of f, a quad's evaluation takes two to
+// three times as long as a lane group's, and only enough merges make up for it
+// (us, quads / lane groups: theta 1/2, 1600 merges 71 / 36, 29400 70 / 69,
+// 47000 98 / 113, 312000 314 / 551; theta 2^-4, 5600 376 / 143, 50300 427 /
+// 390, 103000 697 / 775; theta 2^-8, 3980 672 / 228, 40600 1038 / 1215; C^ in
+// 32-bit words, theta 2^-4, 9500 303 / 219, 22800 379 / 343, 48500 426 / 551).
+// At n = 2 a quad loses little (2360 merges 41 / 32, 29600 43 / 55) and the
+// choice, a second launch, costs 4 us: quads always.
+constexpr uint32_t kQuadMerges3 = 40960, kQuadMergesWide3 = 20480;
 cudaError_t launch_walk_step_q(const LevelCtx &lv, int chunk, const uint64_t *in, uint64_t *out, uint8_t *is_dp,
                                size_t count, cudaStream_t s);
 // DP-owner sharding: insert `count` distinguished points {dp, trail ref}
@@ -459,5 +471,6 @@ struct qcs_problem {
         qcs::WalkLaunch w{};
         int pp = 0;          // dPend[pp] holds the re-walks carried into the next launch
         uint32_t pend_n = 0; // how many
+        uint32_t rw_last = 0; // merges of the last collected re-walk
     } lvl;
 };

@@ -557,10 +557,11 @@ __device__ __forceinline__ void rewalk_eight(const WL &w, uint32_t *cursor, uint
 }
 
 template <int NQ>
-__global__ void __launch_bounds__(qd::Geo<NQ>::kThreads, 1) k_rewalk_q(WalkLaunch w)
+__global__ void __launch_bounds__(qd::Geo<NQ>::kThreads, 1) k_rewalk_q(WalkLaunch w, uint32_t least)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t cnt = w.pend_in_n + min(*w.qhead, w.qcap);
+    if (cnt < least) return; // k_rewalk_pairs takes them
     if (cnt <= 8 * blockIdx.x) return; // no merges for this CTA
     const qd::Level<NQ> L(w.lv);
     const qd::Sm<NQ> sm = qd::set_up<NQ>(w.lv, L.scale, smem_raw);
@@ -660,12 +661,12 @@ cudaError_t walk_step_q(const LevelCtx &lv, int chunk, const uint64_t *in, uint6
 }
 
 template <int NQ>
-cudaError_t rewalk_q(const WalkLaunch &w, cudaStream_t s)
+cudaError_t rewalk_q(const WalkLaunch &w, uint32_t least, cudaStream_t s)
 {
     using G = qd::Geo<NQ>;
     const cudaError_t e = allow_smem<NQ>(k_rewalk_q<NQ>);
     if (e != cudaSuccess) return e;
-    k_rewalk_q<NQ><<<(unsigned)num_sms(), G::kThreads, G::smem_bytes(G::kWarps), s>>>(w);
+    k_rewalk_q<NQ><<<(unsigned)num_sms(), G::kThreads, G::smem_bytes(G::kWarps), s>>>(w, least);
     return cudaGetLastError();
 }
 
@@ -681,10 +682,10 @@ cudaError_t batch_q(const BatchArgs &a, bool rewalk, cudaStream_t s)
 
 } // namespace
 
-cudaError_t launch_rewalk_q(const WalkLaunch &w, cudaStream_t s)
+cudaError_t launch_rewalk_q(const WalkLaunch &w, uint32_t least, cudaStream_t s)
 {
     if (!w.rw_next) return cudaErrorInvalidValue;
-    return w.lv.n == 3 ? rewalk_q<3>(w, s) : w.lv.n == 2 ? rewalk_q<2>(w, s) : cudaErrorInvalidValue;
+    return w.lv.n == 3 ? rewalk_q<3>(w, least, s) : w.lv.n == 2 ? rewalk_q<2>(w, least, s) : cudaErrorInvalidValue;
 }
 
 cudaError_t launch_walks_batch_q(int n, const BatchArgs &a, cudaStream_t s)

@@ -803,11 +803,13 @@ __device__ __forceinline__ void rewalk_job(const WL &w, const Smem<NQ> &sm, uint
     }
 }
 
+// below: lists of this length and longer are left to the quads (k_rewalk_q)
 template <int NQ>
-__global__ void __launch_bounds__(Geo<NQ>::THREADS) k_rewalk_pairs(WalkLaunch w)
+__global__ void __launch_bounds__(Geo<NQ>::THREADS) k_rewalk_pairs(WalkLaunch w, uint32_t below)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint32_t cnt = w.pend_in_n + min(*w.qhead, w.qcap);
+    if (cnt >= below) return;
     if (cnt <= blockIdx.x * Geo<NQ>::WALKS) return; // no pair for this CTA (uniform)
     const Smem<NQ> sm = stage<NQ>(w.lv, smem_raw);
     rewalk_job<NQ>(w, sm, blockIdx.x * Geo<NQ>::WALKS + group_in_cta<NQ>(), cnt, gridDim.x * Geo<NQ>::WALKS,
@@ -1069,10 +1071,24 @@ cudaError_t rewalk_pairs_n(const WalkLaunch &w, cudaStream_t s)
     // against 47 us; 130: 54 / 66; 17320: 115 / 193; 116090: 311 / 869 us at
     // theta 1/2, 431 at 2^-8: 1.25 / 1.42 ms)
     if (NQ == 4 && w.lv.Cm) return launch_rewalk_e4(w, s);
-    if ((NQ == 2 || NQ == 3) && w.lv.Cm) return launch_rewalk_q(w, s);
+    if (NQ == 2 && w.lv.Cm) return launch_rewalk_q(w, 0, s);
+    uint32_t below = ~0u;
+    if (NQ == 3 && w.lv.Cm) {
+        // by the list's length, which only the device knows: both kernels, and
+        // the one whose turn it is not ends at once (4 us).  Where the level's
+        // last list was far from the line one of them is enough: a wrong guess
+        // costs time, no merge.
+        const uint32_t line = w.lv.Cq ? kQuadMerges3 : kQuadMergesWide3;
+        if (w.rw_last >= 2 * line) return launch_rewalk_q(w, 0, s);
+        if ((uint64_t)w.pend_in_n + w.qcap >= line && (w.rw_last == 0 || w.rw_last >= line / 4)) {
+            const cudaError_t e = launch_rewalk_q(w, line, s);
+            if (e != cudaSuccess) return e;
+            below = line;
+        }
+    }
     cudaFuncSetAttribute(k_rewalk_pairs<NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)Geo<NQ>::smem_bytes);
-    k_rewalk_pairs<NQ><<<grid_for<NQ>(w.qcap), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(w);
+    k_rewalk_pairs<NQ><<<grid_for<NQ>(w.qcap), Geo<NQ>::THREADS, Geo<NQ>::smem_bytes, s>>>(w, below);
     return cudaGetLastError();
 }
 

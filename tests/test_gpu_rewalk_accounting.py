@@ -38,3 +38,69 @@ def test_a_budget_of_one_evaluation_loses_no_merge(n, t, k, dpb, walks):
             assert r["queue_overflow"] == 0 and r["false_hash"] == 0
             assert classified(r) + r["rewalk_carried"] == r["merges"], launch
         assert r["merges"] > 100 and r["rewalk_carried"] > 0
+
+
+def smix(z):
+    z = (z ^ (z >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+    z = (z ^ (z >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+    return z ^ (z >> np.uint64(31))
+
+
+def trails(refs, seed, version, L, n_chunks):
+    """Start, chunk and length of the trails that the references name."""
+    u = np.uint64
+    walk, seq, length = refs & u((1 << 24) - 1), (refs >> u(24)) & u((1 << 23) - 1), refs >> u(47)
+    start = smix(u(seed) ^ smix((walk << u(32)) | seq) ^ (u(version) << u(40))) & u((1 << L) - 1)
+    chunk = u(1) + smix(start ^ u(0x5851F42D4C957F2D)) % u(n_chunks) if n_chunks else np.zeros(len(refs), u)
+    return start, chunk, length
+
+
+# n = 3 lists as long as the queue, one merge shorter than the quads take, as
+# long and longer (40960, and 20480 where C^ is not int8); lists far shorter
+# than the queue; a short list after a long one and the other way round; with
+# an evaluation budget, whose carried merges count
+@pytest.mark.parametrize("t,queue,walks,dpb,budget,steps", [
+    (8, 40959, 60000, 1, 0, (12,)), (8, 40960, 60000, 1, 0, (12,)), (8, 60001, 65536, 1, 0, (12,)),
+    (8, 50000, 3000, 3, 0, (12,)), (8, 1 << 19, 65536, 1, 0, (12, 1, 1)), (8, 1 << 19, 20000, 2, 0, (1, 1, 30)),
+    (8, 1 << 17, 50000, 2, 8, (12, 1, 1, 1)), (19, 20479, 40000, 1, 0, (12,)), (19, 20480, 40000, 1, 0, (12,)),
+    (19, 1 << 16, 5000, 2, 0, (12,))])
+def test_list_lengths_around_the_quads(t, queue, walks, dpb, budget, steps):
+    """Every merge of a list, classified by the level's re-walk and, from its
+    two trails' recomputed starts, by qcs_rewalk (one lane group per pair)."""
+    k, version, L = 5, 2, 48
+    gates, _ = W.seeded_target(3, t, 9)
+    p = Q.default_params(3, walks=walks, table_log2=17, rewalk_budget=budget, queue_capacity=queue)
+    with Q.Problem.from_circuit(3, gates, 15, p) as prob:
+        assert prob.sde > k
+        assert (t == 19) == (max(abs(v).max() for v in prob.channel()[:2]) > 127)
+        prob.level_begin(k, version, dpb)
+        lists, r = [], None
+        for count in steps:
+            prob.level_walk(count)
+            lists.append(prob.level_merges())
+            prob.level_rewalk()
+            r = prob.level_collect()
+        m = np.concatenate(lists).astype(np.uint64)
+        lengths = [len(x) for x in lists]
+        if len(steps) == 1:
+            assert lengths[0] == queue if walks >= 40000 else 500 < lengths[0] < queue
+        elif not budget:  # far above the line in one launch, far below it in another
+            assert max(lengths) > 2 * 40960 and min(lengths) < 40960 and r["queue_overflow"] == 0
+        assert classified(r) + r["rewalk_carried"] == len(m) and r["false_hash"] == 0
+        if budget:
+            assert r["queue_overflow"] == 0 and r["rewalk_carried"] > 0
+            return
+        a, b = (trails(m[:, i], p.seed, version, L, 63) for i in (0, 1))
+        want = np.zeros(6, np.int64)
+        want[5] = int((a[1] != b[1]).sum())
+        for chunk in range(1, 64):
+            at = (a[1] == chunk) & (b[1] == chunk)
+            if not at.any():
+                continue
+            sa, sb = (torch.from_numpy(v[0][at].view(np.int64)).cuda() for v in (a, b))
+            la, lb = (torch.from_numpy(v[2][at].astype(np.int32)).cuda() for v in (a, b))
+            cls = torch.empty(len(sa), dtype=torch.int32, device="cuda")
+            prob.rewalk(k, chunk, version, sa, la, sb, lb, cls, torch.empty(2 * len(sa), dtype=torch.int64, device="cuda"))
+            want += np.bincount(cls.cpu().numpy(), minlength=6)
+        got = [r["robin_hood"], r["trivial"], r["same_side"], r["claws"] + r["false_hash"], r["no_merge"]]
+        assert got == [want[0], want[1], want[2], want[3] + want[4], want[5]]
