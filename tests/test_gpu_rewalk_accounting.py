@@ -104,3 +104,72 @@ def test_list_lengths_around_the_quads(t, queue, walks, dpb, budget, steps):
             want += np.bincount(cls.cpu().numpy(), minlength=6)
         got = [r["robin_hood"], r["trivial"], r["same_side"], r["claws"] + r["false_hash"], r["no_merge"]]
         assert got == [want[0], want[1], want[2], want[3] + want[4], want[5]]
+
+
+def job(n, t, seed, layout, dpb):
+    """A problem whose ladder starts at its T-count's level t, where a few
+    rounds find no claw, with states so short that trails meet all the time."""
+    for s in range(seed, seed + 40):
+        prob = Q.Problem.from_circuit(n, W.seeded_target(n, t, s)[0], 7, Q.default_params(
+            n, c_layout=layout, theta_policy=0, dp_bits=dpb, exhaustive_log2=0, version_factor=0,
+            state_bits=25 if n == 4 else 22))
+        if prob.sde == t:
+            return prob
+        prob.close()
+    raise AssertionError("no target with this denominator exponent")
+
+
+# (n, T-count, layout of C^, -log2 theta) of every job: a CTA for one job alone
+# and shares that meet several, on the engine and on quads, trails of different
+# lengths, jobs of the general kernels beside them, two qubit counts together
+@pytest.mark.parametrize("walks,steps,jobs", [
+    (2048, 64, [(4, 7, 0, 1)]),
+    (1024, 40, [(4, 7, 0, 1), (4, 6, 0, 2), (4, 7, 0, 4)] * 3),
+    (256, 40, [(4, 7, 0, 1), (4, 6, 0, 3)] * 25),
+    (1024, 24, [(4, 7, 0, 1), (4, 7, 1, 1), (4, 6, 0, 2), (4, 6, 1, 2)] * 2),
+    (2048, 20, [(3, 7, 0, 1), (3, 6, 0, 2), (3, 7, 0, 4)] * 2),
+    (512, 20, [(3, 7, 0, 1), (3, 6, 0, 3), (3, 7, 0, 2)] * 18),
+    (512, 32, [(3, 7, 0, 1), (3, 7, 1, 1), (4, 7, 0, 2)] * 8),
+    (80, 60, [(3, 7, 0, 1), (4, 7, 0, 1)] * 60),
+])
+def test_batched_rewalks_classify_every_merge_once(walks, steps, jobs):
+    probs = [job(n, t, 300 + 50 * i, layout, dpb) for i, (n, t, layout, dpb) in enumerate(jobs)]
+    bp = Q.default_batch_params(max_jobs=len(jobs), walks_per_job=walks, steps_per_round=steps, table_log2=16,
+                                queue_capacity=1 << 16, rewalk_budget=0)
+    searching = merges = 0
+    with Q.Batch(bp) as batch:
+        ids = [batch.add(p) for p in probs]
+        for _ in range(4):
+            batch.round()
+            for j, (n, t, layout, dpb) in zip(ids, jobs):
+                r = batch.poll(j)
+                assert r["queue_overflow"] == 0 and r["error"] == 0
+                if r["status"] == Q.SEARCHING:  # else the host's check of candidates ended at a claw
+                    assert classified(r) == r["merges"], (n, t, layout, dpb)
+                    assert r["steps"] == r["launches"] * walks * steps
+                    searching += 1
+                    merges += r["merges"]
+    for p in probs:
+        p.close()
+    assert searching > 2 * len(jobs) and merges > 100
+
+
+def test_the_smallest_jobs_stay_within_their_buffers():
+    """Jobs of 16 walks whose first level has fewer points than a warp's walks
+    take steps for: no more walks than the job has, beside jobs of the next
+    kernel class."""
+    jobs = [(2, 2, 1)] * 12 + [(3, 5, 1)] * 4 + [(2, 2, 0)] * 12
+    probs = [Q.Problem.from_circuit(n, W.seeded_target(n, t, 20 + i)[0], 9, Q.default_params(
+        n, c_layout=layout, exhaustive_log2=0)) for i, (n, t, layout) in enumerate(jobs)]
+    with Q.Batch(Q.default_batch_params(max_jobs=len(jobs), walks_per_job=16, table_log2=10)) as batch:
+        ids = [batch.add(p) for p in probs]
+        for _ in range(6):
+            before = [batch.poll(j) for j in ids]
+            batch.round()
+            for a, b in zip(before, (batch.poll(j) for j in ids)):
+                assert b["error"] == 0 and b["steps"] - a["steps"] <= 16 * 64
+                assert b["status"] in (Q.SEARCHING, Q.FOUND)
+                if a["status"] == Q.SEARCHING:
+                    assert b["steps"] > a["steps"] or b["status"] == Q.FOUND
+    for p in probs:
+        p.close()
