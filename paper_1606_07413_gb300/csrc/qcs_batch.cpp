@@ -538,7 +538,10 @@ uint64_t qcs_batch_job_bytes(const qcs_batch *B, const qcs_problem *P)
 {
     if (!B || !P) return 0;
     const size_t D = (size_t)P->D;
-    return job_bytes(B->bp) + D * D * sizeof(uint2) + D * sizeof(uint2) + D * 2 * 8 * sizeof(uint32_t);
+    size_t matrices = D * D * sizeof(uint2) + D * sizeof(uint2) + D * 2 * 8 * sizeof(uint32_t);
+    if (P->dCq) matrices += D * D * 2 * sizeof(int8_t);
+    if (P->dCm) matrices += D * D * 2 * sizeof(uint16_t);
+    return job_bytes(B->bp) + matrices;
 }
 
 int qcs_batch_add(qcs_batch *B, qcs_problem *P, int *job)
