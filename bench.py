@@ -14,8 +14,9 @@ value   = walk steps per second over the timed steps (all ranks).
 e2e     = the same metric through the public API (problem creation from the
           host gate list, qcs_run_walks, qcs_poll_collisions), with the bytes
           the library reports it copied each way.
-Also reported: the roofline of the dominant kernel (contraction multiply-adds
-against twice the measured dp4a rate, and issue slots from its ncu record),
+Also reported: the roofline of the dominant kernel (the contraction against
+the measured tensor rate, or twice the dp4a rate in the other launch shapes,
+and issue slots from its ncu record),
 the time to the optimal T-count of configurations 1-3 by the collision walk
 alone and by the exhaustive pass, the n = 3 level-5 record, the batched and
 serving workloads, and the CPU oracle timed on the host cores.
@@ -75,7 +76,7 @@ def parse():
                     help="walk the headline level sharded by distinguished-point owner even on one rank "
                          "(the form N > 1 ranks always use; under torchrun)")
     ap.add_argument("--shape", type=int, default=0, help="launch shape of the --level-only walk kernel")
-    ap.add_argument("--c-layout", type=int, default=0, help="C^ layout of the --level-only walk (0 int8, 1 words)")
+    ap.add_argument("--c-layout", type=int, default=0, help="C^ layout of the --level-only walk (0 operand and int8, 1 words)")
     ap.add_argument("--theta-shapes", action="store_true",
                     help="only time one n = 4 level-7 walk launch (2^20 walks x 16 steps) of launch shapes 0 "
                          "and 3 at several distinguished fractions, print its JSON and exit")
@@ -116,13 +117,13 @@ def workload_config(c, k=None, steps=None, rewalk_budget=None):
 # the steps, plus 32 bytes per distinguished point (0.5 MB at the headline's
 # 64 steps), so the figure stands for the headline launch.
 WALK_NCU = {
-    "k_walks<4,3>": {"source_sha256_16": "aa142ca1f214460b", "dram_bytes_per_launch": 34704640,
+    "k_walks<4,3>": {"source_sha256_16": "ec00a3f5b0904296", "dram_bytes_per_launch": 35069440,
                      "warp_inst_per_step": 582.3},
-    "k_walks<4,0>": {"source_sha256_16": "aa142ca1f214460b", "dram_bytes_per_launch": 34991872,
+    "k_walks<4,0>": {"source_sha256_16": "ec00a3f5b0904296", "dram_bytes_per_launch": 35166080,
                      "warp_inst_per_step": 1935.6},
     # n = 3, level 5: `bench.py --level-only n3_level5 --steps 2`, one launch of 2^16 walks x 512 steps,
     # the launch of the n3_level5 record (profiles/k_walks_n3_level5_walks65536.md)
-    "k_walks<3,0>": {"source_sha256_16": "aa142ca1f214460b", "dram_bytes_per_launch": 2203392,
+    "k_walks<3,0>": {"source_sha256_16": "ec00a3f5b0904296", "dram_bytes_per_launch": 2208768,
                      "warp_inst_per_step": 145.2},
 }
 
@@ -226,6 +227,14 @@ def walk_roofline(kernel, n, w_steps, steps, walk_s, launches, dp4a_per_s, clock
                 "traffic": traffic, "traffic_unit": "bytes per launch", "hbm": hbm, "issue_slots": issue,
                 "algorithmic_ops": f"2*d^2 = {2 * d * d} 16-bit-weight multiply-adds per W-side walk step, "
                                    "each two f16 byte-plane multiply-adds (4 flops) on the tensor cores"}
+    if kernel == "k_walks<3,0>" and hmma_per_s:
+        # eight walks to a warp (2^16 walks): the contraction is mma.sync on f16 byte planes
+        return {"bound": "tensor", "unit": "G multiply-adds/s", "kernel": kernel,
+                "achieved": 2 * achieved / 1e9, "peak": hmma_per_s / 1e9, "frac": 2 * achieved / hmma_per_s,
+                "peak_source": "measured mma.sync m16n8k16 f16 -> f32 rate (qcs_peak_hmma, this run)",
+                "traffic": traffic, "traffic_unit": "bytes per launch", "hbm": hbm, "issue_slots": issue,
+                "algorithmic_ops": f"2*d^2 = {2 * d * d} 16-bit-weight multiply-adds per W-side walk step, "
+                                   "each two f16 byte-plane multiply-adds; issue slots bound the kernel"}
     return {"bound": "alu", "unit": "Gop/s", "kernel": kernel,
             "achieved": achieved / 1e9, "peak": peak / 1e9, "frac": achieved / peak,
             "traffic": traffic, "traffic_unit": "bytes per launch", "hbm": hbm, "issue_slots": issue,
@@ -467,7 +476,8 @@ def run_batched(Q, W, torch, stream, n_targets=256, mac_peak=None, min_seconds=1
         "identical_work": fev == fev_one,
         "contraction_ops_per_s_batched": imad / bs,
         "contraction_alu_frac_batched": (imad / bs / mac_peak) if mac_peak else None,
-        "alu_peak_note": "contraction multiply-adds of all jobs against twice the measured dp4a rate",
+        "alu_peak_note": "contraction multiply-adds of all jobs against twice the measured dp4a rate: a common scale, "
+                         "not a bound (jobs on the tensor-core kernels contract in f16)",
         "found": len(tts), "time_to_tcount_p50_s": q(0.5), "time_to_tcount_p99_s": q(0.99),
         "graph": "each batched round is one CUDA-graph replay",
     }
@@ -868,7 +878,7 @@ def run_ours(args):
                 "config": workload_config(c2, 5, 512, 0), "walk_steps_per_s": st2 / (sum(s2) / 1e3),
                 "ms_per_step": sum(s2) / len(s2),
                 "roofline": walk_roofline("k_walks<3,0>", 3, q1["w_steps"] - q0["w_steps"], st2, sum(w2) / 1e3, 20,
-                                          dp4a_per_s, clk.get("sm_mhz"), num_sms)}
+                                          dp4a_per_s, clk.get("sm_mhz"), num_sms, hmma_per_s)}
             batched = run_batched(Q, W, torch, stream, mac_peak=2 * dp4a_per_s)
             extra.update({
                 "batched": batched,
@@ -891,7 +901,8 @@ def run_ours(args):
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "int32",
             "data": "synthetic (seeded target C0.R(P7)..R(P1), n=4)",
             "config": dict(workload_config(c), launch_shape=Q.launch_shapes(c["n"])[shape["launch_shape"]],
-                           c_layout=["int8 byte quads (dp4a)", "32-bit words (IMAD)"][shape["c_layout"]]),
+                           c_layout="32-bit words (IMAD)" if shape["c_layout"] else
+                           "f16 operand (tcgen05.mma)" if shape["launch_shape"] == 3 else "int8 byte quads (dp4a)"),
             "autotuned_level_shape": shape_trials, "roofline": roof, "cpu_baseline": cpu_base, "e2e": e2e, "clocks": clk,
             "gpu_launches": (5 if sharded else 2) * args.steps, "wall_s": wall,
             "step_split_ms": dict(step_split or {}, note="per bench step: walk kernel; re-walk kernel and the "

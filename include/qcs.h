@@ -96,7 +96,7 @@ extern "C" {
 typedef struct qcs_params {
     int32_t state_bits;       /* L, 32..64 */
     int32_t dp_bits;          /* d_theta, theta = 2^-d_theta (Sec. 3), 1 .. L-1 */
-    int32_t walks;            /* concurrent walks (one lane group each: min(32, 4^n) lanes) */
+    int32_t walks;            /* concurrent walks */
     int32_t table_log2;       /* distinguished-point table holds 2^table_log2 slots (16 B each) */
     int32_t steps_per_launch; /* walk steps each walk advances per kernel launch */
     int32_t max_trail_factor; /* a trail is abandoned after max_trail_factor * 2^d_theta steps */
@@ -121,9 +121,11 @@ typedef struct qcs_params {
                                  0, C^'s numerators are at most 2048 and its columns' absolute sums
                                  at most 16448 (any C^ up to denominator exponent 19); otherwise it
                                  runs shape 0 */
-    int32_t c_layout;         /* device layout of C^ for the W side's contraction (n >= 3): 0 = signed
-                                 byte quads when every entry fits in int8 (dp4a), else 32-bit words;
-                                 1 = 32-bit words always (IMAD).  Results do not depend on it */
+    int32_t c_layout;         /* device layout of C^ for the W side's contraction (n >= 2): 0 = the
+                                 tensor-core kernels' operand where C^ suits it (see launch_shape), and
+                                 for the other kernels, at n >= 3, signed byte quads when every entry
+                                 fits in int8 (dp4a), else 32-bit words; 1 = 32-bit words alone (IMAD),
+                                 no tensor-core kernel.  Results do not depend on it */
     int32_t rewalk_budget;    /* evaluations of f one re-walk of a merge (Sec. 3, Fig. 2) may take per
                                  launch; an unfinished re-walk is carried to the next launch of the same
                                  level and function version (up to queue_capacity of them; more are
@@ -172,9 +174,14 @@ typedef struct qcs_problem qcs_problem;
  * of shapes (>= 1) and fills, for shape i < max_shapes, warps[i] (warps per
  * CTA of the level walk, each warp evaluating 32 / min(32, 4^n) walks; at
  * n = 4, shape 3 is the tensor-core engine: 24 warps evaluating one walk of
- * each of three sets, and 4 warps for the products and the walks' bookkeeping) and min_blocks[i] (the
- * resident CTAs per SM the kernel is compiled for, capping its registers at
- * 65536 / (32 warps[i] min_blocks[i])).  Either pointer may be NULL.
+ * each of three sets, and 4 warps for the products and the walks'
+ * bookkeeping) and min_blocks[i] (the resident CTAs per SM the kernel is
+ * compiled for, capping its registers at 65536 / (32 warps[i]
+ * min_blocks[i])).  At n = 2 and 3 the figures of shape 0 are those of the
+ * kernel with a lane group to a walk; where C^ suits the tensor cores
+ * (c_layout 0) and a launch has walks enough (n = 2: any number, n = 3: 6144,
+ * or 2048 where C^ does not fit int8), shape 0 runs eight walks to a warp, in
+ * one CTA per SM of up to 24 (n = 2) or 18 warps.  Either pointer may be NULL.
  * QCS_ERR_ARG if n is not in 1..4. */
 QCS_API int qcs_launch_shapes(int n_qubits, int32_t *warps, int32_t *min_blocks, int max_shapes);
 

@@ -9,8 +9,9 @@ every candidate setting and keeps the best, in two stages:
    of GPU time, ties broken by walk steps per second;
 2. for each qubit count n >= 3 in the sample, the walk kernel's launch shape
    (warps per CTA and resident CTAs per SM, ``qcs_launch_shapes``) together
-   with the device layout of C^ (``c_layout``: int8 byte quads for dp4a or
-   32-bit words for IMAD), by the time the same rounds take.  Shapes and
+   with the device layout of C^ (``c_layout``: 0 with the tensor-core operand
+   and int8 byte quads, 1 with 32-bit words alone), by the time the same
+   rounds take.  (At n = 4 shapes 0 and 3 run the same kernels in a batch.)  Shapes and
    layouts change neither the walks nor their results, so every trial of this
    stage does identical work and the fastest wins.
 

@@ -287,7 +287,11 @@ int begin_level(qcs_batch *B, Job &j, int slot)
 
 // The kernels a job runs in: the tensor-core ones where C^ suits them and the
 // batch asks for its qubit count's default shape (or, n = 4, for theirs).  Few
-// n = 3 walks (walks3: of all jobs this round) are left to the others.
+// n = 3 walks (walks3: of all jobs this round) are left to the others; one line
+// for all jobs, that of C^ in int8, which nearly every job's fits.  It holds for
+// short rounds too (n = 3 alone, 512 walks a job, us a round, quads / the best
+// other shape: 16 steps, 12 jobs 254 / 283, 24 jobs 344 / 350, 85 jobs 644 / 985,
+// 256 jobs 1455 / 2314; 64 steps, 24 jobs 721 / 1198).
 int job_class(const qcs_batch *B, const Job &j, uint64_t walks3)
 {
     const int n = j.P->n, shape = B->bp.launch_shape[n - 1];

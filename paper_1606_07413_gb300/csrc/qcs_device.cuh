@@ -97,8 +97,7 @@ __device__ __forceinline__ void new_trail(WalkState &st, uint32_t walk, const Le
 }
 
 // per-walk-group tallies, added to the job's counters by the group's first
-// lane (the tensor-core kernel keeps them in 32 bits and flushes them before
-// they could overflow)
+// lane (the quads keep theirs in 32 bits: a walk's are at most a launch's steps)
 template <typename T>
 struct TallyOf {
     T steps = 0, w = 0, dp = 0, ab = 0, evicted = 0, duplicate = 0, pairs = 0;

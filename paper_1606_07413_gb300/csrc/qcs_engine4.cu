@@ -22,7 +22,9 @@
 // tcgen05.mma with A in tensor memory, 40 in shared memory, whatever N), E
 // (700), control (800).  With 48 points in flight (two sets of 24, or three
 // of 16) that chain was the bound; with 72 it is issue: 75 % active at 582
-// warp instructions a point, half of them the 255 column finalisers.
+// warp instructions a point.  The adjoint stages are the largest piece (88
+// each, and at level 7 a point has 2.5 on average after the table's: 220), then
+// the 255 column finalisers (18 for 32 columns: 144).
 // 2^20 walks x 16 steps at level 7: 11.1 ms (1.51 G steps/s); two sets and
 // 16 workers 14.9 ms; with mma.sync (12 stage and 8 MMA warps, C^'s fragments
 // through tcgen05.ld, the rows through ldmatrix, 1073 instructions) 26.7 ms.
@@ -68,7 +70,7 @@ constexpr int kMmaWarp = kWorkers, kCtlWarp = kWorkers + 1; // control warps kCt
 constexpr int kWarps = kWorkers + 1 + kSets, kThreads = 32 * kWarps;
 constexpr int kN = 2 * kPairs;              // columns of D per set and half
 constexpr int kTmemK = 8;                   // K-blocks of C^'s second half held in tensor memory
-constexpr int kDcol = 256 + 8 * kTmemK;     // tensor-memory column of D (set X, half h: + 96 X + 48 h)
+constexpr int kDcol = 256 + 8 * kTmemK;     // tensor-memory column of D (set X, half h: + 2 kN X + kN h)
 static_assert(kDcol + kSets * 2 * kN <= 512, "tensor memory");
 constexpr uint32_t kInvalid = 1u << 31;
 constexpr int kTaskWalks = 24; // of a batch: a third of the slots, for even shares
@@ -83,7 +85,7 @@ struct alignas(16) Job {
 };
 // shared memory
 constexpr size_t off_A = 0;                                        // C^, second half, K-blocks 8..31: 6 chunks of 64 K
-constexpr size_t off_B = off_A + 6 * 16384;                        // [set]: 8 chunks of 64 K x 48 rows
+constexpr size_t off_B = off_A + 6 * 16384;                        // [set]: 8 chunks of 64 K x kN rows
 constexpr size_t off_job = off_B + (size_t)kSets * 8 * kN * 128;   // Job [set][slot]
 constexpr size_t off_wb = off_job + sizeof(Job) * kSets * kSet;    // HashBase [set][row pair]
 constexpr int kParts = 16; // partial column sums of a W point
@@ -91,7 +93,7 @@ constexpr size_t off_part = off_wb + sizeof(HashBase) * kSets * kPairs; // u64 [
 constexpr size_t off_vsum = off_part + kParts * sizeof(uint64_t) * kSets * kPairs; // u64 [set][slot]
 constexpr size_t off_chunk = off_vsum + sizeof(uint64_t) * kSets * kSet; // HashBase [chunk]
 constexpr size_t off_stage = off_chunk + sizeof(HashBase) * 256;   // stage table: u32 [side][code % 64][lane]
-constexpr size_t off_nw = off_stage + 2 * 64 * 32 * sizeof(uint32_t);                  // u32 [set]: W points; [2 + set]: the set is done
+constexpr size_t off_nw = off_stage + 2 * 64 * 32 * sizeof(uint32_t);                  // u32 [set]: W points; [4 + set]: the set is done
 constexpr size_t off_bar = off_nw + 32;                            // mbarriers: jobs, rows, product, sums [set]
 constexpr size_t off_tmem = off_bar + 4 * kSets * sizeof(uint64_t);
 constexpr size_t smem_bytes = off_tmem + 16;

@@ -179,7 +179,7 @@ enum Counter {
     C_CANDS,       // claw candidates found by the re-walk (including overflowed ones)
     C_RSTEPS,      // walk steps taken by the re-walk (evaluations of f)
     C_CLS0,        // re-walk classes QCS_MERGE_ROBIN_HOOD .. QCS_MERGE_NO_MERGE at C_CLS0 + class
-    C_STALLED = C_CLS0 + 6, // warps of the tensor-core walk whose bounded wait ran out (low word)
+    C_STALLED = C_CLS0 + 6, // CTAs of the n = 4 engine that gave up on a bounded wait, in a batch once for every job left (low word)
     C_NCOUNTERS
 };
 
@@ -220,9 +220,8 @@ struct WalkLaunch {
     // (zeroed before the launch); null: a fixed stride (the batched re-walk)
     uint32_t *rw_next;
     uint32_t rw_last; // merges of the level's last re-walk (0: unknown), for the choice of this one's kernels
-    // the tensor-core walk (n = 4, launch shape 3) counts here the warps
-    // whose bounded wait ran out (the launch's results are then invalid);
-    // it refuses to launch without it
+    // the n = 4 engine counts here the CTAs that gave up on a bounded wait
+    // (the launch's results are then invalid); it refuses to launch without it
     uint32_t *stall;
 };
 

@@ -1042,7 +1042,7 @@ cudaError_t walks_batch_n(int shape, const BatchArgs &a, cudaStream_t s)
     case 1: if constexpr (shape_count(NQ) > 1) return walks_batch_ns<NQ, 1>(a, s); break;
     case 2: if constexpr (shape_count(NQ) > 2) return walks_batch_ns<NQ, 2>(a, s); break;
     case 3:
-        if constexpr (NQ == 4) return walks_batch_ns<4, 0>(a, s); // no batched tensor-core form
+        if constexpr (NQ == 4) return walks_batch_ns<4, 0>(a, s); // the jobs that the engine does not take
         else if constexpr (shape_count(NQ) > 3) return walks_batch_ns<NQ, 3>(a, s);
         break;
     }
